@@ -51,26 +51,26 @@ def _case(kind, job, sets=1, fail_lo=1, fail_hi=1, micro=0, cost=0, order=0, sha
 def listed():
     return [
         # a failure is being handled now: one set, plan wanted as soon as possible
-        dict(_case("one", "8dev"), name="one failure, 8 devices"),
-        dict(_case("one", "32dev", fail_lo=2, fail_hi=2), name="one failure, 32 devices"),
+        dict(_case("one", "8dev"), name="one failure 8 devices"),
+        dict(_case("one", "32dev", fail_lo=2, fail_hi=2), name="one failure 32 devices"),
         # deep pipelines, most compositions rejected by memory; integer nanoseconds
-        dict(_case("one", "64dev", fail_lo=3, fail_hi=3, cost=1), name="one failure, 64 devices, int64"),
+        dict(_case("one", "64dev", fail_lo=3, fail_hi=3, cost=1), name="one failure 64 devices int64"),
         # a node of eight lost from the largest job
-        dict(_case("one", "256dev", fail_lo=8, fail_hi=8), name="one failure, 256 devices"),
+        dict(_case("one", "256dev", fail_lo=8, fail_hi=8), name="one failure 256 devices"),
         # the step-by-step interface: enumerate the three spaces, select, decode the layer cuts
-        dict(_case("select", "32dev", fail_lo=1, fail_hi=1), name="enumerate and select, 32 devices"),
+        dict(_case("select", "32dev", fail_lo=1, fail_hi=1), name="enumerate and select 32 devices"),
         # plans for many potential failure sets, computed ahead of time
-        dict(_case("batch", "32dev", sets=2576, fail_lo=1, fail_hi=4), name="batch 2576, 32 devices"),
-        dict(_case("batch", "64dev", sets=64, fail_lo=1, fail_hi=8, cost=1), name="batch 64, 64 devices, int64"),
-        dict(_case("batch", "256dev", sets=1024, fail_lo=1, fail_hi=16), name="batch 1024, 256 devices"),
+        dict(_case("batch", "32dev", sets=2576, fail_lo=1, fail_hi=4), name="batch 2576 32 devices"),
+        dict(_case("batch", "64dev", sets=64, fail_lo=1, fail_hi=8, cost=1), name="batch 64 64 devices int64"),
+        dict(_case("batch", "256dev", sets=1024, fail_lo=1, fail_hi=16), name="batch 1024 256 devices"),
         # the same with identical searches shared, as the plan cache does
-        dict(_case("batch", "256dev", sets=1000, fail_lo=1, fail_hi=16, sharing=True), name="shared batch 1000, 256 devices"),
+        dict(_case("batch", "256dev", sets=1000, fail_lo=1, fail_hi=16, sharing=True), name="shared batch 1000 256 devices"),
         # the second execution order
-        dict(_case("batch", "32dev", sets=515, fail_lo=1, fail_hi=4, order=1), name="batch 515, 32 devices, all-forward"),
+        dict(_case("batch", "32dev", sets=515, fail_lo=1, fail_hi=4, order=1), name="batch 515 32 devices all-forward"),
         # transition time in the objective: shortlist, migrations, synchronisation rounds
-        dict(_case("objective", "256dev", sets=64, fail_lo=1, fail_hi=8, rounds=1), name="objective 64, 256 devices"),
+        dict(_case("objective", "256dev", sets=64, fail_lo=1, fail_hi=8, rounds=1), name="objective 64 256 devices"),
         # cost and feasibility of many single candidates, by index
-        dict(_case("evaluate", "256dev", fail_lo=3, fail_hi=3, count=200_000, indexed=True), name="evaluate 200000, 256 devices"),
+        dict(_case("evaluate", "256dev", fail_lo=3, fail_hi=3, count=200_000, indexed=True), name="evaluate 200000 256 devices"),
     ]
 
 
