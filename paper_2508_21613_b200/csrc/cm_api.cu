@@ -1147,21 +1147,8 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
         launches += (bd.n_red_blocks && bd.max_red_per_scen > 1) ? 2 : 1;
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
         if (bt.n_tiles) {
-            bool deep = false;
-            for (const TSeg &g : bt.tseg) deep = deep || (g.S > kRegStagesMax && g.K > 0);
-            // few winners (a failure handled on its own): the lock-step kernel completes every deep
-            // pipeline in one launch; many: one plan per lane, a kernel per depth
-            const bool by_warp = deep && (uint64_t)bt.B * bt.dp_max <= kWarpTieMaxPairs;
-            CM_CUDA(ctx, launch_cost_pass2(tb, bd, st, by_warp));
+            CM_CUDA(ctx, launch_tiebreak(tb, bd, st));
             ++launches;
-            if (by_warp) {
-                CM_CUDA(ctx, launch_tiebreak_warp(tb, bd, st));
-                ++launches;
-            } else if (deep) {
-                uint64_t stage_mask = 0;
-                for (const TSeg &g : bt.tseg) stage_mask |= 1ull << (g.S & 63);
-                CM_CUDA(ctx, launch_tiebreak_wide(tb, bd, stage_mask, st, &ctx->side, &launches));
-            }
         }
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[5], st));
     }
@@ -1957,16 +1944,13 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
     ++obj_launches;
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[1], st));
     if (bt.n_tiles) {
-        // the tie-break kernels complete every shortlisted pair exactly as they complete the winner
+        // the tie-break kernel completes every shortlisted pair exactly as it completes the winner
         BatchDev sd = bd;
         sd.winner = od.short_win;
         sd.kappa_sel = od.short_kappa;
         sd.B = (int32_t)slots;
-        CM_CUDA(ctx, launch_cost_pass2(tb, sd, st));
+        CM_CUDA(ctx, launch_tiebreak(tb, sd, st));
         ++obj_launches;
-        uint64_t stage_mask = 0;
-        for (const TSeg &g : bt.tseg) stage_mask |= 1ull << (g.S & 63);
-        CM_CUDA(ctx, launch_tiebreak_wide(tb, sd, stage_mask, st, &ctx->side, &obj_launches));
     }
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[2], st));
     CM_CUDA(ctx, launch_plan_matching(tb, bd, od, st));

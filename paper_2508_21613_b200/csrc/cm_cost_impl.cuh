@@ -647,87 +647,4 @@ cudaError_t launch_deep_range(const Tables &t, const BatchDev &b, const LaunchCl
     return deep_dispatch<T, LO, HI>(t, b, c, st);
 }
 
-// ----------------------------------------------------------------------------------
-// Tie-break pass for the winners' deep pipelines (17..48 stages): the lowest layer
-// composition that is feasible with cost <= T*.  Same grid as the generic tie-break
-// kernel -- x = (scenario, pipeline), y = tiles of kChunk compositions -- one launch per
-// stage count; CTAs whose winner segment has another depth leave at once.
-// ----------------------------------------------------------------------------------
-template <typename T, int S>
-__global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_tiebreak_wide_kernel(Tables tb, BatchDev bd) {
-    __shared__ SProf<T> sp;
-    __shared__ uint64_t red[kChunk / 32];
-    __shared__ SegView g;
-    __shared__ uint64_t found_so_far;
-    extern __shared__ __align__(16) unsigned char dyn[];
-    const uint32_t b = blockIdx.x / bd.dp_max, p = blockIdx.x % bd.dp_max;
-    const Winner &w = bd.winner[b];
-    if (w.cost_bits >= inf_bits<T>() || p >= w.dp) return;            // uniform over the CTA
-    if (bd.tseg[w.seg[p]].S != S) return;
-    stage_profile(sp, tb);
-    FB<T> *fcol = reinterpret_cast<FB<T> *>(dyn) + threadIdx.x;
-    T *xcol = reinterpret_cast<T *>(dyn + sizeof(FB<T>) * S * kChunk) + threadIdx.x;
-    uint64_t *slot = &bd.kappa_sel[b * kMaxP + p];
-    for (uint64_t tile = blockIdx.y; tile < bd.max_tiles_per_seg; tile += gridDim.y) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            g = seg_view(bd, w.scen, w.seg[p]);
-            found_so_far = *(volatile uint64_t *)slot;
-        }
-        __syncthreads();
-        const uint64_t count = walk_count(g);
-        const uint64_t first = tile * kChunk;
-        // uniform: later tiles hold higher compositions than one already found
-        if (first >= count || found_so_far <= walk_kappa(bd.feas, g.feas_first, first)) break;
-        uint64_t hit = ~0ull;
-        if (first + threadIdx.x < count) {
-            const uint64_t kappa = walk_kappa(bd.feas, g.feas_first, first + threadIdx.x);
-            T cost;
-            if (plan_cost_wide_lane<T, S>(sp, tb, bd.layer_mode, g, kappa, fcol, xcol, cost) &&
-                Num<T>::bits(cost) <= w.cost_bits)
-                hit = kappa;
-        }
-        hit = warp_min_u64(hit);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = hit;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int q = 0; q < kChunk / 32; ++q) hit = red[q] < hit ? red[q] : hit;
-            if (hit != ~0ull) atomicMin((unsigned long long *)slot, (unsigned long long)hit);
-            const uint64_t n = count - first < (uint64_t)kChunk ? count - first : (uint64_t)kChunk;
-            atomicAdd(&bd.counters[1], (unsigned long long)n);
-        }
-    }
-}
-
-template <typename T, int S>
-static cudaError_t launch_tiebreak_wide_one(const Tables &t, const BatchDev &b, cudaStream_t st) {
-    constexpr size_t smem = wide_smem_bytes<S, false, T>();
-    static std::atomic<uint64_t> configured{0};   // as in launch_wide_one
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 64 || !((configured.load(std::memory_order_acquire) >> dev) & 1ull)) {
-        cudaError_t e = cudaFuncSetAttribute(cm_tiebreak_wide_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
-    }
-    const uint64_t nx = (uint64_t)b.B * b.dp_max;
-    if (nx >= (1ull << 31)) return cudaErrorInvalidConfiguration;
-    dim3 grid((unsigned)nx, tiebreak_grid_y(nx, b.max_tiles_per_seg), 1);
-    cm_tiebreak_wide_kernel<T, S><<<grid, kChunk, smem, st>>>(t, b);
-    return cudaGetLastError();
-}
-
-template <typename T, int S, int HI>
-static cudaError_t tiebreak_dispatch(const Tables &t, const BatchDev &b, int stages, cudaStream_t st) {
-    if constexpr (S <= kWideStagesMax) {   // deeper winners are completed by the generic tie-break kernel
-        if (stages == S) return launch_tiebreak_wide_one<T, S>(t, b, st);
-    }
-    if constexpr (S < HI) return tiebreak_dispatch<T, S + 1, HI>(t, b, stages, st);
-    else return cudaSuccess;
-}
-template <typename T, int LO, int HI>
-cudaError_t launch_tiebreak_range(const Tables &t, const BatchDev &b, int S, cudaStream_t st) {
-    return tiebreak_dispatch<T, LO, HI>(t, b, S, st);
-}
-
 }  // namespace cm

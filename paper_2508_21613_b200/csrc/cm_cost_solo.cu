@@ -77,40 +77,11 @@ __global__ void __launch_bounds__(kChunk) cm_cost_warp_kernel(Tables tb, BatchDe
     if (seg_local < bk.n_seg && m >= 1) {                       // warp-uniform
         const uint64_t kappa = walk_kappa(bd.feas, bk.feas_first, plan - seg_local * bk.count);
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
-        uint8_t *cuts = cuts_s[warp];
-        CutWalker cw;
-        bool ok = make_walker(cw, tb, bd.layer_mode, sp.L, S, kappa, g.K, tb.mm_slot(S, m));
-        if (ok) {
-            int lo = 0;
-            for (int i = 0; i < S; ++i) {
-                const int hi = cw.next();
-                ok = ok && hi > lo;
-                if (lane == 0) cuts[i + 1] = (uint8_t)hi;
-                lo = hi;
-            }
-            if (lane == 0) cuts[0] = 0;
-        }
-        __syncwarp();
-        long long g_max = 0;
-        if (ok)
-            for (int i = lane; i < S; i += 32) {
-                const int lo = cuts[i], hi = cuts[i + 1];
-                ok = ok && stage_fits(sp.PS[hi] - sp.PS[lo], sp.PA[hi] - sp.PA[lo], i, S, m, sp.cap, sp.sched);
-                const long long gb = sp.PP[hi] - sp.PP[lo];
-                g_max = gb > g_max ? gb : g_max;
-            }
-        ok = __all_sync(0xffffffffu, ok);
-        if (ok) {
-            for (int o = 16; o > 0; o >>= 1) {
-                const long long og = __shfl_xor_sync(0xffffffffu, g_max, o);
-                g_max = og > g_max ? og : g_max;
-            }
-            const T t = warp_pipe_time<T>(sp, cuts, S, m, g.tier, lane);
-            if (lane == 0) {
-                const uint64_t bits = Num<T>::bits(t + Num<T>::sync(g_max, g.n_sync, sp.bw_sync, sp.intval));
-                if (bits < bd.seg_best[g.row]) atomicMin((unsigned long long *)&bd.seg_best[g.row], (unsigned long long)bits);
-                my_cells = one_plan(2ull * S * m);
-            }
+        T cost;
+        if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, kappa, cuts_s[warp], cost) && lane == 0) {
+            const uint64_t bits = Num<T>::bits(cost);
+            if (bits < bd.seg_best[g.row]) atomicMin((unsigned long long *)&bd.seg_best[g.row], (unsigned long long)bits);
+            my_cells = one_plan(2ull * S * m);
         }
     }
     count_cells(&bd.counters[0], my_cells, cells_w);

@@ -14,7 +14,7 @@ constexpr int kMaxL = CM_MAX_LAYERS;
 constexpr int kMaxS = CM_MAX_STAGES;
 constexpr int kMaxP = CM_MAX_PIPES;
 constexpr int kBinomCols = 64;          // binomial table columns 0..64
-constexpr int kTile = 128;              // layer compositions per CTA in the tie-break kernels
+constexpr int kTile = 128;              // layer compositions per tile of BatchDev::max_tiles_per_seg
 constexpr uint64_t kSat = ~0ull;        // saturated binomial
 
 // Per-layer prefix arrays, built on the device by cm_prefix_kernel and staged into shared
@@ -299,18 +299,6 @@ cudaError_t launch_policies(const Tables &t, const BatchDev &b, int n_dp, cudaSt
 cudaError_t launch_useg_keys(const BatchDev &b, const USegDev &u, cudaStream_t st);   // three launches
 cudaError_t launch_useg_copy(const BatchDev &b, const USegDev &u, cudaStream_t st);
 cudaError_t launch_dup_copy(const BatchDev &b, cudaStream_t st);   // duplicate template segments take their first occurrence's minimum
-// Tiles of a segment that the tie-break kernels take side by side (grid.y); the rest is
-// walked serially inside the CTA.  A single scenario gets every tile its own CTA (lowest
-// latency), a large batch about one CTA per (scenario, pipeline): most of those stop after
-// their first tile anyway, and an idle CTA per tile would cost more than the work.
-inline unsigned tiebreak_grid_y(uint64_t nx, uint32_t max_tiles) {
-    const uint64_t target = 2048;   // CTAs worth launching
-    uint64_t y = nx ? (target + nx - 1) / nx : 1;
-    if (y > max_tiles) y = max_tiles;
-    if (y > 65535) y = 65535;
-    return (unsigned)(y ? y : 1);
-}
-
 // side streams (may be NULL / 0): launch classes are independent of one another, so they are
 // spread over the caller's stream and the side streams and joined again before returning
 constexpr int kSideStreams = 7;
@@ -322,15 +310,7 @@ struct SideStreams {
 cudaError_t launch_cost_pass1(const Tables &t, const BatchDev &b, const LaunchClass *classes, int n_classes,
                               cudaStream_t st, const SideStreams *side, int *launches);
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st);
-// deep_elsewhere: winners' pipelines deeper than kRegStagesMax are completed by another kernel
-// (the per-depth ones, or the lock-step one below), this one leaves them alone
-cudaError_t launch_cost_pass2(const Tables &t, const BatchDev &b, cudaStream_t st, bool deep_elsewhere_all = false);
-// Tie-break pass for few winners (one failure at a time): a warp per layer composition walks the
-// pipeline in lock step, every depth above kRegStagesMax in one launch.
-constexpr uint64_t kWarpTieMaxPairs = 64;   // (scenario, pipeline) pairs up to which the lock-step tie-break is used
-cudaError_t launch_tiebreak_warp(const Tables &t, const BatchDev &b, cudaStream_t st);
-cudaError_t launch_tiebreak_wide(const Tables &t, const BatchDev &b, uint64_t stage_mask, cudaStream_t st,
-                                 const SideStreams *side, int *launches);
+cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);   // cm_bound.cu
 cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st);
 // single_policy < 0: candidates of the dynamic-parallelism segments; otherwise the one
 // candidate of that policy (its cost must already be in pol_cost of scenario 0)

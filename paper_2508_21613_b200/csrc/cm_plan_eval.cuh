@@ -633,4 +633,43 @@ __device__ __forceinline__ bool plan_cost_regs_any(const SProf<T> &sp, const Tab
     }
 }
 
+// Cost of candidate kappa of a segment, a warp walking the pipeline in lock step (two stages per
+// lane); `cuts`: kMaxS + 8 bytes of shared memory of the warp.  Warp-uniform arguments and result.
+template <typename T>
+__device__ __forceinline__ bool warp_plan_cost(const SProf<T> &sp, const Tables &tb, int layer_mode, const SegView &g,
+                                               uint64_t kappa, uint8_t *cuts, T &cost) {
+    const int lane = threadIdx.x & 31, S = g.S, m = g.m;
+    CutWalker cw;
+    bool ok = m >= 1 && make_walker(cw, tb, layer_mode, sp.L, S, kappa, g.K, tb.mm_slot(S, m));
+    __syncwarp();   // nobody reads the cuts of an earlier plan any more
+    if (ok) {
+        int lo = 0;
+        for (int i = 0; i < S; ++i) {
+            const int hi = cw.next();
+            ok = ok && hi > lo;
+            if (lane == 0) cuts[i + 1] = (uint8_t)hi;
+            lo = hi;
+        }
+        if (lane == 0) cuts[0] = 0;
+    }
+    __syncwarp();
+    long long g_max = 0;
+    if (ok)
+        for (int i = lane; i < S; i += 32) {
+            const int lo = cuts[i], hi = cuts[i + 1];
+            ok = ok && stage_fits(sp.PS[hi] - sp.PS[lo], sp.PA[hi] - sp.PA[lo], i, S, m, sp.cap, sp.sched);
+            const long long gb = sp.PP[hi] - sp.PP[lo];
+            g_max = gb > g_max ? gb : g_max;
+        }
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) return false;
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long og = __shfl_xor_sync(0xffffffffu, g_max, o);
+        g_max = og > g_max ? og : g_max;
+    }
+    const T t = warp_pipe_time<T>(sp, cuts, S, m, g.tier, lane);
+    cost = t + Num<T>::sync(g_max, g.n_sync, sp.bw_sync, sp.intval);
+    return true;
+}
+
 }  // namespace cm
