@@ -370,7 +370,7 @@ cm_status cm_set_latency_graphs(cm_ctx *ctx, int on);
  * The first search that meets a new (stages, micro-batches) pair builds its list: one small copy
  * each way, one kernel and a stream synchronisation.  Results are identical either way; candidate
  * indices, cm_evaluate and cm_decode_plan are unaffected; cm_last_stats [0] still counts every
- * enumerated pipeline-plan and [16] those whose recurrence ran.  cm_set_memory_screen(ctx, 0)
+ * enumerated pipeline-plan and [16] those that were decided.  cm_set_memory_screen(ctx, 0)
  * makes batches and spaces built afterwards test every composition inside the search pass. */
 cm_status cm_set_memory_screen(cm_ctx *ctx, int on);
 
@@ -381,7 +381,8 @@ cm_status cm_set_memory_screen(cm_ctx *ctx, int on);
  * round m -- so for pipelines of up to 48 stages with m >= stages one thread evaluates both: the
  * common rounds once, then the two tails (shallow pipelines, up to 16 stages, where a group of
  * them holds enough plans to be worth a launch of its own).  Same operations on the same values: results are
- * bit-identical; cm_last_stats [1] counts the recurrence cells that actually ran.
+ * bit-identical; cm_last_stats [1] counts the shared rounds once.  (A search that is decided by
+ * bounds -- see cm_last_stats [16] -- runs the recurrence on a handful of plans, each on its own.)
  * cm_set_micro_batch_pairs(ctx, 0) makes batches and spaces built afterwards evaluate every
  * segment on its own. */
 cm_status cm_set_micro_batch_pairs(cm_ctx *ctx, int on);
@@ -393,7 +394,7 @@ cm_status cm_set_micro_batch_pairs(cm_ctx *ctx, int on);
  * (Section "Estimator": a pipeline's time and memory are functions of its own stages, links and
  * micro-batches), so its least cost is searched once per scenario and the other strategies take
  * the result.  Results are identical; cm_last_stats [0] still counts every pipeline-plan of the
- * search space, [16] those whose recurrence ran.  cm_set_pipeline_reuse(ctx, 0) makes batches and
+ * search space, [16] those that were decided in their own right.  cm_set_pipeline_reuse(ctx, 0) makes batches and
  * spaces built afterwards search every (strategy, pipeline) on its own. */
 cm_status cm_set_pipeline_reuse(cm_ctx *ctx, int on);
 
@@ -409,11 +410,10 @@ cm_status cm_set_pipeline_reuse(cm_ctx *ctx, int on);
  * the device (one small device->host copy and one synchronisation of the context's stream per
  * prepared batch) and each is searched once (as one half of a micro-batch pair where two distinct
  * pipelines differ only by one micro-batch).  A single failure set searched through the latency
- * path of cm_search_batch has its duplicate pipelines removed on the host when enough work is
- * saved to pay for launching its sequence directly instead of replaying the resident graph.
+ * path of cm_search_batch is searched as without sharing.
  * Results are identical either way; cm_last_stats
  * [0] then counts only the plans of the scenarios that were searched and [16] only the plans
- * whose recurrence ran.  cm_cache_build always shares. */
+ * that were decided in their own right.  cm_cache_build always shares. */
 cm_status cm_set_sharing(cm_ctx *ctx, int on);
 
 /* Device time and work of the objective pass of the last cm_search_objective (HOST out[8]):
@@ -461,8 +461,9 @@ cm_status cm_cache_free(cm_cache *cache);
 
 /* Work counters of the last cm_select / cm_search_batch / cm_batch_search on this
  * context (HOST out[24]):
- *  [0] pipeline-plans evaluated by the search pass   [1] recurrence cells simulated by it
- *      (2 * stages * micro-batches per memory-feasible plan, counted on the device)
+ *  [0] pipeline-plans covered by the search pass   [1] recurrence cells of the plans of [16]
+ *      (2 * stages * micro-batches per plan, a micro-batch pair's shared rounds once): what
+ *      deciding each of them by its recurrence takes; [20] has the cells that ran
  *  [2] pipeline-plans re-evaluated by the tie-break pass   [3] kernels launched
  *  [4] device time of the whole launch sequence, ns (CUDA events on the context's stream)
  *  [5] segments  [6] strategies  [7] micro-batch splits reduced
@@ -470,8 +471,11 @@ cm_status cm_cache_free(cm_cache *cache);
  *  [10] bytes copied device->host   [11] device time of the tie-break kernel(s), ns
  *  [12] launches of the search-pass cost kernel   [13] host time building descriptor tables, ns
  *  [14] host time enqueueing the launch sequence, ns   [15] host time waiting for the stream, ns
- *  [16] pipeline-plans whose recurrence ran, i.e. that are searched in their own right ([19]) and
- *       passed the memory estimator (Section "Estimator", memory estimator)
+ *  [16] pipeline-plans decided in their own right: searched in their own right ([19]) and passed by
+ *       the memory estimator (Section "Estimator", memory estimator).  In a small search each of
+ *       them is decided by its recurrence; a search of more than 2*10^8 recurrence cells computes a
+ *       lower bound on the time of each (a dependency path of the transition equation) and runs the
+ *       recurrence only on the plans whose bound does not exclude them: [21] says on how many
  *  [17] host time spent listing memory-feasible compositions (inside [13]; includes one stream
  *       synchronisation when a new (stages, micro-batches) pair is met), ns
  *  [18] host time packing and uploading the descriptor tables, buffer allocation included, ns
@@ -479,7 +483,8 @@ cm_status cm_cache_free(cm_cache *cache);
  *       that another strategy of the same survivor count has as well and take its result
  *       (cm_set_pipeline_reuse); [19] - [16] were rejected by the memory estimator (with sharing
  *       on, [16] also leaves out what other scenarios' segments already covered)
- *  [20..23] reserved, 0. */
+ *  [20] recurrence cells that ran in the search pass  [21] pipeline-plans whose recurrence ran in it
+ *  [22..23] reserved, 0. */
 cm_status cm_last_stats(const cm_ctx *ctx, uint64_t out[24]);
 
 const char *cm_strerror(cm_status status);

@@ -142,12 +142,14 @@ struct Batch {
     DevBuf<uint32_t> d_urep, d_slot_of, d_ucount;
     DevBuf<uint2> d_useg;
     PinnedVec<uint32_t> ucount_host;
-    // A resident one-scenario batch searched with shared segments keeps its template buckets (the
-    // replayed graph uses them) and lays the shared ones out beside them, per search.
-    const Bucket *bucket_override = nullptr;
-    uint64_t single_cells = 0;            // recurrence cells of the one scenario's search pass, every segment on its own
-    DevBuf<Bucket> d_alt_bucket;
-    PinnedVec<unsigned char> alt_stage;   // slot_of | rep | list | buckets, staged for the copies
+    // Bounded search pass (cm_bound.cu): its buckets and its device state.
+    bool bounded = false;
+    bool dense_only = false;              // a list was full: this batch is searched without bounds
+    std::vector<BBucket> bbucket;
+    BoundDev bo{};
+    size_t off_bbucket = 0;
+    DevBuf<SearchWin> d_win;
+    int k_best = 1;                       // (strategy, split) pairs whose step times have to be exact
 };
 
 struct cm_ctx {
@@ -188,6 +190,8 @@ struct cm_ctx {
     size_t feas_used = 0;
     PinnedVec<unsigned char> feas_stage;      // keys, K, offsets out; counts back
     DevBuf<unsigned char> d_feas_stage;
+    DevBuf<uint4> d_bound_list;       // plans the bounded search pass lists for the recurrence
+    bool uniform_p2p = false;         // every stage boundary moves the same bytes
     bool screen = true;               // walk only the listed feasible compositions (cm_set_memory_screen)
     bool dedup = true;                // search a pipeline that several strategies of a survivor count share once (cm_set_pipeline_reuse)
     bool pairs = true;                // one recurrence for a pipeline's m and m+1 micro-batch variants (cm_set_micro_batch_pairs)
@@ -354,10 +358,56 @@ int bucket_kind(bool by_warp, int S, int m, uint64_t n_seg, uint64_t K) {
 
 cm_status layout_buckets(cm_ctx *ctx, Batch &bt, const std::vector<PreBucket> &pre);
 
+cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups);
+
+uint64_t walked(const TSeg &g) { return g.feas_first != kNoFeasList ? (uint64_t)g.feas_count : (g.K ? g.K + 1 : 1); }
+
+// The bounded layout of a batch without shared segments: per template, the segments that are searched
+// in their own right, grouped by (stages, micro-batches, role in the accounting of pairs).
+cm_status build_bound(cm_ctx *ctx, Batch &bt) {
+    std::vector<BBucket> groups;
+    std::vector<uint32_t> idx;
+    for (size_t t = 0; t < bt.tmpl.size(); ++t) {
+        const Tmpl &tp = bt.tmpl[t];
+        if (tp.n_scen == 0) continue;
+        idx.clear();
+        for (uint32_t i = tp.tseg_first; i < tp.tseg_first + tp.n_tseg; ++i)
+            if (bt.tseg_canon[i] == i && bt.tseg[i].m >= 1 && walked(bt.tseg[i]) > 0) idx.push_back(i);
+        std::sort(idx.begin(), idx.end(), [&](uint32_t a, uint32_t b) {
+            const TSeg &x = bt.tseg[a], &y = bt.tseg[b];
+            return x.S != y.S ? x.S > y.S : x.m != y.m ? x.m < y.m : bt.role[a] != bt.role[b] ? bt.role[a] < bt.role[b] : a < b;
+        });
+        for (size_t i = 0, j; i < idx.size(); i = j) {
+            const TSeg &g = bt.tseg[idx[i]];
+            for (j = i; j < idx.size() && bt.tseg[idx[j]].S == g.S && bt.tseg[idx[j]].m == g.m && bt.role[idx[j]] == bt.role[idx[i]]; ++j) {}
+            const uint64_t n_seg = (uint64_t)(j - i) * tp.n_scen;
+            if (n_seg >= (1ull << 31)) return fail(ctx, CM_EOVERFLOW, "too many segments in one bucket");
+            BBucket q{};
+            q.count = walked(g);
+            q.K = g.K;
+            q.list_first = (uint32_t)bt.bucket_tseg.size();
+            q.n_seg = (uint32_t)n_seg;
+            q.tmpl = (uint32_t)t;
+            q.feas_first = g.feas_first;
+            q.S = g.S;
+            q.m = g.m;
+            q.role = bt.role[idx[i]];
+            bt.bucket_tseg.insert(bt.bucket_tseg.end(), idx.begin() + i, idx.begin() + j);
+            groups.push_back(q);
+        }
+    }
+    return layout_bound(ctx, bt, groups);
+}
+
 cm_status build_buckets(cm_ctx *ctx, Batch &bt) {
     bt.bucket.clear();
     bt.classes.clear();
     bt.bucket_tseg.clear();
+    if (ctx->d_prof) {   // (a context without a device only describes: cm_host_describe)
+        cm_status s = build_bound(ctx, bt);
+        if (s != CM_OK || bt.bounded) return s;
+        bt.bucket_tseg.clear();
+    }
     using Pre = PreBucket;
     std::vector<Pre> pre;
     std::vector<uint8_t> role = bt.role;   // pairs too few for the transposed kernel are dissolved here, for this layout only
@@ -443,6 +493,73 @@ cm_status build_buckets(cm_ctx *ctx, Batch &bt) {
         }
     }
     return layout_buckets(ctx, bt, pre);
+}
+
+// Work layout of the bounded search pass from the groups of segments it covers (BBucket: count, K,
+// list_first, n_seg, tmpl, feas_first, S, m, role, second filled in).  bt.bounded stays false where
+// the recurrences are too few to pay for the pass's launches.
+cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups) {
+    bt.bounded = false;
+    bt.bbucket.clear();
+    if (bt.dense_only || groups.empty()) return CM_OK;
+    // The full enumeration of splits gives pipelines every micro-batch count from 1 up; with fewer
+    // micro-batches than stages the bound is loose and hundreds of thousands of plans would be left.
+    if (bt.opts.bm != CM_BATCH_REMAINDER) return CM_OK;
+    double cells = 0.0, plans[2] = {0.0, 0.0};   // plans up to kRegStagesMax stages, deeper
+    uint64_t segs[2] = {0, 0};
+    int max_stages = 1;
+    for (const BBucket &g : groups) {
+        if (g.count >= 0xfffffff0ull) return CM_OK;   // positions are 32-bit
+        cells += 2.0 * (double)g.count * g.n_seg * g.S * g.m;
+        plans[g.S > kRegStagesMax] += (double)g.count * g.n_seg;
+        segs[g.S > kRegStagesMax] += g.n_seg;
+        max_stages = std::max<int>(max_stages, g.S);
+    }
+    if (cells < (double)kBoundMinCells) return CM_OK;
+    std::stable_sort(groups.begin(), groups.end(), [](const BBucket &a, const BBucket &b) { return a.S > b.S; });
+    BoundDev bo{};
+    for (int l = 0; l < 4; ++l) {
+        const uint64_t n = segs[l & 1];
+        const double room = l < 2 ? (double)n : std::min(plans[l & 1], (double)std::max<uint64_t>(n, kBoundListMin));
+        bo.list_first[l + 1] = bo.list_first[l] + (uint32_t)room;
+    }
+    // segments a CTA walks with one set of compositions: as many as shared memory holds comfortably,
+    // fewer where the grid would not fill the GPU
+    const int per_seg = ctx->uniform_p2p ? 16 * ((max_stages + 3) / 4) : 16;
+    uint64_t chunks = 0, n_segs = 0;
+    int max_group = 1;
+    for (int most = std::min(256, 16384 / per_seg);; most /= 2) {
+        chunks = n_segs = 0;
+        max_group = 1;
+        for (BBucket &g : groups) {
+            int width = 1;
+            while (width < 128 && (uint64_t)width < g.count) width *= 2;
+            const int side = 128 / width;
+            int group = std::max(side, most / side * side);
+            group = (int)std::min<uint64_t>((uint64_t)group, ((uint64_t)g.n_seg + side - 1) / side * side);
+            g.width = (uint16_t)width;
+            g.seg_group = (uint16_t)group;
+            g.n_groups = (uint32_t)((g.n_seg + group - 1) / group);
+            g.chunk_first = (uint32_t)chunks;
+            g.seg_first = (uint32_t)n_segs;
+            chunks += (g.count + width - 1) / width * g.n_groups;
+            n_segs += g.n_seg;
+            max_group = std::max(max_group, group);
+            if (chunks >= 0x7fffffffull) return CM_OK;
+        }
+        if (chunks >= 4 * 148 || most <= 8) break;
+    }
+    bo.n_buckets = (uint32_t)groups.size();
+    bo.n_chunks = (uint32_t)chunks;
+    bo.n_segs = (uint32_t)n_segs;
+    bo.uniform_x = ctx->uniform_p2p ? 1 : 0;
+    bo.window = bt.useg ? 0 : 1;
+    bo.dyn_bytes = bound_dyn_bytes(bo, max_stages, max_group, ctx->uniform_p2p);
+    if (bo.dyn_bytes > kBoundDynMax) return CM_OK;
+    bt.bo = bo;
+    bt.bbucket = groups;
+    bt.bounded = true;
+    return CM_OK;
 }
 
 // Buckets and launch classes from the collected (template or shared-list) segment groups.
@@ -586,6 +703,7 @@ cm_status build_segment_classes(cm_ctx *ctx, Batch &bt) {
     bt.utab_slots = slots;
     bt.ulist_len = list;
     bt.bucket.assign(std::max<size_t>(kSharedBucketsPerClass * bt.ucls_info.size(), 1), Bucket{});
+    bt.bbucket.assign(std::max<size_t>(2 * bt.ucls_info.size(), 1), BBucket{});   // (a pair class: both rows)
     bt.classes.clear();
     bt.bucket_tseg.clear();
     return CM_OK;
@@ -601,6 +719,30 @@ cm_status build_shared_buckets(cm_ctx *ctx, Batch &bt, const uint32_t *n_distinc
     auto count_of = [](const Batch::USegInfo &u) {
         return u.feas_first != kNoFeasList ? (uint64_t)u.feas_count : (u.K ? u.K + 1 : 1);
     };
+    {
+        std::vector<BBucket> groups;
+        for (size_t c = 0; c < bt.ucls_info.size(); ++c) {
+            const Batch::USegInfo &u = bt.ucls_info[c];
+            if (n_distinct[c] == 0) continue;
+            if (n_distinct[c] > u.rows) return fail(ctx, CM_ECUDA, "internal: more distinct segments than rows");
+            for (int second = 0; second < (u.pair ? 2 : 1); ++second) {
+                BBucket q{};
+                q.count = count_of(u);
+                q.K = u.K;
+                q.list_first = bt.ucls[c].list_first;
+                q.n_seg = n_distinct[c];
+                q.tmpl = kSharedBucket;
+                q.feas_first = u.feas_first;
+                q.S = u.S;
+                q.m = (uint16_t)(u.m + second);
+                q.role = u.pair ? (second ? 2 : 1) : 0;
+                q.second = (uint16_t)second;
+                groups.push_back(q);
+            }
+        }
+        cm_status s = layout_bound(ctx, bt, groups);
+        if (s != CM_OK || bt.bounded) return s;
+    }
     uint64_t deep_plans = 0;
     for (size_t c = 0; c < bt.ucls_info.size(); ++c) {
         const Batch::USegInfo &u = bt.ucls_info[c];
@@ -855,6 +997,7 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
     bt.tmpl_cand_own.assign(1, 0);   // template 0 has no strategies
     bt.max_tiles_per_seg = 0;
     bt.dp_max = 0;
+    bt.k_best = 1;
     bt.B = B;
     bt.tmpl_of_nsurv.assign((size_t)N + 1, -1);
     bt.tmpl.push_back(Tmpl{});   // template 0: no strategies (scenarios without a dynamic-parallelism search)
@@ -958,6 +1101,8 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
     bt.n_rows = rows;
     bt.n_tiles = bt.max_tiles_per_seg ? 1 : 0;   // only "is there anything to tie-break" matters
     bt.mm_launched = false;
+    bt.bounded = bt.dense_only = false;
+    bt.bbucket.clear();
     if (ctx->d_prof && ctx->screen) {   // (a context without a device only describes: cm_host_describe)
         const uint64_t t0 = now_ns();
         cm_status s = ensure_feasible_lists(ctx, bt);
@@ -993,7 +1138,7 @@ BatchDev dev_view(const cm_ctx *ctx, Batch &bt) {
     v.strat = (const Strat *)(a + bt.off_strat); v.tseg = (const TSeg *)(a + bt.off_tseg);
     v.failed = (const uint32_t *)(a + bt.off_failed); v.cross = (const uint64_t *)(a + bt.off_cross);
     v.tmpl_scen = (const uint32_t *)(a + bt.off_tmpl_scen);
-    v.bucket = bt.bucket_override ? bt.bucket_override : (const Bucket *)(a + bt.off_bucket);
+    v.bucket = (const Bucket *)(a + bt.off_bucket);
     v.bucket_tseg = (const uint32_t *)(a + bt.off_bucket_tseg); v.red_scen = (const uint32_t *)(a + bt.off_red);
     v.feas = ctx->d_feas.p;
     v.useg = bt.d_useg.p;
@@ -1043,6 +1188,19 @@ Tables tables_plain(const cm_ctx *ctx) {   // for kernels that only read the byt
     return t;
 }
 
+constexpr size_t kCounterSlots = 8;                 // kCounters of them in use
+constexpr size_t kStateExtra = kCounterSlots + 2;   // + the counts of four lists (32-bit)
+
+// Room for listed plans.  Captured launch sequences carry the list's address: dropped when it moves.
+cm_status reserve_bound_list(cm_ctx *ctx, size_t want) {
+    if (want <= ctx->d_bound_list.cap) return CM_OK;
+    CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (!ctx->d_bound_list.reserve(want)) return fail(ctx, CM_ENOMEM, "device memory");
+    for (auto &e : ctx->single)
+        if (e->exec) { cudaGraphExecDestroy(e->exec); e->exec = nullptr; }
+    return CM_OK;
+}
+
 // Copy the tables of a batch to the device (one copy) and run the min-max partitions it needs.
 cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
     struct Timer { cm_ctx *c; uint64_t t0; ~Timer() { c->stats[18] += now_ns() - t0; } } timer{ctx, now_ns()};
@@ -1064,12 +1222,14 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
     bt.off_look_head = arena_put(bt.arena, bt.look_head, ok);
     bt.off_look_part = arena_put(bt.arena, bt.look_part, ok);
     bt.off_bucket = arena_put(bt.arena, bt.bucket, ok);
+    bt.off_bbucket = arena_put(bt.arena, bt.bbucket, ok);
     if (!ok) return fail(ctx, CM_ENOMEM, "host memory");
     if (!bt.d_arena.reserve(bt.arena.size())) return fail(ctx, CM_ENOMEM, "device memory");
     CM_CUDA(ctx, cudaMemcpyAsync(bt.d_arena.p, bt.arena.p, bt.arena.size(), cudaMemcpyHostToDevice, ctx->stream));
     ctx->stats[9] += bt.arena.size();
     const size_t B = std::max(bt.B, 1);
-    ok = bt.d_seg_best.reserve(bt.n_rows + 4) &&   // + the four work counters, cleared by the same memset
+    // minima | work counters | list counts | bounds | picks: what one memset clears
+    ok = bt.d_seg_best.reserve(3 * bt.n_rows + kStateExtra) && bt.d_win.reserve(B) &&
          bt.d_partial.reserve(std::max<size_t>(bt.red_scen.size(), 1)) && bt.d_winner.reserve(B) &&
          bt.d_kappa_sel.reserve(B * kMaxP) && bt.d_pol_cost.reserve(B * 2) &&
          bt.d_rc_stages.reserve(B * kMaxP) && bt.d_plans.reserve(B * 4 + 1);   // + room for the counters
@@ -1099,12 +1259,47 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
         if (bt.ucount_host[n_cls] != 0) return fail(ctx, CM_ECUDA, "internal: segment table full");
         cm_status s = build_shared_buckets(ctx, bt, bt.ucount_host.p);
         if (s != CM_OK) return s;
-        if (!bt.bucket.empty()) {
+        if (bt.bounded) {
+            memcpy(bt.arena.p + bt.off_bbucket, bt.bbucket.data(), bt.bbucket.size() * sizeof(BBucket));
+            const size_t bytes = bt.bbucket.size() * sizeof(BBucket);
+            CM_CUDA(ctx, cudaMemcpyAsync(bt.d_arena.p + bt.off_bbucket, bt.arena.p + bt.off_bbucket, bytes, cudaMemcpyHostToDevice, ctx->stream));
+            ctx->stats[9] += bytes;
+        } else if (!bt.bucket.empty()) {
             memcpy(bt.arena.p + bt.off_bucket, bt.bucket.data(), bt.bucket.size() * sizeof(Bucket));
             CM_CUDA(ctx, cudaMemcpyAsync(bt.d_arena.p + bt.off_bucket, bt.arena.p + bt.off_bucket, bt.bucket.size() * sizeof(Bucket),
                                          cudaMemcpyHostToDevice, ctx->stream));
             ctx->stats[9] += bt.bucket.size() * sizeof(Bucket);
         }
+    }
+    if (bt.bounded) return reserve_bound_list(ctx, bt.bo.list_first[4]);
+    return CM_OK;
+}
+
+// Search pass with bounds: see cm_bound.cu.
+cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchDev &bd, cudaStream_t st, int *launches) {
+    BoundDev bo = bt.bo;
+    bo.bucket = (const BBucket *)(bt.d_arena.p + bt.off_bbucket);
+    bo.count = (uint32_t *)(bt.d_seg_best.p + bt.n_rows + kCounterSlots);
+    bo.lbarg = bt.d_seg_best.p + bt.n_rows + kStateExtra;
+    bo.pick = bo.lbarg + bt.n_rows;
+    bo.win = bt.d_win.p;
+    bo.list = ctx->d_bound_list.p;
+    CM_CUDA(ctx, launch_bound(tb, bd, bo, st));
+    ++*launches;
+    for (int phase = 1; phase <= 2; ++phase) {
+        if (bo.window) {
+            CM_CUDA(ctx, launch_window(tb, bd, bo, phase - 1, bt.k_best, st));
+            ++*launches;
+        }
+        CM_CUDA(ctx, launch_refine(tb, bd, bo, phase, st));
+        if (phase == 1) {
+            CM_CUDA(ctx, launch_gather(tb, bd, bo, st));
+            ++*launches;
+        }
+        const int l = 2 * phase - 2;
+        const uint64_t most = std::max(bo.list_first[l + 1] - bo.list_first[l], bo.list_first[l + 2] - bo.list_first[l + 1]);
+        CM_CUDA(ctx, launch_list(tb, bd, bo, l, most, st));
+        *launches += 2;
     }
     return CM_OK;
 }
@@ -1118,7 +1313,8 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     int launches = 0, cost_launches = 0;
     // per-segment minima start at all-ones (above every cost); so do the work counters, which
     // therefore read "value - 1" until cm_finalize_kernel adds the one back
-    CM_CUDA(ctx, cudaMemsetAsync(bt.d_seg_best.p, 0xFF, (bt.n_rows + 4) * sizeof(uint64_t), st));
+    const size_t cleared = (bt.bounded ? 3 * bt.n_rows : bt.n_rows) + kStateExtra;
+    CM_CUDA(ctx, cudaMemsetAsync(bt.d_seg_best.p, 0xFF, cleared * sizeof(uint64_t), st));
     const bool policies = (bt.policy_mask & ((1u << CM_REROUTE) | (1u << CM_REDUNDANT))) != 0;
     const bool beside = policies && (bt.policy_mask & (1u << CM_DYNPAR)) && ctx->pol_stream;
     if (policies) {
@@ -1132,7 +1328,12 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     }
     if (bt.policy_mask & (1u << CM_DYNPAR)) {
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
-        CM_CUDA(ctx, launch_cost_pass1(tb, bd, bt.classes.data(), (int)bt.classes.size(), st, &ctx->side, &cost_launches));
+        if (bt.bounded) {
+            cm_status s = enqueue_bounded(ctx, bt, tb, bd, st, &cost_launches);
+            if (s != CM_OK) return s;
+        } else {
+            CM_CUDA(ctx, launch_cost_pass1(tb, bd, bt.classes.data(), (int)bt.classes.size(), st, &ctx->side, &cost_launches));
+        }
         launches += cost_launches;
         if (bt.useg) {   // rows that share a segment take its representative's minimum
             CM_CUDA(ctx, launch_useg_copy(bd, useg_view(bt), st));
@@ -1156,7 +1357,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     CM_CUDA(ctx, launch_finalize(tb, bd, st));
     ++launches;
     if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
-    const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + 4 * sizeof(unsigned long long);
+    const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
     CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, back_bytes, cudaMemcpyDeviceToHost, st));
     *launches_out = launches;
     *cost_launches_out = cost_launches;
@@ -1168,7 +1369,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
 cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single = nullptr) {
     cudaStream_t st = ctx->stream;
     int launches = 0, cost_launches = 0;
-    const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + 4 * sizeof(unsigned long long);
+    const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
     if (!bt.plans_host.resize((size_t)bt.B * 4 + 1)) return fail(ctx, CM_ENOMEM, "host memory");
     const uint64_t h_enqueue = now_ns();
     bool replay = false;
@@ -1214,172 +1415,27 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
     }
     ctx->stats[10] += back_bytes;
     const unsigned long long *counters_host = reinterpret_cast<const unsigned long long *>(bt.plans_host.p + (size_t)bt.B * 4);
+    if (bt.bounded && counters_host[4]) {
+        // a list was full (plans whose bounds tie in their hundreds of thousands): search again, every plan
+        if (single && single->exec) { cudaGraphExecDestroy(single->exec); single->exec = nullptr; }
+        bt.dense_only = true;
+        cm_status s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
+        if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
+        return s == CM_OK ? run_batch(ctx, bt, launches, single) : s;
+    }
     ctx->stats[0] += (bt.policy_mask & (1u << CM_DYNPAR)) ? bt.n_cand : 0;
     ctx->stats[19] += (bt.policy_mask & (1u << CM_DYNPAR)) ? bt.n_cand_own : 0;
     ctx->stats[1] += counters_host[0];
     ctx->stats[2] += counters_host[1];
     ctx->stats[16] += counters_host[2];
+    ctx->stats[20] += bt.bounded ? counters_host[3] : counters_host[0];
+    ctx->stats[21] += bt.bounded ? counters_host[5] : counters_host[2];
     ctx->stats[3] += (uint64_t)launches;
     ctx->stats[4] += (uint64_t)((double)ms * 1e6);
     ctx->stats[5] += bt.n_rows;
     ctx->stats[6] += bt.strat.size();
     ctx->stats[7] += bt.n_split;
     return CM_OK;
-}
-
-// One resident scenario searched with its duplicate segments removed (sharing on).  A single
-// failure set repeats pipelines too: strategies share stage counts, and a pipeline that starts a
-// whole number of nodes further on sees the same link tiers.  The few hundred template segments
-// are keyed on the host (class, tier word), sorted, and the distinct ones laid out as shared
-// buckets beside the template buckets; the sequence is launched directly (its grids change from
-// failure to failure, so the resident graph does not fit).  *done = false: too little would be
-// saved to pay for the direct launches -- the caller replays the graph as usual.
-constexpr uint64_t kShareSingleMinCells = 250000000ull;   // recurrence cells that sharing must save (~70 us of search pass)
-cm_status run_single_shared(cm_ctx *ctx, Batch &bt, int launches_so_far, bool *done) {
-    *done = false;
-    if (bt.B != 1 || !(bt.policy_mask & (1u << CM_DYNPAR)) || bt.scen.empty()) return CM_OK;
-    const Scen &sc = bt.scen[0];
-    const Tmpl &tp = bt.tmpl[sc.tmpl];
-    if (tp.n_tseg < 2) return CM_OK;
-    if (bt.tseg_cls.size() != bt.tseg.size()) {   // once per resident batch
-        assign_segment_classes(bt);
-        bt.single_cells = 0;
-        for (uint32_t i = 0; i < tp.n_tseg; ++i) {
-            const TSeg &g = bt.tseg[tp.tseg_first + i];
-            if (bt.tseg_cls[tp.tseg_first + i] == kNoSegClass) continue;
-            bt.single_cells += (g.feas_first != kNoFeasList ? (uint64_t)g.feas_count : (g.K ? g.K + 1 : 1)) * 2ull * g.S * g.m;
-        }
-    }
-    if (bt.single_cells < kShareSingleMinCells) return CM_OK;   // not even all of its cells would be worth it
-    const size_t n_cls = bt.ucls_info.size();
-    // The same keying as cm_useg_key_kernel, on the host: the heads of the pair classes first, then
-    // every other row, which joins a pair that holds its tier (as head: its own m; as second row:
-    // m - 1) before it is keyed among the single segments.  `joined`: slot_of value of such a row.
-    struct Key { uint32_t cls; uint64_t tier; uint32_t row; uint32_t joined; };
-    std::vector<Key> heads, others;
-    heads.reserve(tp.n_tseg);
-    others.reserve(tp.n_tseg);
-    const uint64_t *words = bt.cross.data() + sc.cross_first;
-    auto single_cells_of = [&](const TSeg &g) {
-        return (g.feas_first != kNoFeasList ? (uint64_t)g.feas_count : (g.K ? g.K + 1 : 1)) * 2ull * g.S * g.m;
-    };
-    uint64_t all_cells = 0, distinct_cells = 0;
-    for (uint32_t i = 0; i < tp.n_tseg; ++i) {
-        const uint32_t c = bt.tseg_cls[tp.tseg_first + i];
-        if (c == kNoSegClass) continue;
-        const TSeg &g = bt.tseg[tp.tseg_first + i];
-        all_cells += single_cells_of(g);
-        if (c == kPartnerSeg) continue;
-        const int w = g.off >> 6, sh = g.off & 63, n = g.S - 1;
-        uint64_t v = words[w] >> sh;
-        if (sh) v |= words[w + 1] << (64 - sh);
-        (c < bt.n_pair_cls ? heads : others).push_back(Key{c, v & ((1ull << n) - 1ull), i, kNoSegClass});
-    }
-    auto by_key = [](const Key &a, const Key &b) {
-        return a.cls != b.cls ? a.cls < b.cls : a.tier != b.tier ? a.tier < b.tier : a.row < b.row;
-    };
-    auto same_key = [](const Key &a, const Key &b) { return a.cls == b.cls && a.tier == b.tier; };
-    std::sort(heads.begin(), heads.end(), by_key);
-    std::vector<Key> pair_reps;   // distinct pair heads, sorted by (class, tier); index = their slot
-    for (size_t i = 0; i < heads.size(); ++i)
-        if (i == 0 || !same_key(heads[i], heads[i - 1])) pair_reps.push_back(heads[i]);
-    auto find_pair = [&](uint32_t cls, uint64_t tier) -> uint32_t {
-        if (cls == kNoSegClass) return kNoSegClass;
-        const Key probe{cls, tier, 0, 0};
-        auto it = std::lower_bound(pair_reps.begin(), pair_reps.end(), probe, [](const Key &a, const Key &b) {
-            return a.cls != b.cls ? a.cls < b.cls : a.tier < b.tier;
-        });
-        return it != pair_reps.end() && same_key(*it, probe) ? (uint32_t)(it - pair_reps.begin()) : kNoSegClass;
-    };
-    std::vector<Key> singles;
-    singles.reserve(others.size());
-    for (Key &k : others) {
-        const uint32_t t = tp.tseg_first + k.row;
-        uint32_t at = find_pair(bt.look_head[t], k.tier);
-        if (at == kNoSegClass) {
-            at = find_pair(bt.look_part[t], k.tier);
-            if (at != kNoSegClass) at |= kSecondRowFlag;
-        }
-        k.joined = at;
-        if (at == kNoSegClass) singles.push_back(k);
-    }
-    std::sort(singles.begin(), singles.end(), by_key);
-    auto cells_of = [&](uint32_t c) {
-        const Batch::USegInfo &u = bt.ucls_info[c];
-        const uint64_t count = u.feas_first != kNoFeasList ? (uint64_t)u.feas_count : (u.K ? u.K + 1 : 1);
-        return count * (u.pair ? 2ull * u.S * (u.m + 1) + 3ull * u.S * (u.S - 1) / 2 : 2ull * u.S * u.m);
-    };
-    std::vector<uint32_t> counts(n_cls + 1, 0);
-    size_t n_distinct = pair_reps.size();
-    for (const Key &k : pair_reps) { distinct_cells += cells_of(k.cls); ++counts[k.cls]; }
-    for (size_t i = 0; i < singles.size(); ++i)
-        if (i == 0 || !same_key(singles[i], singles[i - 1])) { distinct_cells += cells_of(singles[i].cls); ++counts[singles[i].cls]; ++n_distinct; }
-    if (all_cells < distinct_cells + kShareSingleMinCells) return CM_OK;
-
-    // staging: slot_of [rows] | rep [distinct] | list [distinct] | buckets [2 per class]
-    const size_t rows = bt.n_rows, max_buckets = std::max<size_t>(kSharedBucketsPerClass * n_cls, 1);
-    const size_t off_rep = 4 * rows, off_list = (off_rep + 4 * n_distinct + 7) & ~(size_t)7;
-    const size_t off_bk = (off_list + 8 * n_distinct + 15) & ~(size_t)15, bytes = off_bk + max_buckets * sizeof(Bucket);
-    bool ok = bt.alt_stage.resize(bytes) && bt.d_slot_of.reserve(std::max<size_t>(rows, 1)) && bt.d_urep.reserve(std::max<size_t>(n_distinct, 1)) &&
-              bt.d_useg.reserve(std::max<size_t>(n_distinct, 1)) && bt.d_alt_bucket.reserve(max_buckets);
-    if (!ok) return fail(ctx, CM_ENOMEM, "memory");
-    uint32_t *slot_of = (uint32_t *)bt.alt_stage.p, *rep = (uint32_t *)(bt.alt_stage.p + off_rep);
-    uint2 *list = (uint2 *)(bt.alt_stage.p + off_list);
-    std::fill(slot_of, slot_of + rows, kNoSegClass);
-    bt.ucls.assign(n_cls, USegClass{0, 0, 0, 0});
-    uint32_t first_of = 0;
-    for (size_t c = 0; c < n_cls; ++c) { bt.ucls[c].list_first = first_of; first_of += counts[c]; }
-    // slots (= list positions): the distinct pair heads, then the distinct single segments; pair
-    // classes have the lower class numbers, so the positions follow the class regions
-    uint32_t u = 0;
-    for (size_t i = 0; i < heads.size(); ++i) {
-        if (i == 0 || !same_key(heads[i], heads[i - 1])) {
-            rep[u] = sc.seg_base + heads[i].row;
-            list[u] = make_uint2(0u, tp.tseg_first + heads[i].row);
-            ++u;
-        }
-        slot_of[sc.seg_base + heads[i].row] = u - 1;
-        slot_of[sc.seg_base + heads[i].row + 1] = kPartnerSeg;
-    }
-    for (const Key &k : others)
-        if (k.joined != kNoSegClass) slot_of[sc.seg_base + k.row] = k.joined;
-    for (size_t i = 0; i < singles.size(); ++i) {
-        if (i == 0 || !same_key(singles[i], singles[i - 1])) {
-            rep[u] = sc.seg_base + singles[i].row;
-            list[u] = make_uint2(0u, tp.tseg_first + singles[i].row);
-            ++u;
-        }
-        slot_of[sc.seg_base + singles[i].row] = u - 1;
-    }
-    std::vector<Bucket> keep_buckets;
-    std::vector<LaunchClass> keep_classes;
-    keep_buckets.swap(bt.bucket);
-    keep_classes.swap(bt.classes);
-    bt.bucket.assign(max_buckets, Bucket{});
-    cm_status s = build_shared_buckets(ctx, bt, counts.data());
-    cudaError_t e = cudaSuccess;
-    if (s == CM_OK) {
-        if (!bt.bucket.empty()) memcpy(bt.alt_stage.p + off_bk, bt.bucket.data(), bt.bucket.size() * sizeof(Bucket));
-        cudaStream_t st = ctx->stream;
-        e = cudaMemcpyAsync(bt.d_slot_of.p, slot_of, 4 * rows, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && n_distinct) e = cudaMemcpyAsync(bt.d_urep.p, rep, 4 * n_distinct, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && n_distinct) e = cudaMemcpyAsync(bt.d_useg.p, list, 8 * n_distinct, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && !bt.bucket.empty())
-            e = cudaMemcpyAsync(bt.d_alt_bucket.p, bt.alt_stage.p + off_bk, bt.bucket.size() * sizeof(Bucket), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) {
-            ctx->stats[9] += 4 * rows + 12 * n_distinct + bt.bucket.size() * sizeof(Bucket);
-            bt.bucket_override = bt.d_alt_bucket.p;
-            bt.useg = true;
-            s = run_batch(ctx, bt, launches_so_far, nullptr);
-            *done = s == CM_OK;
-        }
-    }
-    bt.useg = false;
-    bt.bucket_override = nullptr;
-    bt.bucket.swap(keep_buckets);
-    bt.classes.swap(keep_classes);
-    if (e != cudaSuccess) { cudaGetLastError(); return fail(ctx, CM_ECUDA, std::string("shared segments: ") + cudaGetErrorString(e)); }
-    return s;
 }
 
 // Keys of min-max partitions that were scheduled but never computed must be asked for
@@ -1619,6 +1675,8 @@ static cm_status load_profile_host(cm_ctx *ctx, const cm_profile *p) {
         h.act[l] = p->act_bytes[l]; h.par[l] = p->param_bytes[l]; h.opt[l] = p->opt_bytes[l]; h.p2p[l] = p->p2p_bytes[l];
     }
     for (int i = 0; i <= p->n_pp; ++i) h.base_cuts[i] = p->base_cuts[i];
+    ctx->uniform_p2p = true;
+    for (int l = 1; l < p->L; ++l) ctx->uniform_p2p = ctx->uniform_p2p && p->p2p_bytes[l] == p->p2p_bytes[0];
     {
         // Largest value the integer mode can form: all work of all micro-batches in sequence
         // (rerouted and redundant load included: at most three times that), every transfer of
@@ -1861,14 +1919,7 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
         cm_ctx::Single *entry = nullptr;
         if ((s = single_batch(ctx, failed_ids + offsets[b], offsets[b + 1] - offsets[b], *opts, mask, &sb, &launches, &entry)) != CM_OK) return s;
         ctx->stats[13] += now_ns() - h0;
-        bool done = false;
-        if (ctx->share) {
-            const uint64_t h1 = now_ns();
-            s = run_single_shared(ctx, *sb, launches, &done);
-            if (!done) ctx->stats[13] += now_ns() - h1;   // (the keys were built and found not worth using)
-            if (s != CM_OK) return s;
-        }
-        if (!done && (s = run_batch(ctx, *sb, launches, entry)) != CM_OK) return s;
+        if ((s = run_batch(ctx, *sb, launches, entry)) != CM_OK) return s;
         for (int pol = 0; pol < 3; ++pol) {
             cm_plan pl = sb->plans_host[pol];
             scrub(pl);
@@ -1914,6 +1965,7 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
     if ((s = build_batch(ctx, bt, failed_ids, offsets, B, *opts, mask)) != CM_OK) { forget_keys(ctx, bt); return s; }
     ctx->stats[13] += now_ns() - h0;
     if ((s = upload_batch(ctx, bt, &launches)) != CM_OK) { forget_keys(ctx, bt); return s; }
+    bt.k_best = q.topk;   // the shortlist takes that many step times
     if ((s = run_batch(ctx, bt, launches)) != CM_OK) return s;
 
     // the objective pass works on what the search left on the device

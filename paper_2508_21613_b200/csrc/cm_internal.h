@@ -186,6 +186,44 @@ constexpr int kUniItemsMax = 8;
 constexpr int kUniBatchStagesMax = 28;     // deeper transposed classes keep one item per warp
 constexpr uint64_t kUniMinChunks = 4096;   // keep at least this many CTAs (about ten waves) in a class before batching items
 
+// Bounded search pass (cm_bound.cu).  Its work layout groups segments as the buckets above do, every
+// segment on its own; a CTA of the bound kernel takes `width` compositions of a bucket side by side
+// for 128 / width segments at a time and walks a group of seg_group of them.
+struct BBucket {
+    uint64_t count, K;      // candidates walked per segment; enumerated compositions
+    uint32_t chunk_first;   // its first CTA
+    uint32_t seg_first;     // its first segment, counted through all buckets
+    uint32_t list_first;    // its template segments in bucket_tseg, or its range of the list of distinct segments
+    uint32_t n_seg, tmpl;   // tmpl == kSharedBucket: distinct segments
+    uint32_t feas_first;
+    uint32_t n_groups;
+    uint16_t S, m;
+    uint16_t role;          // work accounting: 0 on its own, 1 head of a micro-batch pair, 2 the row after a head
+    uint16_t second;        // distinct segments: the rows after the listed ones (m is theirs)
+    uint16_t width, seg_group;
+    uint32_t pad;
+};
+// Step times that can still be a scenario's answer: lo <= T* <= ub, lo from bounds.
+struct SearchWin { float lo, pad; uint64_t ub; };
+struct BoundDev {
+    const BBucket *bucket;
+    uint64_t *lbarg;              // per row: least bound (float bits) << 32 | its position in the walk; all-ones = no plan fits
+    uint64_t *pick;               // per row: the plan phase 1 takes (cm_bound_lane.cuh)
+    SearchWin *win;               // per scenario (window)
+    uint4 *list;                  // plans for the recurrence: scenario, template segment, position
+    uint32_t *count;              // per list: plans listed minus one
+    uint32_t list_first[5];       // lists: phase 1 up to kRegStagesMax stages, deeper; phase 2 the same
+    uint32_t n_buckets, n_chunks, n_segs;
+    uint32_t dyn_cols, dyn_segs, max_group;
+    size_t dyn_bytes;
+    int window, uniform_x;
+};
+constexpr int kCounters = 6;   // work counters of a search in use (BatchDev::counters)
+// Recurrence cells of a search from which bounds pay for their extra launches.
+constexpr uint64_t kBoundMinCells = 200000000ull;
+constexpr uint32_t kBoundListMin = 65536;        // plans a list has room for, at least (if there are as many)
+constexpr size_t kBoundDynMax = 160 * 1024;      // dynamic shared memory of the bound kernels, at most
+
 // (cost, index) pair carried through the hierarchical argmin of the split reduction.
 struct Partial {
     uint64_t cost_bits;     // cost as an order-preserving 64-bit pattern (inf = infeasible)
@@ -229,7 +267,9 @@ struct BatchDev {
     uint64_t *pol_cost;     // [B][2] rerouting / redundant cost bits
     uint16_t *rc_stages;    // [B][kMaxP] stage counts of the redundant-computation plan
     cm_plan *plans;         // [B][4]: per policy, then the overall best
-    unsigned long long *counters;  // [0] cells simulated in pass 1, [1] plans in pass 2
+    // [0] cells of the plans the search pass decided, [1] plans of the tie-break pass, [2] plans decided;
+    // bounded pass: [3] cells and [5] plans whose recurrence ran, [4] a list was full
+    unsigned long long *counters;
     int32_t B, mode;
     uint32_t n_rows;             // rows of seg_best over all scenarios
     // 1: integer-nanosecond mode evaluated in double arithmetic on integer-valued inputs; every
@@ -309,8 +349,16 @@ struct SideStreams {
 };
 cudaError_t launch_cost_pass1(const Tables &t, const BatchDev &b, const LaunchClass *classes, int n_classes,
                               cudaStream_t st, const SideStreams *side, int *launches);
+// bounded search pass (cm_bound.cu, cm_refine.cu)
+size_t bound_dyn_bytes(BoundDev &bo, int max_stages, int max_group, bool uniform_x);   // also sets the offsets
+cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
+cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st);
+cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st);
+cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
+// lists first_list and first_list + 1, at most `most` plans in either
+cudaError_t launch_list(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, uint64_t most, cudaStream_t st);
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st);
-cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);   // cm_bound.cu
+cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);   // cm_tiebreak.cu
 cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st);
 // single_policy < 0: candidates of the dynamic-parallelism segments; otherwise the one
 // candidate of that policy (its cost must already be in pol_cost of scenario 0)

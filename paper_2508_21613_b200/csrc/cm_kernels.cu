@@ -7,7 +7,7 @@
 //   (the search pass over every pipeline-plan lives in cm_cost.cu)
 //   cm_split_kernel       (cost, index) argmin over (strategy, micro-batch split) per scenario
 //   cm_winner_kernel      finishes that argmin and decodes the winner
-//   (pass 2, the lowest layer composition that meets the winning cost: cm_bound.cu)
+//   (pass 2, the lowest layer composition that meets the winning cost: cm_tiebreak.cu)
 //   cm_finalize_kernel    assembles the plans and picks the best policy
 //   cm_evaluate_kernel    per-candidate cost / feasibility for cm_evaluate
 //   cm_pick_kernel        best of several spaces for cm_select
@@ -481,7 +481,7 @@ __global__ void cm_finalize_kernel(Tables tb, BatchDev bd, uint64_t inf) {
     if (b == 0) {
         // work counters ride home behind the plans (they start at all-ones, i.e. -1)
         unsigned long long *tail = reinterpret_cast<unsigned long long *>(bd.plans + (size_t)bd.B * 4);
-        for (int i = 0; i < 4; ++i) tail[i] = bd.counters[i] + 1ull;
+        for (int i = 0; i < kCounters; ++i) tail[i] = bd.counters[i] + 1ull;
     }
     if (b >= bd.B) return;
     const DevProfile *p = tb.prof;

@@ -1,0 +1,119 @@
+// Tie-break pass of the plan search (sm_100a): among optimal plans the lexicographically smallest
+// tuple wins, so each pipeline of a winning (strategy, split) takes the LOWEST layer composition
+// that is feasible with cost <= T* (not its own argmin).
+#include <algorithm>
+
+#include "cm_bound.cuh"
+
+namespace cm {
+
+// ----------------------------------------------------------------------------------
+// A CTA per (winner record, pipeline) walks the segment's candidates upwards, a thread per
+// composition: a lower bound above T* rules one out (first in O(stages), then, for those that tie,
+// bit for bit along the walk: cm_bound.cuh), and the few that are left are walked by a warp each in
+// lock step, lowest first, n_eval of them at a time.  The bound is tight, so about one recurrence
+// per pipeline remains; what bounds the kernel is the latency of those, 2(S+m) dependent
+// slots.  grid.y: tiles of a segment side by side where the winners alone leave the GPU empty (the
+// uncapped spaces hold 10^8 compositions per pipeline); a tile whose first composition is above one
+// already found stops.
+// ----------------------------------------------------------------------------------
+template <typename T, int kTieThreads>
+__global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, BatchDev bd, int n_eval) {
+    __shared__ SProf<T> sp;
+    __shared__ uint8_t cuts_s[kTieThreads / 32][kMaxS + 8];
+    __shared__ uint32_t left[kTieThreads / 32];
+    __shared__ unsigned long long found;
+    const uint32_t b = blockIdx.x / bd.dp_max, p = blockIdx.x % bd.dp_max;
+    const Winner &w = bd.winner[b];
+    if (w.cost_bits >= inf_bits<T>() || p >= w.dp) return;          // uniform over the CTA
+    const SegView g = seg_view(bd, w.scen, w.seg[p]);
+    if (g.K == 0) return;                                           // one candidate: known already
+    stage_profile(sp, tb);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double goal = std::is_same<T, long long>::value ? __ll2double_ru((long long)w.cost_bits)
+                                                          : __longlong_as_double((long long)w.cost_bits);
+    unsigned long long *slot = reinterpret_cast<unsigned long long *>(&bd.kappa_sel[(size_t)b * kMaxP + p]);
+    const uint64_t count = walk_count(g);
+    unsigned long long evaluated = 0;
+    for (uint64_t base = (uint64_t)blockIdx.y * kTieThreads; base < count; base += (uint64_t)gridDim.y * kTieThreads) {
+        __syncthreads();
+        if (threadIdx.x == 0) found = *(volatile unsigned long long *)slot;
+        __syncthreads();
+        if (found <= walk_kappa(bd.feas, g.feas_first, base)) break;   // uniform: this tile and all later ones are higher
+        const uint64_t pos = base + threadIdx.x;
+        bool maybe = false;
+        if (pos < count) {
+            CutWalker cw;
+            const uint64_t kappa = walk_kappa(bd.feas, g.feas_first, pos);
+            if (make_walker(cw, tb, bd.layer_mode, sp.L, g.S, kappa, g.K, tb.mm_slot(g.S, g.m))) {
+                const CutEdges c = cut_edges(cw);
+                const Walk walk = best_walk<T>(sp, c, g.S, g.m, g.tier, g.n_sync, g.feas_first == kNoFeasList);
+                maybe = walk.value >= 0.0 && walk.value <= goal;
+                if (maybe) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= w.cost_bits;
+            }
+        }
+        const uint32_t vote = __ballot_sync(0xffffffffu, maybe);
+        if (lane == 0) left[warp] = vote;
+        __syncthreads();
+        if (threadIdx.x == 0) found = ~0ull;
+        for (;;) {
+            // this warp's candidate: number `warp` among those left, if it is one of the next n_eval
+            int skip = warp, at = -1, total = 0;
+            for (int q = 0; q < kTieThreads / 32; ++q) {
+                const uint32_t v = left[q];
+                const int c = __popc(v);
+                if (at < 0 && skip < c) at = q * 32 + (int)__fns(v, 0, skip + 1);
+                skip -= c;
+                total += c;
+            }
+            __syncthreads();                                        // everybody has read `left`; `found` is reset
+            if (total == 0) break;                                  // uniform
+            if (warp < n_eval && at >= 0) {
+                const uint64_t kappa = walk_kappa(bd.feas, g.feas_first, base + at);
+                T cost;
+                if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, kappa, cuts_s[warp], cost) && lane == 0 &&
+                    Num<T>::bits(cost) <= w.cost_bits)
+                    atomicMin(&found, (unsigned long long)kappa);
+                if (lane == 0) ++evaluated;
+            }
+            if (threadIdx.x == 0)                                   // strike the candidates being tried
+                for (int q = 0, n = n_eval; q < kTieThreads / 32 && n > 0; ++q)
+                    while (left[q] && n > 0) { left[q] &= left[q] - 1; --n; }
+            __syncthreads();
+            if (found != ~0ull) break;                              // uniform
+        }
+        if (found != ~0ull) {                                       // the lowest of this tile: later tiles are higher
+            if (threadIdx.x == 0) atomicMin(slot, found);
+            break;
+        }
+    }
+    if (lane == 0 && evaluated) atomicAdd(&bd.counters[1], evaluated);
+}
+
+cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st) {
+    if (b.B <= 0 || b.max_tiles_per_seg == 0 || b.dp_max == 0) return cudaSuccess;
+    const uint64_t nx = (uint64_t)b.B * b.dp_max;
+    if (nx >= (1ull << 31)) return cudaErrorInvalidConfiguration;
+    // A failure handled on its own: a wide CTA per pipeline, whose warps try candidates side by side.  A
+    // batch: narrow CTAs, of which an SM holds nine instead of two; the first tile nearly always holds
+    // the answer, and its first candidate nearly always is it.  2576 failure sets of the 32-device job:
+    // 131 us with 64 threads, above 400 us with 256; 290 us for the plan-per-lane kernel this replaced.
+    // 1024 sets of the 256-device job: 147 us, where a plan-per-lane kernel per depth took 1300 us in all.
+    const bool wide = nx <= 148 * 2;
+    const unsigned threads = wide ? 256 : 64;
+    const int n_eval = wide ? 256 / 32 : 1;
+    const uint64_t tiles = ((uint64_t)b.max_tiles_per_seg * kTile + threads - 1) / threads;
+    uint64_t y = (148 * 4 + nx - 1) / nx;
+    y = std::min<uint64_t>(std::min(y, tiles), 65535);
+    const dim3 grid((unsigned)nx, (unsigned)std::max<uint64_t>(y, 1), 1);
+    if (native_i64(b)) {
+        if (wide) cm_tiebreak_kernel<long long, 256><<<grid, threads, 0, st>>>(t, b, n_eval);
+        else cm_tiebreak_kernel<long long, 64><<<grid, threads, 0, st>>>(t, b, n_eval);
+    } else {
+        if (wide) cm_tiebreak_kernel<double, 256><<<grid, threads, 0, st>>>(t, b, n_eval);
+        else cm_tiebreak_kernel<double, 64><<<grid, threads, 0, st>>>(t, b, n_eval);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace cm

@@ -1,0 +1,120 @@
+"""The bounded search pass (lower bounds decide most plans, the recurrence runs on the few they leave)
+and the tie-break pass by bounds, at the sizes where they can go wrong, against the CPU oracle: plan
+tuples bit-exact, costs equal."""
+import itertools
+
+import numpy as np
+import pytest
+
+from paper_2508_21613_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    import torch
+    from paper_2508_21613_b200 import binding, build
+    build.build()
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device; there is no CPU path")
+    return binding
+
+
+def _small(seed, times=None, tight=False, n_micro=7, p2p=None):
+    p = W.random_small(seed, L=13, n_dp=3, n_pp=4, n_micro=n_micro, tight_memory=tight).profile
+    fwd = p.fwd_ns if times is None else times(13)
+    return W.make_profile_ns(13, 3, 4, n_micro, fwd, 2.0 * np.asarray(fwd), p.act_bytes, p.param_bytes, p.opt_bytes,
+                             p.p2p_bytes if p2p is None else p2p, p.base_cuts, p.mem_capacity_bytes, 4, 300, 20)
+
+
+SETS = [list(c) for k in (1, 2) for c in itertools.combinations(range(12), k)]
+CASES = {
+    # transfer times that depend on the layer
+    "layered-transfers": (_small(31), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 40),
+    "tight-memory": (_small(33, tight=True), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 200),
+    # transfer times equal on every boundary; identical layers (most plans tie); fewer micro-batches than stages
+    "equal-transfers": (_small(34, p2p=30_000_000), (1, 3, 2, 7, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 40),
+    "identical-layers": (_small(35, times=lambda n: np.full(n, 3e6), p2p=30_000_000), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 40),
+    "few-micro-batches": (_small(36, n_micro=2), (1, 3, 2, 8, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 160),
+}
+
+
+@pytest.mark.parametrize("schedule", [W.SCHED_1F1B, W.SCHED_GPIPE])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_bounded_search_against_the_oracle(gpu, oracle_factory, name, schedule):
+    """Each failure set many times over, so that the batch is large enough for bounds; in double,
+    integer-valued double and 64-bit integer arithmetic."""
+    profile, window, sets, copies = CASES[name]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        for mode in (0, 1):
+            opts = W.SearchOptions(*window, 1 << 62, mode, schedule)
+            orc = oracle_factory(profile, opts)
+            want = [orc.search(f)[0] for f in sets]
+            for native in (False, True)[:1 + mode]:
+                gpu.cm_set_int64_arithmetic(ctx, native)
+                best, _, _ = gpu.cm_search_batch(ctx, sets * copies, opts)
+                st = gpu.cm_last_stats(ctx)
+                assert st["plans_run"] < st["plans_simulated"]      # bounds decided the rest
+                for b, plan in enumerate(gpu.plans_from_array(best)):
+                    w = want[b % len(sets)]
+                    assert plan.feasible == (w is not None and w.feasible)
+                    if w is not None and w.feasible:
+                        assert plan.key() == w.key(), (sets[b % len(sets)], plan, w)
+                        assert plan.cost == w.cost and plan.cost_ns == w.cost_ns
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_search_with_more_ties_than_the_list_holds(gpu, oracle_factory, mode):
+    """One layer holds all the time, so every composition of a pipeline ties with a quarter of a million
+    others: the list of plans left to the recurrence overflows and the search is repeated in full."""
+    L = 24
+    fwd = np.zeros(L)
+    fwd[0] = 5e6
+    profile = W.make_profile_ns(L, 2, 8, 4, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 0,
+                                list(range(0, 25, 3)), 80_000_000_000, 4, 300, 20)
+    opts = W.SearchOptions(2, 2, 7, 8, W.LAYERS_FULL, W.BATCH_REMAINDER, 1 << 62, mode)
+    sets = [[0], [9]]
+    orc = oracle_factory(profile, opts)
+    want = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        best, _, _ = gpu.cm_search_batch(ctx, sets * 4, opts)
+        st = gpu.cm_last_stats(ctx)
+        assert st["plans_run"] == st["plans_simulated"] > 1 << 20   # the full search ran in the end
+        for b, plan in enumerate(gpu.plans_from_array(best)):
+            assert plan.key() == want[b % 2].key() and plan.cost == want[b % 2].cost and plan.cost_ns == want[b % 2].cost_ns
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+def test_bounded_shortlist_against_the_oracle(gpu, oracle_factory):
+    """The full objective takes the k best step times: every one of them has to be exact, not the first alone."""
+    profile, window, sets, copies = CASES["layered-transfers"]
+    for mode, topk in ((0, 16), (1, 5)):
+        opts = W.SearchOptions(*window, 1 << 62, mode)
+        orc = oracle_factory(profile, opts)
+        obj = W.ObjectiveOptions(topk=topk)
+        want = [orc.search_objective(f, obj) for f in sets[:6]]
+        ctx = gpu.cm_create(0)
+        try:
+            gpu.cm_load_profile(ctx, profile)
+            many = sets[:6] * (copies * 4)
+            best, trans, short, moved, _ = gpu.cm_search_objective(ctx, many, opts, obj, shortlist=True)
+            st = gpu.cm_last_stats(ctx)
+            assert st["plans_run"] < st["plans_simulated"]
+            short = gpu.plans_from_array(short)
+            best = gpu.plans_from_array(best)
+            for b in range(len(many)):
+                plan, tr = want[b % 6]
+                assert best[b].key() == plan.key() and best[b].cost == plan.cost and best[b].cost_ns == plan.cost_ns
+                got = [short[b * topk + r] for r in range(topk) if moved[b, r] >= 0]
+                assert [p.key() for p in got] == [p.key() for p in tr.shortlist]
+                assert [(p.cost, p.cost_ns) for p in got] == [(p.cost, p.cost_ns) for p in tr.shortlist]
+        finally:
+            gpu.cm_destroy(ctx)
