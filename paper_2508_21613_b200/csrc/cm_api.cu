@@ -187,6 +187,7 @@ struct cm_ctx {
     struct FeasEntry { uint32_t first, count; uint64_t K; };
     std::map<uint32_t, FeasEntry> feas[6];   // [layer mode * 2 + execution order]
     DevBuf<uint32_t> d_feas;
+    DevBuf<ulonglong2> d_feas_mask;           // the same entries as masks
     size_t feas_used = 0;
     PinnedVec<unsigned char> feas_stage;      // keys, K, offsets out; counts back
     DevBuf<unsigned char> d_feas_stage;
@@ -523,19 +524,17 @@ cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups) {
         const double room = l < 2 ? (double)n : std::min(plans[l & 1], (double)std::max<uint64_t>(n, kBoundListMin));
         bo.list_first[l + 1] = bo.list_first[l] + (uint32_t)room;
     }
-    // segments a CTA walks with one set of compositions: as many as shared memory holds comfortably,
-    // fewer where the grid would not fill the GPU
-    const int per_seg = ctx->uniform_p2p ? 16 * ((max_stages + 3) / 4) : 16;
+    // segments a CTA walks with one set of compositions; fewer where the grid would not fill the GPU
     uint64_t chunks = 0, n_segs = 0;
     int max_group = 1;
-    for (int most = std::min(256, 16384 / per_seg);; most /= 2) {
+    for (int most = bound_group(max_stages, ctx->uniform_p2p);; most = std::max(most / 2, 1)) {
         chunks = n_segs = 0;
         max_group = 1;
         for (BBucket &g : groups) {
-            int width = 1;
-            while (width < 128 && (uint64_t)width < g.count) width *= 2;
+            int width = 1;   // (segments side by side: at most the group)
+            while (width < 128 && ((uint64_t)width < g.count || 128 / width > most)) width *= 2;
             const int side = 128 / width;
-            int group = std::max(side, most / side * side);
+            int group = most / side * side;
             group = (int)std::min<uint64_t>((uint64_t)group, ((uint64_t)g.n_seg + side - 1) / side * side);
             g.width = (uint16_t)width;
             g.seg_group = (uint16_t)group;
@@ -900,16 +899,25 @@ cm_status grow_feas_pool(cm_ctx *ctx, size_t want) {
     if (want <= ctx->d_feas.cap) return CM_OK;
     size_t nc = std::max<size_t>(want, std::max<size_t>(ctx->d_feas.cap * 2, 1u << 20));
     uint32_t *q = nullptr;
+    ulonglong2 *qm = nullptr;
     CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (cudaMalloc((void **)&q, nc * sizeof(uint32_t)) != cudaSuccess) { cudaGetLastError(); return fail(ctx, CM_ENOMEM, "device memory"); }
+    if (cudaMalloc((void **)&q, nc * sizeof(uint32_t)) != cudaSuccess || cudaMalloc((void **)&qm, nc * sizeof(ulonglong2)) != cudaSuccess) {
+        cudaGetLastError();
+        if (q) cudaFree(q);
+        return fail(ctx, CM_ENOMEM, "device memory");
+    }
     if (ctx->feas_used) {
         cudaError_t e = cudaMemcpyAsync(q, ctx->d_feas.p, ctx->feas_used * sizeof(uint32_t), cudaMemcpyDeviceToDevice, ctx->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(qm, ctx->d_feas_mask.p, ctx->feas_used * sizeof(ulonglong2), cudaMemcpyDeviceToDevice, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) { cudaFree(q); cudaGetLastError(); return fail(ctx, CM_ECUDA, cudaGetErrorString(e)); }
+        if (e != cudaSuccess) { cudaFree(q); cudaFree(qm); cudaGetLastError(); return fail(ctx, CM_ECUDA, cudaGetErrorString(e)); }
     }
     if (ctx->d_feas.p) cudaFree(ctx->d_feas.p);
+    if (ctx->d_feas_mask.p) cudaFree(ctx->d_feas_mask.p);
     ctx->d_feas.p = q;
-    ctx->d_feas.cap = nc;
+    ctx->d_feas_mask.p = qm;
+    ctx->d_feas.cap = ctx->d_feas_mask.cap = nc;
     for (auto &e : ctx->single)
         if (e->exec) { cudaGraphExecDestroy(e->exec); e->exec = nullptr; }
     return CM_OK;
@@ -959,7 +967,7 @@ cm_status ensure_feasible_lists(cm_ctx *ctx, Batch &bt) {
             e = launch_minmax(tb, (const uint32_t *)(d + off_mm), (int)n_mm, bt.intval ? CM_COST_FP64 : bt.opts.cost, ctx->stream);
         if (e == cudaSuccess)
             e = launch_feasible(tb, lm, (const uint32_t *)(d + off_key), (const uint64_t *)d, (const uint32_t *)(d + off_first),
-                                (int)n, ctx->d_feas.p, (uint32_t *)(d + off_cnt), ctx->stream);
+                                (int)n, ctx->d_feas.p, ctx->d_feas_mask.p, (uint32_t *)(d + off_cnt), ctx->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h + off_cnt, d + off_cnt, 4 * n, cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
         if (e != cudaSuccess) { cudaGetLastError(); undo(); return fail(ctx, CM_ECUDA, std::string("feasible-composition lists: ") + cudaGetErrorString(e)); }
@@ -1141,6 +1149,7 @@ BatchDev dev_view(const cm_ctx *ctx, Batch &bt) {
     v.bucket = (const Bucket *)(a + bt.off_bucket);
     v.bucket_tseg = (const uint32_t *)(a + bt.off_bucket_tseg); v.red_scen = (const uint32_t *)(a + bt.off_red);
     v.feas = ctx->d_feas.p;
+    v.feas_mask = ctx->d_feas_mask.p;
     v.useg = bt.d_useg.p;
     v.tseg_canon = bt.n_dup ? (const uint32_t *)(a + bt.off_canon) : nullptr;
     v.n_rep_scen = 0;
@@ -1296,10 +1305,8 @@ cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchD
             CM_CUDA(ctx, launch_gather(tb, bd, bo, st));
             ++*launches;
         }
-        const int l = 2 * phase - 2;
-        const uint64_t most = std::max(bo.list_first[l + 1] - bo.list_first[l], bo.list_first[l + 2] - bo.list_first[l + 1]);
-        CM_CUDA(ctx, launch_list(tb, bd, bo, l, most, st));
-        *launches += 2;
+        ++*launches;
+        CM_CUDA(ctx, launch_lists(tb, bd, bo, 2 * phase - 2, st, launches));
     }
     return CM_OK;
 }
@@ -1596,7 +1603,7 @@ cm_status cm_create(cm_ctx **out, int cuda_device, void *cuda_stream) {
     ok = ok && c->d_scratch.reserve(sizeof(cm_plan *) * 64 + sizeof(cm_plan));   // what cm_select needs
     // the feasible-composition pool and its staging are allocated here, not at the first search:
     // a pinned allocation costs milliseconds, which a failure handler should not pay
-    ok = ok && c->d_feas.reserve(1u << 20) && c->feas_stage.reserve(1u << 16) && c->d_feas_stage.reserve(1u << 16);
+    ok = ok && c->d_feas.reserve(1u << 20) && c->d_feas_mask.reserve(1u << 20) && c->feas_stage.reserve(1u << 16) && c->d_feas_stage.reserve(1u << 16);
     if (!ok || cudaMalloc((void **)&c->d_prof, sizeof(DevProfile)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_prof53, sizeof(DevProfile)) != cudaSuccess) {
         if (c->d_prof) cudaFree(c->d_prof);

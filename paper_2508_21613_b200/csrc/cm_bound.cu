@@ -6,7 +6,7 @@
 //                      the strategies that can reach them
 //   cm_refine_kernel   compares plans whose bounds tie, bit for bit (cm_refine.cu)
 //   cm_gather_kernel   lists the most promising plan of every segment needed
-//   cm_list_kernel     the recurrence on the listed plans
+//   cm_list_*_kernel   the recurrence on the listed plans
 //
 // The sequence is: bounds -> window from the bounds -> refine (phase 1) -> gather -> recurrence ->
 // window from the results -> refine (phase 2) -> recurrence.  Phase 1 is optimistic: it assumes that a
@@ -34,24 +34,20 @@ namespace cm {
 // holds the bucket's candidates, at most all threads), and walks its group of segments with the
 // composition's terms in registers.
 template <typename T, int NB, bool UNI_X>
-__device__ void bound_body(const SProf<T> &sp, const Tables &tb, const BatchDev &bd, const BoundDev &bo, const BBucket &bk,
-                           uint64_t tile0, const SegLite *segs, int n_seg, unsigned long long *seg_min, unsigned char *dyn) {
+__device__ void bound_body(const SProf<T> &sp, const Tables &tb, const BatchDev &bd, const BBucket &bk, uint64_t tile0, int n_seg,
+                           const BoundSmem &sm) {
     const int S = bk.S, m = bk.m, W = bk.width;
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     const int sub = tid / W, n_sub = kBoundThreads / W;
-    float *xs = reinterpret_cast<float *>(dyn);                                            // [n_seg][4 NB] (UNI_X)
-    float *cc = reinterpret_cast<float *>(dyn + bo.dyn_cols) + tid;                        // [S][threads]
-    float *dd = cc + S * kBoundThreads;
-    uint8_t *cutc = dyn + bo.dyn_cols + sizeof(float) * 2 * S * kBoundThreads + tid;
-    const float x1 = __double2float_rd((double)sp.XT[1][0]);
-    if (UNI_X) fill_transfers<T, NB>(xs, sp, S, segs, n_seg);
+    if (UNI_X) fill_transfers<T, NB>(sm, sp, S, m, n_seg);
     const uint64_t pos = tile0 + (tid & (W - 1));
     LaneBound<NB> v;
     v.ok = pos < bk.count;
     if (v.ok) {
         CutWalker w;
-        v.ok = make_walker(w, tb, bd.layer_mode, sp.L, S, walk_kappa(bd.feas, bk.feas_first, pos), bk.K, tb.mm_slot(S, m));
-        if (v.ok) lane_setup<T, NB, UNI_X>(v, sp, cut_edges(w), S, m, bk.feas_first == kNoFeasList, cc, dd, cutc);
+        const CutColumn<kBoundThreads> cuts{sm.cut};
+        v.ok = make_walker(w, tb, bd.layer_mode, sp.L, S, walk_cand(bd, bk.feas_first, pos), bk.K, tb.mm_slot(S, m)) && cuts.fill(w, S);
+        if (v.ok) lane_setup<T, NB, UNI_X>(v, sp, cuts, S, m, bk.feas_first == kNoFeasList, sm.cd);
     }
     const int n_ok = __syncthreads_count(v.ok && sub == 0);
     if (tid == 0 && n_ok) {   // what this pass decides: the plans, and the cells recurrences over them would take
@@ -63,23 +59,23 @@ __device__ void bound_body(const SProf<T> &sp, const Tables &tb, const BatchDev 
     }
     const float slack = sp.intval || std::is_same<T, long long>::value ? 1.0f : 0.0f;
     const int n_it = (n_seg + n_sub - 1) / n_sub;
+    const float none = __uint_as_float(0x7f800000u);
+#pragma unroll 2
     for (int it = 0; it < n_it; ++it) {
         const int s = it * n_sub + sub;
-        const bool have = s < n_seg && v.ok;
-        float lb = __uint_as_float(0x7f800000u);
-        if (have) lb = lane_value<T, NB, UNI_X>(v, sp, S, m, segs[s], xs + s * 4 * NB, x1, slack, cc, dd, cutc);
-        if (W >= 32) {   // (the lanes of a warp share the segment)
-            const uint32_t mine = __float_as_uint(lb), least = __reduce_min_sync(0xffffffffu, mine);
-            const uint32_t who = __ballot_sync(0xffffffffu, mine == least);
-            if (have && lane == (uint32_t)(__ffs(who) - 1))
-                atomicMin(&seg_min[s], ((unsigned long long)mine << 32) | (uint32_t)pos);
+        const float value = s < n_seg && v.ok ? lane_value<T, NB, UNI_X>(v, sp, S, m, s, sm) : none;
+        if (W >= 32) {   // (the lanes of a warp share the segment; one lane works on its minimum)
+            const float least = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(value)));   // (values are not negative)
+            const uint32_t who = __ballot_sync(0xffffffffu, value == least);
+            if (least < none && lane == (uint32_t)(__ffs(who) - 1))
+                sm.word[4 * s + (tid >> 5)] = ((unsigned long long)__float_as_uint(bound_of(value, slack)) << 32) | (uint32_t)pos;
         } else {
-            unsigned long long key = have ? ((unsigned long long)__float_as_uint(lb) << 32) | (uint32_t)pos : ~0ull;
+            unsigned long long key = value < none ? ((unsigned long long)__float_as_uint(bound_of(value, slack)) << 32) | (uint32_t)pos : ~0ull;
             for (int o = W >> 1; o > 0; o >>= 1) {
                 const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
                 key = k2 < key ? k2 : key;
             }
-            if (s < n_seg && (tid & (W - 1)) == 0 && key != ~0ull) seg_min[s] = key;   // the only writer of its segment
+            if (s < n_seg && (tid & (W - 1)) == 0 && key != ~0ull) sm.word[4 * s] = key;   // the only writer of its segment
         }
     }
 }
@@ -95,35 +91,49 @@ __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, Batc
     __syncthreads();
     const BBucket &bk = bks;
     const BoundJob job = bound_job(bk, blockIdx.x);
-    SegLite *segs = reinterpret_cast<SegLite *>(dyn + bo.dyn_segs);
-    unsigned long long *seg_min = reinterpret_cast<unsigned long long *>(dyn + bo.dyn_segs + sizeof(SegLite) * bo.max_group);
+    const BoundSmem sm = bound_smem(dyn, bo);
     const int n_seg = (int)(job.s1 - job.s0);
     for (int q = tid; q < n_seg; q += kBoundThreads) {
-        segs[q] = seg_lite(tb, bound_segment(bd, bk, job.s0 + q));
-        seg_min[q] = ~0ull;
+        sm.segs[q] = seg_lite(tb, bound_segment(bd, bk, job.s0 + q));
+        for (int w = 0; w < 4; ++w) sm.word[4 * q + w] = ~0ull;   // a word per warp
     }
     __syncthreads();
     const int nb = (bk.S + 3) >> 2;
-#define CM_NB(K) if (nb <= K) bound_body<T, K, UNI_X>(sp, tb, bd, bo, bk, job.tile0, segs, n_seg, seg_min, dyn); else
+#define CM_NB(K) if (nb <= K) bound_body<T, K, UNI_X>(sp, tb, bd, bk, job.tile0, n_seg, sm); else
     if constexpr (UNI_X && std::is_same<T, double>::value) { CM_NB(1) CM_NB(2) CM_NB(3) CM_NB(4) CM_NB(6) CM_NB(8) CM_NB(9) CM_NB(12) CM_NB(16) {} }
     else { CM_NB(4) CM_NB(9) CM_NB(16) {} }
 #undef CM_NB
     __syncthreads();
-    for (int q = tid; q < n_seg; q += kBoundThreads)
-        if (seg_min[q] < bo.lbarg[segs[q].row]) atomicMin((unsigned long long *)&bo.lbarg[segs[q].row], seg_min[q]);
+    for (int q = tid; q < n_seg; q += kBoundThreads) {
+        unsigned long long least = sm.word[4 * q];
+        for (int w = 1; w < 4; ++w) least = sm.word[4 * q + w] < least ? sm.word[4 * q + w] : least;
+        if (least < bo.lbarg[sm.segs[q].row]) atomicMin((unsigned long long *)&bo.lbarg[sm.segs[q].row], least);
+    }
 }
 
+// Segments a CTA walks with one set of compositions, and the layout of its shared memory.  Three CTAs per
+// SM are wanted up to 36 stages; a deeper pipeline's columns alone take a third of an SM.
+int bound_group(int max_stages, bool uniform_x) {
+    BoundDev bo{};
+    const size_t fixed = bound_dyn_bytes(bo, max_stages, 0, uniform_x), per = (bound_dyn_bytes(bo, max_stages, 1024, uniform_x) - fixed) / 1024;
+    const size_t target = std::max<size_t>(kBoundDynTarget, fixed + 16 * 1024);
+    return (int)std::min<size_t>(255, std::max<size_t>(16, (target - fixed) / std::max<size_t>(per, 1)));
+}
 size_t bound_dyn_bytes(BoundDev &bo, int max_stages, int max_group, bool uniform_x) {
     size_t nb = (size_t)(max_stages + 3) / 4;
     for (size_t k : kBoundNb)
         if (nb <= k) { nb = k; break; }
-    size_t off = uniform_x ? (size_t)max_group * 16 * nb : 0;
+    const size_t n = (size_t)max_group, columns = (size_t)max_stages * kBoundThreads;
+    size_t off = uniform_x ? n * 16 * nb : 0;
+    bo.dyn_far = (uint32_t)off;
+    off += uniform_x ? n * kFarMax * sizeof(FarVisit) : 0;
     bo.dyn_cols = (uint32_t)off;
-    off += sizeof(float) * 2 * max_stages * kBoundThreads + (uniform_x ? 0 : (size_t)max_stages * kBoundThreads);
-    off = (off + 15) & ~(size_t)15;
+    off += columns * sizeof(float2);
+    bo.dyn_cuts = (uint32_t)off;
+    off += columns;
     bo.dyn_segs = (uint32_t)off;
     bo.max_group = (uint32_t)max_group;
-    return off + (size_t)max_group * (sizeof(SegLite) + sizeof(unsigned long long));
+    return off + n * (sizeof(SegLite) + sizeof(unsigned long long) + kRefineSegBytes);   // (cm_bound_kernel: four words, nothing else)
 }
 
 template <typename T, bool UNI_X>
@@ -144,14 +154,14 @@ cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo,
 // pipelines, every choice of them a split, so its best step time is the least value t among its
 // pipelines' two costs such that those that cannot do with their smaller share (cost above t) number
 // at most R, all pipelines that can take the larger one (cost at most t) number at least R, and the
-// former are among the latter; C(may - must, R - must) splits then stay within t.  A thread per
+// former are among the latter; C(may - must, R - must) splits then stay within t.  A warp per
 // strategy; phase 0 works on the bounds, phase 1 on the results.  Either then marks the segments of the
 // strategies whose step time from bounds is still within reach.
 // ----------------------------------------------------------------------------------
-struct StratCosts { uint64_t lo[kMaxP], hi[kMaxP]; int dp, R; };
 // Phase 0 marks strategies this far above the best step time from bounds: one plan of each of their
 // segments is evaluated, so that a result that misses its bound a little still leaves phase 2 nothing to do.
 constexpr float kReach = 1.0f / (1 << 13);
+constexpr int kWinThreads = 128;
 
 __device__ __forceinline__ uint32_t canon_row(const BatchDev &bd, const Tmpl &tp, const Scen &sc, const Strat &s, int p, int k) {
     uint32_t t = s.seg_first + p * s.n_m + k;
@@ -159,51 +169,63 @@ __device__ __forceinline__ uint32_t canon_row(const BatchDev &bd, const Tmpl &tp
     return sc.seg_base + (t - tp.tseg_first);
 }
 
-__device__ __forceinline__ void strat_costs(const BatchDev &bd, const BoundDev &bo, const Tmpl &tp, const Scen &sc, uint32_t si, int phase,
-                                            uint64_t inf, StratCosts &c) {
-    const Strat &s = bd.strat[tp.strat_first + si];
-    c.dp = s.dp;
-    c.R = s.R;
-    for (int p = 0; p < s.dp; ++p)
-        for (int k = 0; k < 2; ++k) {
-            uint64_t v = inf;
-            if (k < s.n_m && s.m_lo[p] + k >= 1) {
-                const uint32_t row = canon_row(bd, tp, sc, s, p, k);
-                v = phase ? bd.seg_best[row] : (uint64_t)(bo.lbarg[row] >> 32);
-                v = v > inf ? inf : v;
-            }
-            (k ? c.hi : c.lo)[p] = v;
-        }
+// The two costs of every pipeline of a strategy, a lane each: lane 2p + k holds pipeline p with its
+// smaller (k = 0) or larger share (2 kMaxP = 32 lanes).
+__device__ __forceinline__ uint64_t strat_cost(const BatchDev &bd, const BoundDev &bo, const Tmpl &tp, const Scen &sc, const Strat &s,
+                                               int phase, uint64_t inf) {
+    const int p = (threadIdx.x & 31) >> 1, k = threadIdx.x & 1;
+    uint64_t v = inf;
+    if (p < s.dp && k < s.n_m && s.m_lo[p] + k >= 1) {
+        const uint32_t row = canon_row(bd, tp, sc, s, p, k);
+        v = phase ? bd.seg_best[row] : (uint64_t)(bo.lbarg[row] >> 32);
+    }
+    return v < inf ? v : inf;
 }
 
-__device__ __forceinline__ bool splits_within(const StratCosts &c, uint64_t t, int &free_ones, int &left) {
+// Is there a split of the strategy within this lane's t, and how many?
+__device__ __forceinline__ bool splits_within(uint64_t v, int dp, int R, uint64_t t, int &free_ones, int &left) {
     int may = 0, must = 0;
     bool ok = true;
-    for (int p = 0; p < c.dp; ++p) {
-        const bool can = c.hi[p] <= t, need = c.lo[p] > t;
+    for (int p = 0; p < dp; ++p) {
+        const bool need = __shfl_sync(0xffffffffu, v, 2 * p) > t, can = __shfl_sync(0xffffffffu, v, 2 * p + 1) <= t;
         may += can;
         must += need;
         ok = ok && (can || !need);
     }
     free_ones = may - must;
-    left = c.R - must;
-    return ok && left >= 0 && may >= c.R;
+    left = R - must;
+    return ok && left >= 0 && may >= R;
 }
 
-__device__ __forceinline__ uint64_t strat_best(const StratCosts &c, uint64_t after, uint64_t inf) {   // least t > after (after = ~0: any)
-    uint64_t best = inf;
-    int f, l;
-    for (int p = 0; p < c.dp; ++p)
-        for (int k = 0; k < 2; ++k) {
-            const uint64_t t = k ? c.hi[p] : c.lo[p];
-            if (t < best && (after == ~0ull || t > after) && splits_within(c, t, f, l)) best = t;
+// Least step time above `after` (~0: any) of a strategy, in every lane.
+__device__ __forceinline__ uint64_t strat_best(uint64_t v, const Strat &s, uint64_t after, uint64_t inf) {
+    const int lane = threadIdx.x & 31, dp = s.dp, R = s.R;
+    const bool mine = lane < 2 * dp;
+    if (after == ~0ull) {
+        // Where no pipeline is cheaper with the larger share (always so for bounds, and for results that
+        // are all there): everybody's smaller share, and the R cheapest larger ones.
+        const uint64_t other = __shfl_xor_sync(0xffffffffu, v, 1);
+        if (!R || __all_sync(0xffffffffu, !mine || (lane & 1 ? v >= other : v <= other))) {
+            uint64_t t = ~warp_min_u64(mine && !(lane & 1) ? ~v : ~0ull);   // largest of the smaller shares
+            if (R) {
+                int below = 0;
+                for (int p = 0; p < dp; ++p) {
+                    const uint64_t h = __shfl_sync(0xffffffffu, v, 2 * p + 1);
+                    below += h < v || (h == v && 2 * p + 1 < lane);
+                }
+                const uint32_t who = __ballot_sync(0xffffffffu, mine && (lane & 1) && below == R - 1);
+                const uint64_t at = who ? __shfl_sync(0xffffffffu, v, __ffs(who) - 1) : inf;
+                t = at > t ? at : t;
+            }
+            return t;
         }
-    return best;
+    }
+    int f, l;
+    const bool ok = splits_within(v, dp, R, v, f, l) && mine && v < inf && (after == ~0ull || v > after);
+    return warp_min_u64(ok ? v : inf);
 }
 
-constexpr int kWinThreads = 128;
-__device__ __forceinline__ uint64_t block_min_u64(uint64_t v, uint64_t *red) {
-    v = warp_min_u64(v);
+__device__ __forceinline__ uint64_t block_min_u64(uint64_t v /* warp-uniform */, uint64_t *red) {
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -217,15 +239,16 @@ __global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, Batch
     const uint32_t b = blockIdx.x;
     const Scen sc = bd.scen[b];
     const Tmpl tp = bd.tmpl[sc.tmpl];
+    const Strat *strat = bd.strat + tp.strat_first;
+    const uint32_t warp = threadIdx.x >> 5, warps = kWinThreads / 32;
+    const int lane = threadIdx.x & 31;
     const uint64_t inf = phase ? inf_cost : 0xffffffffull;
     uint64_t first = ~0ull, t = ~0ull;
     bool enough = false;
     for (int r = 0; r < k_best && !enough; ++r) {
         uint64_t mine = inf;
-        for (uint32_t si = threadIdx.x; si < tp.n_strat; si += kWinThreads) {
-            StratCosts c;
-            strat_costs(bd, bo, tp, sc, si, phase, inf, c);
-            const uint64_t v = strat_best(c, t, inf);
+        for (uint32_t si = warp; si < tp.n_strat; si += warps) {
+            const uint64_t v = strat_best(strat_cost(bd, bo, tp, sc, strat[si], phase, inf), strat[si], t, inf);
             mine = v < mine ? v : mine;
         }
         t = block_min_u64(mine, red);
@@ -233,14 +256,11 @@ __global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, Batch
         if (t >= inf || k_best == 1) break;
         if (threadIdx.x == 0) total = 0;
         __syncthreads();
-        unsigned long long n = 0;
-        for (uint32_t si = threadIdx.x; si < tp.n_strat; si += kWinThreads) {
-            StratCosts c;
+        for (uint32_t si = warp; si < tp.n_strat; si += warps) {
             int f, l;
-            strat_costs(bd, bo, tp, sc, si, phase, inf, c);
-            if (splits_within(c, t, f, l)) n += binom_at(tb.binom, f, l);
+            const bool ok = splits_within(strat_cost(bd, bo, tp, sc, strat[si], phase, inf), strat[si].dp, strat[si].R, t, f, l);
+            if (ok && lane == 0) atomicAdd(&total, (unsigned long long)binom_at(tb.binom, f, l));
         }
-        if (n) atomicAdd(&total, n);
         __syncthreads();
         enough = total >= (unsigned long long)k_best;
         __syncthreads();
@@ -248,24 +268,25 @@ __global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, Batch
     if (k_best > 1 && !enough && t < inf) t = inf;
     float reach = -1.0f;   // step times from bounds up to here (-1: none)
     if (phase) {
-        if (t < ~0ull) reach = __double2float_ru(cost_up(t, native_i64_dev(bd)));
+        reach = __double2float_ru(cost_up(t, native_i64_dev(bd)));
+        const float marked = bo.win[b].reach;
+        __syncthreads();
         if (threadIdx.x == 0) bo.win[b].ub = t;
+        if (reach <= marked) return;   // (uniform) phase 0 has marked them all: the results came out as promised
     } else {
         const float lo = first < inf ? __uint_as_float((uint32_t)first) : 0.0f;
         if (first < inf) reach = t < inf ? __fmul_ru(__uint_as_float((uint32_t)t), 1.0f + kReach) : __uint_as_float(0x7f800000u);
-        if (threadIdx.x == 0) bo.win[b] = SearchWin{lo, 0.0f, inf_cost};
+        if (threadIdx.x == 0) bo.win[b] = SearchWin{lo, reach, inf_cost};
     }
-    for (uint32_t si = threadIdx.x; si < tp.n_strat; si += kWinThreads) {
-        StratCosts c;
-        strat_costs(bd, bo, tp, sc, si, 0, 0xffffffffull, c);
-        const uint64_t v = strat_best(c, ~0ull, 0xffffffffull);
-        if (v >= 0xffffffffull || __uint_as_float((uint32_t)v) > reach) continue;
-        const Strat &s = bd.strat[tp.strat_first + si];
-        for (int p = 0; p < s.dp; ++p)
-            for (int k = 0; k < s.n_m; ++k) {
-                const uint32_t row = canon_row(bd, tp, sc, s, p, k);
-                if (bo.pick[row] == ~0ull) bo.pick[row] = kPickWanted;   // (every writer writes the same)
-            }
+    for (uint32_t si = warp; si < tp.n_strat; si += warps) {
+        const Strat &s = strat[si];
+        const uint64_t v = strat_best(strat_cost(bd, bo, tp, sc, s, 0, 0xffffffffull), s, ~0ull, 0xffffffffull);
+        if (v >= 0xffffffffull || __uint_as_float((uint32_t)v) > reach) continue;   // warp-uniform
+        const int p = lane >> 1, k = lane & 1;
+        if (p < s.dp && k < s.n_m) {
+            const uint32_t row = canon_row(bd, tp, sc, s, p, k);
+            if (bo.pick[row] == ~0ull) bo.pick[row] = kPickWanted;   // (every writer writes the same)
+        }
     }
 }
 
@@ -303,53 +324,84 @@ cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo
 // ----------------------------------------------------------------------------------
 // The recurrence on the listed plans.  Pipelines of at most 16 stages: a thread per plan, state in
 // registers; deeper ones: a warp per plan in lock step, 2(S+m) slots of ~45 cycles (a thread would
-// need ~100 us for its chain of 2 S m cells, and the lists are short).  Even CTAs take the shallow
-// list, odd ones the deep one.
+// need ~100 us for its chain of 2 S m cells, and the lists are short).
 // ----------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kChunk) cm_list_kernel(Tables tb, BatchDev bd, BoundDev bo, int first_list) {
-    __shared__ SProf<T> sp;
-    __shared__ uint8_t cuts_s[kChunk / 32][kMaxS + 8];
-    const bool deep = blockIdx.x & 1;
-    const uint32_t cta = blockIdx.x >> 1, ctas = gridDim.x >> 1;
-    const int list = first_list + (deep ? 1 : 0);
-    const uint32_t room = bo.list_first[list + 1] - bo.list_first[list];
-    uint32_t n = bo.count[list] + 1u;
-    n = n < room ? n : room;
-    const uint32_t per = deep ? kChunk / 32 : kChunk;
-    if ((uint64_t)cta * per >= n) return;
-    stage_profile(sp, tb);
-    __syncthreads();
-    const uint4 *entries = bo.list + bo.list_first[list];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long work = 0;   // cells in the low 40 bits, plans above
-    for (uint32_t i = cta * per + (deep ? warp : threadIdx.x); i < n; i += ctas * per) {
-        const uint4 e = entries[i];
-        const SegView g = seg_view(bd, e.x, e.y);
-        const uint64_t kappa = walk_kappa(bd.feas, g.feas_first, e.z);
-        T cost;
-        bool ok;
-        if (deep) ok = warp_plan_cost<T>(sp, tb, bd.layer_mode, g, kappa, cuts_s[warp], cost);
-        else if (g.m >= g.S - 1) ok = plan_cost_regs_any<T>(sp, tb, bd.layer_mode, g, kappa, cost);
-        else ok = plan_cost_regs_any<T, true>(sp, tb, bd.layer_mode, g, kappa, cost);
-        if (deep && lane) continue;
-        if (ok) {
-            const uint64_t bits = Num<T>::bits(cost);
-            if (bits < bd.seg_best[g.row]) atomicMin((unsigned long long *)&bd.seg_best[g.row], (unsigned long long)bits);
-        }
-        work += 2ull * g.S * g.m + (1ull << 40);
-    }
+__device__ __forceinline__ uint32_t list_length(const BoundDev &bo, int list) {
+    const uint32_t n = bo.count[list] + 1u, room = bo.list_first[list + 1] - bo.list_first[list];
+    return n < room ? n : room;
+}
+template <typename T> __device__ __forceinline__ void list_commit(const BatchDev &bd, uint32_t row, T cost) {
+    const uint64_t bits = Num<T>::bits(cost);
+    if (bits < bd.seg_best[row]) atomicMin((unsigned long long *)&bd.seg_best[row], (unsigned long long)bits);
+}
+// work: cells in the low 40 bits, plans above
+__device__ __forceinline__ void count_list_work(const BatchDev &bd, unsigned long long work) {
     for (int o = 16; o > 0; o >>= 1) work += __shfl_xor_sync(0xffffffffu, work, o);
-    if (lane == 0 && work) {
+    if ((threadIdx.x & 31) == 0 && work) {
         atomicAdd(&bd.counters[3], work & ((1ull << 40) - 1ull));
         atomicAdd(&bd.counters[5], work >> 40);
     }
 }
 
-cudaError_t launch_list(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, uint64_t most, cudaStream_t st) {
-    const unsigned grid = 2 * (unsigned)std::min<uint64_t>(std::max<uint64_t>((most + 3) / 4, 1), 148 * 6);
-    if (native_i64(b)) cm_list_kernel<long long><<<grid, kChunk, 0, st>>>(t, b, bo, first_list);
-    else cm_list_kernel<double><<<grid, kChunk, 0, st>>>(t, b, bo, first_list);
+template <typename T>
+__global__ void __launch_bounds__(kChunk) cm_list_shallow_kernel(Tables tb, BatchDev bd, BoundDev bo, int list) {
+    __shared__ SProf<T> sp;
+    const uint32_t n = list_length(bo, list);
+    if ((uint64_t)blockIdx.x * kChunk >= n) return;
+    stage_profile(sp, tb);
+    __syncthreads();
+    const uint4 *entries = bo.list + bo.list_first[list];
+    unsigned long long work = 0;
+    for (uint32_t i = blockIdx.x * kChunk + threadIdx.x; i < n; i += gridDim.x * kChunk) {
+        const uint4 e = entries[i];
+        const SegView g = seg_view(bd, e.x, e.y);
+        const Cand cand = walk_cand(bd, g.feas_first, e.z);
+        T cost;
+        const bool ok = g.m >= g.S - 1 ? plan_cost_regs_any<T>(sp, tb, bd.layer_mode, g, cand, cost)
+                                       : plan_cost_regs_any<T, true>(sp, tb, bd.layer_mode, g, cand, cost);
+        if (ok) list_commit<T>(bd, g.row, cost);
+        work += 2ull * g.S * g.m + (1ull << 40);
+    }
+    count_list_work(bd, work);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kChunk, 5) cm_list_deep_kernel(Tables tb, BatchDev bd, BoundDev bo, int list) {
+    __shared__ SProf<T> sp;
+    __shared__ uint8_t cuts_s[kChunk / 32][kMaxS + 8];
+    const uint32_t n = list_length(bo, list);
+    if ((uint64_t)blockIdx.x * (kChunk / 32) >= n) return;
+    stage_profile(sp, tb);
+    __syncthreads();
+    const uint4 *entries = bo.list + bo.list_first[list];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long work = 0;
+    for (uint32_t i = blockIdx.x * (kChunk / 32) + warp; i < n; i += gridDim.x * (kChunk / 32)) {
+        const uint4 e = entries[i];
+        const SegView g = seg_view(bd, e.x, e.y);
+        T cost;
+        if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, walk_cand(bd, g.feas_first, e.z), cuts_s[warp], cost) && lane == 0)
+            list_commit<T>(bd, g.row, cost);
+        if (lane == 0) work += 2ull * g.S * g.m + (1ull << 40);
+    }
+    count_list_work(bd, work);
+}
+
+cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches) {
+    const uint64_t shallow = bo.list_first[first_list + 1] - bo.list_first[first_list];
+    const uint64_t deep = bo.list_first[first_list + 2] - bo.list_first[first_list + 1];
+    if (shallow) {
+        const unsigned grid = (unsigned)std::min<uint64_t>((shallow + kChunk - 1) / kChunk, 148 * 4);
+        if (native_i64(b)) cm_list_shallow_kernel<long long><<<grid, kChunk, 0, st>>>(t, b, bo, first_list);
+        else cm_list_shallow_kernel<double><<<grid, kChunk, 0, st>>>(t, b, bo, first_list);
+        ++*launches;
+    }
+    if (deep) {
+        const unsigned grid = (unsigned)std::min<uint64_t>((deep + kChunk / 32 - 1) / (kChunk / 32), 148 * 5);
+        if (native_i64(b)) cm_list_deep_kernel<long long><<<grid, kChunk, 0, st>>>(t, b, bo, first_list + 1);
+        else cm_list_deep_kernel<double><<<grid, kChunk, 0, st>>>(t, b, bo, first_list + 1);
+        ++*launches;
+    }
     return cudaGetLastError();
 }
 

@@ -35,30 +35,25 @@ namespace cm {
 // has at most 2 (m + S) <= 8320 additions of one rounding each (2^-53), on either side.
 constexpr double kBoundSlack = 1.0 - 1.0 / (1ull << 36);
 
-// Layer cuts of a plan, any of them in O(1) or nearly: edge(i) = first layer of stage i, edge(S) = L.
-struct CutEdges {
-    uint64_t a, b;
-    const uint8_t *row;
-    int kind, q, L, S;
-    static __device__ __forceinline__ int select(uint64_t v, int n) {   // position of set bit number n (from 0)
-        int at = 0;
-        for (int w = 32; w; w >>= 1) {
-            const int c = __popcll((v >> at) & ((1ull << w) - 1ull));
-            if (n >= c) { n -= c; at += w; }
+// Layer cuts of a plan in a shared-memory column, one byte per stage, a plan per thread:
+// edge(i) = first layer of stage i, edge(S) = L.
+template <int STRIDE> struct CutColumn {
+    uint8_t *col;   // col[i * STRIDE] = upper cut of stage i
+    __device__ __forceinline__ int edge(int i) const { return i ? col[(i - 1) * STRIDE] : 0; }
+    // Returns false if a stage would be empty.
+    __device__ __forceinline__ bool fill(CutWalker w, int S) const {
+        bool ok = true;
+        int lo = 0;
+#pragma unroll 4
+        for (int i = 0; i < S; ++i) {
+            const int hi = w.next();
+            col[i * STRIDE] = (uint8_t)hi;
+            ok = ok && hi > lo;
+            lo = hi;
         }
-        return at;
-    }
-    __device__ __forceinline__ int edge(int i) const {
-        if (i == S) return L;
-        if (kind == 0) return q * i + __popcll(a & ((1ull << i) - 1ull));
-        if (kind == 2) return row[i];
-        if (i == 0) return 0;
-        const int na = __popcll(a);
-        return i <= na ? select(a, i - 1) + 1 : 64 + select(b, i - 1 - na) + 1;
+        return ok;
     }
 };
-
-__device__ __forceinline__ CutEdges cut_edges(const CutWalker &w) { return CutEdges{w.a, w.b, w.row, w.kind, w.q, w.L, w.S}; }
 
 // The best walk of a plan and its value (synchronisation included), in double arithmetic for either
 // cost type; value -1 if the plan does not fit in memory (looked at only where no feasible list
@@ -70,8 +65,8 @@ struct Walk {
     int a, kind, d;     // stage it stays at; what it does there; (kWalkAfab: the stage of the backwards)
 };
 
-template <typename T>
-__device__ __forceinline__ Walk best_walk(const SProf<T> &s, const CutEdges &c, int S, int m, uint64_t tier, int n_sync, bool check) {
+template <typename T, typename Cuts>
+__device__ __forceinline__ Walk best_walk(const SProf<T> &s, const Cuts &c, int S, int m, uint64_t tier, int n_sync, bool check) {
     const bool gpipe = s.sched == CM_SCHED_GPIPE;
     double U = 0.0, best = -1.0, fmax = -1.0, bmax = -1.0;
     double base_n = 0.0, w_n = 0.0, q_n = 0.0;   // stage i+1: the value of its own walk (without U_0), w, pairs of stays
@@ -79,8 +74,9 @@ __device__ __forceinline__ Walk best_walk(const SProf<T> &s, const CutEdges &c, 
     long long g_max = 0;
     int hi = s.L;
     auto take = [&](double v, int at, int k) { if (v > best) { best = v; a = at; kind = k; } };
+#pragma unroll 2
     for (int i = S - 1; i >= 0; --i) {
-        const int lo = i ? c.edge(i) : 0;
+        const int lo = c.edge(i);
         if (check && (hi <= lo || !stage_fits(s.PS[hi] - s.PS[lo], s.PA[hi] - s.PA[lo], i, S, m, s.cap, s.sched)))
             return Walk{-1.0, 0, 0, 0, 0};
         const double f = (double)(s.PF[hi] - s.PF[lo]), bk = (double)(s.PB[hi] - s.PB[lo]), wi = f + bk;
@@ -118,36 +114,36 @@ __device__ __forceinline__ Walk best_walk(const SProf<T> &s, const CutEdges &c, 
 
 // Cost along the walk in the arithmetic and the order of the recurrence: a lower bound of the plan's
 // computed cost, bit for bit.
-template <typename T>
-__device__ __forceinline__ T walk_cost(const SProf<T> &s, const CutEdges &c, int S, int m, uint64_t tier, int n_sync, const Walk &w) {
+template <typename T, typename Cuts>
+__device__ __forceinline__ T walk_cost(const SProf<T> &s, const Cuts &c, int S, int m, uint64_t tier, int n_sync, const Walk &w) {
     T t = (T)0;
-    auto climb = [&](int from, bool first) {   // forwards of stages from .. S-1; `first`: repeated ones on the way
+    // forwards of stages from .. to-1, each with the transfer above it; backwards of stages from .. to,
+    // each with the transfer above it first.  (The additions are one dependent chain; the loads are not.)
+    auto climb = [&](int from, int to) {
         int lo = c.edge(from);
-        for (int i = from; i < S; ++i) {
+#pragma unroll 4
+        for (int i = from; i < to; ++i) {
             const int hi = c.edge(i + 1);
-            const T f = s.PF[hi] - s.PF[lo];
-            const int times = first && i == w.a && (w.kind == kWalkForward || w.kind == kWalkAfab) ? m : 1;
-            for (int k = 0; k < times; ++k) t = t + f;
+            t = t + (s.PF[hi] - s.PF[lo]);
             if (i < S - 1) t = t + s.XT[(tier >> i) & 1ull][hi - 1];
             lo = hi;
         }
     };
-    auto drop = [&](int to, bool last) {       // backwards of stages S-1 .. to; `last`: repeated ones on the way
-        int hi = s.L;
-        for (int i = S - 1; i >= to; --i) {
+    auto drop = [&](int from, int to) {
+        int hi = c.edge(from + 1);
+#pragma unroll 4
+        for (int i = from; i >= to; --i) {
             const int lo = c.edge(i);
-            const T bk = s.PB[hi] - s.PB[lo];
             if (i < S - 1) t = t + s.XT[(tier >> i) & 1ull][hi - 1];
-            const int times = last && ((w.kind == kWalkBackward && i == w.a) || (w.kind == kWalkAfab && i == w.d)) ? m : 1;
-            for (int k = 0; k < times; ++k) t = t + bk;
+            t = t + (s.PB[hi] - s.PB[lo]);
             hi = lo;
         }
     };
-    climb(0, true);
+    const int a = w.a, lo = c.edge(a), hi = c.edge(a + 1);
+    const T f = s.PF[hi] - s.PF[lo], bk = s.PB[hi] - s.PB[lo];
     if (w.kind <= kWalkDown) {
-        const int a = w.a, lo = c.edge(a), hi = c.edge(a + 1);
-        drop(a, false);
-        const T f = s.PF[hi] - s.PF[lo], bk = s.PB[hi] - s.PB[lo];
+        climb(0, S);
+        drop(S - 1, a);
         int n = m - 1 + a - S;
         if (w.kind == kWalkUp) {
             const int hi2 = c.edge(a + 2);
@@ -159,9 +155,19 @@ __device__ __forceinline__ T walk_cost(const SProf<T> &s, const CutEdges &c, int
             for (; n > 1; n -= 2) t = ((((((t + x) + b2) + f2) + x) + f) + bk);
         }
         for (; n > 0; --n) t = (t + f) + bk;
-        climb(a, false);
+        climb(a, S);
+        drop(S - 1, 0);
+    } else {
+        const bool forwards = w.kind != kWalkBackward, backwards = w.kind != kWalkForward;
+        climb(0, a);
+        for (int k = forwards ? m - 1 : 0; k > 0; --k) t = t + f;
+        climb(a, S);
+        const int d = w.kind == kWalkAfab ? w.d : a, dlo = c.edge(d), dhi = c.edge(d + 1);
+        const T db = s.PB[dhi] - s.PB[dlo];
+        drop(S - 1, d);
+        for (int k = backwards ? m - 1 : 0; k > 0; --k) t = t + db;
+        if (d > 0) drop(d - 1, 0);
     }
-    drop(0, true);
     return t + Num<T>::sync(w.g_max, n_sync, s.bw_sync, s.intval);
 }
 

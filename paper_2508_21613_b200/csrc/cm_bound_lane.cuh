@@ -9,20 +9,40 @@ namespace cm {
 // Bounds of whole buckets are floats rounded down: the per-plan inner loop costs one addition and one
 // maximum per stage at full rate (in double arithmetic an addition and a compare-and-select take six
 // issue slots).
-constexpr float kFloatSlack = 1.0f - 1.0f / (1 << 23);
+constexpr float kFloatSlack = 1.0f - 1.0f / (1 << 22);
 constexpr float kTieWindow = 1.0f / (1 << 18);     // bounds this close to the least one of a segment are compared bit for bit
 constexpr int kBoundThreads = 128;
 constexpr float kNoWalk = -__builtin_huge_valf();   // value of a walk that does not exist
 
-struct SegLite {
-    uint64_t tier;
-    uint64_t lim_bits;   // phase 2: list a plan whose walk costs at most this
-    double lim;          // phases 1, 2: look at plans whose bound is at most lim ...
-    float ev;            //   ... and above ev (what phase 1 has settled already)
-    float coef;          // synchronisation time per gradient byte
-    uint32_t scen, tseg, row;
-    int n_sync;
+// What the bound of a segment needs: its link tiers, its row, the synchronisation time per gradient byte,
+// how many of its inter-node boundaries are in the list of visits (kFarLong: too many, see lane_value).
+struct SegLite { uint64_t tier; uint32_t row; float coef; int n_sync, n_far; };
+// A visit across an inter-node boundary between stages `at` and at+1: what it adds to the lane's terms.
+struct FarVisit { float up, down; int at, pad; };
+constexpr int kFarMax = 6, kFarLong = kFarMax + 1;
+// Shared memory of a bound CTA, in this order: transfers above every stage [group][4 NB] floats (UNI_X) |
+// visits [group][kFarMax] (UNI_X) | visit terms [stages][threads] float2 | cuts [stages][threads] bytes |
+// segments [group] | a 64-bit word per segment | what else the kernel keeps per segment.
+struct BoundSmem {
+    float *xs;
+    FarVisit *far;
+    float2 *cd;       // this thread's column
+    uint8_t *cut;     // this thread's column
+    SegLite *segs;
+    unsigned long long *word;
+    unsigned char *rest;
 };
+__device__ __forceinline__ BoundSmem bound_smem(unsigned char *dyn, const BoundDev &bo) {
+    BoundSmem m;
+    m.xs = reinterpret_cast<float *>(dyn);
+    m.far = reinterpret_cast<FarVisit *>(dyn + bo.dyn_far);
+    m.cd = reinterpret_cast<float2 *>(dyn + bo.dyn_cols) + threadIdx.x;
+    m.cut = dyn + bo.dyn_cuts + threadIdx.x;
+    m.segs = reinterpret_cast<SegLite *>(dyn + bo.dyn_segs);
+    m.word = reinterpret_cast<unsigned long long *>(dyn + bo.dyn_segs + sizeof(SegLite) * bo.max_group);
+    m.rest = reinterpret_cast<unsigned char *>(m.word + bo.max_group);
+    return m;
+}
 
 __device__ __forceinline__ bool native_i64_dev(const BatchDev &b) { return b.mode == CM_COST_INT64NS && !b.intval; }
 __device__ __forceinline__ float lb_of(uint64_t lbarg) { return __uint_as_float((uint32_t)(lbarg >> 32)); }
@@ -63,10 +83,8 @@ __device__ __forceinline__ BoundSeg bound_segment(const BatchDev &bd, const BBuc
     return v;
 }
 __device__ __forceinline__ SegLite seg_lite(const Tables &tb, const BoundSeg &g) {
-    SegLite s;
-    s.tier = g.tier; s.scen = g.scen; s.tseg = g.tseg; s.row = g.row; s.n_sync = g.n_sync;
-    s.lim = 0.0; s.lim_bits = 0; s.ev = -1.0f;
-    s.coef = g.n_sync <= 1 ? 0.0f : __double2float_rd((2.0 * (double)(g.n_sync - 1)) / ((double)g.n_sync * (double)tb.prof->bw_sync));
+    SegLite s{g.tier, g.row, 0.0f, g.n_sync, 0};
+    if (g.n_sync > 1) s.coef = __double2float_rd((2.0 * (double)(g.n_sync - 1)) / ((double)g.n_sync * (double)tb.prof->bw_sync));
     return s;
 }
 
@@ -91,127 +109,181 @@ __device__ __forceinline__ BoundJob bound_job(const BBucket &bk, uint32_t cta) {
     return j;
 }
 
+// Maximum of three and two additions (rounded down) in one instruction each.
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float2 add2_rd(float2 a, float2 b) {
+    uint64_t x, y, z;
+    float2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(z) : "l"(x), "l"(y));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(z));
+    return r;
+}
+
 // Everything a lane knows about its layer composition: b[i] + X_i is the best walk through stage i
 // whose visits stay on the cheaper link tier, X_i = 2 * (transfers of boundaries i .. S-2).
 template <int NB> struct LaneBound {
-    float b[4 * NB];
+    float2 b[2 * NB];
     float u0, once, g;
     bool ok;
+    __device__ __forceinline__ float get(int i) const { return i & 1 ? b[i >> 1].y : b[i >> 1].x; }
+    __device__ __forceinline__ void set(int i, float v) { if (i & 1) b[i >> 1].y = v; else b[i >> 1].x = v; }
 };
 
-// cc / dd (shared memory, a column per thread): stage i's walk with visits upwards / downwards, what
-// a boundary on the slower tier adds comes on top.
+// Stays at stage i in its own walk (negative: the walk does not exist), and the pairs of them that
+// visits can replace.
+__device__ __forceinline__ int stays(int i, int S, int m) { return m - 1 + i - S; }
+__device__ __forceinline__ float stay_pairs(int i, int S, int m) {
+    const int n = stays(i, S, m);
+    return n > 1 ? (float)(n >> 1) : 0.0f;
+}
+
+// cd (shared memory, a column per thread): entry i = the walks that visit across boundary i, from stage i
+// upwards and from stage i+1 downwards, without the boundary's transfers.
+//
+// This is a third of the kernel's instructions, so double arithmetic is kept to the sums that cancel or
+// grow (six operations a stage); what is left is done in floats rounded down, and the slowest single
+// forward and backward are compared by the upper halves of their bit patterns.
 template <typename T, int NB, bool UNI_X>
-__device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, const CutEdges &w, int S, int m, bool check,
-                                           float *cc, float *dd, uint8_t *cutc) {
+__device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, const CutColumn<kBoundThreads> &w, int S, int m, bool check, float2 *cd) {
     const bool gpipe = s.sched == CM_SCHED_GPIPE;
-    constexpr double none = (double)kNoWalk;
-    double U = 0.0, fmax = 0.0, bmax = 0.0;
-    double base_n = none, c_n = none, w_n = 0.0, xm_n = 0.0, q_n = 0.0;   // of stage i+1
+    double U = 0.0, w_n = 0.0;                        // w_n: of stage i+1
+    float base_n = kNoWalk, c_n = kNoWalk, xq_n = 0.0f, q_n = 0.0f;
+    const float xm_all = __double2float_rd((double)(s.XT[0][0] < s.XT[1][0] ? s.XT[0][0] : s.XT[1][0]));
+    int fmax = 0, bmax = 0;
     long long g_max = 0;
     int hi = s.L;
 #pragma unroll
     for (int i = 4 * NB - 1; i >= 0; --i) {
-        v.b[i] = kNoWalk;
+        v.set(i, kNoWalk);
         if (i < S) {
             const int lo = w.edge(i);
             if (check && (hi <= lo || !stage_fits(s.PS[hi] - s.PS[lo], s.PA[hi] - s.PA[lo], i, S, m, s.cap, s.sched))) v.ok = false;
             const double f = (double)(s.PF[hi] - s.PF[lo]), bk = (double)(s.PB[hi] - s.PB[lo]), wi = f + bk;
             const long long g = s.PP[hi] - s.PP[lo];
             g_max = g > g_max ? g : g_max;
-            fmax = tmax(fmax, f);
-            bmax = tmax(bmax, bk);
+            fmax = max(fmax, __double2hiint(f));
+            bmax = max(bmax, __double2hiint(bk));
             U += wi;
             if (!gpipe) {
-                const bool below_top = i < S - 1;
-                const double xm = below_top ? (double)(s.XT[0][hi - 1] < s.XT[1][hi - 1] ? s.XT[0][hi - 1] : s.XT[1][hi - 1]) : 0.0;
-                const int n = m - 1 + i - S;
-                const double q = n > 1 ? (double)(n >> 1) : 0.0;
-                if (below_top) {   // stage i+1 is complete now that its lower neighbour is known
-                    const double d = q_n > 0.0 ? base_n + q_n * (wi - w_n) : none;
-                    const double best = tmax(base_n, tmax(c_n + 2.0 * q_n * xm_n, d + 2.0 * q_n * xm));
-                    if (i + 1 < 4 * NB) v.b[i + 1 < 4 * NB ? i + 1 : 0] = __double2float_rd(best);
-                    dd[(i + 1) * kBoundThreads] = __double2float_rd(d);
+                const int n = stays(i, S, m);
+                const float q = stay_pairs(i, S, m);
+                float xm = xm_all, d = kNoWalk;
+                if (!UNI_X) xm = __double2float_rd((double)(s.XT[0][hi - 1] < s.XT[1][hi - 1] ? s.XT[0][hi - 1] : s.XT[1][hi - 1]));
+                const double dw = wi - w_n;
+                if (i < S - 1) {   // stage i+1 is complete now that its lower neighbour is known
+                    if (q_n > 0.0f) d = __fmaf_rd(q_n, __double2float_rd(dw), base_n);
+                    const float up = c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n);
+                    const float best = max3(base_n, up, __fmaf_rd(2.0f * q_n, xm, d));
+                    if (i + 1 < 4 * NB) v.set(i + 1 < 4 * NB ? i + 1 : 0, best);
                 }
-                base_n = n >= 0 ? U + (double)n * wi : none;
-                c_n = q > 0.0 && below_top ? base_n + q * (w_n - wi) : none;
-                cc[i * kBoundThreads] = __double2float_rd(c_n);
-                w_n = wi; xm_n = xm; q_n = q;
-                if (i == 0) v.b[0] = __double2float_rd(tmax(base_n, c_n + 2.0 * q_n * xm_n));
+                base_n = n >= 0 ? __double2float_rd(__fma_rd((double)n, wi, U)) : kNoWalk;
+                c_n = q > 0.0f && i < S - 1 ? __fmaf_rd(q, __double2float_rd(-dw), base_n) : kNoWalk;
+                cd[i * kBoundThreads] = make_float2(c_n, d);
+                w_n = wi; q_n = q; xq_n = __fmul_rd(2.0f * q, xm);
+                if (i == 0) v.set(0, fmaxf(base_n, c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n)));
             }
-            if (!UNI_X) cutc[i * kBoundThreads] = (uint8_t)hi;
             hi = lo;
         }
     }
+    const double f1 = __hiloint2double(fmax, 0), b1 = __hiloint2double(bmax, 0);
     v.u0 = __double2float_rd(U);
-    v.once = __double2float_rd((double)(m - 1) * (gpipe ? fmax + bmax : tmax(fmax, bmax)));
+    v.once = __double2float_rd((double)(m - 1) * (gpipe ? f1 + b1 : tmax(f1, b1)));
     v.g = __ll2float_rd(g_max);
 }
 
-// pairs of stays at stage i that visits can replace
-__device__ __forceinline__ float stay_pairs(int i, int S, int m) {
-    const int n = m - 1 + i - S;
-    return n > 1 ? (float)(n >> 1) : 0.0f;
-}
-
-// Bound of the lane's composition in one segment.  What a segment adds -- the transfers of its link
-// tiers -- is summed once per CTA where the transfer times do not depend on the layer (UNI_X: xr), else
-// per plan.  slack: 1 where the synchronisation quotient floors.
-template <typename T, int NB, bool UNI_X>
-__device__ __forceinline__ float lane_value(const LaneBound<NB> &v, const SProf<T> &sp, int S, int m, const SegLite &sg, const float *xr,
-                                            float x1, float slack, const float *cc, const float *dd, const uint8_t *cutc) {
-                float best = v.once, x_all;
-                const uint64_t tier = sg.tier;
-                if (UNI_X) {
-                        #pragma unroll
-                    for (int k = 0; k < NB; ++k) {
-                        const float4 x = reinterpret_cast<const float4 *>(xr)[k];
-                        best = fmaxf(best, fmaxf(fmaxf(__fadd_rd(v.b[4 * k], x.x), __fadd_rd(v.b[4 * k + 1], x.y)),
-                                                 fmaxf(__fadd_rd(v.b[4 * k + 2], x.z), __fadd_rd(v.b[4 * k + 3], x.w))));
-                    }
-                    x_all = xr[0];
-                    if (sp.sched != CM_SCHED_GPIPE)
-                        for (uint64_t t = tier; t; t &= t - 1) {   // visits across an inter-node boundary
-                            const int i = __ffsll((long long)t) - 1;
-                            best = fmaxf(best, __fadd_rd(cc[i * kBoundThreads], __fmaf_rd(2.0f * stay_pairs(i, S, m), x1, xr[i])));
-                            best = fmaxf(best, __fadd_rd(dd[(i + 1) * kBoundThreads],
-                                                         __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x1, i + 1 < S - 1 ? xr[i + 1] : 0.0f)));
-                        }
-                } else {
-                    float X = 0.0f;
-    #pragma unroll
-                    for (int i = 4 * NB - 1; i >= 0; --i) {
-                        if (i < S) {
-                            if (i < S - 1) {
-                                const bool far = (tier >> i) & 1ull;
-                                const float x = __double2float_rd((double)sp.XT[far ? 1 : 0][cutc[i * kBoundThreads] - 1]);
-                                const float X_up = X;
-                                X = __fadd_rd(X, 2.0f * x);
-                                if (far && sp.sched != CM_SCHED_GPIPE) {
-                                    best = fmaxf(best, __fadd_rd(cc[i * kBoundThreads], __fmaf_rd(2.0f * stay_pairs(i, S, m), x, X)));
-                                    best = fmaxf(best, __fadd_rd(dd[(i + 1) * kBoundThreads], __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x, X_up)));
-                                }
-                            }
-                            best = fmaxf(best, __fadd_rd(v.b[i], X));
-                        }
-                    }
-                    x_all = X;
-                }
-                const float lb = __fmaf_rd(v.g, sg.coef, __fadd_rd(__fadd_rd(v.u0, x_all), best));
-                return fmaxf(__fmul_rd(__fsub_rd(lb, slack), kFloatSlack), 0.0f);
-}
-
-// Transfers above every stage, per segment of the CTA (UNI_X).
+// Transfers above every stage and the visits across inter-node boundaries, per segment of the CTA, where
+// the transfer times do not depend on the layer (UNI_X).
 template <typename T, int NB>
-__device__ __forceinline__ void fill_transfers(float *xs, const SProf<T> &sp, int S, const SegLite *segs, int n_act) {
+__device__ __forceinline__ void fill_transfers(const BoundSmem &sm, const SProf<T> &sp, int S, int m, int n_seg) {
     const float x0 = __double2float_rd((double)sp.XT[0][0]), x1 = __double2float_rd((double)sp.XT[1][0]);
-    for (int s = threadIdx.x; s < n_act; s += kBoundThreads) {
+    for (int s = threadIdx.x; s < n_seg; s += kBoundThreads) {
+        const uint64_t tier = sm.segs[s].tier;
         float X = 0.0f;
+        int n = 0;
         for (int i = 4 * NB - 1; i >= 0; --i) {
-            if (i < S - 1) X = __fadd_rd(X, 2.0f * (((segs[s].tier >> i) & 1ull) ? x1 : x0));
-            xs[s * 4 * NB + i] = X;
+            if (i < S - 1) {
+                const bool far = (tier >> i) & 1ull;
+                const float X_up = X;
+                X = __fadd_rd(X, 2.0f * (far ? x1 : x0));
+                if (far && sp.sched != CM_SCHED_GPIPE) {
+                    if (n < kFarMax)
+                        sm.far[s * kFarMax + n] = FarVisit{__fmaf_rd(2.0f * stay_pairs(i, S, m), x1, X),
+                                                           __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x1, X_up), i, 0};
+                    n = n < kFarMax ? n + 1 : kFarLong;
+                }
+            }
+            sm.xs[s * 4 * NB + i] = X;
         }
+        sm.segs[s].n_far = n;
     }
+}
+
+// Bound of the lane's composition in one segment, without the slack (bound_of).  What a segment adds -- the
+// transfers of its link tiers -- is prepared once per CTA (UNI_X) or worked out per plan.
+template <typename T, int NB, bool UNI_X>
+__device__ __forceinline__ float lane_value(const LaneBound<NB> &v, const SProf<T> &sp, int S, int m, int s, const BoundSmem &sm) {
+    const SegLite &sg = sm.segs[s];
+    float best = v.once, x_all;
+    if (UNI_X) {
+        const float4 *xr = reinterpret_cast<const float4 *>(sm.xs + s * 4 * NB);
+        float other = kNoWalk;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            const float4 x = xr[k];
+            const float2 p = add2_rd(v.b[2 * k], make_float2(x.x, x.y)), q = add2_rd(v.b[2 * k + 1], make_float2(x.z, x.w));
+            best = max3(best, p.x, p.y);
+            other = max3(other, q.x, q.y);
+            if (k == 0) x_all = x.x;
+        }
+        if (sg.n_far <= kFarMax) {
+            for (int k = 0; k < sg.n_far; ++k) {
+                const FarVisit f = sm.far[s * kFarMax + k];
+                const float2 r = add2_rd(sm.cd[f.at * kBoundThreads], make_float2(f.up, f.down));
+                best = max3(best, r.x, r.y);
+            }
+        } else {
+            const float x1 = __double2float_rd((double)sp.XT[1][0]);
+            const float *xf = sm.xs + s * 4 * NB;
+            for (uint64_t t = sg.tier; t; t &= t - 1) {
+                const int i = __ffsll((long long)t) - 1;
+                const float2 cd = sm.cd[i * kBoundThreads];
+                best = fmaxf(best, __fadd_rd(cd.x, __fmaf_rd(2.0f * stay_pairs(i, S, m), x1, xf[i])));
+                best = fmaxf(best, __fadd_rd(cd.y, __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x1, i + 1 < S - 1 ? xf[i + 1] : 0.0f)));
+            }
+        }
+        best = fmaxf(best, other);
+    } else {
+        float X = 0.0f;
+#pragma unroll
+        for (int i = 4 * NB - 1; i >= 0; --i) {
+            if (i < S) {
+                if (i < S - 1) {
+                    const bool far = (sg.tier >> i) & 1ull;
+                    const float x = __double2float_rd((double)sp.XT[far ? 1 : 0][sm.cut[i * kBoundThreads] - 1]);
+                    const float X_up = X;
+                    X = __fadd_rd(X, 2.0f * x);
+                    if (far && sp.sched != CM_SCHED_GPIPE) {
+                        const float2 cd = sm.cd[i * kBoundThreads];
+                        best = fmaxf(best, __fadd_rd(cd.x, __fmaf_rd(2.0f * stay_pairs(i, S, m), x, X)));
+                        best = fmaxf(best, __fadd_rd(cd.y, __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x, X_up)));
+                    }
+                }
+                best = fmaxf(best, __fadd_rd(v.get(i), X));
+            }
+        }
+        x_all = X;
+    }
+    return __fmaf_rd(v.g, sg.coef, __fadd_rd(__fadd_rd(v.u0, x_all), best));
+}
+// slack: 1 where the synchronisation quotient floors
+__device__ __forceinline__ float bound_of(float value, float slack) {
+    return fmaxf(__fmul_rd(__fsub_rd(value, slack), kFloatSlack), 0.0f);
 }
 
 // Append a plan to a list (any subset of a warp's lanes).

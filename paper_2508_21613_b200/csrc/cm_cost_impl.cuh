@@ -128,7 +128,8 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_kernel(Tables tb, BatchDe
     const uint64_t base = (chunk - bk.chunk_first) * kChunk;
     uint64_t seg_local, kappa;
     plan_of_thread(base, bk.count, threadIdx.x, seg_local, kappa);
-    if (seg_local < bk.n_seg) kappa = walk_kappa(bd.feas, bk.feas_first, kappa);
+    Cand cand{};
+    if (seg_local < bk.n_seg) cand = walk_cand(bd, bk.feas_first, kappa);
     uint32_t row = 0xffffffffu;
     uint64_t bits = inf_bits<T>();
     unsigned long long my_cells = 0;
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_kernel(Tables tb, BatchDe
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
         row = g.row;
         T cost;
-        if (plan_cost_regs<T, S>(sp, tb, bd.layer_mode, g, kappa, cost)) {
+        if (plan_cost_regs<T, S>(sp, tb, bd.layer_mode, g, cand, cost)) {
             bits = Num<T>::bits(cost);
             my_cells = one_plan(2ull * S * g.m);
         }
@@ -159,7 +160,8 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_pair_kernel(Tables tb, Ba
     const uint64_t base = (chunk - bk.chunk_first) * kChunk;
     uint64_t seg_local, kappa;
     plan_of_thread(base, bk.count, threadIdx.x, seg_local, kappa);
-    if (seg_local < bk.n_seg) kappa = walk_kappa(bd.feas, bk.feas_first, kappa);
+    Cand cand{};
+    if (seg_local < bk.n_seg) cand = walk_cand(bd, bk.feas_first, kappa);
     uint32_t row = 0xffffffffu;
     uint64_t bits0 = inf_bits<T>(), bits1 = inf_bits<T>();
     unsigned long long my_cells = 0;
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_pair_kernel(Tables tb, Ba
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
         row = g.row;
         T c0, c1;
-        if (plan_cost_regs_pair<T, S>(sp, tb, bd.layer_mode, g, kappa, c0, c1)) {
+        if (plan_cost_regs_pair<T, S>(sp, tb, bd.layer_mode, g, cand, c0, c1)) {
             bits0 = Num<T>::bits(c0);
             bits1 = Num<T>::bits(c1);
             my_cells = pair_plans<S>(g.m);
@@ -191,7 +193,8 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_any_kernel(Tables tb, Bat
     const uint64_t base = (chunk - bk.chunk_first) * kChunk;
     uint64_t seg_local, kappa;
     plan_of_thread(base, bk.count, threadIdx.x, seg_local, kappa);
-    if (seg_local < bk.n_seg) kappa = walk_kappa(bd.feas, bk.feas_first, kappa);
+    Cand cand{};
+    if (seg_local < bk.n_seg) cand = walk_cand(bd, bk.feas_first, kappa);
     uint32_t row = 0xffffffffu;
     uint64_t bits = inf_bits<T>();
     unsigned long long my_cells = 0;
@@ -199,7 +202,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_any_kernel(Tables tb, Bat
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
         row = g.row;
         T cost;
-        if (plan_cost_regs_any<T>(sp, tb, bd.layer_mode, g, kappa, cost)) {
+        if (plan_cost_regs_any<T>(sp, tb, bd.layer_mode, g, cand, cost)) {
             bits = Num<T>::bits(cost);
             my_cells = one_plan(2ull * g.S * g.m);
         }
@@ -235,10 +238,10 @@ template <int S> constexpr int wide_ctas_per_sm() { return S <= CM_WIDE3 ? 3 : (
 // are shared out over the lanes for the sums and the check.  Returns, warp-uniform, whether
 // the composition is feasible; g_max = largest gradient bytes of a stage (in every lane).
 template <typename T, int S>
-__device__ __forceinline__ bool uni_composition(const SProf<T> &sp, const Tables &tb, int layer_mode, int m, uint64_t kappa,
+__device__ __forceinline__ bool uni_composition(const SProf<T> &sp, const Tables &tb, int layer_mode, int m, const Cand &cand,
                                                 uint64_t K, FB<T> *fb, uint8_t *cuts, uint32_t lane, long long &g_max) {
     CutWalker cw;
-    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, kappa, K, tb.mm_slot(S, m));
+    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, cand, K, tb.mm_slot(S, m));
     if (ok) {
         int lo = 0;
         for (int i = 0; i < S; ++i) {
@@ -308,13 +311,14 @@ __global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_cost_wide_ke
             const uint32_t n_groups = (bks.n_seg + 31) / 32;
             const uint64_t pos = item / n_groups;              // position in the bucket's walk
             if (pos >= bks.count || m < 1) break;              // warp-uniform; items ascend
-            const uint64_t kappa = walk_kappa(bd.feas, bks.feas_first, pos);
+            const Cand cand = walk_cand(bd, bks.feas_first, pos);
+            const uint64_t kappa = cand.kappa;
             const uint32_t seg_local = (uint32_t)(item - pos * n_groups) * 32 + lane;
             const bool active = seg_local < bks.n_seg;
             const SegView g = bucket_segment(bd, bks, active ? seg_local : 0);
             if (kappa != st_kappa[warp]) {
                 long long g_max;
-                const bool ok = uni_composition<T, S>(sp, tb, bd.layer_mode, m, kappa, g.K, fb, cuts, lane, g_max);
+                const bool ok = uni_composition<T, S>(sp, tb, bd.layer_mode, m, cand, g.K, fb, cuts, lane, g_max);
                 if (lane == 0) { st_kappa[warp] = kappa; st_ok[warp] = ok ? 1 : 0; st_gmax[warp] = g_max; }
                 __syncwarp();
             }
@@ -356,14 +360,15 @@ __global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_cost_wide_ke
         const uint64_t base = (chunk - bk.chunk_first) * kChunk;
         uint64_t seg_local, kappa;
         plan_of_thread(base, bk.count, tid, seg_local, kappa);
-        if (seg_local < bk.n_seg) kappa = walk_kappa(bd.feas, bk.feas_first, kappa);
+        Cand cand{};
+        if (seg_local < bk.n_seg) cand = walk_cand(bd, bk.feas_first, kappa);
         uint32_t row = 0xffffffffu;
         uint64_t bits = inf_bits<T>();
         if (seg_local < bk.n_seg && m >= 1) {
             const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
             row = g.row;
             T cost;
-            if (plan_cost_wide_lane<T, S>(sp, tb, bd.layer_mode, g, kappa, fcol, xcol, cost)) {
+            if (plan_cost_wide_lane<T, S>(sp, tb, bd.layer_mode, g, cand, fcol, xcol, cost)) {
                 bits = Num<T>::bits(cost);
                 my_cells = one_plan(2ull * S * m);
             }
@@ -410,13 +415,14 @@ __global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_cost_pair_ke
         const uint32_t n_groups = (bks.n_seg + 31) / 32;
         const uint64_t pos = item / n_groups;
         if (pos >= bks.count) break;                       // warp-uniform; items ascend
-        const uint64_t kappa = walk_kappa(bd.feas, bks.feas_first, pos);
+        const Cand cand = walk_cand(bd, bks.feas_first, pos);
+        const uint64_t kappa = cand.kappa;
         const uint32_t seg_local = (uint32_t)(item - pos * n_groups) * 32 + lane;
         const bool active = seg_local < bks.n_seg;
         const SegView g = bucket_segment(bd, bks, active ? seg_local : 0);
         if (kappa != st_kappa[warp]) {
             long long g_max;
-            const bool ok = uni_composition<T, S>(sp, tb, bd.layer_mode, m, kappa, g.K, fb, cuts, lane, g_max);
+            const bool ok = uni_composition<T, S>(sp, tb, bd.layer_mode, m, cand, g.K, fb, cuts, lane, g_max);
             if (lane == 0) { st_kappa[warp] = kappa; st_ok[warp] = ok ? 1 : 0; st_gmax[warp] = g_max; }
             __syncwarp();
         }
@@ -467,7 +473,8 @@ __global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_cost_lane_pa
     const uint64_t base = (chunk - bk.chunk_first) * kChunk;
     uint64_t seg_local, kappa;
     plan_of_thread(base, bk.count, tid, seg_local, kappa);
-    if (seg_local < bk.n_seg) kappa = walk_kappa(bd.feas, bk.feas_first, kappa);
+    Cand cand{};
+    if (seg_local < bk.n_seg) cand = walk_cand(bd, bk.feas_first, kappa);
     uint32_t row = 0xffffffffu;
     uint64_t bits0 = inf_bits<T>(), bits1 = inf_bits<T>();
     unsigned long long my_cells = 0;
@@ -475,7 +482,7 @@ __global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_cost_lane_pa
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
         row = g.row;
         T c0, c1;
-        if (plan_cost_wide_lane_pair<T, S>(sp, tb, bd.layer_mode, g, kappa, fcol, xcol, c0, c1)) {
+        if (plan_cost_wide_lane_pair<T, S>(sp, tb, bd.layer_mode, g, cand, fcol, xcol, c0, c1)) {
             bits0 = Num<T>::bits(c0);
             bits1 = Num<T>::bits(c1);
             my_cells = pair_plans<S>(bk.m);
@@ -499,7 +506,8 @@ __global__ void __launch_bounds__(kChunk) cm_cost_short_kernel(Tables tb, BatchD
     const uint64_t base = (chunk - bk.chunk_first) * kChunk;
     uint64_t seg_local, kappa;
     plan_of_thread(base, bk.count, threadIdx.x, seg_local, kappa);
-    if (seg_local < bk.n_seg) kappa = walk_kappa(bd.feas, bk.feas_first, kappa);
+    Cand cand{};
+    if (seg_local < bk.n_seg) cand = walk_cand(bd, bk.feas_first, kappa);
     uint32_t row = 0xffffffffu;
     uint64_t bits = inf_bits<T>();
     unsigned long long my_cells = 0;
@@ -507,7 +515,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_short_kernel(Tables tb, BatchD
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
         row = g.row;
         T cost;
-        if (plan_cost_regs_any<T, true>(sp, tb, bd.layer_mode, g, kappa, cost)) {
+        if (plan_cost_regs_any<T, true>(sp, tb, bd.layer_mode, g, cand, cost)) {
             bits = Num<T>::bits(cost);
             my_cells = one_plan(2ull * g.S * g.m);
         }

@@ -75,10 +75,10 @@ __global__ void __launch_bounds__(kChunk) cm_cost_warp_kernel(Tables tb, BatchDe
     const uint64_t seg_local = plan / bk.count;
     unsigned long long my_cells = 0;
     if (seg_local < bk.n_seg && m >= 1) {                       // warp-uniform
-        const uint64_t kappa = walk_kappa(bd.feas, bk.feas_first, plan - seg_local * bk.count);
+        const Cand cand = walk_cand(bd, bk.feas_first, plan - seg_local * bk.count);
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
         T cost;
-        if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, kappa, cuts_s[warp], cost) && lane == 0) {
+        if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, cand, cuts_s[warp], cost) && lane == 0) {
             const uint64_t bits = Num<T>::bits(cost);
             if (bits < bd.seg_best[g.row]) atomicMin((unsigned long long *)&bd.seg_best[g.row], (unsigned long long)bits);
             my_cells = one_plan(2ull * S * m);

@@ -285,6 +285,18 @@ __device__ __forceinline__ uint64_t walk_kappa(const uint32_t *feas, uint32_t fe
     return feas_first != kNoFeasList ? (uint64_t)feas[feas_first + idx] : idx;
 }
 
+// The same with the composition itself where it is listed: a listed candidate needs no unranking (a
+// chain of dependent look-ups in the binomial table, 3-10 us of latency in a cold kernel).
+struct Cand {
+    uint64_t kappa, a, b;   // a, b: CutWalker's mask of an enumerated composition
+    bool masked;
+};
+__device__ __forceinline__ Cand walk_cand(const BatchDev &bd, uint32_t feas_first, uint64_t idx) {
+    if (feas_first == kNoFeasList) return Cand{idx, 0, 0, false};
+    const ulonglong2 mask = bd.feas_mask[feas_first + idx];
+    return Cand{(uint64_t)bd.feas[feas_first + idx], mask.x, mask.y, true};
+}
+
 __device__ __forceinline__ uint64_t cut_bits(const uint64_t *words, int off, int n /* <= 63 */) {
     const int w = off >> 6, sh = off & 63;
     uint64_t v = words[w] >> sh;

@@ -204,7 +204,8 @@ struct BBucket {
     uint32_t pad;
 };
 // Step times that can still be a scenario's answer: lo <= T* <= ub, lo from bounds.
-struct SearchWin { float lo, pad; uint64_t ub; };
+// reach: strategies whose step time from bounds is at most this had their segments marked.
+struct SearchWin { float lo, reach; uint64_t ub; };
 struct BoundDev {
     const BBucket *bucket;
     uint64_t *lbarg;              // per row: least bound (float bits) << 32 | its position in the walk; all-ones = no plan fits
@@ -214,7 +215,7 @@ struct BoundDev {
     uint32_t *count;              // per list: plans listed minus one
     uint32_t list_first[5];       // lists: phase 1 up to kRegStagesMax stages, deeper; phase 2 the same
     uint32_t n_buckets, n_chunks, n_segs;
-    uint32_t dyn_cols, dyn_segs, max_group;
+    uint32_t dyn_far, dyn_cols, dyn_cuts, dyn_segs, max_group;   // shared memory of a CTA (BoundSmem)
     size_t dyn_bytes;
     int window, uniform_x;
 };
@@ -223,6 +224,8 @@ constexpr int kCounters = 6;   // work counters of a search in use (BatchDev::co
 constexpr uint64_t kBoundMinCells = 200000000ull;
 constexpr uint32_t kBoundListMin = 65536;        // plans a list has room for, at least (if there are as many)
 constexpr size_t kBoundDynMax = 160 * 1024;      // dynamic shared memory of the bound kernels, at most
+constexpr size_t kBoundDynTarget = 64 * 1024;    //   and wanted: three CTAs per SM
+constexpr size_t kRefineSegBytes = 32;
 
 // (cost, index) pair carried through the hierarchical argmin of the split reduction.
 struct Partial {
@@ -250,7 +253,8 @@ struct BatchDev {
     const uint32_t *tmpl_scen;    // scenario ids grouped by template
     const Bucket *bucket;         // search-pass work layout
     const uint32_t *bucket_tseg;  // template segment rows grouped by bucket
-    const uint32_t *feas;         // feasible-composition pool of the context
+    const uint32_t *feas;         // feasible-composition pool of the context: ranks,
+    const ulonglong2 *feas_mask;  //   and the compositions as masks (zero for the min-max partition)
     const uint2 *useg;            // distinct segments of a batch searched with sharing (buckets with tmpl == kSharedBucket)
     // Strategies of one survivor count repeat pipelines: the same stages over the same survivors with
     // the same micro-batches and peers (the tuples (30,31,..) and (30,32,..) start with the same
@@ -332,7 +336,8 @@ cudaError_t launch_minmax(const Tables &t, const uint32_t *keys_dev, int n_keys,
 // feasible compositions of n_keys (S << 16 | m) keys: list of key q written at pool + first[q]
 // (room for K[q] + 1 entries), its length to count[q]
 cudaError_t launch_feasible(const Tables &t, int layer_mode, const uint32_t *keys_dev, const uint64_t *K_dev,
-                            const uint32_t *first_dev, int n_keys, uint32_t *pool, uint32_t *count_dev, cudaStream_t st);
+                            const uint32_t *first_dev, int n_keys, uint32_t *pool, ulonglong2 *masks, uint32_t *count_dev,
+                            cudaStream_t st);
 cudaError_t launch_policies(const Tables &t, const BatchDev &b, int n_dp, cudaStream_t st);
 // segments shared between scenarios: key every row and list the distinct ones (tab, rep, count
 // cleared by the caller); after the search pass, give every other row its representative's result
@@ -351,12 +356,12 @@ cudaError_t launch_cost_pass1(const Tables &t, const BatchDev &b, const LaunchCl
                               cudaStream_t st, const SideStreams *side, int *launches);
 // bounded search pass (cm_bound.cu, cm_refine.cu)
 size_t bound_dyn_bytes(BoundDev &bo, int max_stages, int max_group, bool uniform_x);   // also sets the offsets
+int bound_group(int max_stages, bool uniform_x);   // segments per CTA
 cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
 cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st);
 cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st);
 cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
-// lists first_list and first_list + 1, at most `most` plans in either
-cudaError_t launch_list(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, uint64_t most, cudaStream_t st);
+cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches);   // first_list and the next
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st);
 cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);   // cm_tiebreak.cu
 cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st);

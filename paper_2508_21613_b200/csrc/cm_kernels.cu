@@ -149,7 +149,8 @@ cudaError_t launch_minmax(const Tables &t, const uint32_t *keys_dev, int n_keys,
 constexpr int kFeasThreads = 1024;
 __global__ void __launch_bounds__(kFeasThreads) cm_feasible_kernel(Tables tb, int layer_mode, const uint32_t *keys,
                                                                    const uint64_t *Ks, const uint32_t *first,
-                                                                   uint32_t *pool, uint32_t *count_out, int binom_rows_staged) {
+                                                                   uint32_t *pool, ulonglong2 *masks, uint32_t *count_out,
+                                                                   int binom_rows_staged) {
     __shared__ long long PA[kMaxL + 1], PS[kMaxL + 1];
     __shared__ uint32_t warp_cnt[kFeasThreads / 32];
     __shared__ uint32_t running;
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kFeasThreads) cm_feasible_kernel(Tables tb, in
     const int S = (int)(key >> 16), m = (int)(key & 0xffffu);
     const uint64_t K = Ks[blockIdx.x];
     uint32_t *out = pool + first[blockIdx.x];
+    ulonglong2 *out_mask = masks + first[blockIdx.x];
     const long long cap = p->cap;
     for (int l = threadIdx.x; l <= L; l += blockDim.x) { PA[l] = p->PA[l]; PS[l] = p->PS[l]; }
     if (threadIdx.x == 0) running = 0;
@@ -173,9 +175,11 @@ __global__ void __launch_bounds__(kFeasThreads) cm_feasible_kernel(Tables tb, in
     for (uint64_t base = 0; base < K; base += kFeasThreads) {
         const uint64_t kappa = base + threadIdx.x;
         bool ok = kappa < K;
+        ulonglong2 mask = make_ulonglong2(0, 0);
         if (ok) {
             CutWalker cw;
-            make_walker(cw, tb, layer_mode, L, S, kappa, K, 0);
+            make_walker(cw, tb, layer_mode, L, S, Cand{kappa, 0, 0, false}, K, 0);
+            mask = make_ulonglong2(cw.a, cw.b);
             int lo = 0;
             for (int i = 0; i < S && ok; ++i) {
                 const int hi = cw.next();
@@ -192,20 +196,25 @@ __global__ void __launch_bounds__(kFeasThreads) cm_feasible_kernel(Tables tb, in
             if (w < warp) before += c;
             total += c;
         }
-        if (ok) out[before + __popc(vote & ((1u << lane) - 1u))] = (uint32_t)kappa;
+        if (ok) {
+            const uint32_t at = before + __popc(vote & ((1u << lane) - 1u));
+            out[at] = (uint32_t)kappa;
+            out_mask[at] = mask;
+        }
         __syncthreads();
         if (threadIdx.x == 0) running += total;
         __syncthreads();
     }
     if (threadIdx.x == 0) {
         uint32_t n = running;
-        if (tb.mm_cuts[(size_t)tb.mm_slot(S, m) * (kMaxS + 1)] == 0) out[n++] = (uint32_t)K;
+        if (tb.mm_cuts[(size_t)tb.mm_slot(S, m) * (kMaxS + 1)] == 0) { out_mask[n] = make_ulonglong2(0, 0); out[n++] = (uint32_t)K; }
         count_out[blockIdx.x] = n;
     }
 }
 
 cudaError_t launch_feasible(const Tables &t, int layer_mode, const uint32_t *keys_dev, const uint64_t *K_dev,
-                            const uint32_t *first_dev, int n_keys, uint32_t *pool, uint32_t *count_dev, cudaStream_t st) {
+                            const uint32_t *first_dev, int n_keys, uint32_t *pool, ulonglong2 *masks, uint32_t *count_dev,
+                            cudaStream_t st) {
     if (n_keys <= 0) return cudaSuccess;
     // rows 0 .. 64 (remainder rule: n <= CM_MAX_STAGES) or 0 .. 127 (full enumeration: n < CM_MAX_LAYERS)
     const int rows = std::min(t.binom_rows, layer_mode == CM_LAYERS_REMAINDER ? kMaxS + 1 : kMaxL);
@@ -219,7 +228,7 @@ cudaError_t launch_feasible(const Tables &t, int layer_mode, const uint32_t *key
         if (e != cudaSuccess) return e;
         if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
     }
-    cm_feasible_kernel<<<n_keys, kFeasThreads, smem, st>>>(t, layer_mode, keys_dev, K_dev, first_dev, pool, count_dev, rows);
+    cm_feasible_kernel<<<n_keys, kFeasThreads, smem, st>>>(t, layer_mode, keys_dev, K_dev, first_dev, pool, masks, count_dev, rows);
     return cudaGetLastError();
 }
 

@@ -35,19 +35,21 @@ struct CutWalker {
 };
 
 __device__ __forceinline__ bool make_walker(CutWalker &w, const Tables &tb, int layer_mode, int L, int S,
-                                            uint64_t kappa, uint64_t K, uint32_t mm_slot) {
+                                            const Cand &cand, uint64_t K, uint32_t mm_slot) {
     w.a = 0; w.b = 0; w.row = nullptr; w.q = 0; w.L = L; w.S = S; w.i = 0; w.pos = 0;
-    if (kappa < K) {
-        if (layer_mode == CM_LAYERS_REMAINDER) {
-            w.kind = 0;
-            w.q = L / S;
+    if (cand.kappa < K) {
+        w.kind = layer_mode == CM_LAYERS_REMAINDER ? 0 : 1;
+        if (w.kind == 0) w.q = L / S;
+        if (cand.masked) {
+            w.a = cand.a;
+            w.b = cand.b;
+        } else if (w.kind == 0) {
             uint64_t mask = 0;
-            unrank_subset(tb.binom, kappa, S, L % S, [&](int, int v) { mask |= 1ull << v; });
+            unrank_subset(tb.binom, cand.kappa, S, L % S, [&](int, int v) { mask |= 1ull << v; });
             w.a = mask;
         } else {
-            w.kind = 1;
             uint64_t m0 = 0, m1 = 0;
-            unrank_subset(tb.binom, kappa, L - 1, S - 1, [&](int, int v) {
+            unrank_subset(tb.binom, cand.kappa, L - 1, S - 1, [&](int, int v) {
                 if (v < 64) m0 |= 1ull << v; else m1 |= 1ull << (v - 64);
             });
             w.a = m0; w.b = m1;
@@ -492,10 +494,10 @@ __device__ __forceinline__ void sim_regs_pair(int m, const FB<T> (&st)[S], const
 // of the unrolled triangles -- for the few segments with fewer micro-batches than warm-up slots.
 template <typename T, int S, bool ANY_M = false>
 __device__ __forceinline__ bool plan_cost_regs(const SProf<T> &sp, const Tables &tb, int layer_mode,
-                                               const SegView &g, uint64_t kappa, T &cost) {
+                                               const SegView &g, const Cand &cand, T &cost) {
     const int m = g.m;
     CutWalker cw;
-    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, kappa, g.K, tb.mm_slot(S, m));
+    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, cand, g.K, tb.mm_slot(S, m));
     FB<T> st[S];
     T xts[S];
     long long g_max = 0;
@@ -531,10 +533,10 @@ __device__ __forceinline__ bool plan_cost_regs(const SProf<T> &sp, const Tables 
 // micro-batches and with m + 1, one composition, one recurrence.
 template <typename T, int S>
 __device__ __forceinline__ bool plan_cost_regs_pair(const SProf<T> &sp, const Tables &tb, int layer_mode,
-                                                    const SegView &g, uint64_t kappa, T &cost_m, T &cost_m1) {
+                                                    const SegView &g, const Cand &cand, T &cost_m, T &cost_m1) {
     const int m = g.m;
     CutWalker cw;
-    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, kappa, g.K, tb.mm_slot(S, m));
+    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, cand, g.K, tb.mm_slot(S, m));
     FB<T> st[S];
     T xts[S];
     long long g_max = 0;
@@ -563,11 +565,11 @@ __device__ __forceinline__ bool plan_cost_regs_pair(const SProf<T> &sp, const Ta
 // ----------------------------------------------------------------------------------
 template <typename T, int S>
 __device__ __forceinline__ bool plan_cost_wide_lane(const SProf<T> &sp, const Tables &tb, int layer_mode,
-                                                    const SegView &g, uint64_t kappa, FB<T> *fcol, T *xcol, T &cost) {
+                                                    const SegView &g, const Cand &cand, FB<T> *fcol, T *xcol, T &cost) {
     const int m = g.m;
     if (m < 1) return false;
     CutWalker cw;
-    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, kappa, g.K, tb.mm_slot(S, m));
+    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, cand, g.K, tb.mm_slot(S, m));
     long long g_max = 0;
     int lo = 0;
     for (int i = 0; i < S && ok; ++i) {
@@ -593,10 +595,10 @@ __device__ __forceinline__ bool plan_cost_wide_lane(const SProf<T> &sp, const Ta
 // and with m + 1, one composition, one recurrence.
 template <typename T, int S>
 __device__ __forceinline__ bool plan_cost_wide_lane_pair(const SProf<T> &sp, const Tables &tb, int layer_mode, const SegView &g,
-                                                         uint64_t kappa, FB<T> *fcol, T *xcol, T &cost_m, T &cost_m1) {
+                                                         const Cand &cand, FB<T> *fcol, T *xcol, T &cost_m, T &cost_m1) {
     const int m = g.m;
     CutWalker cw;
-    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, kappa, g.K, tb.mm_slot(S, m));
+    bool ok = make_walker(cw, tb, layer_mode, sp.L, S, cand, g.K, tb.mm_slot(S, m));
     long long g_max = 0;
     int lo = 0;
     for (int i = 0; i < S && ok; ++i) {
@@ -623,9 +625,9 @@ __device__ __forceinline__ bool plan_cost_wide_lane_pair(const SProf<T> &sp, con
 // m >= S-1 unless ANY_M.
 template <typename T, bool ANY_M = false>
 __device__ __forceinline__ bool plan_cost_regs_any(const SProf<T> &sp, const Tables &tb, int layer_mode,
-                                                   const SegView &g, uint64_t kappa, T &cost) {
+                                                   const SegView &g, const Cand &cand, T &cost) {
     switch (g.S) {
-#define CM_CASE(S) case S: return plan_cost_regs<T, S, ANY_M>(sp, tb, layer_mode, g, kappa, cost);
+#define CM_CASE(S) case S: return plan_cost_regs<T, S, ANY_M>(sp, tb, layer_mode, g, cand, cost);
         CM_CASE(1) CM_CASE(2) CM_CASE(3) CM_CASE(4) CM_CASE(5) CM_CASE(6) CM_CASE(7) CM_CASE(8)
         CM_CASE(9) CM_CASE(10) CM_CASE(11) CM_CASE(12) CM_CASE(13) CM_CASE(14) CM_CASE(15) CM_CASE(16)
 #undef CM_CASE
@@ -633,14 +635,14 @@ __device__ __forceinline__ bool plan_cost_regs_any(const SProf<T> &sp, const Tab
     }
 }
 
-// Cost of candidate kappa of a segment, a warp walking the pipeline in lock step (two stages per
+// Cost of one candidate of a segment, a warp walking the pipeline in lock step (two stages per
 // lane); `cuts`: kMaxS + 8 bytes of shared memory of the warp.  Warp-uniform arguments and result.
 template <typename T>
 __device__ __forceinline__ bool warp_plan_cost(const SProf<T> &sp, const Tables &tb, int layer_mode, const SegView &g,
-                                               uint64_t kappa, uint8_t *cuts, T &cost) {
+                                               const Cand &cand, uint8_t *cuts, T &cost) {
     const int lane = threadIdx.x & 31, S = g.S, m = g.m;
     CutWalker cw;
-    bool ok = m >= 1 && make_walker(cw, tb, layer_mode, sp.L, S, kappa, g.K, tb.mm_slot(S, m));
+    bool ok = m >= 1 && make_walker(cw, tb, layer_mode, sp.L, S, cand, g.K, tb.mm_slot(S, m));
     __syncwarp();   // nobody reads the cuts of an earlier plan any more
     if (ok) {
         int lo = 0;

@@ -8,21 +8,31 @@
 
 namespace cm {
 
+// What a segment is looked at for.
+struct RefineSeg {
+    uint64_t lim_bits;   // phase 2: list a plan whose walk costs at most this
+    double lim;          // plans whose bound is at most lim ...
+    float ev;            //   ... and above ev (what phase 1 has settled already)
+    uint32_t scen, tseg, pad;
+};
+static_assert(sizeof(RefineSeg) <= kRefineSegBytes, "room per segment in bound_dyn_bytes");
+
 // What a segment still needs.  False: nothing.
 template <typename T>
-__device__ __forceinline__ bool seg_open(const BatchDev &bd, const BoundDev &bo, const BBucket &bk, int phase, SegLite &s) {
+__device__ __forceinline__ bool seg_open(const BatchDev &bd, const BoundDev &bo, const BBucket &bk, int phase, uint32_t row, RefineSeg &s) {
     constexpr bool native = std::is_same<T, long long>::value;
-    const uint64_t la = bo.lbarg[s.row], key = bo.pick[s.row];
+    const uint64_t la = bo.lbarg[row], key = bo.pick[row];
     if (la == ~0ull) return false;                                   // nothing fits in memory
     if (bo.window && key == ~0ull) return false;                     // part of no strategy within reach
     const float lb = lb_of(la), near = __fmul_ru(lb, 1.0f + kTieWindow);
     const SearchWin w = bo.window ? bo.win[s.scen] : SearchWin{-1.0f, 0.0f, inf_bits<T>()};
-    const bool least = lb <= __fmul_rd(w.lo, 1.0f - kTieWindow);     // well below the best step time: any plan will do
+    s.ev = -1.0f;
+    s.lim_bits = 0;
     if (phase == 1) {
         s.lim = (double)near;
-        return !least;
+        return !(lb <= __fmul_rd(w.lo, 1.0f - kTieWindow));          // well below the best step time: any plan will do
     }
-    const uint64_t best = bd.seg_best[s.row];
+    const uint64_t best = bd.seg_best[row];
     if (best == 0) return false;
     const double sb = cost_up(best, native), ub = cost_up(w.ub, native);
     if (sb <= (double)w.lo) return false;
@@ -33,31 +43,24 @@ __device__ __forceinline__ bool seg_open(const BatchDev &bd, const BoundDev &bo,
     return (double)lb <= s.lim && s.lim > (double)s.ev;
 }
 
-struct RefineShared {
-    uint64_t a[kBoundThreads], b[kBoundThreads];       // layer composition of every thread (CutEdges)
-    uint8_t minmax[kBoundThreads];
-    uint32_t buf[kBoundThreads / 32][64];              // per warp: (segment << 8 | thread) of collected plans
-};
-
-// Lanes 0 .. n-1 take one collected plan each.
+// Lanes 0 .. n-1 take one collected plan each: entry = segment << 8 | thread whose composition it is.
 template <typename T>
-__device__ __noinline__ void refine_flush(const SProf<T> &sp, const Tables &tb, const BatchDev &bd, const BoundDev &bo, const BBucket &bk,
-                                          int phase, uint64_t tile0, const SegLite *segs, unsigned long long *seg_key,
-                                          const RefineShared &rs, const uint32_t *ent, int n) {
+__device__ __noinline__ void refine_flush(const SProf<T> &sp, const BatchDev &bd, const BoundDev &bo, const BBucket &bk,
+                                          int phase, uint64_t tile0, const BoundSmem &sm, const uint32_t *ent, int n) {
     const int lane = threadIdx.x & 31;
     if (lane < n) {
         const uint32_t e = ent[lane], t = e & 0xffu;
-        const SegLite &sg = segs[e >> 8];
+        const SegLite &sg = sm.segs[e >> 8];
+        const RefineSeg &rg = reinterpret_cast<const RefineSeg *>(sm.rest)[e >> 8];
         const uint64_t pos = tile0 + (t & (bk.width - 1));
-        CutEdges c{rs.a[t], rs.b[t], nullptr, bd.layer_mode == CM_LAYERS_REMAINDER ? 0 : 1, sp.L / bk.S, sp.L, bk.S};
-        if (rs.minmax[t]) { c.kind = 2; c.row = tb.mm_cuts + (size_t)tb.mm_slot(bk.S, bk.m) * (kMaxS + 1); }
+        const CutColumn<kBoundThreads> c{sm.cut - threadIdx.x + t};
         const Walk w = best_walk<T>(sp, c, bk.S, bk.m, sg.tier, sg.n_sync, false);
         const uint64_t bits = Num<T>::bits(walk_cost<T>(sp, c, bk.S, bk.m, sg.tier, sg.n_sync, w));
         if (phase == 1) {
             const float lb = lb_of(bo.lbarg[sg.row]);
-            atomicMin(&seg_key[e >> 8], (unsigned long long)pick_key(bits, pick_base(lb, std::is_same<T, long long>::value), pos, pick_bits(bk.count)));
-        } else if (bits <= sg.lim_bits) {
-            list_append(bd, bo, bk.S <= kRegStagesMax ? 2 : 3, sg.scen, sg.tseg, (uint32_t)pos);
+            atomicMin(&sm.word[e >> 8], (unsigned long long)pick_key(bits, pick_base(lb, std::is_same<T, long long>::value), pos, pick_bits(bk.count)));
+        } else if (bits <= rg.lim_bits) {
+            list_append(bd, bo, bk.S <= kRegStagesMax ? 2 : 3, rg.scen, rg.tseg, (uint32_t)pos);
         }
     }
     __syncwarp();
@@ -65,38 +68,31 @@ __device__ __noinline__ void refine_flush(const SProf<T> &sp, const Tables &tb, 
 
 template <typename T, int NB, bool UNI_X>
 __device__ void refine_body(const SProf<T> &sp, const Tables &tb, const BatchDev &bd, const BoundDev &bo, const BBucket &bk, int phase,
-                            uint64_t tile0, const SegLite *segs, int n_act, unsigned long long *seg_key, unsigned char *dyn, RefineShared &rs) {
+                            uint64_t tile0, int n_act, const BoundSmem &sm, uint32_t *buf /* [64] of this warp */) {
     const int S = bk.S, m = bk.m, W = bk.width;
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     const int sub = tid / W, n_sub = kBoundThreads / W;
-    float *xs = reinterpret_cast<float *>(dyn);                                            // as in cm_bound.cu
-    float *cc = reinterpret_cast<float *>(dyn + bo.dyn_cols) + tid;
-    float *dd = cc + S * kBoundThreads;
-    uint8_t *cutc = dyn + bo.dyn_cols + sizeof(float) * 2 * S * kBoundThreads + tid;
-    const float x1 = __double2float_rd((double)sp.XT[1][0]);
-    if (UNI_X) fill_transfers<T, NB>(xs, sp, S, segs, n_act);
+    if (UNI_X) fill_transfers<T, NB>(sm, sp, S, m, n_act);
     const uint64_t pos = tile0 + (tid & (W - 1));
     LaneBound<NB> v;
     v.ok = pos < bk.count;
     if (v.ok) {
         CutWalker w;
-        const uint64_t kappa = walk_kappa(bd.feas, bk.feas_first, pos);
-        v.ok = make_walker(w, tb, bd.layer_mode, sp.L, S, kappa, bk.K, tb.mm_slot(S, m));
-        rs.a[tid] = w.a; rs.b[tid] = w.b; rs.minmax[tid] = kappa >= bk.K ? 1 : 0;
-        if (v.ok) lane_setup<T, NB, UNI_X>(v, sp, cut_edges(w), S, m, bk.feas_first == kNoFeasList, cc, dd, cutc);
+        const CutColumn<kBoundThreads> cuts{sm.cut};
+        v.ok = make_walker(w, tb, bd.layer_mode, sp.L, S, walk_cand(bd, bk.feas_first, pos), bk.K, tb.mm_slot(S, m)) && cuts.fill(w, S);
+        if (v.ok) lane_setup<T, NB, UNI_X>(v, sp, cuts, S, m, bk.feas_first == kNoFeasList, sm.cd);
     }
     __syncthreads();
     const float slack = sp.intval || std::is_same<T, long long>::value ? 1.0f : 0.0f;
     const int n_it = (n_act + n_sub - 1) / n_sub;
-    uint32_t *buf = rs.buf[tid >> 5];
+    const RefineSeg *rsegs = reinterpret_cast<const RefineSeg *>(sm.rest);
     int n_buf = 0;
     for (int it = 0; it < n_it; ++it) {
         const int s = it * n_sub + sub;
         bool take = false;
         if (s < n_act && v.ok) {
-            const SegLite &sg = segs[s];
-            const float lb = lane_value<T, NB, UNI_X>(v, sp, S, m, sg, xs + s * 4 * NB, x1, slack, cc, dd, cutc);
-            take = (double)lb <= sg.lim && lb > sg.ev;
+            const float lb = bound_of(lane_value<T, NB, UNI_X>(v, sp, S, m, s, sm), slack);
+            take = (double)lb <= rsegs[s].lim && lb > rsegs[s].ev;
         }
         const uint32_t who = __ballot_sync(0xffffffffu, take);
         if (!who) continue;
@@ -105,17 +101,17 @@ __device__ void refine_body(const SProf<T> &sp, const Tables &tb, const BatchDev
         __syncwarp();
         if (n_buf >= 32) {
             n_buf -= 32;
-            refine_flush<T>(sp, tb, bd, bo, bk, phase, tile0, segs, seg_key, rs, buf + n_buf, 32);
+            refine_flush<T>(sp, bd, bo, bk, phase, tile0, sm, buf + n_buf, 32);
         }
     }
-    if (n_buf) refine_flush<T>(sp, tb, bd, bo, bk, phase, tile0, segs, seg_key, rs, buf, n_buf);
+    if (n_buf) refine_flush<T>(sp, bd, bo, bk, phase, tile0, sm, buf, n_buf);
 }
 
 template <typename T, bool UNI_X>
 __global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, BatchDev bd, BoundDev bo, int phase) {
     __shared__ SProf<T> sp;
     __shared__ BBucket bks;
-    __shared__ RefineShared rs;
+    __shared__ uint32_t buf[kBoundThreads / 32][64];
     __shared__ int n_act_s;
     extern __shared__ __align__(16) unsigned char dyn[];
     const uint32_t tid = threadIdx.x;
@@ -126,26 +122,31 @@ __global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, Bat
     __syncthreads();
     const BBucket &bk = bks;
     const BoundJob job = bound_job(bk, blockIdx.x);
-    SegLite *segs = reinterpret_cast<SegLite *>(dyn + bo.dyn_segs);
-    unsigned long long *seg_key = reinterpret_cast<unsigned long long *>(dyn + bo.dyn_segs + sizeof(SegLite) * bo.max_group);
+    const BoundSmem sm = bound_smem(dyn, bo);
     for (uint32_t q = job.s0 + tid; q < job.s1; q += kBoundThreads) {
-        SegLite s = seg_lite(tb, bound_segment(bd, bk, q));
-        if (seg_open<T>(bd, bo, bk, phase, s)) segs[atomicAdd(&n_act_s, 1)] = s;
+        const BoundSeg g = bound_segment(bd, bk, q);
+        RefineSeg s;
+        s.scen = g.scen; s.tseg = g.tseg; s.pad = 0;
+        if (seg_open<T>(bd, bo, bk, phase, g.row, s)) {
+            const int at = atomicAdd(&n_act_s, 1);
+            sm.segs[at] = seg_lite(tb, g);
+            reinterpret_cast<RefineSeg *>(sm.rest)[at] = s;
+        }
     }
     __syncthreads();
     const int n_act = n_act_s;
     if (n_act == 0) return;   // uniform
     stage_profile(sp, tb);
-    for (int q = tid; q < n_act; q += kBoundThreads) seg_key[q] = ~0ull;
+    for (int q = tid; q < n_act; q += kBoundThreads) sm.word[q] = ~0ull;
     __syncthreads();
     const int nb = (bk.S + 3) >> 2;
-#define CM_NB(K) if (nb <= K) refine_body<T, K, UNI_X>(sp, tb, bd, bo, bk, phase, job.tile0, segs, n_act, seg_key, dyn, rs); else
+#define CM_NB(K) if (nb <= K) refine_body<T, K, UNI_X>(sp, tb, bd, bo, bk, phase, job.tile0, n_act, sm, buf[tid >> 5]); else
     CM_NB(4) CM_NB(9) CM_NB(16) {}
 #undef CM_NB
     if (phase != 1) return;
     __syncthreads();
     for (int q = tid; q < n_act; q += kBoundThreads)
-        if (seg_key[q] < bo.pick[segs[q].row]) atomicMin((unsigned long long *)&bo.pick[segs[q].row], seg_key[q]);
+        if (sm.word[q] < bo.pick[sm.segs[q].row]) atomicMin((unsigned long long *)&bo.pick[sm.segs[q].row], sm.word[q]);
 }
 
 template <typename T, bool UNI_X>

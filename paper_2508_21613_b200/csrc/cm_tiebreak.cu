@@ -21,6 +21,7 @@ template <typename T, int kTieThreads>
 __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, BatchDev bd, int n_eval) {
     __shared__ SProf<T> sp;
     __shared__ uint8_t cuts_s[kTieThreads / 32][kMaxS + 8];
+    __shared__ uint8_t cut_col[kMaxS * kTieThreads];
     __shared__ uint32_t left[kTieThreads / 32];
     __shared__ unsigned long long found;
     const uint32_t b = blockIdx.x / bd.dp_max, p = blockIdx.x % bd.dp_max;
@@ -44,9 +45,9 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
         bool maybe = false;
         if (pos < count) {
             CutWalker cw;
-            const uint64_t kappa = walk_kappa(bd.feas, g.feas_first, pos);
-            if (make_walker(cw, tb, bd.layer_mode, sp.L, g.S, kappa, g.K, tb.mm_slot(g.S, g.m))) {
-                const CutEdges c = cut_edges(cw);
+            if (make_walker(cw, tb, bd.layer_mode, sp.L, g.S, walk_cand(bd, g.feas_first, pos), g.K, tb.mm_slot(g.S, g.m))) {
+                const CutColumn<kTieThreads> c{cut_col + threadIdx.x};
+                c.fill(cw, g.S);
                 const Walk walk = best_walk<T>(sp, c, g.S, g.m, g.tier, g.n_sync, g.feas_first == kNoFeasList);
                 maybe = walk.value >= 0.0 && walk.value <= goal;
                 if (maybe) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= w.cost_bits;
@@ -69,11 +70,11 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
             __syncthreads();                                        // everybody has read `left`; `found` is reset
             if (total == 0) break;                                  // uniform
             if (warp < n_eval && at >= 0) {
-                const uint64_t kappa = walk_kappa(bd.feas, g.feas_first, base + at);
+                const Cand cand = walk_cand(bd, g.feas_first, base + at);
                 T cost;
-                if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, kappa, cuts_s[warp], cost) && lane == 0 &&
+                if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, cand, cuts_s[warp], cost) && lane == 0 &&
                     Num<T>::bits(cost) <= w.cost_bits)
-                    atomicMin(&found, (unsigned long long)kappa);
+                    atomicMin(&found, (unsigned long long)cand.kappa);
                 if (lane == 0) ++evaluated;
             }
             if (threadIdx.x == 0)                                   // strike the candidates being tried
