@@ -191,6 +191,7 @@ struct cm_ctx {
     size_t feas_used = 0;
     PinnedVec<unsigned char> feas_stage;      // keys, K, offsets out; counts back
     DevBuf<unsigned char> d_feas_stage;
+    DevBuf<uint4> d_eval;             // cm_evaluate: candidates listed by depth
     DevBuf<uint4> d_bound_list;       // plans the bounded search pass lists for the recurrence
     bool uniform_p2p = false;         // every stage boundary moves the same bytes
     bool screen = true;               // walk only the listed feasible compositions (cm_set_memory_screen)
@@ -1780,6 +1781,13 @@ cm_status cm_host_describe(const cm_profile *p, const uint32_t *failed_ids, int3
     CM_API_END(nullptr)
 }
 
+// Depths of the space's pipelines, bit S-1.
+static uint64_t stage_mask(const Batch &bt) {
+    uint64_t mask = 0;
+    for (const TSeg &g : bt.tseg) mask |= 1ull << ((g.S - 1) & 63);
+    return mask;
+}
+
 cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids, int32_t n_failed,
                        const cm_enum_opts *opts, cm_space **out, uint64_t *n_candidates) {
     if (!ctx) return CM_EINVAL;
@@ -1814,6 +1822,13 @@ cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids
         forget_keys(ctx, sp->batch);
         return s;
     }
+    // cm_evaluate only enqueues: the workspace it bins candidates in (once per context) is found here
+    uint32_t slab = 0;
+    const uint64_t want = policy == CM_DYNPAR ? eval_workspace(stage_mask(sp->batch), &slab) : 0;
+    if (want > ctx->d_eval.cap) {
+        CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // growing frees the old block
+        if (!ctx->d_eval.reserve(want)) return fail(ctx, CM_ENOMEM, "device memory");
+    }
     if (n_candidates) *n_candidates = policy == CM_DYNPAR ? sp->batch.n_cand : 1;
     *out = sp.release();
     return CM_OK;
@@ -1840,9 +1855,16 @@ cm_status cm_evaluate(cm_ctx *ctx, const cm_space *space, uint64_t first, uint64
     if (stale(ctx, bt)) return fail(ctx, CM_EINVAL, kStaleMsg);
     const uint64_t n_cand = space->policy == CM_DYNPAR ? bt.n_cand : 1;
     if (!idx_dev && (first > n_cand || count > n_cand - first)) return fail(ctx, CM_EINVAL, "candidate range out of bounds");
-    CM_CUDA(ctx, launch_evaluate(tables(ctx, bt), dev_view(ctx, bt), n_cand,
-                                 space->policy == CM_DYNPAR ? -1 : space->policy, first, count, idx_dev,
-                                 cost_dev, cost_ns_dev, feasible_dev, ctx->stream));
+    EvalDev ev{};
+    ev.idx = idx_dev;
+    ev.first = first;
+    ev.count = count;
+    ev.n_cand = n_cand;
+    ev.cost = cost_dev;
+    ev.cost_ns = cost_ns_dev;
+    ev.feas = feasible_dev;
+    CM_CUDA(ctx, launch_evaluate(tables(ctx, bt), dev_view(ctx, bt), ev, space->policy == CM_DYNPAR ? -1 : space->policy,
+                                 stage_mask(bt), ctx->d_eval.p, ctx->stream, &ctx->side));
     return CM_OK;
     CM_API_END(ctx)
 }

@@ -9,6 +9,7 @@ template <typename T> cudaError_t launch_shallow_any(const Tables &, const Batch
 template <typename T> cudaError_t launch_shallow_pair_class(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 template <typename T> cudaError_t launch_short_class(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 template <typename T, int LO, int HI> cudaError_t launch_deep_range(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
+template <typename T, int LO, int HI> cudaError_t launch_evaluate_range(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t);
 template <typename T> cudaError_t launch_solo_class(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 template <typename T> cudaError_t launch_warp_class(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 
@@ -26,13 +27,25 @@ CM_EXTERN(long long)
 // the deep-pipeline kernels: one translation unit per cost type and range of stage counts
 #define CM_DEEP_RANGE(LO, HI)                                                                                                     \
     extern template cudaError_t launch_deep_range<double, LO, HI>(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t); \
-    extern template cudaError_t launch_deep_range<long long, LO, HI>(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
+    extern template cudaError_t launch_deep_range<long long, LO, HI>(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t); \
+    extern template cudaError_t launch_evaluate_range<double, LO, HI>(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t); \
+    extern template cudaError_t launch_evaluate_range<long long, LO, HI>(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t);
 CM_DEEP_RANGES(CM_DEEP_RANGE)
 #undef CM_DEEP_RANGE
 
 template <typename T>
 static cudaError_t launch_deep_class(const Tables &t, const BatchDev &b, const LaunchClass &c, cudaStream_t st) {
 #define CM_DEEP_RANGE(LO, HI) if (c.stages >= LO && c.stages <= HI) return launch_deep_range<T, LO, HI>(t, b, c, st);
+    CM_DEEP_RANGES(CM_DEEP_RANGE)
+#undef CM_DEEP_RANGE
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_evaluate_deep(const Tables &t, const BatchDev &b, const EvalDev &ev, int stages, cudaStream_t st) {
+#define CM_DEEP_RANGE(LO, HI)                                                                                      \
+    if (stages >= LO && stages <= HI)                                                                              \
+        return native_i64(b) ? launch_evaluate_range<long long, LO, HI>(t, b, ev, stages, st)                      \
+                             : launch_evaluate_range<double, LO, HI>(t, b, ev, stages, st);
     CM_DEEP_RANGES(CM_DEEP_RANGE)
 #undef CM_DEEP_RANGE
     return cudaErrorInvalidValue;

@@ -26,7 +26,7 @@
 
 #include <atomic>
 
-#include "cm_plan_eval.cuh"
+#include "cm_eval_out.cuh"
 
 namespace cm {
 
@@ -639,6 +639,58 @@ template <typename T>
 cudaError_t launch_short_class(const Tables &t, const BatchDev &b, const LaunchClass &c, cudaStream_t st) {
     cm_cost_short_kernel<T><<<chunk_grid(c.n_chunks), kChunk, 0, st>>>(t, b, c.bucket_begin, c.bucket_end, c.chunk_begin);
     return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------------
+// cm_evaluate, one region of its binned candidates (cm_evaluate.cu), 17 <= S <= 48: one candidate per
+// lane, stage times in a per-lane shared-memory column, as the per-lane cm_cost_wide_kernel.
+// ----------------------------------------------------------------------------------
+template <typename T, int S>
+__global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_evaluate_deep_kernel(Tables tb, BatchDev bd, EvalDev ev) {
+    __shared__ SProf<T> sp;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    const uint32_t n = ev.n_list[S];
+    if ((uint64_t)blockIdx.x * kChunk >= n) return;
+    stage_profile(sp, tb);
+    __syncthreads();
+    FB<T> *fcol = reinterpret_cast<FB<T> *>(dyn) + threadIdx.x;
+    T *xcol = reinterpret_cast<T *>(dyn + sizeof(FB<T>) * S * kChunk) + threadIdx.x;
+    for (uint32_t i = blockIdx.x * kChunk + threadIdx.x; i < n; i += gridDim.x * kChunk) {
+        const EvalEntry x = eval_entry(bd, ev, S, i);
+        T cost;
+        const bool ok = plan_cost_wide_lane<T, S>(sp, tb, bd.layer_mode, x.g, x.cand, fcol, xcol, cost);
+        eval_out<T>(bd, ev, x.t, ok, ok ? cost : Num<T>::inf());
+    }
+}
+
+template <typename T, int S>
+static cudaError_t launch_evaluate_one(const Tables &t, const BatchDev &b, const EvalDev &ev, cudaStream_t st) {
+    constexpr size_t smem = wide_smem_bytes<S, false, T>();
+    static std::atomic<uint64_t> configured{0};   // as in launch_wide_one
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 64 || !((configured.load(std::memory_order_acquire) >> dev) & 1ull)) {
+        cudaError_t e = cudaFuncSetAttribute(cm_evaluate_deep_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
+    }
+    const uint64_t round = ev.count - ev.base < ev.slab ? ev.count - ev.base : ev.slab;
+    const uint64_t chunks = (round + kChunk - 1) / kChunk, most = 148 * wide_ctas_per_sm<S>();
+    cm_evaluate_deep_kernel<T, S><<<(unsigned)(chunks < most ? chunks : most), kChunk, smem, st>>>(t, b, ev);
+    return cudaGetLastError();
+}
+
+template <typename T, int S, int HI>
+static cudaError_t evaluate_dispatch(const Tables &t, const BatchDev &b, const EvalDev &ev, int stages, cudaStream_t st) {
+    if constexpr (S <= kWideStagesMax) {
+        if (stages == S) return launch_evaluate_one<T, S>(t, b, ev, st);
+    }
+    if constexpr (S < HI) return evaluate_dispatch<T, S + 1, HI>(t, b, ev, stages, st);
+    else return cudaErrorInvalidValue;
+}
+template <typename T, int LO, int HI>
+cudaError_t launch_evaluate_range(const Tables &t, const BatchDev &b, const EvalDev &ev, int stages, cudaStream_t st) {
+    return evaluate_dispatch<T, LO, HI>(t, b, ev, stages, st);
 }
 
 // Deep pipelines are instantiated per stage count; the stage counts LO .. HI of one cost type

@@ -365,11 +365,31 @@ cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo,
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st);
 cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);   // cm_tiebreak.cu
 cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st);
+// Candidates of a space one by one (cm_evaluate.cu).  EvalDev: outputs (any may be NULL) and, for the
+// binned path, the lists of candidates by depth.
+struct EvalDev {
+    const uint64_t *idx;      // candidate indices, or NULL: first, first + 1, ..
+    uint64_t first, count, n_cand;
+    double *cost;
+    int64_t *cost_ns;
+    uint8_t *feas;
+    uint4 *list;              // region q holds up to `slab` entries: slot | flags, template segment, 64 bits of composition
+    uint32_t *n_list;         // entries per region
+    uint8_t place[64];        // region -> its place in the list, in units of `slab`
+    uint32_t slab;            // candidates per round
+    uint64_t base;            // first candidate of the round
+};
+constexpr uint32_t kEvalMinMax = 0x80000000u, kEvalMasked = 0x40000000u;   // flags of an entry's slot
+constexpr int kEvalShallow = kRegStagesMax, kEvalRest = kWideStagesMax + 1, kEvalRegions = kEvalRest + 1;   // regions by depth: up to 16, 17 .. 48, deeper
+constexpr uint32_t kEvalSlabMax = 1u << 18, kEvalListMax = 1u << 20;
+constexpr uint64_t kEvalWarpMax = 8192;    // deep spaces: calls of up to this many candidates are evaluated a warp per candidate
+// Entries of the binned path's workspace for a space whose depths are `stages` (bit S-1), counters included; 0 = not needed.
+uint64_t eval_workspace(uint64_t stages, uint32_t *slab);
 // single_policy < 0: candidates of the dynamic-parallelism segments; otherwise the one
 // candidate of that policy (its cost must already be in pol_cost of scenario 0)
-cudaError_t launch_evaluate(const Tables &t, const BatchDev &b, uint64_t n_cand, int single_policy,
-                            uint64_t first, uint64_t count, const uint64_t *idx, double *cost,
-                            int64_t *cost_ns, uint8_t *feas, cudaStream_t st);
+cudaError_t launch_evaluate(const Tables &t, const BatchDev &b, EvalDev ev, int single_policy, uint64_t stages, uint4 *workspace,
+                            cudaStream_t st, const SideStreams *side);
+cudaError_t launch_evaluate_deep(const Tables &t, const BatchDev &b, const EvalDev &ev, int stages, cudaStream_t st);   // one region of 17 .. 48 stages
 // cm_restore.cu
 cudaError_t launch_shortlist(const Tables &t, const BatchDev &b, const ObjDev &o, cudaStream_t st);
 cudaError_t launch_plan_matching(const Tables &t, const BatchDev &b, const ObjDev &o, cudaStream_t st);

@@ -9,7 +9,7 @@
 //   cm_winner_kernel      finishes that argmin and decodes the winner
 //   (pass 2, the lowest layer composition that meets the winning cost: cm_tiebreak.cu)
 //   cm_finalize_kernel    assembles the plans and picks the best policy
-//   cm_evaluate_kernel    per-candidate cost / feasibility for cm_evaluate
+//   (per-candidate cost / feasibility for cm_evaluate: cm_evaluate.cu)
 //   cm_pick_kernel        best of several spaces for cm_select
 #include <algorithm>
 #include <atomic>
@@ -360,19 +360,6 @@ cudaError_t launch_useg_copy(const BatchDev &b, const USegDev &u, cudaStream_t s
 }
 
 // ----------------------------------------------------------------------------------
-// Locate the segment that owns a tile / a candidate: the last row whose first index is
-// not above the query (rows are sorted and every segment owns at least one).
-// ----------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t find_row(const TSeg *seg, uint32_t n, uint64_t q) {
-    uint32_t lo = 0, hi = n - 1;
-    while (lo < hi) {
-        uint32_t mid = (lo + hi + 1) >> 1;
-        if (seg[mid].cand_first <= q) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// ----------------------------------------------------------------------------------
 // Split reduction: item = (strategy, split rank) of one scenario; its step time is the
 // slowest pipeline's best cost (Section "Estimator": step time = max over pipelines).
 // Hierarchical argmin carrying (cost, item) with the lowest item on ties:
@@ -546,61 +533,6 @@ cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st)
     if (b.B <= 0) return cudaSuccess;
     const uint64_t inf = batch_inf_bits(b);
     cm_finalize_kernel<<<(b.B + 127) / 128, 128, 0, st>>>(t, b, inf);
-    return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------------
-// cm_evaluate: one thread per requested candidate.
-// ----------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(128) cm_evaluate_kernel(Tables tb, BatchDev bd, uint64_t first, uint64_t count,
-                                                          const uint64_t *idx, uint64_t n_cand, double *cost,
-                                                          int64_t *cost_ns, uint8_t *feas) {
-    __shared__ SProf<T> sp;
-    stage_profile(sp, tb);
-    __syncthreads();
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count) return;
-    const uint64_t e = idx ? idx[t] : first + t;
-    T c = Num<T>::inf();
-    bool ok = false;
-    if (e < n_cand) {
-        // spaces hold one scenario: its template's segments are sorted by first candidate
-        const Tmpl tp = bd.tmpl[bd.scen[0].tmpl];
-        const uint32_t s = tp.tseg_first + find_row(bd.tseg + tp.tseg_first, tp.n_tseg, e);
-        const SegView g = seg_view(bd, 0, s);
-        T v;
-        if (segment_candidate_cost<T>(sp, tb, g, bd.layer_mode, e - bd.tseg[s].cand_first, v)) { c = v; ok = true; }
-    }
-    if (cost && bd.mode == CM_COST_FP64) cost[t] = __longlong_as_double((long long)Num<T>::bits(c));
-    if (cost_ns && bd.mode == CM_COST_INT64NS) cost_ns[t] = batch_cost_ns(bd, Num<T>::bits(c));
-    if (feas) feas[t] = ok ? 1 : 0;
-}
-
-// One-candidate policies through cm_evaluate: the cost cm_policy_kernel left behind.
-__global__ void cm_evaluate_single_kernel(BatchDev bd, int policy, uint64_t inf, uint64_t first, uint64_t count,
-                                          const uint64_t *idx, double *cost, int64_t *cost_ns, uint8_t *feas) {
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count) return;
-    const uint64_t e = idx ? idx[t] : first + t;
-    uint64_t c = e == 0 ? bd.pol_cost[policy] : inf;
-    if (cost && bd.mode == CM_COST_FP64) cost[t] = __longlong_as_double((long long)c);
-    if (cost_ns && bd.mode == CM_COST_INT64NS) cost_ns[t] = batch_cost_ns(bd, c);
-    if (feas) feas[t] = c < inf ? 1 : 0;
-}
-
-cudaError_t launch_evaluate(const Tables &t, const BatchDev &b, uint64_t n_cand, int single_policy,
-                            uint64_t first, uint64_t count, const uint64_t *idx, double *cost,
-                            int64_t *cost_ns, uint8_t *feas, cudaStream_t st) {
-    if (count == 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((count + 127) / 128);
-    const uint64_t inf = batch_inf_bits(b);
-    if (single_policy >= 0)
-        cm_evaluate_single_kernel<<<blocks, 128, 0, st>>>(b, single_policy, inf, first, count, idx, cost, cost_ns, feas);
-    else if (native_i64(b))
-        cm_evaluate_kernel<long long><<<blocks, 128, 0, st>>>(t, b, first, count, idx, n_cand, cost, cost_ns, feas);
-    else
-        cm_evaluate_kernel<double><<<blocks, 128, 0, st>>>(t, b, first, count, idx, n_cand, cost, cost_ns, feas);
     return cudaGetLastError();
 }
 
