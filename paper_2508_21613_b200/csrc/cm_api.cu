@@ -149,6 +149,12 @@ struct Batch {
     BoundDev bo{};
     size_t off_bbucket = 0;
     DevBuf<SearchWin> d_win;
+    // device memory held (what a spare batch ties up)
+    size_t bytes() const {
+        return d_arena.cap + 8 * (d_seg_best.cap + d_kappa_sel.cap + d_pol_cost.cap + d_utab.cap + d_useg.cap + d_short_kappa.cap) +
+               sizeof(Partial) * d_partial.cap + sizeof(Winner) * (d_winner.cap + d_short_win.cap) + sizeof(cm_plan) * (d_plans.cap + d_short_plans.cap) +
+               4 * (d_urep.cap + d_slot_of.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
+    }
     int k_best = 1;                       // (strategy, split) pairs whose step times have to be exact
 };
 
@@ -160,7 +166,7 @@ struct cm_ctx {
     // the generation they were built under: their segment shapes, min-max keys and candidate
     // counts describe that profile's L and G, so they are refused once another profile is loaded.
     uint64_t profile_gen = 0;
-    DevBuf<unsigned char> d_scratch;  // small per-call device scratch (cm_select, cm_transfer_matching): grown, never shrunk
+    DevBuf<unsigned char> d_scratch;  // per-call device scratch of cm_transfer_matching: grown, never shrunk
     DevProfile hp{};                  // host copy: scalars, raw inputs, base cuts
     DevProfile *d_prof = nullptr;
     // The integer-nanosecond mode normally runs in double arithmetic: its inputs are integers,
@@ -198,6 +204,10 @@ struct cm_ctx {
     bool dedup = true;                // search a pipeline that several strategies of a survivor count share once (cm_set_pipeline_reuse)
     bool pairs = true;                // one recurrence for a pipeline's m and m+1 micro-batch variants (cm_set_micro_batch_pairs)
     Batch batch;                      // reused by cm_search_batch
+    // Batches of freed spaces and prepared batches, kept for the next ones: a batch is a dozen device
+    // and pinned buffers, and allocating them costs more than building and searching a 32-device space.
+    // At most kSpareBatches of them and none above kSpareBytes; released with the context.
+    std::vector<std::unique_ptr<Batch>> spare;
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     cudaEvent_t ev_obj[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // phases of the objective pass
     uint64_t obj_stats[8] = {0};
@@ -232,17 +242,30 @@ struct cm_ctx {
 struct cm_space {
     cm_ctx *ctx = nullptr;
     int policy = 0;
-    Batch batch;
+    std::unique_ptr<Batch> own;           // taken from the context's spare batches, given back by cm_space_free
     std::vector<uint32_t> failed;
 };
 
 struct cm_batch {
     cm_ctx *ctx = nullptr;
-    Batch batch;
+    std::unique_ptr<Batch> own;           // as above
     int prep_launches = 0;
 };
 
 namespace {
+
+constexpr size_t kSpareBatches = 8, kSpareBytes = 16u << 20;
+
+std::unique_ptr<Batch> take_batch(cm_ctx *c) {
+    if (c->spare.empty()) return std::unique_ptr<Batch>(new (std::nothrow) Batch());
+    std::unique_ptr<Batch> b = std::move(c->spare.back());
+    c->spare.pop_back();
+    return b;
+}
+// The caller has synchronised the context's stream: nothing queued uses the batch any more.
+void give_batch(cm_ctx *c, std::unique_ptr<Batch> b) {
+    if (b && c->spare.size() < kSpareBatches && b->bytes() <= kSpareBytes) c->spare.push_back(std::move(b));
+}
 
 cm_status fail(cm_ctx *c, cm_status s, const std::string &msg) {
     if (c) c->err = msg;
@@ -885,7 +908,7 @@ cm_status build_template(cm_ctx *ctx, Batch &bt, int n_surv, uint32_t *out) {
     }
     tp.n_split_total = split_first;
     tp.n_cand = cand;
-    tp.n_red = split_first ? (uint32_t)std::min<uint64_t>((split_first + 1023) / 1024, 64) : 0;
+    tp.n_red = split_first && o.bm == CM_BATCH_FULL ? (uint32_t)std::min<uint64_t>((split_first + 1023) / 1024, 64) : 0;   // (the remainder rule reduces strategies)
     *out = (uint32_t)bt.tmpl.size();
     bt.tmpl.push_back(tp);
     return CM_OK;
@@ -1347,13 +1370,9 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
             CM_CUDA(ctx, launch_useg_copy(bd, useg_view(bt), st));
             ++launches;
         }
-        if (bt.n_dup) {  // pipelines that strategies have in common were searched once
-            CM_CUDA(ctx, launch_dup_copy(bd, st));
-            ++launches;
-        }
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
         CM_CUDA(ctx, launch_split_reduce(tb, bd, st));
-        launches += (bd.n_red_blocks && bd.max_red_per_scen > 1) ? 2 : 1;
+        launches += (bd.batch_mode == CM_BATCH_FULL && bd.n_red_blocks && bd.max_red_per_scen > 1) ? 2 : 1;
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
         if (bt.n_tiles) {
             CM_CUDA(ctx, launch_tiebreak(tb, bd, st));
@@ -1367,9 +1386,28 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
     const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
     CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, back_bytes, cudaMemcpyDeviceToHost, st));
-    *launches_out = launches;
-    *cost_launches_out = cost_launches;
+    *launches_out += launches;
+    *cost_launches_out += cost_launches;
     return CM_OK;
+}
+
+// Work counters of a finished search (they came back behind its plans).
+const unsigned long long *search_counters(const Batch &bt) {
+    return reinterpret_cast<const unsigned long long *>(bt.plans_host.p + (size_t)bt.B * 4);
+}
+void account_search(cm_ctx *ctx, const Batch &bt, int launches) {
+    const unsigned long long *counters_host = search_counters(bt);
+    ctx->stats[0] += (bt.policy_mask & (1u << CM_DYNPAR)) ? bt.n_cand : 0;
+    ctx->stats[19] += (bt.policy_mask & (1u << CM_DYNPAR)) ? bt.n_cand_own : 0;
+    ctx->stats[1] += counters_host[0];
+    ctx->stats[2] += counters_host[1];
+    ctx->stats[16] += counters_host[2];
+    ctx->stats[20] += bt.bounded ? counters_host[3] : counters_host[0];
+    ctx->stats[21] += bt.bounded ? counters_host[5] : counters_host[2];
+    ctx->stats[3] += (uint64_t)launches;
+    ctx->stats[5] += bt.n_rows;
+    ctx->stats[6] += bt.strat.size();
+    ctx->stats[7] += bt.n_split;
 }
 
 // The search over an uploaded batch; results land in bt.plans_host ([B][4]) after the stream is
@@ -1387,6 +1425,7 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
             cudaGraph_t graph = nullptr;
             bool ok = cudaStreamBeginCapture(ctx->graph_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
             if (ok) {
+                single->launches = 0;
                 const cm_status cs = enqueue_search(ctx, bt, ctx->graph_stream, false, &single->launches, &cost_launches);
                 const cudaError_t ce = cudaStreamEndCapture(ctx->graph_stream, &graph);
                 ok = cs == CM_OK && ce == cudaSuccess && graph;
@@ -1422,8 +1461,7 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
         ctx->stats[12] += (uint64_t)cost_launches;
     }
     ctx->stats[10] += back_bytes;
-    const unsigned long long *counters_host = reinterpret_cast<const unsigned long long *>(bt.plans_host.p + (size_t)bt.B * 4);
-    if (bt.bounded && counters_host[4]) {
+    if (bt.bounded && search_counters(bt)[4]) {
         // a list was full (plans whose bounds tie in their hundreds of thousands): search again, every plan
         if (single && single->exec) { cudaGraphExecDestroy(single->exec); single->exec = nullptr; }
         bt.dense_only = true;
@@ -1431,18 +1469,8 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
         if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
         return s == CM_OK ? run_batch(ctx, bt, launches, single) : s;
     }
-    ctx->stats[0] += (bt.policy_mask & (1u << CM_DYNPAR)) ? bt.n_cand : 0;
-    ctx->stats[19] += (bt.policy_mask & (1u << CM_DYNPAR)) ? bt.n_cand_own : 0;
-    ctx->stats[1] += counters_host[0];
-    ctx->stats[2] += counters_host[1];
-    ctx->stats[16] += counters_host[2];
-    ctx->stats[20] += bt.bounded ? counters_host[3] : counters_host[0];
-    ctx->stats[21] += bt.bounded ? counters_host[5] : counters_host[2];
-    ctx->stats[3] += (uint64_t)launches;
+    account_search(ctx, bt, launches);
     ctx->stats[4] += (uint64_t)((double)ms * 1e6);
-    ctx->stats[5] += bt.n_rows;
-    ctx->stats[6] += bt.strat.size();
-    ctx->stats[7] += bt.n_split;
     return CM_OK;
 }
 
@@ -1542,7 +1570,7 @@ int cm_internal_grid_devices(const cm_ctx *ctx) { return ctx && ctx->has_profile
 
 cm_status cm_internal_space_view(cm_ctx *ctx, const cm_space *space, SpaceView *out) {
     if (!space || space->ctx != ctx) return fail(ctx, CM_EINVAL, "space does not belong to this context");
-    Batch &bt = const_cast<Batch &>(space->batch);
+    Batch &bt = *space->own;
     if (stale(ctx, bt)) return fail(ctx, CM_EINVAL, kStaleMsg);
     out->tb = tables(ctx, bt);
     out->bd = dev_view(ctx, bt);
@@ -1601,7 +1629,6 @@ cm_status cm_create(cm_ctx **out, int cuda_device, void *cuda_stream) {
              cudaEventCreateWithFlags(&c->side.join[i], cudaEventDisableTiming) == cudaSuccess;
         if (ok) c->side.n = i + 1;
     }
-    ok = ok && c->d_scratch.reserve(sizeof(cm_plan *) * 64 + sizeof(cm_plan));   // what cm_select needs
     // the feasible-composition pool and its staging are allocated here, not at the first search:
     // a pinned allocation costs milliseconds, which a failure handler should not pay
     ok = ok && c->d_feas.reserve(1u << 20) && c->d_feas_mask.reserve(1u << 20) && c->feas_stage.reserve(1u << 16) && c->d_feas_stage.reserve(1u << 16);
@@ -1807,29 +1834,31 @@ cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids
     if (!sp) return fail(ctx, CM_ENOMEM, "host memory");
     sp->ctx = ctx;
     sp->policy = policy;
+    sp->own = take_batch(ctx);
+    if (!sp->own) return fail(ctx, CM_ENOMEM, "host memory");
     sp->failed.assign(failed_ids, failed_ids + n_failed);
     const int32_t offsets[2] = {0, n_failed};
-    s = build_batch(ctx, sp->batch, failed_ids, offsets, 1, o, 1u << policy);
-    if (s == CM_OK) s = upload_batch(ctx, sp->batch, nullptr);
+    s = build_batch(ctx, *sp->own, failed_ids, offsets, 1, o, 1u << policy);
+    if (s == CM_OK) s = upload_batch(ctx, *sp->own, nullptr);
     if (s == CM_OK && policy != CM_DYNPAR) {
         // the one candidate of these policies is evaluated right away so that
         // cm_evaluate can hand its cost out
-        cudaError_t e = launch_policies(tables(ctx, sp->batch), dev_view(ctx, sp->batch), ctx->hp.n_dp, ctx->stream);
+        cudaError_t e = launch_policies(tables(ctx, *sp->own), dev_view(ctx, *sp->own), ctx->hp.n_dp, ctx->stream);
         if (e != cudaSuccess) s = fail(ctx, CM_ECUDA, cudaGetErrorString(e));
     }
     if (s != CM_OK) {
         cudaStreamSynchronize(ctx->stream);
-        forget_keys(ctx, sp->batch);
+        forget_keys(ctx, *sp->own);
         return s;
     }
     // cm_evaluate only enqueues: the workspace it bins candidates in (once per context) is found here
     uint32_t slab = 0;
-    const uint64_t want = policy == CM_DYNPAR ? eval_workspace(stage_mask(sp->batch), &slab) : 0;
+    const uint64_t want = policy == CM_DYNPAR ? eval_workspace(stage_mask(*sp->own), &slab) : 0;
     if (want > ctx->d_eval.cap) {
         CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // growing frees the old block
         if (!ctx->d_eval.reserve(want)) return fail(ctx, CM_ENOMEM, "device memory");
     }
-    if (n_candidates) *n_candidates = policy == CM_DYNPAR ? sp->batch.n_cand : 1;
+    if (n_candidates) *n_candidates = policy == CM_DYNPAR ? sp->own->n_cand : 1;
     *out = sp.release();
     return CM_OK;
     CM_API_END(ctx)
@@ -1837,10 +1866,13 @@ cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids
 
 cm_status cm_space_free(cm_space *sp) {
     if (!sp) return CM_EINVAL;
+    CM_API_BEGIN
     cudaSetDevice(sp->ctx->device);
     cudaStreamSynchronize(sp->ctx->stream);   // queued copies still read its host tables
-    delete sp;
+    std::unique_ptr<cm_space> gone(sp);
+    give_batch(sp->ctx, std::move(sp->own));
     return CM_OK;
+    CM_API_END(nullptr)
 }
 
 cm_status cm_evaluate(cm_ctx *ctx, const cm_space *space, uint64_t first, uint64_t count,
@@ -1851,7 +1883,7 @@ cm_status cm_evaluate(cm_ctx *ctx, const cm_space *space, uint64_t first, uint64
     // one thread per candidate, 128 per block, the block count a 31-bit grid dimension
     if (count > 0x7fffffffull * 128ull) return fail(ctx, CM_EINVAL, "count too large: at most (2^31 - 1) * 128 candidates per call");
     CM_CUDA(ctx, cudaSetDevice(ctx->device));
-    Batch &bt = const_cast<Batch &>(space->batch);
+    Batch &bt = *space->own;
     if (stale(ctx, bt)) return fail(ctx, CM_EINVAL, kStaleMsg);
     const uint64_t n_cand = space->policy == CM_DYNPAR ? bt.n_cand : 1;
     if (!idx_dev && (first > n_cand || count > n_cand - first)) return fail(ctx, CM_EINVAL, "candidate range out of bounds");
@@ -1875,30 +1907,74 @@ cm_status cm_select(cm_ctx *ctx, cm_space *const *spaces, int32_t n_spaces, cm_p
     if (!spaces || n_spaces < 1 || n_spaces > 64 || !best) return fail(ctx, CM_EINVAL, "bad arguments");
     for (int i = 0; i < n_spaces; ++i) {
         if (!spaces[i] || spaces[i]->ctx != ctx) return fail(ctx, CM_EINVAL, "space does not belong to this context");
-        if (stale(ctx, spaces[i]->batch)) return fail(ctx, CM_EINVAL, kStaleMsg);
-        if (spaces[i]->batch.opts.cost != spaces[0]->batch.opts.cost) return fail(ctx, CM_EINVAL, "spaces mix cost modes");
+        if (stale(ctx, *spaces[i]->own)) return fail(ctx, CM_EINVAL, kStaleMsg);
+        if (spaces[i]->own->opts.cost != spaces[0]->own->opts.cost) return fail(ctx, CM_EINVAL, "spaces mix cost modes");
     }
     CM_CUDA(ctx, cudaSetDevice(ctx->device));
     memset(ctx->stats, 0, sizeof(ctx->stats));
-    const int mode = spaces[0]->batch.opts.cost;
-    std::vector<const cm_plan *> ptrs(n_spaces);
-    for (int i = 0; i < n_spaces; ++i) {
-        cm_status s = run_batch(ctx, spaces[i]->batch, 0);
-        if (s != CM_OK) return s;
-        ptrs[i] = spaces[i]->batch.d_plans.p + spaces[i]->policy;
+    // Enqueue every space -- the one-plan policies beside the dynamic-parallelism search, which does not
+    // wait for them -- and synchronise once.  (Several dynamic-parallelism spaces go one after the other:
+    // they share the list of the bounded search pass.)
+    cudaStream_t st = ctx->stream;
+    int n_dyn = 0, launches = 0, cost_launches = 0;
+    for (int i = 0; i < n_spaces; ++i) n_dyn += spaces[i]->policy == CM_DYNPAR;
+    for (int i = 0; i < n_spaces; ++i)
+        if (!spaces[i]->own->plans_host.resize((size_t)spaces[i]->own->B * 4 + 1)) return fail(ctx, CM_ENOMEM, "host memory");
+    const bool beside = n_dyn && n_dyn < n_spaces && ctx->pol_stream;
+    const uint64_t h_enqueue = now_ns();
+    CM_CUDA(ctx, cudaEventRecord(ctx->ev[0], st));
+    if (beside) {
+        CM_CUDA(ctx, cudaEventRecord(ctx->pol_fork, st));
+        CM_CUDA(ctx, cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0));
     }
-    // best over the spaces, on the device as well (scratch of the context: 64 pointers and a plan
-    // were reserved by cm_create, so this call allocates nothing)
-    if (!ctx->d_scratch.reserve(sizeof(cm_plan *) * 64 + sizeof(cm_plan))) return fail(ctx, CM_ENOMEM, "device memory");
-    const cm_plan **d_ptrs = reinterpret_cast<const cm_plan **>(ctx->d_scratch.p);
-    cm_plan *d_out = reinterpret_cast<cm_plan *>(ctx->d_scratch.p + sizeof(cm_plan *) * 64);
+    cm_status s = CM_OK;
+    for (int i = 0; i < n_spaces && s == CM_OK; ++i)
+        if (spaces[i]->policy != CM_DYNPAR || n_dyn == 1)
+            s = enqueue_search(ctx, *spaces[i]->own, spaces[i]->policy != CM_DYNPAR && beside ? ctx->pol_stream : st,
+                               spaces[i]->policy == CM_DYNPAR, &launches, &cost_launches);
+    if (beside) {   // joined even after a failure, so that no side stream runs ahead unobserved
+        const cudaError_t e1 = cudaEventRecord(ctx->pol_join, ctx->pol_stream), e2 = cudaStreamWaitEvent(st, ctx->pol_join, 0);
+        if (s == CM_OK) { CM_CUDA(ctx, e1); CM_CUDA(ctx, e2); }
+    }
+    if (s != CM_OK) return s;
+    CM_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
+    const uint64_t h_wait = now_ns();
+    CM_CUDA(ctx, cudaStreamSynchronize(st));
+    ctx->stats[14] += h_wait - h_enqueue;
+    ctx->stats[15] += now_ns() - h_wait;
+    float ms = 0.f;
+    CM_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]));
+    ctx->stats[4] += (uint64_t)((double)ms * 1e6);
+    if (n_dyn == 1) {
+        float ms_cost = 0.f, ms_tie = 0.f;
+        CM_CUDA(ctx, cudaEventElapsedTime(&ms_cost, ctx->ev[2], ctx->ev[3]));
+        CM_CUDA(ctx, cudaEventElapsedTime(&ms_tie, ctx->ev[4], ctx->ev[5]));
+        ctx->stats[8] += (uint64_t)((double)ms_cost * 1e6);
+        ctx->stats[11] += (uint64_t)((double)ms_tie * 1e6);
+        ctx->stats[12] += (uint64_t)cost_launches;
+    }
+    for (int i = 0; i < n_spaces; ++i) {
+        Batch &bt = *spaces[i]->own;
+        if (spaces[i]->policy == CM_DYNPAR && (n_dyn > 1 || (bt.bounded && search_counters(bt)[4]))) {
+            s = run_batch(ctx, bt, 0);
+            if (s != CM_OK) return s;
+            continue;
+        }
+        ctx->stats[10] += (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
+        account_search(ctx, bt, 0);
+    }
+    ctx->stats[3] += (uint64_t)launches;
+    // least cost, ties to the lowest policy id, then to the earlier space
+    const bool whole = spaces[0]->own->opts.cost == CM_COST_INT64NS;
     cm_plan result;
-    cudaError_t e = cudaMemcpyAsync(d_ptrs, ptrs.data(), sizeof(cm_plan *) * n_spaces, cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess) e = launch_pick(d_ptrs, n_spaces, d_out, mode, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&result, d_out, sizeof(cm_plan), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) { cudaGetLastError(); return fail(ctx, CM_ECUDA, cudaGetErrorString(e)); }
-    ctx->stats[3] += 1;
+    memset(&result, 0, sizeof(result));
+    for (int i = 0; i < n_spaces; ++i) {
+        const cm_plan &q = spaces[i]->own->plans_host[spaces[i]->policy];
+        if (!q.feasible) continue;
+        const bool less = whole ? q.cost_ns < result.cost_ns : q.cost < result.cost;
+        const bool equal = whole ? q.cost_ns == result.cost_ns : q.cost == result.cost;
+        if (!result.feasible || less || (equal && q.policy < result.policy)) result = q;
+    }
     scrub(result);
     *best = result;
     if (!result.feasible) return fail(ctx, CM_ENOFEASIBLE, "no feasible plan in the given spaces");
@@ -2215,16 +2291,18 @@ cm_status cm_batch_prepare(cm_ctx *ctx, const uint32_t *failed_ids, const int32_
     std::unique_ptr<cm_batch> bp(new (std::nothrow) cm_batch());
     if (!bp) return fail(ctx, CM_ENOMEM, "host memory");
     bp->ctx = ctx;
+    bp->own = take_batch(ctx);
+    if (!bp->own) return fail(ctx, CM_ENOMEM, "host memory");
     memset(ctx->stats, 0, sizeof(ctx->stats));
     const uint32_t mask = (1u << CM_REROUTE) | (1u << CM_REDUNDANT) | (1u << CM_DYNPAR);
-    s = build_batch(ctx, bp->batch, failed_ids, offsets, B, *opts, mask);
-    if (s == CM_OK) s = upload_batch(ctx, bp->batch, &bp->prep_launches);
+    s = build_batch(ctx, *bp->own, failed_ids, offsets, B, *opts, mask);
+    if (s == CM_OK) s = upload_batch(ctx, *bp->own, &bp->prep_launches);
     if (s != CM_OK) {
         cudaStreamSynchronize(ctx->stream);
-        forget_keys(ctx, bp->batch);
+        forget_keys(ctx, *bp->own);
         return s;
     }
-    if (n_candidates) *n_candidates = bp->batch.n_cand;
+    if (n_candidates) *n_candidates = bp->own->n_cand;
     *out = bp.release();
     return CM_OK;
     CM_API_END(ctx)
@@ -2234,10 +2312,10 @@ cm_status cm_batch_search(cm_ctx *ctx, cm_batch *bp, cm_plan *best_per_scenario,
     if (!ctx) return CM_EINVAL;
     CM_API_BEGIN
     if (!bp || bp->ctx != ctx || !best_per_scenario) return fail(ctx, CM_EINVAL, "bad arguments");
-    if (stale(ctx, bp->batch)) return fail(ctx, CM_EINVAL, kStaleMsg);
+    if (stale(ctx, *bp->own)) return fail(ctx, CM_EINVAL, kStaleMsg);
     CM_CUDA(ctx, cudaSetDevice(ctx->device));
     memset(ctx->stats, 0, sizeof(ctx->stats));
-    Batch &bt = bp->batch;
+    Batch &bt = *bp->own;
     if (bt.B == 0) return CM_OK;
     cm_status s = run_batch(ctx, bt, 0);
     if (s != CM_OK) return s;
@@ -2257,10 +2335,13 @@ cm_status cm_batch_search(cm_ctx *ctx, cm_batch *bp, cm_plan *best_per_scenario,
 
 cm_status cm_batch_free(cm_batch *bp) {
     if (!bp) return CM_EINVAL;
+    CM_API_BEGIN
     cudaSetDevice(bp->ctx->device);
     cudaStreamSynchronize(bp->ctx->stream);
-    delete bp;
+    std::unique_ptr<cm_batch> gone(bp);
+    give_batch(bp->ctx, std::move(bp->own));
     return CM_OK;
+    CM_API_END(nullptr)
 }
 
 cm_status cm_last_stats(const cm_ctx *ctx, uint64_t out[24]) {
@@ -2273,7 +2354,7 @@ cm_status cm_decode_plan(cm_ctx *ctx, const cm_space *space, const cm_plan *plan
     if (!ctx) return CM_EINVAL;
     CM_API_BEGIN
     if (!space || space->ctx != ctx || !plan || !cuts_out) return fail(ctx, CM_EINVAL, "bad arguments");
-    if (stale(ctx, space->batch)) return fail(ctx, CM_EINVAL, kStaleMsg);
+    if (stale(ctx, *space->own)) return fail(ctx, CM_EINVAL, kStaleMsg);
     if (plan->policy != space->policy) return fail(ctx, CM_EINVAL, "plan was not found in this space");
     const DevProfile &hp = ctx->hp;
     CM_CUDA(ctx, cudaSetDevice(ctx->device));
@@ -2294,7 +2375,7 @@ cm_status cm_decode_plan(cm_ctx *ctx, const cm_space *space, const cm_plan *plan
             }
         }
     } else {
-        const Batch &bt = space->batch;
+        const Batch &bt = *space->own;
         const Tmpl &tp = bt.tmpl[bt.scen[0].tmpl];
         if (plan->strategy >= tp.n_strat) return fail(ctx, CM_EINVAL, "strategy index out of range");
         const Strat &st = bt.strat[tp.strat_first + plan->strategy];

@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "cm_bound_lane.cuh"
+#include "cm_split.cuh"
 
 namespace cm {
 
@@ -150,80 +151,15 @@ cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo,
 }
 
 // ----------------------------------------------------------------------------------
-// Window of a scenario under the remainder rule: a strategy hands one more micro-batch to R of its
-// pipelines, every choice of them a split, so its best step time is the least value t among its
-// pipelines' two costs such that those that cannot do with their smaller share (cost above t) number
-// at most R, all pipelines that can take the larger one (cost at most t) number at least R, and the
-// former are among the latter; C(may - must, R - must) splits then stay within t.  A warp per
-// strategy; phase 0 works on the bounds, phase 1 on the results.  Either then marks the segments of the
-// strategies whose step time from bounds is still within reach.
+// Window of a scenario: the best step time of any of its strategies (cm_split.cuh), from the bounds
+// (phase 0) or the results (phase 1).  Either then marks the segments of the strategies whose step time
+// from bounds is still within reach.
+// ----------------------------------------------------------------------------------
 // ----------------------------------------------------------------------------------
 // Phase 0 marks strategies this far above the best step time from bounds: one plan of each of their
 // segments is evaluated, so that a result that misses its bound a little still leaves phase 2 nothing to do.
 constexpr float kReach = 1.0f / (1 << 13);
 constexpr int kWinThreads = 128;
-
-__device__ __forceinline__ uint32_t canon_row(const BatchDev &bd, const Tmpl &tp, const Scen &sc, const Strat &s, int p, int k) {
-    uint32_t t = s.seg_first + p * s.n_m + k;
-    if (bd.tseg_canon) t = bd.tseg_canon[t];
-    return sc.seg_base + (t - tp.tseg_first);
-}
-
-// The two costs of every pipeline of a strategy, a lane each: lane 2p + k holds pipeline p with its
-// smaller (k = 0) or larger share (2 kMaxP = 32 lanes).
-__device__ __forceinline__ uint64_t strat_cost(const BatchDev &bd, const BoundDev &bo, const Tmpl &tp, const Scen &sc, const Strat &s,
-                                               int phase, uint64_t inf) {
-    const int p = (threadIdx.x & 31) >> 1, k = threadIdx.x & 1;
-    uint64_t v = inf;
-    if (p < s.dp && k < s.n_m && s.m_lo[p] + k >= 1) {
-        const uint32_t row = canon_row(bd, tp, sc, s, p, k);
-        v = phase ? bd.seg_best[row] : (uint64_t)(bo.lbarg[row] >> 32);
-    }
-    return v < inf ? v : inf;
-}
-
-// Is there a split of the strategy within this lane's t, and how many?
-__device__ __forceinline__ bool splits_within(uint64_t v, int dp, int R, uint64_t t, int &free_ones, int &left) {
-    int may = 0, must = 0;
-    bool ok = true;
-    for (int p = 0; p < dp; ++p) {
-        const bool need = __shfl_sync(0xffffffffu, v, 2 * p) > t, can = __shfl_sync(0xffffffffu, v, 2 * p + 1) <= t;
-        may += can;
-        must += need;
-        ok = ok && (can || !need);
-    }
-    free_ones = may - must;
-    left = R - must;
-    return ok && left >= 0 && may >= R;
-}
-
-// Least step time above `after` (~0: any) of a strategy, in every lane.
-__device__ __forceinline__ uint64_t strat_best(uint64_t v, const Strat &s, uint64_t after, uint64_t inf) {
-    const int lane = threadIdx.x & 31, dp = s.dp, R = s.R;
-    const bool mine = lane < 2 * dp;
-    if (after == ~0ull) {
-        // Where no pipeline is cheaper with the larger share (always so for bounds, and for results that
-        // are all there): everybody's smaller share, and the R cheapest larger ones.
-        const uint64_t other = __shfl_xor_sync(0xffffffffu, v, 1);
-        if (!R || __all_sync(0xffffffffu, !mine || (lane & 1 ? v >= other : v <= other))) {
-            uint64_t t = ~warp_min_u64(mine && !(lane & 1) ? ~v : ~0ull);   // largest of the smaller shares
-            if (R) {
-                int below = 0;
-                for (int p = 0; p < dp; ++p) {
-                    const uint64_t h = __shfl_sync(0xffffffffu, v, 2 * p + 1);
-                    below += h < v || (h == v && 2 * p + 1 < lane);
-                }
-                const uint32_t who = __ballot_sync(0xffffffffu, mine && (lane & 1) && below == R - 1);
-                const uint64_t at = who ? __shfl_sync(0xffffffffu, v, __ffs(who) - 1) : inf;
-                t = at > t ? at : t;
-            }
-            return t;
-        }
-    }
-    int f, l;
-    const bool ok = splits_within(v, dp, R, v, f, l) && mine && v < inf && (after == ~0ull || v > after);
-    return warp_min_u64(ok ? v : inf);
-}
 
 __device__ __forceinline__ uint64_t block_min_u64(uint64_t v /* warp-uniform */, uint64_t *red) {
     __syncthreads();
@@ -243,12 +179,15 @@ __global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, Batch
     const uint32_t warp = threadIdx.x >> 5, warps = kWinThreads / 32;
     const int lane = threadIdx.x & 31;
     const uint64_t inf = phase ? inf_cost : 0xffffffffull;
+    auto cost_of = [&](const Strat &s, int from_results, uint64_t most) {
+        return strat_cost(bd, tp, sc, s, most, [&](uint32_t row) { return from_results ? bd.seg_best[row] : (uint64_t)(bo.lbarg[row] >> 32); });
+    };
     uint64_t first = ~0ull, t = ~0ull;
     bool enough = false;
     for (int r = 0; r < k_best && !enough; ++r) {
         uint64_t mine = inf;
         for (uint32_t si = warp; si < tp.n_strat; si += warps) {
-            const uint64_t v = strat_best(strat_cost(bd, bo, tp, sc, strat[si], phase, inf), strat[si], t, inf);
+            const uint64_t v = strat_best(cost_of(strat[si], phase, inf), strat[si], t, inf);
             mine = v < mine ? v : mine;
         }
         t = block_min_u64(mine, red);
@@ -258,7 +197,7 @@ __global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, Batch
         __syncthreads();
         for (uint32_t si = warp; si < tp.n_strat; si += warps) {
             int f, l;
-            const bool ok = splits_within(strat_cost(bd, bo, tp, sc, strat[si], phase, inf), strat[si].dp, strat[si].R, t, f, l);
+            const bool ok = splits_within(cost_of(strat[si], phase, inf), strat[si].dp, strat[si].R, t, f, l);
             if (ok && lane == 0) atomicAdd(&total, (unsigned long long)binom_at(tb.binom, f, l));
         }
         __syncthreads();
@@ -280,7 +219,7 @@ __global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, Batch
     }
     for (uint32_t si = warp; si < tp.n_strat; si += warps) {
         const Strat &s = strat[si];
-        const uint64_t v = strat_best(strat_cost(bd, bo, tp, sc, s, 0, 0xffffffffull), s, ~0ull, 0xffffffffull);
+        const uint64_t v = strat_best(cost_of(s, 0, 0xffffffffull), s, ~0ull, 0xffffffffull);
         if (v >= 0xffffffffull || __uint_as_float((uint32_t)v) > reach) continue;   // warp-uniform
         const int p = lane >> 1, k = lane & 1;
         if (p < s.dp && k < s.n_m) {

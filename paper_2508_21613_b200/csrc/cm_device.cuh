@@ -379,7 +379,11 @@ __device__ __forceinline__ uint64_t item_step_time(const Tables &tb, const Batch
     for (int p = 0; p < s.dp; ++p) {
         uint64_t c = inf;
         const int off = (int)micro[p] - (int)s.m_lo[p];
-        if (micro[p] >= 1 && off >= 0 && off < s.n_m) c = best[s.seg_first - tp.tseg_first + p * s.n_m + off];
+        if (micro[p] >= 1 && off >= 0 && off < s.n_m) {
+            uint32_t t = s.seg_first + p * s.n_m + off;
+            if (bd.tseg_canon) t = bd.tseg_canon[t];   // (repeated pipelines: the first occurrence has the result)
+            c = best[t - tp.tseg_first];
+        }
         c = c > inf ? inf : c;   // a segment nobody improved still holds its all-ones initial value
         T = c > T ? c : T;
     }

@@ -259,8 +259,8 @@ struct BatchDev {
     // Strategies of one survivor count repeat pipelines: the same stages over the same survivors with
     // the same micro-batches and peers (the tuples (30,31,..) and (30,32,..) start with the same
     // pipeline).  Such template segments have the same candidates with the same costs in every
-    // scenario, so only the first of them -- tseg_canon[t] == t -- is searched; the others take its
-    // per-segment minimum afterwards (cm_dup_copy_kernel).  NULL: the batch has no duplicates.
+    // scenario, so only the first of them -- tseg_canon[t] == t -- is searched, and whoever wants the
+    // result of another looks there.  NULL: the batch has no duplicates.
     const uint32_t *tseg_canon;
     uint32_t n_rep_scen;          // scenarios that own result rows (entries of tmpl_scen in use)
     uint64_t *seg_best;     // [n_seg] min cost over kappa, order-preserving bits
@@ -343,7 +343,6 @@ cudaError_t launch_policies(const Tables &t, const BatchDev &b, int n_dp, cudaSt
 // cleared by the caller); after the search pass, give every other row its representative's result
 cudaError_t launch_useg_keys(const BatchDev &b, const USegDev &u, cudaStream_t st);   // three launches
 cudaError_t launch_useg_copy(const BatchDev &b, const USegDev &u, cudaStream_t st);
-cudaError_t launch_dup_copy(const BatchDev &b, cudaStream_t st);   // duplicate template segments take their first occurrence's minimum
 // side streams (may be NULL / 0): launch classes are independent of one another, so they are
 // spread over the caller's stream and the side streams and joined again before returning
 constexpr int kSideStreams = 7;
@@ -399,7 +398,6 @@ cudaError_t launch_objective(const Tables &t, const BatchDev &b, const ObjDev &o
 cudaError_t launch_range_matching(const Tables &t, int n_problems, const int32_t *sizes, const uint8_t *old_lo,
                                   const uint8_t *old_hi, const uint8_t *new_lo, const uint8_t *new_hi,
                                   int64_t *total, uint16_t *assign, cudaStream_t st);
-cudaError_t launch_pick(const cm_plan *const *plans_dev, int n, cm_plan *out_dev, int mode, cudaStream_t st);
 
 // What an entry point implemented outside cm_api.cu needs to know about a space.
 struct SpaceView {

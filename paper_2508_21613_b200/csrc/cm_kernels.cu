@@ -5,16 +5,17 @@
 //   cm_feasible_kernel    memory-feasible layer compositions per (stages, micro-batches), listed once
 //   (data rerouting / redundant computation: cm_policy.cu)
 //   (the search pass over every pipeline-plan lives in cm_cost.cu)
-//   cm_split_kernel       (cost, index) argmin over (strategy, micro-batch split) per scenario
+//   cm_best_split_kernel  best (strategy, micro-batch split) per scenario under the remainder rule
+//   cm_split_kernel       the same under the full enumeration of splits: (cost, index) argmin
 //   cm_winner_kernel      finishes that argmin and decodes the winner
 //   (pass 2, the lowest layer composition that meets the winning cost: cm_tiebreak.cu)
 //   cm_finalize_kernel    assembles the plans and picks the best policy
 //   (per-candidate cost / feasibility for cm_evaluate: cm_evaluate.cu)
-//   cm_pick_kernel        best of several spaces for cm_select
 #include <algorithm>
 #include <atomic>
 
 #include "cm_plan_eval.cuh"
+#include "cm_split.cuh"
 
 namespace cm {
 
@@ -330,21 +331,6 @@ __global__ void __launch_bounds__(256) cm_useg_copy_kernel(BatchDev bd, USegDev 
     if (r != row) bd.seg_best[row] = bd.seg_best[r];   // representatives and their second rows are only read here
 }
 
-__global__ void __launch_bounds__(128) cm_dup_copy_kernel(BatchDev bd) {
-    const Scen sc = bd.scen[bd.tmpl_scen[blockIdx.x]];
-    const Tmpl tp = bd.tmpl[sc.tmpl];
-    for (uint32_t i = threadIdx.x; i < tp.n_tseg; i += blockDim.x) {
-        const uint32_t c = bd.tseg_canon[tp.tseg_first + i];
-        if (c != tp.tseg_first + i) bd.seg_best[sc.seg_base + i] = bd.seg_best[sc.seg_base + (c - tp.tseg_first)];
-    }
-}
-
-cudaError_t launch_dup_copy(const BatchDev &b, cudaStream_t st) {
-    if (!b.tseg_canon || b.n_rep_scen == 0) return cudaSuccess;
-    cm_dup_copy_kernel<<<b.n_rep_scen, 128, 0, st>>>(b);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_useg_keys(const BatchDev &b, const USegDev &u, cudaStream_t st) {
     if (u.n_rep_scen == 0) return cudaSuccess;
     cm_useg_key_kernel<<<u.n_rep_scen, 128, 0, st>>>(b, u, 0);
@@ -360,7 +346,7 @@ cudaError_t launch_useg_copy(const BatchDev &b, const USegDev &u, cudaStream_t s
 }
 
 // ----------------------------------------------------------------------------------
-// Split reduction: item = (strategy, split rank) of one scenario; its step time is the
+// Split reduction under the full enumeration of splits: item = (strategy, split rank) of one scenario; its step time is the
 // slowest pipeline's best cost (Section "Estimator": step time = max over pipelines).
 // Hierarchical argmin carrying (cost, item) with the lowest item on ties:
 // thread-serial over a strided range -> warp shuffle -> shared memory -> one partial
@@ -452,9 +438,80 @@ __global__ void __launch_bounds__(256) cm_split_winner_kernel(Tables tb, BatchDe
     if (threadIdx.x < kMaxP) init_kappa_sel(bd, bd.winner[b], bd.kappa_sel + (size_t)b * kMaxP, (int)threadIdx.x);
 }
 
+// The remainder rule: a warp per strategy finds its best step time directly (cm_split.cuh); the first
+// strategy with the least one wins, and of its splits the one of lowest rank -- the smaller share wherever
+// it will do, the R larger ones to the lowest pipelines that may have them (colexicographic ranks grow
+// with the highest element first).  One CTA per scenario, no split is enumerated.
+__global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev bd, uint64_t inf) {
+    __shared__ uint64_t rc[32];
+    __shared__ uint32_t ri[32];
+    const uint32_t b = blockIdx.x;
+    const Scen sc = bd.scen[b];
+    const Tmpl tp = bd.tmpl[sc.tmpl];
+    const Strat *strat = bd.strat + tp.strat_first;
+    const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31;
+    auto cost_of = [&](const Strat &s) { return strat_cost(bd, tp, sc, s, inf, [&](uint32_t row) { return bd.seg_best[row]; }); };
+    uint64_t best_c = inf;
+    uint32_t best_i = 0;
+    if (sc.rep == b)   // (else it shares another scenario's search: nothing to tie-break here)
+        for (uint32_t si = warp; si < tp.n_strat; si += warps) {
+            const uint64_t v = strat_best(cost_of(strat[si]), strat[si], ~0ull, inf);
+            if (v < best_c) { best_c = v; best_i = si; }
+        }
+    if (lane == 0) { rc[warp] = best_c; ri[warp] = best_i; }
+    __syncthreads();
+    if (warp) return;
+    best_c = lane < (int)warps ? rc[lane] : inf;
+    best_i = lane < (int)warps ? ri[lane] : 0;
+    for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o);
+        const uint32_t oi = __shfl_xor_sync(0xffffffffu, best_i, o);
+        if (oc < best_c || (oc == best_c && oi < best_i)) { best_c = oc; best_i = oi; }
+    }
+    Winner &w = bd.winner[b];
+    uint64_t *kappa = bd.kappa_sel + (size_t)b * kMaxP;
+    if (best_c >= inf) {
+        if (lane == 0) { w.cost_bits = inf; w.item = ~0ull; w.strat = 0; w.dp = 0; w.scen = b; w.pad = 0; }
+        if (lane < kMaxP) { w.seg[lane] = 0; w.micro[lane] = 0; kappa[lane] = ~0ull; }
+        return;
+    }
+    const Strat &s = strat[best_i];
+    const uint64_t v = cost_of(s);
+    const uint64_t lo = __shfl_sync(0xffffffffu, v, (2 * lane) & 31), hi = __shfl_sync(0xffffffffu, v, (2 * lane + 1) & 31);
+    const bool mine = lane < (int)s.dp;                               // lane = pipeline from here on
+    const uint32_t must = __ballot_sync(0xffffffffu, mine && lo > best_c);
+    const uint32_t may = s.R ? __ballot_sync(0xffffffffu, mine && hi <= best_c) & ~must : 0u;
+    const int need = (int)s.R - __popc(must);
+    const bool extra = mine && (((must >> lane) & 1u) || (((may >> lane) & 1u) && __popc(may & ((1u << lane) - 1u)) < need));
+    const uint32_t set = __ballot_sync(0xffffffffu, extra);
+    uint64_t rank = extra ? binom_at(tb.binom, lane, __popc(set & ((1u << lane) - 1u)) + 1) : 0ull;
+    for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (lane == 0) {
+        w.cost_bits = best_c;
+        w.item = s.split_first + rank;
+        w.strat = tp.strat_first + best_i;
+        w.dp = s.dp;
+        w.scen = b;
+        w.pad = 0;
+    }
+    if (lane < kMaxP) {
+        const uint32_t seg = mine ? s.seg_first + lane * s.n_m + (extra ? 1 : 0) : 0u;
+        w.seg[lane] = seg;
+        w.micro[lane] = mine ? (uint16_t)(s.m_lo[lane] + (extra ? 1 : 0)) : (uint16_t)0;
+        // a segment whose only candidate is the min-max partition has nothing to search (init_kappa_sel)
+        kappa[lane] = mine && bd.tseg[seg].K == 0 ? 0ull : ~0ull;
+    }
+}
+
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
     const uint64_t inf = batch_inf_bits(b);
+    if (b.batch_mode == CM_BATCH_REMAINDER) {
+        // a failure handled on its own: a warp for every strategy; a batch: enough to keep the SMs busy
+        cm_best_split_kernel<<<b.B, b.B <= 148 ? 1024 : 128, 0, st>>>(t, b, inf);
+        return cudaGetLastError();
+    }
     if (b.n_red_blocks <= (uint32_t)b.B && b.max_red_per_scen <= 1) {
         cm_split_winner_kernel<<<b.B, 256, 0, st>>>(t, b, inf);
         return cudaGetLastError();
@@ -470,95 +527,57 @@ cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t
 
 // ----------------------------------------------------------------------------------
 // Assemble the per-policy plans and the overall best: least cost, ties to the lowest
-// policy id (Algorithm 1 keeps the plan with the least estimated time).
+// policy id (Algorithm 1 keeps the plan with the least estimated time).  Sixteen threads per plan, one
+// per pipeline; four plans per scenario, the last a copy of the winner.
 // ----------------------------------------------------------------------------------
-__global__ void cm_finalize_kernel(Tables tb, BatchDev bd, uint64_t inf) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b == 0) {
+constexpr int kFinalThreads = 64;
+__global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, BatchDev bd, uint64_t inf) {
+    const uint32_t b = blockIdx.x;
+    const int slot = threadIdx.x >> 4, k = threadIdx.x & 15;
+    if (b == 0 && threadIdx.x < kCounters) {
         // work counters ride home behind the plans (they start at all-ones, i.e. -1)
         unsigned long long *tail = reinterpret_cast<unsigned long long *>(bd.plans + (size_t)bd.B * 4);
-        for (int i = 0; i < kCounters; ++i) tail[i] = bd.counters[i] + 1ull;
+        tail[threadIdx.x] = bd.counters[threadIdx.x] + 1ull;
     }
-    if (b >= bd.B) return;
     const DevProfile *p = tb.prof;
     const Scen sc = bd.scen[b];
-    cm_plan *out = bd.plans + (size_t)b * 4;
-    uint64_t cost[3] = {inf, inf, inf};
-    for (int pol = 0; pol < 2; ++pol) {
-        cm_plan pl;
-        plan_clear(pl, pol);
-        pl.n_pipes = (uint32_t)p->n_dp;
-        for (int k = 0; k < p->n_dp && k < kMaxP; ++k) {
-            pl.stages[k] = (uint16_t)p->n_pp;
-            pl.micro[k] = (uint16_t)p->n_micro;
-        }
-        uint64_t c = (sc.policy_mask & (1u << pol)) ? bd.pol_cost[2 * b + pol] : inf;
-        if (c < inf) {
-            pl.feasible = 1;
-            plan_set_cost(pl, c, bd);
-            if (pol == CM_REDUNDANT)
-                for (int k = 0; k < p->n_dp && k < kMaxP; ++k) pl.stages[k] = bd.rc_stages[b * kMaxP + k];
-            cost[pol] = c;
-        }
-        out[pol] = pl;
+    const Winner &w = bd.winner[sc.rep];   // its own search, or the one it shares
+    uint64_t cost[3];
+    for (int pol = 0; pol < 3; ++pol) {
+        const uint64_t c = !(sc.policy_mask & (1u << pol)) ? inf : pol < 2 ? bd.pol_cost[2 * b + pol] : w.cost_bits;
+        cost[pol] = c < inf ? c : inf;
     }
-    {
-        cm_plan pl;
-        plan_clear(pl, CM_DYNPAR);
-        const Winner &w = bd.winner[sc.rep];   // its own search, or the one it shares
-        if ((sc.policy_mask & (1u << CM_DYNPAR)) && w.cost_bits < inf) {
-            const Strat &s = bd.strat[w.strat];
-            pl.feasible = 1;
-            plan_set_cost(pl, w.cost_bits, bd);
-            pl.strategy = w.strat - bd.tmpl[sc.tmpl].strat_first;
-            pl.n_pipes = w.dp;
-            pl.split_rank = w.item - s.split_first;
-            for (uint32_t q = 0; q < w.dp; ++q) {
-                pl.stages[q] = s.S[q];
-                pl.micro[q] = w.micro[q];
-                pl.kappa[q] = bd.kappa_sel[sc.rep * kMaxP + q];
-            }
-            cost[2] = w.cost_bits;
-        }
-        out[2] = pl;
+    int pol = slot;
+    bool any = true;
+    if (slot == 3) {
+        pol = 0;
+        for (int q = 1; q < 3; ++q)
+            if (cost[q] < cost[pol]) pol = q;
+        any = cost[pol] < inf;             // (else an empty plan)
     }
-    int win = -1;
-    for (int pol = 0; pol < 3; ++pol)
-        if (cost[pol] < inf && (win < 0 || cost[pol] < cost[win])) win = pol;
-    if (win >= 0) out[3] = out[win];
-    else { cm_plan pl; plan_clear(pl, 0); out[3] = pl; }
+    const bool dyn = pol == CM_DYNPAR, feasible = cost[pol] < inf, filled = any && (!dyn || feasible);
+    const int n = !filled ? 0 : dyn ? (int)w.dp : p->n_dp < kMaxP ? p->n_dp : kMaxP;
+    cm_plan &out = bd.plans[(size_t)b * 4 + slot];
+    if (k == 0) {
+        out.policy = any ? pol : 0;
+        out.feasible = feasible ? 1 : 0;
+        out.cost = 0.0;
+        out.cost_ns = 0;
+        if (feasible) plan_set_cost(out, cost[pol], bd);
+        out.strategy = filled && dyn ? w.strat - bd.tmpl[sc.tmpl].strat_first : 0u;
+        out.n_pipes = !filled ? 0u : dyn ? w.dp : (uint32_t)p->n_dp;
+        out.split_rank = filled && dyn ? w.item - bd.strat[w.strat].split_first : 0ull;
+    }
+    out.stages[k] = k >= n ? (uint16_t)0 : dyn ? bd.strat[w.strat].S[k]
+                    : pol == CM_REDUNDANT && feasible ? bd.rc_stages[b * kMaxP + k] : (uint16_t)p->n_pp;
+    out.micro[k] = k >= n ? (uint16_t)0 : dyn ? w.micro[k] : (uint16_t)p->n_micro;
+    out.kappa[k] = k < n && dyn ? bd.kappa_sel[(size_t)sc.rep * kMaxP + k] : 0ull;
 }
 
 cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
     const uint64_t inf = batch_inf_bits(b);
-    cm_finalize_kernel<<<(b.B + 127) / 128, 128, 0, st>>>(t, b, inf);
-    return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------------
-// cm_select over several spaces: least cost, ties to the lowest policy id, then to the
-// earlier space.
-// ----------------------------------------------------------------------------------
-__global__ void cm_pick_kernel(const cm_plan *const *plans, int n, cm_plan *out, int mode) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int win = -1;
-    for (int i = 0; i < n; ++i) {
-        const cm_plan &q = *plans[i];
-        if (!q.feasible) continue;
-        if (win < 0) { win = i; continue; }
-        const cm_plan &w = *plans[win];
-        bool less, equal;
-        if (mode == CM_COST_INT64NS) { less = q.cost_ns < w.cost_ns; equal = q.cost_ns == w.cost_ns; }
-        else { less = q.cost < w.cost; equal = q.cost == w.cost; }
-        if (less || (equal && q.policy < w.policy)) win = i;
-    }
-    if (win >= 0) *out = *plans[win];
-    else { cm_plan pl; plan_clear(pl, 0); *out = pl; }
-}
-
-cudaError_t launch_pick(const cm_plan *const *plans_dev, int n, cm_plan *out_dev, int mode, cudaStream_t st) {
-    cm_pick_kernel<<<1, 32, 0, st>>>(plans_dev, n, out_dev, mode);
+    cm_finalize_kernel<<<b.B, kFinalThreads, 0, st>>>(t, b, inf);
     return cudaGetLastError();
 }
 

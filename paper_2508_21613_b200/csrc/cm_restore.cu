@@ -26,6 +26,7 @@ namespace cm {
 // Shortlist: topk rounds of a block-wide argmin over the scenario's (strategy, split)
 // items; round r takes the least (step time, item) pair that comes after round r-1's.
 // ----------------------------------------------------------------------------------
+constexpr uint64_t kShortKept = 4096;
 __global__ void __launch_bounds__(256) cm_shortlist_kernel(Tables tb, BatchDev bd, ObjDev od, uint64_t inf) {
     __shared__ uint64_t rc[8], ri[8];
     __shared__ uint64_t last_c, last_i;
@@ -35,12 +36,17 @@ __global__ void __launch_bounds__(256) cm_shortlist_kernel(Tables tb, BatchDev b
     const uint64_t *best = bd.seg_best + sc.seg_base;
     const bool searched = (sc.policy_mask & (1u << CM_DYNPAR)) != 0;
     bool exhausted = !searched || tp.n_split_total == 0;
+    // the step times of the items, worked out once where they fit (they are read topk times)
+    __shared__ uint64_t kept[kShortKept];
+    const uint64_t n_kept = exhausted ? 0 : tp.n_split_total < kShortKept ? tp.n_split_total : kShortKept;
+    for (uint64_t item = threadIdx.x; item < n_kept; item += blockDim.x) kept[item] = item_step_time(tb, bd, tp, best, item, inf);
+    __syncthreads();
     for (int r = 0; r < od.topk; ++r) {
         uint64_t best_c = inf, best_i = ~0ull;
         if (!exhausted) {
             const uint64_t lc = r ? last_c : 0, li = r ? last_i : 0;
             for (uint64_t item = threadIdx.x; item < tp.n_split_total; item += blockDim.x) {
-                const uint64_t T = item_step_time(tb, bd, tp, best, item, inf);
+                const uint64_t T = item < n_kept ? kept[item] : item_step_time(tb, bd, tp, best, item, inf);
                 if (T >= inf) continue;
                 if (r && !pair_less(lc, li, T, item)) continue;     // taken by an earlier round
                 if (pair_less(T, item, best_c, best_i)) { best_c = T; best_i = item; }
