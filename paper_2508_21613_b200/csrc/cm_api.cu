@@ -155,6 +155,10 @@ struct Batch {
                sizeof(Partial) * d_partial.cap + sizeof(Winner) * (d_winner.cap + d_short_win.cap) + sizeof(cm_plan) * (d_plans.cap + d_short_plans.cap) +
                4 * (d_urep.cap + d_slot_of.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
     }
+    // One scenario handled on its own: its first kernel reads the failed ids and the node-crossing bits
+    // from the pinned arena and its last one writes the plans to pinned memory, so that no copy sits on the
+    // path (two copies in, one out: ~8 us of a 95 us call).
+    bool direct = false;
     int k_best = 1;                       // (strategy, split) pairs whose step times have to be exact
 };
 
@@ -535,7 +539,9 @@ cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups) {
     int max_stages = 1;
     for (const BBucket &g : groups) {
         if (g.count >= 0xfffffff0ull) return CM_OK;   // positions are 32-bit
-        cells += 2.0 * (double)g.count * g.n_seg * g.S * g.m;
+        // a shallow cell costs the direct search a quarter of a deep one while the GPU is not full (chains of
+        // hundreds, not thousands of dependent cells)
+        cells += 2.0 * (double)g.count * g.n_seg * g.S * g.m * (g.S <= kRegStagesMax ? 0.25 : 1.0);
         plans[g.S > kRegStagesMax] += (double)g.count * g.n_seg;
         segs[g.S > kRegStagesMax] += g.n_seg;
         max_stages = std::max<int>(max_stages, g.S);
@@ -1030,6 +1036,7 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
     bt.max_tiles_per_seg = 0;
     bt.dp_max = 0;
     bt.k_best = 1;
+    bt.direct = false;
     bt.B = B;
     bt.tmpl_of_nsurv.assign((size_t)N + 1, -1);
     bt.tmpl.push_back(Tmpl{});   // template 0: no strategies (scenarios without a dynamic-parallelism search)
@@ -1180,7 +1187,7 @@ BatchDev dev_view(const cm_ctx *ctx, Batch &bt) {
     for (const Tmpl &tp : bt.tmpl) v.n_rep_scen += tp.n_scen;
     v.seg_best = bt.d_seg_best.p; v.partial = bt.d_partial.p;
     v.winner = bt.d_winner.p; v.kappa_sel = bt.d_kappa_sel.p; v.pol_cost = bt.d_pol_cost.p;
-    v.rc_stages = bt.d_rc_stages.p; v.plans = bt.d_plans.p;
+    v.rc_stages = bt.d_rc_stages.p; v.plans = bt.direct ? bt.plans_host.p : bt.d_plans.p;
     v.counters = reinterpret_cast<unsigned long long *>(bt.d_seg_best.p + bt.n_rows);
     v.B = bt.B; v.mode = bt.opts.cost; v.intval = bt.intval ? 1u : 0u;
     v.n_rows = (uint32_t)bt.n_rows;
@@ -1345,7 +1352,14 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     // per-segment minima start at all-ones (above every cost); so do the work counters, which
     // therefore read "value - 1" until cm_finalize_kernel adds the one back
     const size_t cleared = (bt.bounded ? 3 * bt.n_rows : bt.n_rows) + kStateExtra;
-    CM_CUDA(ctx, cudaMemsetAsync(bt.d_seg_best.p, 0xFF, cleared * sizeof(uint64_t), st));
+    if (bt.direct) {
+        CM_CUDA(ctx, launch_prologue(bt.d_seg_best.p, cleared, (const uint32_t *)(bt.arena.p + bt.off_failed), (uint32_t *)(bt.d_arena.p + bt.off_failed),
+                                     (int)bt.failed.size(), (const uint64_t *)(bt.arena.p + bt.off_cross),
+                                     (uint64_t *)(bt.d_arena.p + bt.off_cross), (int)bt.cross.size(), st));
+        ++launches;
+    } else {
+        CM_CUDA(ctx, cudaMemsetAsync(bt.d_seg_best.p, 0xFF, cleared * sizeof(uint64_t), st));
+    }
     const bool policies = (bt.policy_mask & ((1u << CM_REROUTE) | (1u << CM_REDUNDANT))) != 0;
     const bool beside = policies && (bt.policy_mask & (1u << CM_DYNPAR)) && ctx->pol_stream;
     if (policies) {
@@ -1384,8 +1398,10 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     CM_CUDA(ctx, launch_finalize(tb, bd, st));
     ++launches;
     if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
-    const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
-    CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, back_bytes, cudaMemcpyDeviceToHost, st));
+    if (!bt.direct) {
+        const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
+        CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, back_bytes, cudaMemcpyDeviceToHost, st));
+    }
     *launches_out += launches;
     *cost_launches_out += cost_launches;
     return CM_OK;
@@ -1465,8 +1481,10 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
         // a list was full (plans whose bounds tie in their hundreds of thousands): search again, every plan
         if (single && single->exec) { cudaGraphExecDestroy(single->exec); single->exec = nullptr; }
         bt.dense_only = true;
+        const bool direct = bt.direct;
         cm_status s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
         if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
+        bt.direct = direct;
         return s == CM_OK ? run_batch(ctx, bt, launches, single) : s;
     }
     account_search(ctx, bt, launches);
@@ -1520,6 +1538,7 @@ cm_status single_batch(cm_ctx *ctx, const uint32_t *ids, int n, const cm_enum_op
         cm_status s = build_batch(ctx, *b, ids, off, 1, o, mask);
         if (s == CM_OK) s = upload_batch(ctx, *b, launches);
         if (s != CM_OK) { cudaStreamSynchronize(ctx->stream); forget_keys(ctx, *b); return s; }
+        b->direct = true;
         if (ctx->single.size() >= 64) {   // bounded: start over rather than grow without limit
             cudaStreamSynchronize(ctx->stream);
             ctx->single.clear();
@@ -1548,8 +1567,6 @@ cm_status single_batch(cm_ctx *ctx, const uint32_t *ids, int n, const cm_enum_op
     }
     if (n) memcpy(bt.arena.p + bt.off_failed, bt.failed.data(), sizeof(uint32_t) * n);
     memcpy(bt.arena.p + bt.off_cross, bt.cross.data(), sizeof(uint64_t) * cross_words);
-    if (n) CM_CUDA(ctx, cudaMemcpyAsync(bt.d_arena.p + bt.off_failed, bt.arena.p + bt.off_failed, sizeof(uint32_t) * n, cudaMemcpyHostToDevice, ctx->stream));
-    CM_CUDA(ctx, cudaMemcpyAsync(bt.d_arena.p + bt.off_cross, bt.arena.p + bt.off_cross, sizeof(uint64_t) * cross_words, cudaMemcpyHostToDevice, ctx->stream));
     ctx->stats[9] += sizeof(uint32_t) * n + sizeof(uint64_t) * cross_words;
     *out = &bt;
     return CM_OK;
@@ -1858,6 +1875,7 @@ cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids
         CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // growing frees the old block
         if (!ctx->d_eval.reserve(want)) return fail(ctx, CM_ENOMEM, "device memory");
     }
+    sp->own->direct = true;
     if (n_candidates) *n_candidates = policy == CM_DYNPAR ? sp->own->n_cand : 1;
     *out = sp.release();
     return CM_OK;

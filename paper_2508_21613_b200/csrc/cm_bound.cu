@@ -159,24 +159,23 @@ cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo,
 // Phase 0 marks strategies this far above the best step time from bounds: one plan of each of their
 // segments is evaluated, so that a result that misses its bound a little still leaves phase 2 nothing to do.
 constexpr float kReach = 1.0f / (1 << 13);
-constexpr int kWinThreads = 128;
 
 __device__ __forceinline__ uint64_t block_min_u64(uint64_t v /* warp-uniform */, uint64_t *red) {
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int w = 0; w < kWinThreads / 32; ++w) v = red[w] < v ? red[w] : v;
+    for (uint32_t w = 0; w < blockDim.x / 32; ++w) v = red[w] < v ? red[w] : v;
     return v;
 }
 
-__global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, BatchDev bd, BoundDev bo, int phase, int k_best, uint64_t inf_cost) {
-    __shared__ uint64_t red[kWinThreads / 32];
+__global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd, BoundDev bo, int phase, int k_best, uint64_t inf_cost) {
+    __shared__ uint64_t red[32];
     __shared__ unsigned long long total;
     const uint32_t b = blockIdx.x;
     const Scen sc = bd.scen[b];
     const Tmpl tp = bd.tmpl[sc.tmpl];
     const Strat *strat = bd.strat + tp.strat_first;
-    const uint32_t warp = threadIdx.x >> 5, warps = kWinThreads / 32;
+    const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint64_t inf = phase ? inf_cost : 0xffffffffull;
     auto cost_of = [&](const Strat &s, int from_results, uint64_t most) {
@@ -231,7 +230,7 @@ __global__ void __launch_bounds__(kWinThreads) cm_window_kernel(Tables tb, Batch
 
 cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
-    cm_window_kernel<<<b.B, kWinThreads, 0, st>>>(t, b, bo, phase, k_best, batch_inf_bits(b));
+    cm_window_kernel<<<b.B, b.B <= 148 ? 1024 : 128, 0, st>>>(t, b, bo, phase, k_best, batch_inf_bits(b));
     return cudaGetLastError();
 }
 

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_any_kernel(Tables tb, Bat
         const SegView g = bucket_segment(bd, bk, (uint32_t)seg_local);
         row = g.row;
         T cost;
-        if (plan_cost_regs_any<T>(sp, tb, bd.layer_mode, g, cand, cost)) {
+        if (plan_cost_regs_any<T, true>(sp, tb, bd.layer_mode, g, cand, cost)) {
             bits = Num<T>::bits(cost);
             my_cells = one_plan(2ull * g.S * g.m);
         }

@@ -220,7 +220,7 @@ struct BoundDev {
     int window, uniform_x;
 };
 constexpr int kCounters = 6;   // work counters of a search in use (BatchDev::counters)
-// Recurrence cells of a search from which bounds pay for their extra launches.
+// Recurrence cells of a search (a shallow one counting a quarter) from which bounds pay for their extra launches.
 constexpr uint64_t kBoundMinCells = 200000000ull;
 constexpr uint32_t kBoundListMin = 65536;        // plans a list has room for, at least (if there are as many)
 constexpr size_t kBoundDynMax = 160 * 1024;      // dynamic shared memory of the bound kernels, at most
@@ -363,6 +363,9 @@ cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo
 cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches);   // first_list and the next
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st);
 cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);   // cm_tiebreak.cu
+// first kernel of a scenario handled on its own: clear n_words result words, fetch its ids and bits from host memory
+cudaError_t launch_prologue(uint64_t *words, size_t n_words, const uint32_t *ids_host, uint32_t *ids, int n_ids,
+                            const uint64_t *bits_host, uint64_t *bits, int n_bits, cudaStream_t st);
 cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st);
 // Candidates of a space one by one (cm_evaluate.cu).  EvalDev: outputs (any may be NULL) and, for the
 // binned path, the lists of candidates by depth.

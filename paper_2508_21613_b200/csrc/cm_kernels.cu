@@ -526,6 +526,27 @@ cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t
 }
 
 // ----------------------------------------------------------------------------------
+// One scenario handled on its own: clears the result words and fetches the few bytes that say which
+// devices failed from the host's pinned memory.
+// ----------------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) cm_prologue_kernel(uint64_t *words, size_t n_words, const uint32_t *ids_host, uint32_t *ids, int n_ids,
+                                                          const uint64_t *bits_host, uint64_t *bits, int n_bits) {
+    const size_t at = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (blockIdx.x == 0) {
+        for (int i = threadIdx.x; i < n_ids; i += 256) ids[i] = ids_host[i];
+        for (int i = threadIdx.x; i < n_bits; i += 256) bits[i] = bits_host[i];
+    }
+    for (size_t i = at; i < n_words; i += (size_t)gridDim.x * 256) words[i] = ~0ull;
+}
+
+cudaError_t launch_prologue(uint64_t *words, size_t n_words, const uint32_t *ids_host, uint32_t *ids, int n_ids,
+                            const uint64_t *bits_host, uint64_t *bits, int n_bits, cudaStream_t st) {
+    const size_t ctas = (n_words + 255) / 256;
+    cm_prologue_kernel<<<(unsigned)(ctas < 148 ? (ctas ? ctas : 1) : 148), 256, 0, st>>>(words, n_words, ids_host, ids, n_ids, bits_host, bits, n_bits);
+    return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------------
 // Assemble the per-policy plans and the overall best: least cost, ties to the lowest
 // policy id (Algorithm 1 keeps the plan with the least estimated time).  Sixteen threads per plan, one
 // per pipeline; four plans per scenario, the last a copy of the winner.

@@ -31,12 +31,12 @@ def _small(seed, times=None, tight=False, n_micro=7, p2p=None):
 SETS = [list(c) for k in (1, 2) for c in itertools.combinations(range(12), k)]
 CASES = {
     # transfer times that depend on the layer
-    "layered-transfers": (_small(31), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 40),
-    "tight-memory": (_small(33, tight=True), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 200),
+    "layered-transfers": (_small(31), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 160),
+    "tight-memory": (_small(33, tight=True), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 800),
     # transfer times equal on every boundary; identical layers (most plans tie); fewer micro-batches than stages
-    "equal-transfers": (_small(34, p2p=30_000_000), (1, 3, 2, 7, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 40),
-    "identical-layers": (_small(35, times=lambda n: np.full(n, 3e6), p2p=30_000_000), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 40),
-    "few-micro-batches": (_small(36, n_micro=2), (1, 3, 2, 8, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 160),
+    "equal-transfers": (_small(34, p2p=30_000_000), (1, 3, 2, 7, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 160),
+    "identical-layers": (_small(35, times=lambda n: np.full(n, 3e6), p2p=30_000_000), (1, 3, 2, 6, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 160),
+    "few-micro-batches": (_small(36, n_micro=2), (1, 3, 2, 8, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:20], 640),
 }
 
 
@@ -104,7 +104,7 @@ def test_bounded_shortlist_against_the_oracle(gpu, oracle_factory):
         ctx = gpu.cm_create(0)
         try:
             gpu.cm_load_profile(ctx, profile)
-            many = sets[:6] * (copies * 4)
+            many = sets[:6] * (copies * 2)
             best, trans, short, moved, _ = gpu.cm_search_objective(ctx, many, opts, obj, shortlist=True)
             st = gpu.cm_last_stats(ctx)
             assert st["plans_run"] < st["plans_simulated"]
