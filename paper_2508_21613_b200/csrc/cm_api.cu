@@ -80,7 +80,7 @@ struct Batch {
     std::vector<Tmpl> tmpl;
     std::vector<Strat> strat;
     std::vector<TSeg> tseg;
-    std::vector<uint32_t> failed, red_scen, keys, tmpl_scen, bucket_tseg;
+    std::vector<uint32_t> failed, keys, tmpl_scen, bucket_tseg;
     std::vector<uint32_t> tseg_canon;      // first template segment with the same (stages, micro-batches, peers, offset): itself if none before
     uint32_t n_dup = 0;                    // template segments that are not their own first occurrence
     size_t off_canon = 0;
@@ -90,11 +90,10 @@ struct Batch {
     std::vector<int> tmpl_of_nsurv;        // survivor count -> template, -1 = not built
     PinnedVec<unsigned char> arena;        // host image of the tables
     DevBuf<unsigned char> d_arena;
-    size_t off_scen = 0, off_tmpl = 0, off_strat = 0, off_tseg = 0, off_failed = 0, off_red = 0, off_keys = 0,
+    size_t off_scen = 0, off_tmpl = 0, off_strat = 0, off_tseg = 0, off_failed = 0, off_keys = 0,
            off_tmpl_scen = 0, off_bucket_tseg = 0, off_cross = 0, off_bucket = 0;
     PinnedVec<cm_plan> plans_host;
     DevBuf<uint64_t> d_seg_best, d_kappa_sel, d_pol_cost;
-    DevBuf<Partial> d_partial;
     DevBuf<Winner> d_winner;
     DevBuf<uint16_t> d_rc_stages;
     DevBuf<cm_plan> d_plans;
@@ -152,7 +151,7 @@ struct Batch {
     // device memory held (what a spare batch ties up)
     size_t bytes() const {
         return d_arena.cap + 8 * (d_seg_best.cap + d_kappa_sel.cap + d_pol_cost.cap + d_utab.cap + d_useg.cap + d_short_kappa.cap) +
-               sizeof(Partial) * d_partial.cap + sizeof(Winner) * (d_winner.cap + d_short_win.cap) + sizeof(cm_plan) * (d_plans.cap + d_short_plans.cap) +
+               sizeof(Winner) * (d_winner.cap + d_short_win.cap) + sizeof(cm_plan) * (d_plans.cap + d_short_plans.cap) +
                4 * (d_urep.cap + d_slot_of.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
     }
     // One scenario handled on its own: its first kernel reads the failed ids and the node-crossing bits
@@ -194,8 +193,10 @@ struct cm_ctx {
     int mm_stride_m = 0;
     // Memory-feasible layer compositions per (layer mode, stages, micro-batches), listed once per
     // profile (cm_feasible_kernel) into one device pool that only grows; key = S << 16 | m.
-    struct FeasEntry { uint32_t first, count; uint64_t K; };
-    std::map<uint32_t, FeasEntry> feas[6];   // [layer mode * 2 + execution order]
+    // Their places: a table over (stages, micro-batches) per [layer mode * 2 + execution order], made at
+    // first use (listed = 0: not yet).
+    struct FeasEntry { uint32_t first, count, listed; };
+    std::vector<FeasEntry> feas[6];
     DevBuf<uint32_t> d_feas;
     DevBuf<ulonglong2> d_feas_mask;           // the same entries as masks
     size_t feas_used = 0;
@@ -914,7 +915,6 @@ cm_status build_template(cm_ctx *ctx, Batch &bt, int n_surv, uint32_t *out) {
     }
     tp.n_split_total = split_first;
     tp.n_cand = cand;
-    tp.n_red = split_first && o.bm == CM_BATCH_FULL ? (uint32_t)std::min<uint64_t>((split_first + 1023) / 1024, 64) : 0;   // (the remainder rule reduces strategies)
     *out = (uint32_t)bt.tmpl.size();
     bt.tmpl.push_back(tp);
     return CM_OK;
@@ -961,7 +961,9 @@ cm_status grow_feas_pool(cm_ctx *ctx, size_t want) {
 cm_status ensure_feasible_lists(cm_ctx *ctx, Batch &bt) {
     const int lm = bt.opts.lm;
     if (lm == CM_LAYERS_MINMAX) return CM_OK;
-    std::map<uint32_t, cm_ctx::FeasEntry> &known = ctx->feas[lm * 2 + (int)bt.opts.sched];
+    std::vector<cm_ctx::FeasEntry> &known = ctx->feas[lm * 2 + (int)bt.opts.sched];
+    if (known.empty()) known.assign((size_t)CM_MAX_STAGES * ctx->mm_stride_m, cm_ctx::FeasEntry{0, 0, 0});
+    auto entry = [&](uint32_t key) -> cm_ctx::FeasEntry & { return known[((key >> 16) - 1) * (size_t)ctx->mm_stride_m + (key & 0xffffu)]; };
     std::vector<uint32_t> new_keys;
     std::vector<uint64_t> new_K;
     std::vector<uint32_t> new_first;
@@ -969,16 +971,16 @@ cm_status ensure_feasible_lists(cm_ctx *ctx, Batch &bt) {
     for (const TSeg &g : bt.tseg) {
         if (g.K == 0 || g.K > kFeasMaxK || g.m < 1) continue;
         const uint32_t key = ((uint32_t)g.S << 16) | g.m;
-        if (known.count(key)) continue;
+        if (entry(key).listed) continue;
         if (used + g.K + 1 >= 0xfffffff0ull) break;   // pool offsets are 32-bit: later keys stay unscreened
-        known[key] = cm_ctx::FeasEntry{(uint32_t)used, kNoFeasList, g.K};   // count filled in below
+        entry(key) = cm_ctx::FeasEntry{(uint32_t)used, kNoFeasList, 1};   // count filled in below
         new_keys.push_back(key);
         new_K.push_back(g.K);
         new_first.push_back((uint32_t)used);
         used += g.K + 1;
     }
     if (!new_keys.empty()) {
-        auto undo = [&]() { for (uint32_t k : new_keys) known.erase(k); };
+        auto undo = [&]() { for (uint32_t k : new_keys) entry(k).listed = 0; };
         cm_status s = grow_feas_pool(ctx, used);
         if (s != CM_OK) { undo(); return s; }
         const size_t n = new_keys.size(), n_mm = bt.keys.size();
@@ -1003,27 +1005,29 @@ cm_status ensure_feasible_lists(cm_ctx *ctx, Batch &bt) {
         if (e != cudaSuccess) { cudaGetLastError(); undo(); return fail(ctx, CM_ECUDA, std::string("feasible-composition lists: ") + cudaGetErrorString(e)); }
         bt.mm_launched = n_mm > 0;
         const uint32_t *cnt = (const uint32_t *)(h + off_cnt);
-        for (size_t q = 0; q < n; ++q) known[new_keys[q]].count = cnt[q];
+        for (size_t q = 0; q < n; ++q) entry(new_keys[q]).count = cnt[q];
         ctx->feas_used = used;
         ctx->stats[9] += off_cnt;
         ctx->stats[10] += 4 * n;
     }
     for (TSeg &g : bt.tseg) {
         if (g.K == 0 || g.K > kFeasMaxK || g.m < 1) continue;
-        auto it = known.find(((uint32_t)g.S << 16) | g.m);
-        if (it == known.end() || it->second.count == kNoFeasList) continue;
-        g.feas_first = it->second.first;
-        g.feas_count = it->second.count;
+        const cm_ctx::FeasEntry &e = entry(((uint32_t)g.S << 16) | g.m);
+        if (!e.listed || e.count == kNoFeasList) continue;
+        g.feas_first = e.first;
+        g.feas_count = e.count;
     }
     return CM_OK;
 }
+
+int crossing_bits(const DevProfile &hp, const uint32_t *failed, int n_failed, std::vector<int> &alive, uint64_t *words);
 
 // Build the descriptor tables of a batch on the host: integers only, no cost arithmetic.
 cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const int32_t *offsets, int B,
                       const cm_enum_opts &o, uint32_t policy_mask) {
     const DevProfile &hp = ctx->hp;
     const int N = hp.n_dp * hp.n_pp;
-    bt.scen.clear(); bt.tmpl.clear(); bt.strat.clear(); bt.tseg.clear(); bt.failed.clear(); bt.red_scen.clear();
+    bt.scen.clear(); bt.tmpl.clear(); bt.strat.clear(); bt.tseg.clear(); bt.failed.clear();
     bt.keys.clear(); bt.tmpl_scen.clear(); bt.cross.clear(); bt.tseg_canon.clear();
     bt.n_dup = 0;
     bt.opts = o;
@@ -1042,7 +1046,8 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
     bt.tmpl.push_back(Tmpl{});   // template 0: no strategies (scenarios without a dynamic-parallelism search)
     const int cross_words = (N + 63) / 64 + 1;
     std::vector<char> dead(N);
-    std::map<std::string, uint32_t> seen;   // sharing: (node-crossing string, survivor count) -> first scenario
+    std::vector<int> alive;
+    std::unordered_map<std::string, uint32_t> seen;   // sharing: (node-crossing string, survivor count) -> first scenario
     bt.scen.reserve(B);
     bt.cross.reserve((size_t)B * cross_words);
 
@@ -1069,14 +1074,7 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
         sc.cross_first = (uint32_t)bt.cross.size();
         bt.cross.resize(bt.cross.size() + cross_words, 0);
         uint64_t *cw = bt.cross.data() + sc.cross_first;
-        int n_surv = 0, prev_node = -1;
-        for (int d = 0; d < N; ++d) {
-            if (dead[d]) continue;
-            const int node = d / hp.devices_per_node;
-            if (n_surv > 0 && node != prev_node) cw[(n_surv - 1) >> 6] |= 1ull << ((n_surv - 1) & 63);
-            prev_node = node;
-            ++n_surv;
-        }
+        const int n_surv = crossing_bits(hp, failed_ids + f0, f1 - f0, alive, cw);
         for (int f = f0; f < f1; ++f) dead[failed_ids[f]] = 0;
         sc.rep = (uint32_t)b;
         if (policy_mask & (1u << CM_DYNPAR)) {
@@ -1112,29 +1110,25 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
         bt.tmpl[sc.tmpl].n_scen++;
         bt.scen.push_back(sc);
     }
-    // scenarios grouped by template; result rows and reduction blocks per scenario
+    // scenarios grouped by template; result rows and rows per scenario
     uint32_t first = 0;
     for (Tmpl &tp : bt.tmpl) { tp.scen_first = first; first += tp.n_scen; tp.n_scen = 0; }
     bt.tmpl_scen.resize(B);
-    uint64_t rows = 0, red = 0;
+    uint64_t rows = 0;
     for (int b = 0; b < B; ++b) {
         Scen &sc = bt.scen[b];
         Tmpl &tp = bt.tmpl[sc.tmpl];
         if (sc.rep != (uint32_t)b) {   // shares the rows of an earlier scenario; nothing of its own to search
             sc.seg_base = bt.scen[sc.rep].seg_base;
-            sc.red_first = 0;
             continue;
         }
         bt.tmpl_scen[tp.scen_first + tp.n_scen++] = (uint32_t)b;
         sc.seg_base = (uint32_t)rows;
-        sc.red_first = (uint32_t)red;
         rows += tp.n_tseg;
-        red += tp.n_red;
-        for (uint32_t r = 0; r < tp.n_red; ++r) bt.red_scen.push_back((uint32_t)b);
         bt.n_cand = sat_add(bt.n_cand, tp.n_cand);
         bt.n_cand_own = sat_add(bt.n_cand_own, bt.tmpl_cand_own[sc.tmpl]);
         bt.n_split = sat_add(bt.n_split, tp.n_split_total);
-        if (rows >= (1ull << 31) || red >= (1ull << 31) || bt.n_cand >= (1ull << 62))
+        if (rows >= (1ull << 31) || bt.n_cand >= (1ull << 62))
             return fail(ctx, CM_EOVERFLOW, "batch too large for the index type");
     }
     bt.n_rows = rows;
@@ -1178,23 +1172,21 @@ BatchDev dev_view(const cm_ctx *ctx, Batch &bt) {
     v.failed = (const uint32_t *)(a + bt.off_failed); v.cross = (const uint64_t *)(a + bt.off_cross);
     v.tmpl_scen = (const uint32_t *)(a + bt.off_tmpl_scen);
     v.bucket = (const Bucket *)(a + bt.off_bucket);
-    v.bucket_tseg = (const uint32_t *)(a + bt.off_bucket_tseg); v.red_scen = (const uint32_t *)(a + bt.off_red);
+    v.bucket_tseg = (const uint32_t *)(a + bt.off_bucket_tseg);
     v.feas = ctx->d_feas.p;
     v.feas_mask = ctx->d_feas_mask.p;
     v.useg = bt.d_useg.p;
     v.tseg_canon = bt.n_dup ? (const uint32_t *)(a + bt.off_canon) : nullptr;
     v.n_rep_scen = 0;
     for (const Tmpl &tp : bt.tmpl) v.n_rep_scen += tp.n_scen;
-    v.seg_best = bt.d_seg_best.p; v.partial = bt.d_partial.p;
+    v.seg_best = bt.d_seg_best.p;
     v.winner = bt.d_winner.p; v.kappa_sel = bt.d_kappa_sel.p; v.pol_cost = bt.d_pol_cost.p;
     v.rc_stages = bt.d_rc_stages.p; v.plans = bt.direct ? bt.plans_host.p : bt.d_plans.p;
     v.counters = reinterpret_cast<unsigned long long *>(bt.d_seg_best.p + bt.n_rows);
     v.B = bt.B; v.mode = bt.opts.cost; v.intval = bt.intval ? 1u : 0u;
     v.n_rows = (uint32_t)bt.n_rows;
     v.n_tiles = bt.n_tiles; v.max_tiles_per_seg = bt.max_tiles_per_seg;
-    v.n_red_blocks = (uint32_t)bt.red_scen.size(); v.dp_max = bt.dp_max;
-    v.max_red_per_scen = 0;
-    for (const Tmpl &tp : bt.tmpl) v.max_red_per_scen = std::max(v.max_red_per_scen, tp.n_scen ? tp.n_red : 0u);
+    v.dp_max = bt.dp_max;
     v.layer_mode = bt.opts.lm; v.batch_mode = bt.opts.bm;
     return v;
 }
@@ -1251,7 +1243,6 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
     bt.off_strat = arena_put(bt.arena, bt.strat, ok);
     bt.off_tseg = arena_put(bt.arena, bt.tseg, ok);
     bt.off_failed = arena_put(bt.arena, bt.failed, ok);
-    bt.off_red = arena_put(bt.arena, bt.red_scen, ok);
     bt.off_keys = arena_put(bt.arena, bt.keys, ok);
     bt.off_tmpl_scen = arena_put(bt.arena, bt.tmpl_scen, ok);
     bt.off_bucket_tseg = arena_put(bt.arena, bt.bucket_tseg, ok);
@@ -1270,7 +1261,7 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
     const size_t B = std::max(bt.B, 1);
     // minima | work counters | list counts | bounds | picks: what one memset clears
     ok = bt.d_seg_best.reserve(3 * bt.n_rows + kStateExtra) && bt.d_win.reserve(B) &&
-         bt.d_partial.reserve(std::max<size_t>(bt.red_scen.size(), 1)) && bt.d_winner.reserve(B) &&
+         bt.d_winner.reserve(B) &&
          bt.d_kappa_sel.reserve(B * kMaxP) && bt.d_pol_cost.reserve(B * 2) &&
          bt.d_rc_stages.reserve(B * kMaxP) && bt.d_plans.reserve(B * 4 + 1);   // + room for the counters
     if (!ok) return fail(ctx, CM_ENOMEM, "device memory");
@@ -1386,7 +1377,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
         }
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
         CM_CUDA(ctx, launch_split_reduce(tb, bd, st));
-        launches += (bd.batch_mode == CM_BATCH_FULL && bd.n_red_blocks && bd.max_red_per_scen > 1) ? 2 : 1;
+        ++launches;
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
         if (bt.n_tiles) {
             CM_CUDA(ctx, launch_tiebreak(tb, bd, st));
@@ -1510,6 +1501,27 @@ void scrub(cm_plan &pl) {
         if (pl.kappa[p] == ~0ull) { pl.kappa[p] = 0; pl.feasible = 0; }
 }
 
+// Plans of a finished search to the caller's arrays (per_policy may be NULL).
+void hand_out(const Batch &bt, cm_plan *best, cm_plan *per_policy) {
+    memcpy(best, bt.plans_host.p, sizeof(cm_plan) * bt.B);
+    if (per_policy) memcpy(per_policy, bt.plans_host.p + bt.B, sizeof(cm_plan) * 3 * (size_t)bt.B);
+}
+
+// Node boundaries among the survivors, ascending (bit j: survivors j and j+1 sit on different nodes), from
+// how many of every node's devices survive.  `alive`: scratch.  Returns the survivor count.
+int crossing_bits(const DevProfile &hp, const uint32_t *failed, int n_failed, std::vector<int> &alive, uint64_t *words) {
+    const int N = hp.n_dp * hp.n_pp, dpn = hp.devices_per_node, nodes = (N + dpn - 1) / dpn;
+    alive.assign(nodes, dpn);
+    alive[nodes - 1] = N - (nodes - 1) * dpn;
+    for (int f = 0; f < n_failed; ++f) --alive[failed[f] / (uint32_t)dpn];
+    int n = 0;
+    for (int a : alive) {
+        if (a > 0 && n > 0) words[(n - 1) >> 6] |= 1ull << ((n - 1) & 63);
+        n += a;
+    }
+    return n;
+}
+
 // A prepared one-scenario batch for this failure set: found among the context's resident ones
 // (same survivor count, same options, same arithmetic) and patched, or built and uploaded.
 // *entry: the resident entry that was reused (its launch sequence may replay as a graph), NULL
@@ -1554,17 +1566,9 @@ cm_status single_batch(cm_ctx *ctx, const uint32_t *ids, int n, const cm_enum_op
     // patch what depends on WHICH devices failed: the ids and the node-crossing bits
     const size_t cross_words = bt.cross.size();
     std::fill(bt.cross.begin(), bt.cross.end(), 0ull);
-    int n_surv = 0, prev_node = -1, f = 0;
-    uint32_t sorted[CM_MAX_PIPES * CM_MAX_STAGES];
-    for (int i = 0; i < n; ++i) { bt.failed[i] = ids[i]; sorted[i] = ids[i]; }
-    std::sort(sorted, sorted + n);
-    for (int d = 0; d < N; ++d) {
-        if (f < n && sorted[f] == (uint32_t)d) { ++f; continue; }
-        const int node = d / hp.devices_per_node;
-        if (n_surv > 0 && node != prev_node) bt.cross[(n_surv - 1) >> 6] |= 1ull << ((n_surv - 1) & 63);
-        prev_node = node;
-        ++n_surv;
-    }
+    std::vector<int> alive;
+    for (int i = 0; i < n; ++i) bt.failed[i] = ids[i];
+    crossing_bits(hp, ids, n, alive, bt.cross.data());
     if (n) memcpy(bt.arena.p + bt.off_failed, bt.failed.data(), sizeof(uint32_t) * n);
     memcpy(bt.arena.p + bt.off_cross, bt.cross.data(), sizeof(uint64_t) * cross_words);
     ctx->stats[9] += sizeof(uint32_t) * n + sizeof(uint64_t) * cross_words;
@@ -1987,7 +1991,7 @@ cm_status cm_select(cm_ctx *ctx, cm_space *const *spaces, int32_t n_spaces, cm_p
     cm_plan result;
     memset(&result, 0, sizeof(result));
     for (int i = 0; i < n_spaces; ++i) {
-        const cm_plan &q = spaces[i]->own->plans_host[spaces[i]->policy];
+        const cm_plan &q = spaces[i]->own->plans_host[spaces[i]->own->B + spaces[i]->policy];
         if (!q.feasible) continue;
         const bool less = whole ? q.cost_ns < result.cost_ns : q.cost < result.cost;
         const bool equal = whole ? q.cost_ns == result.cost_ns : q.cost == result.cost;
@@ -2014,16 +2018,6 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
     if (B == 0) return CM_OK;
     const uint32_t mask = (1u << CM_REROUTE) | (1u << CM_REDUNDANT) | (1u << CM_DYNPAR);
     Batch &bt = ctx->batch;
-    auto copy_out = [&](int b_dst, int b_src) {
-        for (int pol = 0; pol < 3; ++pol) {
-            cm_plan pl = bt.plans_host[(size_t)b_src * 4 + pol];
-            scrub(pl);
-            if (best_per_policy) best_per_policy[(size_t)b_dst * 3 + pol] = pl;
-        }
-        cm_plan pl = bt.plans_host[(size_t)b_src * 4 + 3];
-        scrub(pl);
-        best_per_scenario[b_dst] = pl;
-    };
     if (!latency_us) {
         int launches = 0;
         const uint64_t h0 = now_ns();
@@ -2031,7 +2025,7 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
         ctx->stats[13] += now_ns() - h0;
         if ((s = upload_batch(ctx, bt, &launches)) != CM_OK) { forget_keys(ctx, bt); return s; }
         if ((s = run_batch(ctx, bt, launches)) != CM_OK) return s;
-        for (int b = 0; b < B; ++b) copy_out(b, b);
+        hand_out(bt, best_per_scenario, best_per_policy);
         return CM_OK;
     }
     for (int b = 0; b < B; ++b) {
@@ -2043,14 +2037,7 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
         if ((s = single_batch(ctx, failed_ids + offsets[b], offsets[b + 1] - offsets[b], *opts, mask, &sb, &launches, &entry)) != CM_OK) return s;
         ctx->stats[13] += now_ns() - h0;
         if ((s = run_batch(ctx, *sb, launches, entry)) != CM_OK) return s;
-        for (int pol = 0; pol < 3; ++pol) {
-            cm_plan pl = sb->plans_host[pol];
-            scrub(pl);
-            if (best_per_policy) best_per_policy[(size_t)b * 3 + pol] = pl;
-        }
-        cm_plan pl = sb->plans_host[3];
-        scrub(pl);
-        best_per_scenario[b] = pl;
+        hand_out(*sb, best_per_scenario + b, best_per_policy ? best_per_policy + (size_t)b * 3 : nullptr);
         const auto t1 = std::chrono::steady_clock::now();
         latency_us[b] = (float)std::chrono::duration<double, std::micro>(t1 - t0).count();
     }
@@ -2172,7 +2159,7 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
     }
     uint64_t solved = 0;
     for (size_t i = 0; i < slots; ++i) {
-        if (shortlist) { cm_plan pl = bt.short_plans_host[i]; scrub(pl); shortlist[i] = pl; }
+        if (shortlist) { shortlist[i] = bt.short_plans_host[i]; scrub(shortlist[i]); }
         if (shortlist_bytes) { shortlist_bytes[i] = bt.short_bytes_host[i]; solved += bt.short_bytes_host[i] >= 0; }
         if (shortlist_rounds) shortlist_rounds[i] = q.sync_rounds ? bt.short_rounds_host[i * 2] : 0;
     }
@@ -2337,16 +2324,7 @@ cm_status cm_batch_search(cm_ctx *ctx, cm_batch *bp, cm_plan *best_per_scenario,
     if (bt.B == 0) return CM_OK;
     cm_status s = run_batch(ctx, bt, 0);
     if (s != CM_OK) return s;
-    for (int b = 0; b < bt.B; ++b) {
-        for (int pol = 0; pol < 3 && best_per_policy; ++pol) {
-            cm_plan pl = bt.plans_host[(size_t)b * 4 + pol];
-            scrub(pl);
-            best_per_policy[(size_t)b * 3 + pol] = pl;
-        }
-        cm_plan pl = bt.plans_host[(size_t)b * 4 + 3];
-        scrub(pl);
-        best_per_scenario[b] = pl;
-    }
+    hand_out(bt, best_per_scenario, best_per_policy);
     return CM_OK;
     CM_API_END(ctx)
 }

@@ -76,7 +76,6 @@ struct Tmpl {
     uint32_t strat_first, n_strat;
     uint32_t tseg_first, n_tseg;
     uint32_t scen_first, n_scen;   // its scenarios, as a range of the tmpl_scen list
-    uint32_t n_red, pad;           // blocks of the split reduction per scenario
 };
 
 // One failure scenario of a batch.  Its segments own rows seg_base .. seg_base+n_tseg-1 of
@@ -84,7 +83,7 @@ struct Tmpl {
 struct Scen {              // 32 bytes
     uint32_t tmpl, seg_base;
     uint32_t failed_first, n_failed;   // into the failed-id array
-    uint32_t cross_first, red_first;   // into the node-crossing bit words; first reduction block
+    uint32_t cross_first, pad;         // into the node-crossing bit words
     uint32_t policy_mask;
     uint32_t rep;                      // scenario whose dynamic-parallelism search this one shares (itself if none)
 };
@@ -227,12 +226,6 @@ constexpr size_t kBoundDynMax = 160 * 1024;      // dynamic shared memory of the
 constexpr size_t kBoundDynTarget = 64 * 1024;    //   and wanted: three CTAs per SM
 constexpr size_t kRefineSegBytes = 32;
 
-// (cost, index) pair carried through the hierarchical argmin of the split reduction.
-struct Partial {
-    uint64_t cost_bits;     // cost as an order-preserving 64-bit pattern (inf = infeasible)
-    uint64_t item;          // split item index within the scenario
-};
-
 // Per-scenario winner of the split reduction, decoded for the tie-break pass.
 struct Winner {
     uint64_t cost_bits;
@@ -264,13 +257,11 @@ struct BatchDev {
     const uint32_t *tseg_canon;
     uint32_t n_rep_scen;          // scenarios that own result rows (entries of tmpl_scen in use)
     uint64_t *seg_best;     // [n_seg] min cost over kappa, order-preserving bits
-    const uint32_t *red_scen;  // [n_red_blocks] scenario of every block of the split reduction
-    Partial *partial;       // [n_red_blocks]
     Winner *winner;         // [B]
     uint64_t *kappa_sel;    // [B][kMaxP] lowest kappa with cost <= T*
     uint64_t *pol_cost;     // [B][2] rerouting / redundant cost bits
     uint16_t *rc_stages;    // [B][kMaxP] stage counts of the redundant-computation plan
-    cm_plan *plans;         // [B][4]: per policy, then the overall best
+    cm_plan *plans;         // [B] the overall best, then [B][3] per policy, then the work counters
     // [0] cells of the plans the search pass decided, [1] plans of the tie-break pass, [2] plans decided;
     // bounded pass: [3] cells and [5] plans whose recurrence ran, [4] a list was full
     unsigned long long *counters;
@@ -280,9 +271,8 @@ struct BatchDev {
     // cost on the device is then a double bit pattern and becomes an integer only on the way out
     uint32_t intval;
     uint64_t n_tiles;
-    uint32_t max_tiles_per_seg, n_red_blocks;
+    uint32_t max_tiles_per_seg;
     uint32_t dp_max;
-    uint32_t max_red_per_scen;   // most blocks of the split reduction any scenario has
     int32_t layer_mode, batch_mode;
 };
 

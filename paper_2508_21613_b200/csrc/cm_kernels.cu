@@ -5,9 +5,7 @@
 //   cm_feasible_kernel    memory-feasible layer compositions per (stages, micro-batches), listed once
 //   (data rerouting / redundant computation: cm_policy.cu)
 //   (the search pass over every pipeline-plan lives in cm_cost.cu)
-//   cm_best_split_kernel  best (strategy, micro-batch split) per scenario under the remainder rule
-//   cm_split_kernel       the same under the full enumeration of splits: (cost, index) argmin
-//   cm_winner_kernel      finishes that argmin and decodes the winner
+//   cm_best_split_kernel  best (strategy, micro-batch split) per scenario, the winner decoded
 //   (pass 2, the lowest layer composition that meets the winning cost: cm_tiebreak.cu)
 //   cm_finalize_kernel    assembles the plans and picks the best policy
 //   (per-candidate cost / feasibility for cm_evaluate: cm_evaluate.cu)
@@ -346,128 +344,119 @@ cudaError_t launch_useg_copy(const BatchDev &b, const USegDev &u, cudaStream_t s
 }
 
 // ----------------------------------------------------------------------------------
-// Split reduction under the full enumeration of splits: item = (strategy, split rank) of one scenario; its step time is the
-// slowest pipeline's best cost (Section "Estimator": step time = max over pipelines).
-// Hierarchical argmin carrying (cost, item) with the lowest item on ties:
-// thread-serial over a strided range -> warp shuffle -> shared memory -> one partial
-// per block -> cm_winner_kernel over the scenario's partials.
+// Best (strategy, micro-batch split) of a scenario: the slowest pipeline's best cost (Section "Estimator":
+// step time = max over pipelines), ties to the first strategy and to its split of lowest rank.  A warp per
+// strategy; no split is enumerated.
+//
+// Remainder rule: cm_split.cuh gives the step time; the R larger shares go where they must and then to the
+// lowest pipelines that may have them (colexicographic ranks grow with the highest element first).
+//
+// Full enumeration: a pipeline's best cost does not fall when it gets one more micro-batch, so a step time
+// t is within reach if the most micro-batches that every pipeline can take within t add up to G.  The
+// pipelines start with one each, t with the slowest of them; whoever can take one more within t does, and
+// where nobody can t moves to the least next cost.  The split of lowest rank gives the last pipelines as
+// many as they can take.  (Costs can fall only where the min-max partition is the only candidate and
+// memory forces a luckier one; such a strategy is seen and goes through its splits.)
 // ----------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) cm_split_kernel(Tables tb, BatchDev bd, uint64_t inf) {
-    __shared__ uint64_t rc[8], ri[8];
-    const uint32_t b = bd.red_scen[blockIdx.x];
-    const Scen sc = bd.scen[b];
-    const Tmpl tp = bd.tmpl[sc.tmpl];
-    const uint32_t local = blockIdx.x - sc.red_first;
-    const uint64_t *best = bd.seg_best + sc.seg_base;   // this scenario's rows, in template order
-    uint64_t best_c = inf, best_i = ~0ull;
-    for (uint64_t item = (uint64_t)local * blockDim.x + threadIdx.x; item < tp.n_split_total;
-         item += (uint64_t)tp.n_red * blockDim.x) {
-        const uint64_t T = item_step_time(tb, bd, tp, best, item, inf);
-        if (pair_less(T, item, best_c, best_i)) { best_c = T; best_i = item; }
+struct FullSplit {   // full enumeration, lane = pipeline
+    const BatchDev &bd; const Tmpl &tp; const Scen &sc; const Strat &s;
+    uint64_t inf;
+    __device__ __forceinline__ uint64_t cost(int m) const {   // of this lane's pipeline with m micro-batches
+        const int lane = threadIdx.x & 31;
+        if (lane >= (int)s.dp || m > (int)s.n_m) return inf;
+        const uint64_t v = bd.seg_best[canon_row(bd, tp, sc, s, lane, m - 1)];
+        return v < inf ? v : inf;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o);
-        uint64_t oi = __shfl_xor_sync(0xffffffffu, best_i, o);
-        if (pair_less(oc, oi, best_c, best_i)) { best_c = oc; best_i = oi; }
-    }
-    if ((threadIdx.x & 31) == 0) { rc[threadIdx.x >> 5] = best_c; ri[threadIdx.x >> 5] = best_i; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w)
-            if (pair_less(rc[w], ri[w], best_c, best_i)) { best_c = rc[w]; best_i = ri[w]; }
-        bd.partial[blockIdx.x].cost_bits = best_c;
-        bd.partial[blockIdx.x].item = best_i;
-    }
-}
-
-// Grid level of the argmin: one warp per scenario over its block partials, then decode
-// the winner (strategy, split -> micro-batches, segment rows) for the tie-break pass.
-__global__ void __launch_bounds__(32) cm_winner_kernel(Tables tb, BatchDev bd, uint64_t inf) {
-    const uint32_t b = blockIdx.x;
-    const Scen sc = bd.scen[b];
-    const Tmpl tp = bd.tmpl[sc.tmpl];
-    uint64_t best_c = inf, best_i = ~0ull;
-    for (uint32_t r = threadIdx.x; r < (sc.rep == b ? tp.n_red : 0u); r += 32) {
-        const Partial q = bd.partial[sc.red_first + r];
-        if (pair_less(q.cost_bits, q.item, best_c, best_i)) { best_c = q.cost_bits; best_i = q.item; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o);
-        uint64_t oi = __shfl_xor_sync(0xffffffffu, best_i, o);
-        if (pair_less(oc, oi, best_c, best_i)) { best_c = oc; best_i = oi; }
-    }
-    if (threadIdx.x == 0) {
-        Winner w;
-        if (sc.rep != b) { best_c = inf; best_i = ~0ull; }   // shares another scenario's search: nothing to tie-break here
-        decode_winner(tb, bd, tp, b, best_c, best_i, inf, w);
-        bd.winner[b] = w;
-    }
-    __syncthreads();   // the record is written: one thread per pipeline sets its start value
-    if (threadIdx.x < kMaxP) init_kappa_sel(bd, bd.winner[b], bd.kappa_sel + (size_t)b * kMaxP, (int)threadIdx.x);
-}
-
-// Both levels in one launch, for batches in which no scenario needs more than one block of the
-// split reduction (up to 1024 (strategy, split) pairs each): one CTA per scenario.
-__global__ void __launch_bounds__(256) cm_split_winner_kernel(Tables tb, BatchDev bd, uint64_t inf) {
-    __shared__ uint64_t rc[8], ri[8];
-    const uint32_t b = blockIdx.x;
-    const Scen sc = bd.scen[b];
-    const Tmpl tp = bd.tmpl[sc.tmpl];
-    const uint64_t *best = bd.seg_best + sc.seg_base;
-    uint64_t best_c = inf, best_i = ~0ull;
-    if (sc.rep == b)
-        for (uint64_t item = threadIdx.x; item < tp.n_split_total; item += blockDim.x) {
-            const uint64_t T = item_step_time(tb, bd, tp, best, item, inf);
-            if (pair_less(T, item, best_c, best_i)) { best_c = T; best_i = item; }
+    __device__ __forceinline__ bool monotone() const {
+        bool ok = true;
+        for (int q = threadIdx.x & 31; q < (int)s.dp * (int)(s.n_m - 1); q += 32) {
+            const int p = q / (s.n_m - 1), k = q - p * (s.n_m - 1);
+            const uint64_t a = bd.seg_best[canon_row(bd, tp, sc, s, p, k)], c = bd.seg_best[canon_row(bd, tp, sc, s, p, k + 1)];
+            ok = ok && (a < inf ? a : inf) <= (c < inf ? c : inf);
         }
-    for (int o = 16; o > 0; o >>= 1) {
-        uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o);
-        uint64_t oi = __shfl_xor_sync(0xffffffffu, best_i, o);
-        if (pair_less(oc, oi, best_c, best_i)) { best_c = oc; best_i = oi; }
+        return __all_sync(0xffffffffu, ok);
     }
-    if ((threadIdx.x & 31) == 0) { rc[threadIdx.x >> 5] = best_c; ri[threadIdx.x >> 5] = best_i; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w)
-            if (pair_less(rc[w], ri[w], best_c, best_i)) { best_c = rc[w]; best_i = ri[w]; }
-        Winner w;
-        decode_winner(tb, bd, tp, b, best_c, best_i, inf, w);
-        bd.winner[b] = w;
+    __device__ __forceinline__ uint64_t best(int G) const {
+        const int dp = s.dp;
+        uint64_t t = ~warp_min_u64((threadIdx.x & 31) < dp ? ~cost(1) : ~0ull);
+        int m = 1, sum = dp;
+        uint64_t next = cost(2);
+        while (sum < G && t < inf) {
+            const bool more = next <= t;
+            const uint32_t who = __ballot_sync(0xffffffffu, more && next < inf);
+            if (who) {
+                sum += __popc(who);
+                if (more && next < inf) next = cost(++m + 1);
+            } else {
+                t = warp_min_u64(next);
+            }
+        }
+        return t < inf ? t : inf;
     }
-    __syncthreads();   // the record is written: one thread per pipeline sets its start value
-    if (threadIdx.x < kMaxP) init_kappa_sel(bd, bd.winner[b], bd.kappa_sel + (size_t)b * kMaxP, (int)threadIdx.x);
-}
+    // micro-batches of this lane's pipeline in the split of lowest rank within t, and that rank
+    __device__ __forceinline__ int micro(const uint64_t *binom, int G, uint64_t t, uint64_t &rank) const {
+        const int lane = threadIdx.x & 31, dp = s.dp;
+        int most = 1;
+        while (cost(most + 1) <= t && most < (int)s.n_m && lane < dp) ++most;
+        int left = G, mine = 0, before = 0;
+        for (int p = dp - 1; p >= 0; --p) {
+            const int can = __shfl_sync(0xffffffffu, most, p), room = left - p;   // (the p pipelines below get one each at least)
+            const int take = can < room ? can : room;
+            left -= take;
+            if (lane == p) { mine = take; before = left; }                        // before: micro-batches of the pipelines below
+        }
+        rank = lane > 0 && lane < dp ? binom_at(binom, before - 1, lane) : 0ull;
+        for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        return mine;
+    }
+};
 
-// The remainder rule: a warp per strategy finds its best step time directly (cm_split.cuh); the first
-// strategy with the least one wins, and of its splits the one of lowest rank -- the smaller share wherever
-// it will do, the R larger ones to the lowest pipelines that may have them (colexicographic ranks grow
-// with the highest element first).  One CTA per scenario, no split is enumerated.
 __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev bd, uint64_t inf) {
-    __shared__ uint64_t rc[32];
+    __shared__ uint64_t rc[32], rx[32];
     __shared__ uint32_t ri[32];
     const uint32_t b = blockIdx.x;
     const Scen sc = bd.scen[b];
     const Tmpl tp = bd.tmpl[sc.tmpl];
     const Strat *strat = bd.strat + tp.strat_first;
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, G = tb.prof->G;
+    const bool full = bd.batch_mode == CM_BATCH_FULL;
     auto cost_of = [&](const Strat &s) { return strat_cost(bd, tp, sc, s, inf, [&](uint32_t row) { return bd.seg_best[row]; }); };
-    uint64_t best_c = inf;
+    uint64_t best_c = inf, best_x = ~0ull;   // best_x: the item, where the splits were gone through
     uint32_t best_i = 0;
     if (sc.rep == b)   // (else it shares another scenario's search: nothing to tie-break here)
         for (uint32_t si = warp; si < tp.n_strat; si += warps) {
-            const uint64_t v = strat_best(cost_of(strat[si]), strat[si], ~0ull, inf);
-            if (v < best_c) { best_c = v; best_i = si; }
+            const Strat &s = strat[si];
+            uint64_t v = inf, x = ~0ull;
+            if (!full) {
+                v = strat_best(cost_of(s), s, ~0ull, inf);
+            } else if (s.n_m >= 1) {
+                const FullSplit fs{bd, tp, sc, s, inf};
+                if (fs.monotone()) {
+                    v = fs.best(G);
+                } else {
+                    for (uint64_t q = lane; q < s.n_split; q += 32) {
+                        const uint64_t item = s.split_first + q, t = item_step_time(tb, bd, tp, bd.seg_best + sc.seg_base, item, inf);
+                        if (pair_less(t, item, v, x)) { v = t; x = item; }
+                    }
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const uint64_t ov = __shfl_xor_sync(0xffffffffu, v, o), ox = __shfl_xor_sync(0xffffffffu, x, o);
+                        if (pair_less(ov, ox, v, x)) { v = ov; x = ox; }
+                    }
+                }
+            }
+            if (v < best_c) { best_c = v; best_i = si; best_x = x; }
         }
-    if (lane == 0) { rc[warp] = best_c; ri[warp] = best_i; }
+    if (lane == 0) { rc[warp] = best_c; ri[warp] = best_i; rx[warp] = best_x; }
     __syncthreads();
     if (warp) return;
     best_c = lane < (int)warps ? rc[lane] : inf;
-    best_i = lane < (int)warps ? ri[lane] : 0;
+    best_i = lane < (int)warps ? ri[lane] : 0xffffffffu;
+    best_x = lane < (int)warps ? rx[lane] : ~0ull;
     for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o);
+        const uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o), ox = __shfl_xor_sync(0xffffffffu, best_x, o);
         const uint32_t oi = __shfl_xor_sync(0xffffffffu, best_i, o);
-        if (oc < best_c || (oc == best_c && oi < best_i)) { best_c = oc; best_i = oi; }
+        if (oc < best_c || (oc == best_c && oi < best_i)) { best_c = oc; best_i = oi; best_x = ox; }
     }
     Winner &w = bd.winner[b];
     uint64_t *kappa = bd.kappa_sel + (size_t)b * kMaxP;
@@ -477,16 +466,29 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
         return;
     }
     const Strat &s = strat[best_i];
-    const uint64_t v = cost_of(s);
-    const uint64_t lo = __shfl_sync(0xffffffffu, v, (2 * lane) & 31), hi = __shfl_sync(0xffffffffu, v, (2 * lane + 1) & 31);
     const bool mine = lane < (int)s.dp;                               // lane = pipeline from here on
-    const uint32_t must = __ballot_sync(0xffffffffu, mine && lo > best_c);
-    const uint32_t may = s.R ? __ballot_sync(0xffffffffu, mine && hi <= best_c) & ~must : 0u;
-    const int need = (int)s.R - __popc(must);
-    const bool extra = mine && (((must >> lane) & 1u) || (((may >> lane) & 1u) && __popc(may & ((1u << lane) - 1u)) < need));
-    const uint32_t set = __ballot_sync(0xffffffffu, extra);
-    uint64_t rank = extra ? binom_at(tb.binom, lane, __popc(set & ((1u << lane) - 1u)) + 1) : 0ull;
-    for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    int micro;
+    uint64_t rank;
+    if (best_x != ~0ull) {
+        uint16_t split[kMaxP];
+        rank = best_x - s.split_first;
+        split_micro(tb.binom, bd.batch_mode, G, s, rank, split);
+        micro = mine ? split[lane & (kMaxP - 1)] : 0;
+    } else if (full) {
+        micro = FullSplit{bd, tp, sc, s, inf}.micro(tb.binom, G, best_c, rank);
+    } else {
+        const uint64_t v = cost_of(s);
+        const uint64_t lo = __shfl_sync(0xffffffffu, v, (2 * lane) & 31), hi = __shfl_sync(0xffffffffu, v, (2 * lane + 1) & 31);
+        const uint32_t must = __ballot_sync(0xffffffffu, mine && lo > best_c);
+        const uint32_t may = s.R ? __ballot_sync(0xffffffffu, mine && hi <= best_c) & ~must : 0u;
+        const int need = (int)s.R - __popc(must);
+        const uint32_t below = (1u << lane) - 1u;
+        const bool extra = mine && (((must >> lane) & 1u) || (((may >> lane) & 1u) && __popc(may & below) < need));
+        const uint32_t set = __ballot_sync(0xffffffffu, extra);
+        rank = extra ? binom_at(tb.binom, lane, __popc(set & below) + 1) : 0ull;
+        for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        micro = mine ? s.m_lo[lane] + (extra ? 1 : 0) : 0;
+    }
     if (lane == 0) {
         w.cost_bits = best_c;
         w.item = s.split_first + rank;
@@ -496,9 +498,9 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
         w.pad = 0;
     }
     if (lane < kMaxP) {
-        const uint32_t seg = mine ? s.seg_first + lane * s.n_m + (extra ? 1 : 0) : 0u;
+        const uint32_t seg = mine ? s.seg_first + lane * s.n_m + (micro - s.m_lo[lane]) : 0u;
         w.seg[lane] = seg;
-        w.micro[lane] = mine ? (uint16_t)(s.m_lo[lane] + (extra ? 1 : 0)) : (uint16_t)0;
+        w.micro[lane] = mine ? (uint16_t)micro : (uint16_t)0;
         // a segment whose only candidate is the min-max partition has nothing to search (init_kappa_sel)
         kappa[lane] = mine && bd.tseg[seg].K == 0 ? 0ull : ~0ull;
     }
@@ -506,22 +508,8 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
 
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
-    const uint64_t inf = batch_inf_bits(b);
-    if (b.batch_mode == CM_BATCH_REMAINDER) {
-        // a failure handled on its own: a warp for every strategy; a batch: enough to keep the SMs busy
-        cm_best_split_kernel<<<b.B, b.B <= 148 ? 1024 : 128, 0, st>>>(t, b, inf);
-        return cudaGetLastError();
-    }
-    if (b.n_red_blocks <= (uint32_t)b.B && b.max_red_per_scen <= 1) {
-        cm_split_winner_kernel<<<b.B, 256, 0, st>>>(t, b, inf);
-        return cudaGetLastError();
-    }
-    if (b.n_red_blocks) {
-        cm_split_kernel<<<b.n_red_blocks, 256, 0, st>>>(t, b, inf);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    cm_winner_kernel<<<b.B, 32, 0, st>>>(t, b, inf);
+    // a failure handled on its own: a warp for every strategy; a batch: enough to keep the SMs busy
+    cm_best_split_kernel<<<b.B, b.B <= 148 ? 1024 : 128, 0, st>>>(t, b, batch_inf_bits(b));
     return cudaGetLastError();
 }
 
@@ -549,7 +537,8 @@ cudaError_t launch_prologue(uint64_t *words, size_t n_words, const uint32_t *ids
 // ----------------------------------------------------------------------------------
 // Assemble the per-policy plans and the overall best: least cost, ties to the lowest
 // policy id (Algorithm 1 keeps the plan with the least estimated time).  Sixteen threads per plan, one
-// per pipeline; four plans per scenario, the last a copy of the winner.
+// per pipeline; four plans per scenario, the last the winner: it goes to the front of the array, the plans
+// per policy follow scenario by scenario, so that the host hands both out in one piece each.
 // ----------------------------------------------------------------------------------
 constexpr int kFinalThreads = 64;
 __global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, BatchDev bd, uint64_t inf) {
@@ -578,10 +567,14 @@ __global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, B
     }
     const bool dyn = pol == CM_DYNPAR, feasible = cost[pol] < inf, filled = any && (!dyn || feasible);
     const int n = !filled ? 0 : dyn ? (int)w.dp : p->n_dp < kMaxP ? p->n_dp : kMaxP;
-    cm_plan &out = bd.plans[(size_t)b * 4 + slot];
+    uint64_t kappa = k < n && dyn ? bd.kappa_sel[(size_t)sc.rep * kMaxP + k] : 0ull;
+    // (a composition that was not found cannot happen for a feasible winner, but is never handed out as a rank)
+    const uint32_t lost = __ballot_sync(0xffffffffu, kappa == ~0ull) >> (threadIdx.x & 16) & 0xffffu;
+    if (kappa == ~0ull) kappa = 0ull;
+    cm_plan &out = bd.plans[slot == 3 ? (size_t)b : (size_t)bd.B + 3 * (size_t)b + slot];
     if (k == 0) {
         out.policy = any ? pol : 0;
-        out.feasible = feasible ? 1 : 0;
+        out.feasible = feasible && !lost ? 1 : 0;
         out.cost = 0.0;
         out.cost_ns = 0;
         if (feasible) plan_set_cost(out, cost[pol], bd);
@@ -592,7 +585,7 @@ __global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, B
     out.stages[k] = k >= n ? (uint16_t)0 : dyn ? bd.strat[w.strat].S[k]
                     : pol == CM_REDUNDANT && feasible ? bd.rc_stages[b * kMaxP + k] : (uint16_t)p->n_pp;
     out.micro[k] = k >= n ? (uint16_t)0 : dyn ? w.micro[k] : (uint16_t)p->n_micro;
-    out.kappa[k] = k < n && dyn ? bd.kappa_sel[(size_t)sc.rep * kMaxP + k] : 0ull;
+    out.kappa[k] = kappa;
 }
 
 cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st) {
