@@ -138,7 +138,7 @@ struct Batch {
     size_t off_ucls = 0, off_tseg_cls = 0, off_look_head = 0, off_look_part = 0;
     uint64_t utab_slots = 0, ulist_len = 0;
     DevBuf<unsigned long long> d_utab;
-    DevBuf<uint32_t> d_urep, d_slot_of, d_ucount;
+    DevBuf<uint32_t> d_urep, d_slot_of, d_row_rep, d_ucount;
     DevBuf<uint2> d_useg;
     PinnedVec<uint32_t> ucount_host;
     // Bounded search pass (cm_bound.cu): its buckets and its device state.
@@ -152,7 +152,7 @@ struct Batch {
     size_t bytes() const {
         return d_arena.cap + 8 * (d_seg_best.cap + d_kappa_sel.cap + d_pol_cost.cap + d_utab.cap + d_useg.cap + d_short_kappa.cap) +
                sizeof(Winner) * (d_winner.cap + d_short_win.cap) + sizeof(cm_plan) * (d_plans.cap + d_short_plans.cap) +
-               4 * (d_urep.cap + d_slot_of.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
+               4 * (d_urep.cap + d_slot_of.cap + d_row_rep.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
     }
     // One scenario handled on its own: its first kernel reads the failed ids and the node-crossing bits
     // from the pinned arena and its last one writes the plans to pinned memory, so that no copy sits on the
@@ -583,7 +583,6 @@ cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups) {
     bo.n_chunks = (uint32_t)chunks;
     bo.n_segs = (uint32_t)n_segs;
     bo.uniform_x = ctx->uniform_p2p ? 1 : 0;
-    bo.window = bt.useg ? 0 : 1;
     bo.dyn_bytes = bound_dyn_bytes(bo, max_stages, max_group, ctx->uniform_p2p);
     if (bo.dyn_bytes > kBoundDynMax) return CM_OK;
     bt.bo = bo;
@@ -1198,7 +1197,7 @@ USegDev useg_view(const Batch &bt) {
     u.look_head = (const uint32_t *)(bt.d_arena.p + bt.off_look_head);
     u.look_part = (const uint32_t *)(bt.d_arena.p + bt.off_look_part);
     u.n_pair_cls = bt.n_pair_cls;
-    u.tab = bt.d_utab.p; u.rep = bt.d_urep.p; u.slot_of = bt.d_slot_of.p; u.count = bt.d_ucount.p; u.list = bt.d_useg.p;
+    u.tab = bt.d_utab.p; u.rep = bt.d_urep.p; u.slot_of = bt.d_slot_of.p; u.row_rep = bt.d_row_rep.p; u.count = bt.d_ucount.p; u.list = bt.d_useg.p;
     u.n_cls = (uint32_t)bt.ucls.size();
     u.n_rep_scen = 0;
     for (const Tmpl &tp : bt.tmpl) u.n_rep_scen += tp.n_scen;
@@ -1259,8 +1258,8 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
     CM_CUDA(ctx, cudaMemcpyAsync(bt.d_arena.p, bt.arena.p, bt.arena.size(), cudaMemcpyHostToDevice, ctx->stream));
     ctx->stats[9] += bt.arena.size();
     const size_t B = std::max(bt.B, 1);
-    // minima | work counters | list counts | bounds | picks: what one memset clears
-    ok = bt.d_seg_best.reserve(3 * bt.n_rows + kStateExtra) && bt.d_win.reserve(B) &&
+    // minima | work counters | list counts | bounds | picks | windows of shared rows: what one memset clears
+    ok = bt.d_seg_best.reserve((bt.useg ? 5 : 3) * bt.n_rows + kStateExtra) && bt.d_win.reserve(B) &&
          bt.d_winner.reserve(B) &&
          bt.d_kappa_sel.reserve(B * kMaxP) && bt.d_pol_cost.reserve(B * 2) &&
          bt.d_rc_stages.reserve(B * kMaxP) && bt.d_plans.reserve(B * 4 + 1);   // + room for the counters
@@ -1276,7 +1275,7 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
         // are laid out and their table -- the last section of the arena -- is copied again
         const size_t n_cls = bt.ucls.size();
         ok = bt.d_utab.reserve(std::max<uint64_t>(bt.utab_slots, 1)) && bt.d_urep.reserve(std::max<uint64_t>(bt.utab_slots, 1)) &&
-             bt.d_slot_of.reserve(std::max<uint64_t>(bt.n_rows, 1)) && bt.d_ucount.reserve(n_cls + 1) &&
+             bt.d_slot_of.reserve(std::max<uint64_t>(bt.n_rows, 1)) && bt.d_row_rep.reserve(std::max<uint64_t>(bt.n_rows, 1)) && bt.d_ucount.reserve(n_cls + 1) &&
              bt.d_useg.reserve(std::max<uint64_t>(bt.ulist_len, 1)) && bt.ucount_host.resize(n_cls + 1);
         if (!ok) return fail(ctx, CM_ENOMEM, "memory");
         CM_CUDA(ctx, cudaMemsetAsync(bt.d_utab.p, 0xFF, bt.utab_slots * sizeof(unsigned long long), ctx->stream));
@@ -1314,20 +1313,22 @@ cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchD
     bo.lbarg = bt.d_seg_best.p + bt.n_rows + kStateExtra;
     bo.pick = bo.lbarg + bt.n_rows;
     bo.win = bt.d_win.p;
+    if (bt.useg) {
+        bo.row_rep = bt.d_row_rep.p;
+        bo.row_lo = bo.pick + bt.n_rows;
+        bo.row_ub = bo.row_lo + bt.n_rows;
+    }
     bo.list = ctx->d_bound_list.p;
     CM_CUDA(ctx, launch_bound(tb, bd, bo, st));
     ++*launches;
     for (int phase = 1; phase <= 2; ++phase) {
-        if (bo.window) {
-            CM_CUDA(ctx, launch_window(tb, bd, bo, phase - 1, bt.k_best, st));
-            ++*launches;
-        }
+        CM_CUDA(ctx, launch_window(tb, bd, bo, phase - 1, bt.k_best, st));
         CM_CUDA(ctx, launch_refine(tb, bd, bo, phase, st));
         if (phase == 1) {
             CM_CUDA(ctx, launch_gather(tb, bd, bo, st));
             ++*launches;
         }
-        ++*launches;
+        *launches += 2;
         CM_CUDA(ctx, launch_lists(tb, bd, bo, 2 * phase - 2, st, launches));
     }
     return CM_OK;
@@ -1342,7 +1343,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     int launches = 0, cost_launches = 0;
     // per-segment minima start at all-ones (above every cost); so do the work counters, which
     // therefore read "value - 1" until cm_finalize_kernel adds the one back
-    const size_t cleared = (bt.bounded ? 3 * bt.n_rows : bt.n_rows) + kStateExtra;
+    const size_t cleared = (bt.bounded ? (bt.useg ? 5 : 3) * bt.n_rows : bt.n_rows) + kStateExtra;
     if (bt.direct) {
         CM_CUDA(ctx, launch_prologue(bt.d_seg_best.p, cleared, (const uint32_t *)(bt.arena.p + bt.off_failed), (uint32_t *)(bt.d_arena.p + bt.off_failed),
                                      (int)bt.failed.size(), (const uint64_t *)(bt.arena.p + bt.off_cross),

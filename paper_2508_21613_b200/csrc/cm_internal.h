@@ -143,6 +143,7 @@ struct USegDev {
     unsigned long long *tab;        // tier words, all-ones = empty
     uint32_t *rep;                  // per slot: lowest row with that key
     uint32_t *slot_of;              // per row: its slot (kNoSegClass: none)
+    uint32_t *row_rep;              // per row: the row that is searched for it
     uint32_t *count;                // per class: distinct segments; count[n_cls]: probes that found no slot (never)
     uint2 *list;                    // (scenario, template segment) of every distinct segment, by class
     uint32_t n_cls, n_rep_scen;
@@ -209,14 +210,19 @@ struct BoundDev {
     const BBucket *bucket;
     uint64_t *lbarg;              // per row: least bound (float bits) << 32 | its position in the walk; all-ones = no plan fits
     uint64_t *pick;               // per row: the plan phase 1 takes (cm_bound_lane.cuh)
-    SearchWin *win;               // per scenario (window)
+    SearchWin *win;               // per scenario
+    // Segments shared between scenarios (else null): the row searched for a row; per searched row the
+    // least lo (float bits) and the largest ub (its complement, so that all-ones is "none") of the
+    // scenarios that mark it.
+    const uint32_t *row_rep;
+    uint64_t *row_lo, *row_ub;
     uint4 *list;                  // plans for the recurrence: scenario, template segment, position
     uint32_t *count;              // per list: plans listed minus one
     uint32_t list_first[5];       // lists: phase 1 up to kRegStagesMax stages, deeper; phase 2 the same
     uint32_t n_buckets, n_chunks, n_segs;
     uint32_t dyn_far, dyn_cols, dyn_cuts, dyn_segs, max_group;   // shared memory of a CTA (BoundSmem)
     size_t dyn_bytes;
-    int window, uniform_x;
+    int uniform_x;
 };
 constexpr int kCounters = 6;   // work counters of a search in use (BatchDev::counters)
 // Recurrence cells of a search (a shallow one counting a quarter) from which bounds pay for their extra launches.

@@ -237,7 +237,8 @@ cudaError_t launch_feasible(const Tables &t, int layer_mode, const uint32_t *key
 // class's table (linear probing, at most as many probes as the table has slots; a table holds
 // at least twice the rows of its class) and leaves the lowest row per slot as its
 // representative; cm_useg_list_kernel appends every representative to its class's list (the
-// order within a class is whatever the atomics give: results do not depend on it);
+// order within a class is whatever the atomics give: results do not depend on it) and writes down
+// which row is searched for each;
 // cm_useg_copy_kernel, after the search pass, gives every other row its representative's minimum.
 // ----------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t mix64(uint64_t x) {
@@ -305,7 +306,12 @@ __global__ void __launch_bounds__(128) cm_useg_list_kernel(BatchDev bd, USegDev 
     for (uint32_t i = threadIdx.x; i < tp.n_tseg; i += blockDim.x) {
         const uint32_t trow = tp.tseg_first + i, row = sc.seg_base + i;
         const uint32_t slot = ud.slot_of[row];
-        if (slot == kNoSegClass || slot == kPartnerSeg || (slot & kSecondRowFlag) || ud.rep[slot] != row) continue;
+        if (slot == kNoSegClass) { ud.row_rep[row] = row; continue; }
+        if (slot == kPartnerSeg) { ud.row_rep[row] = ud.rep[ud.slot_of[row - 1]] + 1; continue; }   // second row of a keyed pair head
+        if (slot & kSecondRowFlag) { ud.row_rep[row] = ud.rep[slot & ~kSecondRowFlag] + 1; continue; }
+        const uint32_t rep = ud.rep[slot];
+        ud.row_rep[row] = rep;
+        if (rep != row) continue;
         const uint32_t ci = ud.tseg_cls[trow];   // a representative was keyed in its own class
         const uint32_t pos = atomicAdd(&ud.count[ci], 1u);
         ud.list[ud.cls[ci].list_first + pos] = make_uint2(scen_id, trow);
@@ -315,17 +321,7 @@ __global__ void __launch_bounds__(128) cm_useg_list_kernel(BatchDev bd, USegDev 
 __global__ void __launch_bounds__(256) cm_useg_copy_kernel(BatchDev bd, USegDev ud) {
     const uint32_t row = blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= bd.n_rows) return;
-    uint32_t slot = ud.slot_of[row];
-    if (slot == kNoSegClass) return;
-    uint32_t second = 0;
-    if (slot == kPartnerSeg) {   // second row of a keyed pair head
-        slot = ud.slot_of[row - 1];
-        second = 1;
-    } else if (slot & kSecondRowFlag) {
-        slot &= ~kSecondRowFlag;
-        second = 1;
-    }
-    const uint32_t r = ud.rep[slot] + second;
+    const uint32_t r = ud.row_rep[row];
     if (r != row) bd.seg_best[row] = bd.seg_best[r];   // representatives and their second rows are only read here
 }
 

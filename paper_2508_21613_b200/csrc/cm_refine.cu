@@ -23,9 +23,9 @@ __device__ __forceinline__ bool seg_open(const BatchDev &bd, const BoundDev &bo,
     constexpr bool native = std::is_same<T, long long>::value;
     const uint64_t la = bo.lbarg[row], key = bo.pick[row];
     if (la == ~0ull) return false;                                   // nothing fits in memory
-    if (bo.window && key == ~0ull) return false;                     // part of no strategy within reach
+    if (key == ~0ull) return false;                                  // part of no strategy within reach
     const float lb = lb_of(la), near = __fmul_ru(lb, 1.0f + kTieWindow);
-    const SearchWin w = bo.window ? bo.win[s.scen] : SearchWin{-1.0f, 0.0f, inf_bits<T>()};
+    const SearchWin w = bo.row_rep ? SearchWin{__uint_as_float((uint32_t)bo.row_lo[row]), 0.0f, ~bo.row_ub[row]} : bo.win[s.scen];
     s.ev = -1.0f;
     s.lim_bits = 0;
     if (phase == 1) {

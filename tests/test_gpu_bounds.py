@@ -118,3 +118,29 @@ def test_bounded_shortlist_against_the_oracle(gpu, oracle_factory):
                 assert [(p.cost, p.cost_ns) for p in got] == [(p.cost, p.cost_ns) for p in tr.shortlist]
         finally:
             gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_bounded_search_of_shared_segments_against_the_oracle(gpu, oracle_factory, mode):
+    """Segments that several failure sets have in common are searched once for all of them: each must come
+    out exact for the set that needs it most.  Five nodes, sets with equal losses per node among them."""
+    rng = np.random.default_rng(61)
+    L, n_dp, n_pp = 40, 2, 20
+    fwd = rng.uniform(2e6, 6e6, L).round()
+    profile = W.make_profile_ns(L, n_dp, n_pp, 48, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 8_000_000,
+                                list(range(0, L + 1, 2)), 80_000_000_000, 8, 300, 20)
+    sets = [[3], [5], [12], [20], [27], [38], [0, 1], [2, 7], [0, 9], [8, 30], [39, 15], [17, 31], [1, 6, 33], [4, 35, 2]]
+    opts = W.SearchOptions(2, 2, 17, 22, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15, mode)
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_set_sharing(ctx, True)
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets, opts)[0])
+        st = gpu.cm_last_stats(ctx)
+        assert st["plans_run"] < st["plans_simulated"], st
+        orc = oracle_factory(profile, opts)
+        for f, plan in zip(sets, best):
+            want = orc.search(f)[0]
+            assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (f, plan, want)
+    finally:
+        gpu.cm_destroy(ctx)
