@@ -310,29 +310,50 @@ uint64_t hbinom(const cm_ctx *c, int n, int k) {
 }
 
 // Strategies (Algorithm 1, get_parallel_strategy): non-decreasing stage counts that use
-// every survivor, dp ascending, tuples in lexicographic order.
-void enum_strategies(int n_surv, int dp_lo, int dp_hi, int lo, int hi,
-                     std::vector<std::vector<uint16_t>> &out) {
-    std::vector<uint16_t> cur;
-    struct Rec {
-        static void go(int dp, int pos, int remaining, int min_part, int hi, std::vector<uint16_t> &cur,
-                       std::vector<std::vector<uint16_t>> &out) {
-            if (pos == dp) {
-                if (remaining == 0) out.push_back(cur);
-                return;
-            }
-            const int left = dp - pos - 1;
-            for (int s = min_part; s <= hi; ++s) {
-                if (remaining - s < left * s) break;            // later parts are >= s
-                if (remaining - s > left * hi) continue;        // later parts are <= hi
-                cur.push_back((uint16_t)s);
-                go(dp, pos + 1, remaining - s, s, hi, cur, out);
-                cur.pop_back();
-            }
+// every survivor, dp ascending, tuples in lexicographic order.  `out`: a dp and its parts, one after another.
+struct StrategyList {
+    uint16_t cur[CM_MAX_PIPES];
+    std::vector<uint16_t> &out;
+    void go(int dp, int pos, int remaining, int min_part, int hi) {
+        const int left = dp - pos - 1;
+        if (left == 0) {
+            if (remaining < min_part || remaining > hi) return;
+            out.push_back((uint16_t)dp);
+            out.insert(out.end(), cur, cur + pos);
+            out.push_back((uint16_t)remaining);
+            return;
         }
-    };
-    for (int dp = dp_lo; dp <= dp_hi; ++dp) Rec::go(dp, 0, n_surv, lo, hi, cur, out);
+        for (int s = std::max(min_part, remaining - left * hi); s <= hi && remaining - s >= left * s; ++s) {   // later parts are s .. hi
+            cur[pos] = (uint16_t)s;
+            go(dp, pos + 1, remaining - s, s, hi);
+        }
+    }
+};
+void enum_strategies(int n_surv, int dp_lo, int dp_hi, int lo, int hi, std::vector<uint16_t> &out) {
+    StrategyList list{{}, out};
+    for (int dp = dp_lo; dp <= dp_hi; ++dp) list.go(dp, 0, n_surv, lo, hi);
 }
+
+// 64-bit keys (never all-ones) to 32-bit values, open addressing; as many slots as twice the keys.
+class FlatMap {
+    std::vector<uint64_t> key_;
+    std::vector<uint32_t> val_;
+    uint64_t mask_ = 0;
+public:
+    void reset(size_t n) {
+        size_t cap = 16;
+        while (cap < 2 * n) cap *= 2;
+        key_.assign(cap, ~0ull);
+        if (val_.size() < cap) val_.resize(cap);
+        mask_ = cap - 1;
+    }
+    uint32_t put(uint64_t key, uint32_t value) {   // the value that the key has: an earlier one, or now this
+        uint64_t h = key * 0x9e3779b97f4a7c15ull;
+        for (h = (h ^ (h >> 32)) & mask_; key_[h] != key; h = (h + 1) & mask_)
+            if (key_[h] == ~0ull) { key_[h] = key; val_[h] = value; break; }
+        return val_[h];
+    }
+};
 
 cm_status check_opts(cm_ctx *ctx, const cm_enum_opts *o) {
     if (!o) return fail(ctx, CM_EINVAL, "opts is NULL");
@@ -396,20 +417,21 @@ uint64_t walked(const TSeg &g) { return g.feas_first != kNoFeasList ? (uint64_t)
 // in their own right, grouped by (stages, micro-batches, role in the accounting of pairs).
 cm_status build_bound(cm_ctx *ctx, Batch &bt) {
     std::vector<BBucket> groups;
-    std::vector<uint32_t> idx;
+    std::vector<uint64_t> idx;   // deepest first, then by micro-batches and role; low half: the segment
     for (size_t t = 0; t < bt.tmpl.size(); ++t) {
         const Tmpl &tp = bt.tmpl[t];
         if (tp.n_scen == 0) continue;
         idx.clear();
-        for (uint32_t i = tp.tseg_first; i < tp.tseg_first + tp.n_tseg; ++i)
-            if (bt.tseg_canon[i] == i && bt.tseg[i].m >= 1 && walked(bt.tseg[i]) > 0) idx.push_back(i);
-        std::sort(idx.begin(), idx.end(), [&](uint32_t a, uint32_t b) {
-            const TSeg &x = bt.tseg[a], &y = bt.tseg[b];
-            return x.S != y.S ? x.S > y.S : x.m != y.m ? x.m < y.m : bt.role[a] != bt.role[b] ? bt.role[a] < bt.role[b] : a < b;
-        });
+        for (uint32_t i = tp.tseg_first; i < tp.tseg_first + tp.n_tseg; ++i) {
+            const TSeg &g = bt.tseg[i];
+            if (bt.tseg_canon[i] == i && g.m >= 1 && walked(g) > 0)
+                idx.push_back(((uint64_t)(CM_MAX_STAGES - g.S) << 50) | ((uint64_t)g.m << 34) | ((uint64_t)bt.role[i] << 32) | i);
+        }
+        std::sort(idx.begin(), idx.end());
         for (size_t i = 0, j; i < idx.size(); i = j) {
-            const TSeg &g = bt.tseg[idx[i]];
-            for (j = i; j < idx.size() && bt.tseg[idx[j]].S == g.S && bt.tseg[idx[j]].m == g.m && bt.role[idx[j]] == bt.role[idx[i]]; ++j) {}
+            const uint32_t first = (uint32_t)idx[i];
+            const TSeg &g = bt.tseg[first];
+            for (j = i + 1; j < idx.size() && idx[j] >> 32 == idx[i] >> 32; ++j) {}
             const uint64_t n_seg = (uint64_t)(j - i) * tp.n_scen;
             if (n_seg >= (1ull << 31)) return fail(ctx, CM_EOVERFLOW, "too many segments in one bucket");
             BBucket q{};
@@ -421,8 +443,8 @@ cm_status build_bound(cm_ctx *ctx, Batch &bt) {
             q.feas_first = g.feas_first;
             q.S = g.S;
             q.m = g.m;
-            q.role = bt.role[idx[i]];
-            bt.bucket_tseg.insert(bt.bucket_tseg.end(), idx.begin() + i, idx.begin() + j);
+            q.role = bt.role[first];
+            for (size_t k = i; k < j; ++k) bt.bucket_tseg.push_back((uint32_t)idx[k]);
             groups.push_back(q);
         }
     }
@@ -825,12 +847,13 @@ cm_status build_template(cm_ctx *ctx, Batch &bt, int n_surv, uint32_t *out) {
     Tmpl tp{};
     tp.strat_first = (uint32_t)bt.strat.size();
     tp.tseg_first = (uint32_t)bt.tseg.size();
-    std::vector<std::vector<uint16_t>> strategies;
+    std::vector<uint16_t> strategies;
     if (n_surv > 0 && pp_lo <= pp_hi) enum_strategies(n_surv, dp_lo, dp_hi, pp_lo, pp_hi, strategies);
     uint64_t split_first = 0, cand = 0;
-    for (const auto &tuple : strategies) {
+    for (size_t at = 0; at < strategies.size(); at += 1 + strategies[at]) {
         Strat st{};
-        const int dp = (int)tuple.size();
+        const int dp = strategies[at];
+        const uint16_t *tuple = strategies.data() + at + 1;
         st.dp = (uint16_t)dp;
         st.seg_first = (uint32_t)bt.tseg.size();
         st.split_first = split_first;
@@ -896,15 +919,15 @@ cm_status build_template(cm_ctx *ctx, Batch &bt, int n_surv, uint32_t *out) {
     tp.n_tseg = (uint32_t)bt.tseg.size() - tp.tseg_first;
     // pipelines that strategies of this survivor count have in common: searched once (BatchDev::tseg_canon)
     {
-        std::unordered_map<uint64_t, uint32_t> first_of;
-        first_of.reserve(2 * (size_t)tp.n_tseg);
+        FlatMap first_of;
+        first_of.reset(tp.n_tseg);
         uint64_t own = 0;
         bt.tseg_canon.resize(bt.tseg.size());
         for (uint32_t i = 0; i < tp.n_tseg; ++i) {
             const uint32_t t = tp.tseg_first + i;
             const TSeg &g = bt.tseg[t];
             const uint64_t key = ((uint64_t)g.S << 48) | ((uint64_t)g.m << 32) | ((uint64_t)g.n_sync << 16) | g.off;
-            const uint32_t c = ctx->dedup ? first_of.emplace(key, t).first->second : t;
+            const uint32_t c = ctx->dedup ? first_of.put(key, t) : t;
             bt.tseg_canon[t] = c;
             if (c != t) ++bt.n_dup;
             else own = sat_add(own, g.K ? g.K + 1 : 1);
@@ -1044,58 +1067,45 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
     bt.tmpl_of_nsurv.assign((size_t)N + 1, -1);
     bt.tmpl.push_back(Tmpl{});   // template 0: no strategies (scenarios without a dynamic-parallelism search)
     const int cross_words = (N + 63) / 64 + 1;
-    std::vector<char> dead(N);
+    std::vector<int> dead(N, -1);   // last scenario a device has failed in
     std::vector<int> alive;
-    std::unordered_map<std::string, uint32_t> seen;   // sharing: (node-crossing string, survivor count) -> first scenario
+    std::vector<uint32_t> seen;     // sharing: first scenario of every (survivor count, node crossings), by hash
+    if (ctx->share) {
+        size_t cap = 16;
+        while (cap < 2 * (size_t)B) cap *= 2;
+        seen.assign(cap, ~0u);
+    }
     bt.scen.reserve(B);
-    bt.cross.reserve((size_t)B * cross_words);
+    bt.cross.assign((size_t)B * cross_words, 0);
+    size_t cross_used = 0;
 
     for (int b = 0; b < B; ++b) {
         const int f0 = offsets[b], f1 = offsets[b + 1];
         if (f1 < f0) return fail(ctx, CM_EINVAL, "offsets must be non-decreasing");
         Scen sc{};
-        sc.failed_first = (uint32_t)bt.failed.size();
+        sc.failed_first = (uint32_t)(f0 - offsets[0]);
         sc.n_failed = (uint32_t)(f1 - f0);
         sc.policy_mask = policy_mask;
         bool bad = false;
         for (int f = f0; f < f1; ++f) {
             const uint32_t d = failed_ids[f];
-            if (d >= (uint32_t)N || dead[d]) { bad = true; break; }
-            dead[d] = 1;
-            bt.failed.push_back(d);
+            if (d >= (uint32_t)N || dead[d] == b) { bad = true; break; }
+            dead[d] = b;
         }
         if (bad) {
             const bool range = std::any_of(failed_ids + f0, failed_ids + f1, [&](uint32_t d) { return d >= (uint32_t)N; });
-            for (int f = f0; f < f1; ++f) if (failed_ids[f] < (uint32_t)N) dead[failed_ids[f]] = 0;
             return fail(ctx, CM_EINVAL, range ? "failed device id out of range" : "failed device ids must be distinct");
         }
         // survivors ascending; bit j: survivors j and j+1 sit on different nodes
-        sc.cross_first = (uint32_t)bt.cross.size();
-        bt.cross.resize(bt.cross.size() + cross_words, 0);
-        uint64_t *cw = bt.cross.data() + sc.cross_first;
+        sc.cross_first = (uint32_t)cross_used;
+        uint64_t *cw = bt.cross.data() + cross_used;
         const int n_surv = crossing_bits(hp, failed_ids + f0, f1 - f0, alive, cw);
-        for (int f = f0; f < f1; ++f) dead[failed_ids[f]] = 0;
         sc.rep = (uint32_t)b;
         if (policy_mask & (1u << CM_DYNPAR)) {
             // The dynamic-parallelism space of a scenario is a function of how many devices survive
             // and of where node boundaries fall among them (survivors are placed in consecutive
             // blocks; which device failed enters nowhere else).  With sharing on, scenarios that
             // agree in both are searched once and the others point at that result.
-            if (ctx->share) {
-                std::string key((const char *)cw, sizeof(uint64_t) * cross_words);
-                key.append((const char *)&n_surv, sizeof(n_surv));
-                auto it = seen.find(key);
-                if (it != seen.end()) {
-                    const Scen &r = bt.scen[it->second];
-                    sc.rep = it->second;
-                    sc.tmpl = r.tmpl;
-                    sc.cross_first = r.cross_first;
-                    bt.cross.resize(bt.cross.size() - cross_words);
-                    bt.scen.push_back(sc);
-                    continue;
-                }
-                seen.emplace(std::move(key), (uint32_t)b);
-            }
             int t = bt.tmpl_of_nsurv[n_surv];
             if (t < 0) {
                 uint32_t nt = 0;
@@ -1105,10 +1115,31 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
                 bt.tmpl_of_nsurv[n_surv] = t;
             }
             sc.tmpl = (uint32_t)t;
+            if (ctx->share) {
+                uint64_t h = (uint64_t)n_surv;
+                for (int k = 0; k < cross_words; ++k) h = (h ^ cw[k] ^ (h >> 29)) * 0x9e3779b97f4a7c15ull;
+                const size_t mask = seen.size() - 1;
+                size_t at = (h >> 20) & mask;
+                for (; seen[at] != ~0u; at = (at + 1) & mask) {
+                    const Scen &r = bt.scen[seen[at]];
+                    if (r.tmpl == sc.tmpl && !memcmp(bt.cross.data() + r.cross_first, cw, sizeof(uint64_t) * cross_words)) break;
+                }
+                if (seen[at] != ~0u) {
+                    sc.rep = seen[at];
+                    sc.cross_first = bt.scen[seen[at]].cross_first;
+                    std::fill(cw, cw + cross_words, 0ull);   // the next scenario's
+                    bt.scen.push_back(sc);
+                    continue;
+                }
+                seen[at] = (uint32_t)b;
+            }
         }
+        cross_used += cross_words;
         bt.tmpl[sc.tmpl].n_scen++;
         bt.scen.push_back(sc);
     }
+    bt.cross.resize(cross_used);
+    bt.failed.assign(failed_ids + offsets[0], failed_ids + offsets[B]);
     // scenarios grouped by template; result rows and rows per scenario
     uint32_t first = 0;
     for (Tmpl &tp : bt.tmpl) { tp.scen_first = first; first += tp.n_scen; tp.n_scen = 0; }
