@@ -149,6 +149,9 @@ __device__ __forceinline__ float stay_pairs(int i, int S, int m) {
 // This is a third of the kernel's instructions, so double arithmetic is kept to the sums that cancel or
 // grow (six operations a stage); what is left is done in floats rounded down, and the slowest single
 // forward and backward are compared by the upper halves of their bit patterns.
+// The stages are a loop of four at a time whose results move up the registers: all of them in a row are
+// tens of kilobytes of code per depth that every CTA runs through once, and the warps waited for
+// instructions most of the time (1024 sets of the 256-device job: 2023 -> 1997 us a call; one: 148 -> 146 us).
 template <typename T, int NB, bool UNI_X>
 __device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, const CutColumn<kBoundThreads> &w, int S, int m, bool check, float2 *cd) {
     const bool gpipe = s.sched == CM_SCHED_GPIPE;
@@ -159,38 +162,47 @@ __device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, 
     long long g_max = 0;
     int hi = s.L;
 #pragma unroll
-    for (int i = 4 * NB - 1; i >= 0; --i) {
-        v.set(i, kNoWalk);
-        if (i < S) {
-            const int lo = w.edge(i);
-            if (check && (hi <= lo || !stage_fits(s.PS[hi] - s.PS[lo], s.PA[hi] - s.PA[lo], i, S, m, s.cap, s.sched))) v.ok = false;
-            const double f = (double)(s.PF[hi] - s.PF[lo]), bk = (double)(s.PB[hi] - s.PB[lo]), wi = f + bk;
-            const long long g = s.PP[hi] - s.PP[lo];
-            g_max = g > g_max ? g : g_max;
-            fmax = max(fmax, __double2hiint(f));
-            bmax = max(bmax, __double2hiint(bk));
-            U += wi;
-            if (!gpipe) {
-                const int n = stays(i, S, m);
-                const float q = stay_pairs(i, S, m);
-                float xm = xm_all, d = kNoWalk;
-                if (!UNI_X) xm = __double2float_rd((double)(s.XT[0][hi - 1] < s.XT[1][hi - 1] ? s.XT[0][hi - 1] : s.XT[1][hi - 1]));
-                const double dw = wi - w_n;
-                if (i < S - 1) {   // stage i+1 is complete now that its lower neighbour is known
-                    if (q_n > 0.0f) d = __fmaf_rd(q_n, __double2float_rd(dw), base_n);
-                    const float up = c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n);
-                    const float best = max3(base_n, up, __fmaf_rd(2.0f * q_n, xm, d));
-                    if (i + 1 < 4 * NB) v.set(i + 1 < 4 * NB ? i + 1 : 0, best);
+    for (int j = 0; j < 2 * NB; ++j) v.b[j] = make_float2(kNoWalk, kNoWalk);
+#pragma unroll 1
+    for (int k = (S - 1) >> 2; k >= 0; --k) {   // four stages a turn, topmost first
+#pragma unroll
+        for (int r = 3; r >= 0; --r) {
+            const int i = 4 * k + r;
+            if (i < S) {
+                const int lo = w.edge(i);
+                if (check && (hi <= lo || !stage_fits(s.PS[hi] - s.PS[lo], s.PA[hi] - s.PA[lo], i, S, m, s.cap, s.sched))) v.ok = false;
+                const double f = (double)(s.PF[hi] - s.PF[lo]), bk = (double)(s.PB[hi] - s.PB[lo]), wi = f + bk;
+                const long long g = s.PP[hi] - s.PP[lo];
+                g_max = g > g_max ? g : g_max;
+                fmax = max(fmax, __double2hiint(f));
+                bmax = max(bmax, __double2hiint(bk));
+                U += wi;
+                if (!gpipe) {
+                    const int n = stays(i, S, m);
+                    const float q = stay_pairs(i, S, m);
+                    float xm = xm_all, d = kNoWalk;
+                    if (!UNI_X) xm = __double2float_rd((double)(s.XT[0][hi - 1] < s.XT[1][hi - 1] ? s.XT[0][hi - 1] : s.XT[1][hi - 1]));
+                    const double dw = wi - w_n;
+                    if (i < S - 1) {   // stage i+1 is complete now that its lower neighbour is known
+                        if (q_n > 0.0f) d = __fmaf_rd(q_n, __double2float_rd(dw), base_n);
+                        const float up = c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n);
+                        v.set(r == 3 ? 0 : r + 1, max3(base_n, up, __fmaf_rd(2.0f * q_n, xm, d)));   // (r == 3: not shifted yet)
+                    }
+                    base_n = n >= 0 ? __double2float_rd(__fma_rd((double)n, wi, U)) : kNoWalk;
+                    c_n = q > 0.0f && i < S - 1 ? __fmaf_rd(q, __double2float_rd(-dw), base_n) : kNoWalk;
+                    cd[i * kBoundThreads] = make_float2(c_n, d);
+                    w_n = wi; q_n = q; xq_n = __fmul_rd(2.0f * q, xm);
                 }
-                base_n = n >= 0 ? __double2float_rd(__fma_rd((double)n, wi, U)) : kNoWalk;
-                c_n = q > 0.0f && i < S - 1 ? __fmaf_rd(q, __double2float_rd(-dw), base_n) : kNoWalk;
-                cd[i * kBoundThreads] = make_float2(c_n, d);
-                w_n = wi; q_n = q; xq_n = __fmul_rd(2.0f * q, xm);
-                if (i == 0) v.set(0, fmaxf(base_n, c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n)));
+                hi = lo;
             }
-            hi = lo;
+            if (r == 3) {   // the stages so far move up by four
+#pragma unroll
+                for (int j = 2 * NB - 1; j > 1; --j) v.b[j] = v.b[j - 2];
+                v.b[0] = v.b[1] = make_float2(kNoWalk, kNoWalk);
+            }
         }
     }
+    if (!gpipe) v.set(0, fmaxf(base_n, c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n)));
     const double f1 = __hiloint2double(fmax, 0), b1 = __hiloint2double(bmax, 0);
     v.u0 = __double2float_rd(U);
     v.once = __double2float_rd((double)(m - 1) * (gpipe ? f1 + b1 : tmax(f1, b1)));
@@ -206,6 +218,7 @@ __device__ __forceinline__ void fill_transfers(const BoundSmem &sm, const SProf<
         const uint64_t tier = sm.segs[s].tier;
         float X = 0.0f;
         int n = 0;
+#pragma unroll 4
         for (int i = 4 * NB - 1; i >= 0; --i) {
             if (i < S - 1) {
                 const bool far = (tier >> i) & 1ull;
