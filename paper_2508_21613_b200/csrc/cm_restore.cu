@@ -131,42 +131,42 @@ __device__ __forceinline__ long long warp_min_nonneg(long long x) {
     return (long long)(((unsigned long long)mhi << 32) | mlo);
 }
 
-// Returns the total of the matching (same value in every lane), -1 if the iteration broke
-// down (cannot happen for n >= 1; guards the loops).  On return w.match[j] = row of column j.
-template <int NC>
-__device__ long long warp_match(MatchWork &w, const long long *PW, int n, int lane) {
-    const long long INF = LLONG_MAX / 4;
-    // ---- fold equal rows into classes, numbered by their first row
-    for (int i = lane; i < n; i += 32) {
-        int first = i;
-        for (int k = 0; k < i; ++k)
-            if (w.olo[k] == w.olo[i] && w.ohi[k] == w.ohi[i]) { first = k; break; }
-        w.tcol[i] = (short)first;                 // scratch: first row of i's class
-        w.cap[i] = 0; w.cnt[i] = 0; w.head[i] = -1; w.match[i] = -1; w.next_col[i] = -1;
-    }
+// Fold equal rows into classes, numbered by their first row; their number.  32 rows at a time: those whose
+// range is among the classes so far, then the first of every new range.
+__device__ __forceinline__ int fold_rows(MatchWork &w, int n, int lane) {
+    for (int i = lane; i < n; i += 32) { w.cap[i] = 0; w.cnt[i] = 0; w.head[i] = -1; w.match[i] = -1; w.next_col[i] = -1; }
     __syncwarp();
     int R = 0;
     for (int base = 0; base < n; base += 32) {
         const int i = base + lane;
-        const bool is_first = i < n && w.tcol[i] == i;
-        const uint32_t mask = __ballot_sync(0xffffffffu, is_first);
-        if (is_first) {
-            const int r = R + __popc(mask & ((1u << lane) - 1u));
-            w.row_class[i] = (short)r;
-            w.clo[r] = w.olo[i];
-            w.chi[r] = w.ohi[i];
+        const int lo = i < n ? (int)w.olo[i] : -1 - lane, hi = i < n ? (int)w.ohi[i] : 0;
+        int r = -1;
+        for (int k = 0; k < R; ++k)
+            if (w.clo[k] == lo && w.chi[k] == hi) r = k;
+        const uint32_t mates = __match_any_sync(0xffffffffu, (lo << 8) | hi);
+        const int lead = __ffs((int)mates) - 1;
+        const uint32_t fresh = __ballot_sync(0xffffffffu, i < n && r < 0 && lane == lead);
+        if ((fresh >> lane) & 1u) {
+            r = R + __popc(fresh & ((1u << lane) - 1u));
+            w.clo[r] = (uint8_t)lo;
+            w.chi[r] = (uint8_t)hi;
         }
-        R += __popc(mask);
+        r = __shfl_sync(0xffffffffu, r, lead);
+        if (i < n) {
+            w.row_class[i] = (short)r;
+            if (lane == lead) w.cap[r] = (short)(w.cap[r] + __popc(mates));
+        }
+        R += __popc(fresh);
+        __syncwarp();
     }
-    __syncwarp();
-    for (int i = lane; i < n; i += 32) {
-        const int r = w.row_class[w.tcol[i]];
-        if (w.tcol[i] != i) w.row_class[i] = (short)r;
-        atomicAdd(&w.cnt[r], 1);                  // counted in cnt, moved to cap below
-    }
-    __syncwarp();
-    for (int r = lane; r < R; r += 32) { w.cap[r] = (short)w.cnt[r]; w.cnt[r] = 0; }
-    __syncwarp();
+    return R;
+}
+
+// Returns the total of the matching (same value in every lane), -1 if the iteration broke
+// down (cannot happen for n >= 1; guards the loops).  On return w.match[j] = row of column j.
+template <int NC>
+__device__ long long warp_match(MatchWork &w, const long long *PW, int n, int R, int lane) {
+    const long long INF = LLONG_MAX / 4;
     // ---- start: v[j] = cheapest class of column j (u = 0), then every column claims a class that
     // attains it and still has room, lowest class first.  Most positions find a device that
     // already holds most of their layers, so few columns are left for the augmenting phase.
@@ -192,11 +192,12 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int la
     __syncwarp();
     // ---- augmenting phase: class potentials and slacks in registers of the owning lane
     long long u[NC], slack[NC], ubase[NC];
-    int clo[NC], chi[NC];
+    int clo[NC], chi[NC], way[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         const int r = c * 32 + lane;
         u[c] = 0;
+        way[c] = 0;
         clo[c] = r < R ? (int)w.clo[r] : 0;
         chi[c] = r < R ? (int)w.chi[r] : 0;
     }
@@ -212,6 +213,7 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int la
         __syncwarp();
         for (int iter = 0; iter <= 2 * (n + R) + 4 && found < 0; ++iter) {
             // 1. scan the tree columns that have not been scanned yet
+#pragma unroll 4
             for (; scanned < nt; ++scanned) {
                 const int j = w.tcol[scanned];
                 const int x = w.nlo[j], y = w.nhi[j];
@@ -222,7 +224,7 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int la
                     const int r = c * 32 + lane;
                     if (r >= R || ((tree >> c) & 1u)) continue;
                     const long long red = range_cost(PW, need, clo[c], chi[c], x, y) - u[c] - vj;
-                    if (red < slack[c]) { slack[c] = red; w.way[r] = (short)j; }
+                    if (red < slack[c]) { slack[c] = red; way[c] = j; }
                 }
             }
             // 2. classes at zero slack join the tree; one with room ends the search, a full one
@@ -233,7 +235,7 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int la
                 const int r = c * 32 + lane;
                 const bool tight = r < R && !((tree >> c) & 1u) && slack[c] == 0;
                 uint32_t mask = __ballot_sync(0xffffffffu, tight);
-                if (tight) { tree |= 1u << c; ubase[c] = D; }
+                if (tight) { tree |= 1u << c; ubase[c] = D; w.way[r] = (short)way[c]; }
                 any_tight = any_tight || mask != 0;
                 while (mask && found < 0) {
                     const int rr = c * 32 + (__ffs((int)mask) - 1);
@@ -324,11 +326,14 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int la
 }
 
 __device__ __forceinline__ long long warp_match_any(MatchWork &w, const long long *PW, int n, int lane) {
-    // the class count is known only inside; NC is chosen for the row count, which bounds it
-    if (n <= 32) return warp_match<1>(w, PW, n, lane);
-    if (n <= 64) return warp_match<2>(w, PW, n, lane);
-    if (n <= 128) return warp_match<4>(w, PW, n, lane);
-    return warp_match<8>(w, PW, n, lane);
+    // The classes, not the rows, decide how many of them a lane owns: the survivors of a job with 32 stages
+    // make 32 classes, however many pipelines it has (64 failure sets of the 256-device job, eight plans
+    // each: 586 us with eight slots per lane for 250 rows, 346 us with one and the rows folded 32 at a time).
+    const int R = fold_rows(w, n, lane);
+    if (R <= 32) return warp_match<1>(w, PW, n, R, lane);
+    if (R <= 64) return warp_match<2>(w, PW, n, R, lane);
+    if (R <= 128) return warp_match<4>(w, PW, n, R, lane);
+    return warp_match<8>(w, PW, n, R, lane);
 }
 
 __device__ __forceinline__ void stage_state_bytes(long long *PW, const DevProfile *p) {
