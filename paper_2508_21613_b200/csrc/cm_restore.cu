@@ -456,90 +456,94 @@ cudaError_t launch_range_matching(const Tables &t, int n_problems, const int32_t
 }
 
 // ----------------------------------------------------------------------------------
-// Asymmetric synchronisation (Section "Restorer", Asymmetric Communication).  One warp per
-// shortlisted plan: lane q evaluates the bare time of pipeline q (one participant: no
-// synchronisation term) and writes the stage of every layer; the layer graph (edge = some
-// pipeline keeps both layers on one device) is coloured greedily in layer order, lanes
-// sharing the earlier layers and OR-reducing the colours their neighbours took; a round
-// lasts as long as its largest all-reduce, rounds add up in colour order.
+// Asymmetric synchronisation (Section "Restorer", Asymmetric Communication).  A CTA per shortlisted
+// plan, a warp per pipeline: the bare time of the pipeline (one participant: no synchronisation
+// term), a chain of 2(S+m) dependent slots that bounds the kernel, and the stage of every layer; the
+// last warp, which has the fewest pipelines, colours the layer graph (edge = some pipeline keeps both
+// layers on one device) greedily in layer order.  Stages are runs of layers, so the earlier neighbours of
+// a layer are one run too, from the lowest start of its stages to the layer before it; the lanes
+// OR-reduce the colours taken there.  A round lasts as long as its largest all-reduce, rounds add up in
+// colour order.  512 plans of the 256-device job (eight pipelines of 32 stages, 128 micro-batches):
+// XXXX us; with one warp for all pipelines of a plan, and every pair of layers looked up in every
+// pipeline, 196 us.
 // ----------------------------------------------------------------------------------
-struct RoundsWork {
-    uint8_t stage_of[kMaxP][kMaxL];
-    uint8_t cuts[kMaxP][kMaxS + 4];
-    uint8_t colour[kMaxL];
-};
+constexpr int kRoundsWarps = 8;
 
 template <typename T>
-__global__ void __launch_bounds__(kMatchWarps * 32) cm_plan_rounds_kernel(Tables tb, BatchDev bd, ObjDev od) {
+__global__ void __launch_bounds__(kRoundsWarps * 32) cm_plan_rounds_kernel(Tables tb, BatchDev bd, ObjDev od) {
     __shared__ SProf<T> sp;
-    __shared__ RoundsWork work[kMatchWarps];
-    stage_profile(sp, tb);
-    __syncthreads();
+    __shared__ uint8_t cuts[kMaxP][kMaxS + 4], stage_of[kMaxP][kMaxL], colour[kMaxL], low[kMaxL];
+    __shared__ T pipe_time[kMaxP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t slot = (size_t)blockIdx.x * kMatchWarps + warp;
-    if (slot >= (size_t)bd.B * od.topk) return;
-    if (lane < 2) { od.short_step[slot * 2 + lane] = inf_bits<T>(); od.short_rounds[slot * 2 + lane] = 0; }
+    const size_t slot = blockIdx.x;
+    if (threadIdx.x < 2) { od.short_step[slot * 2 + lane] = inf_bits<T>(); od.short_rounds[slot * 2 + lane] = 0; }
     const Winner &w = od.short_win[slot];
-    if (w.cost_bits >= inf_bits<T>() || w.dp == 0) return;
-    RoundsWork &rw = work[warp];
-    const int L = sp.L, dp = (int)w.dp;
+    if (w.cost_bits >= inf_bits<T>() || w.dp == 0) return;   // uniform
+    stage_profile(sp, tb);
+    const int dp = (int)w.dp;
     bool ok = true;
-    if (lane < dp) {
-        uint8_t cuts[kMaxS + 1];
-        ok = pipeline_cuts(tb, bd, od, slot, w, lane, cuts);
-        if (ok) {
-            const int S = bd.tseg[w.seg[lane]].S;
-            for (int i = 0; i <= S; ++i) rw.cuts[lane][i] = cuts[i];
-            for (int i = 0; i < S; ++i)
-                for (int l = cuts[i]; l < cuts[i + 1]; ++l) rw.stage_of[lane][l] = (uint8_t)i;
-        }
-    }
-    ok = __all_sync(0xffffffffu, ok);
-    if (!ok) return;
-    __syncwarp();
-    T t_pipe = (T)0;
-    for (int q = 0; q < dp; ++q) {            // one pipeline after the other, each over the whole warp
-        const SegView g = seg_view(bd, w.scen, w.seg[q]);
-        t_pipe = tmax(t_pipe, warp_pipe_time<T>(sp, rw.cuts[q], g.S, g.m, g.tier, lane));
-    }
-    int rounds = 0;
-    for (int l = 0; l < L; ++l) {
-        uint32_t used[4] = {0u, 0u, 0u, 0u};
-        for (int k = lane; k < l; k += 32) {
-            bool adjacent = false;
-            for (int q = 0; q < dp; ++q) adjacent = adjacent || rw.stage_of[q][l] == rw.stage_of[q][k];
-            if (adjacent) { const int c = rw.colour[k]; used[c >> 5] |= 1u << (c & 31); }
-        }
-        int c = -1;
-#pragma unroll
-        for (int word = 0; word < 4; ++word) {
-            const uint32_t all = __reduce_or_sync(0xffffffffu, used[word]);
-            if (c < 0 && all != 0xffffffffu) c = word * 32 + __ffs((int)~all) - 1;
-        }
-        if (lane == 0) rw.colour[l] = (uint8_t)c;
-        rounds = c + 1 > rounds ? c + 1 : rounds;
+    for (int q = warp; q < dp; q += kRoundsWarps) {
+        bool mine = true;
+        if (lane == 0) mine = pipeline_cuts(tb, bd, od, slot, w, q, cuts[q]);
+        mine = __all_sync(0xffffffffu, mine);
+        ok = ok && mine;
         __syncwarp();
+        if (mine)
+            for (int i = lane; i < (int)bd.tseg[w.seg[q]].S; i += 32)
+                for (int l = cuts[q][i]; l < cuts[q][i + 1]; ++l) stage_of[q][l] = (uint8_t)i;
+    }
+    if (!__syncthreads_and(ok)) return;
+    const int L = sp.L;
+    for (int q = warp; q < dp; q += kRoundsWarps) {
+        const SegView g = seg_view(bd, w.scen, w.seg[q]);
+        const T t = warp_pipe_time<T>(sp, cuts[q], g.S, g.m, g.tier, lane);
+        if (lane == 0) pipe_time[q] = t;
     }
     T t_sync = (T)0;
-    for (int c = 0; c < rounds; ++c) {
-        T longest = (T)0;
-        for (int l = lane; l < L; l += 32)
-            if (rw.colour[l] == c) longest = tmax(longest, Num<T>::sync(sp.PP[l + 1] - sp.PP[l], dp, sp.bw_sync, sp.intval));
-        for (int o = 16; o > 0; o >>= 1) {
-            const uint64_t other = __shfl_xor_sync(0xffffffffu, Num<T>::bits(longest), o);
-            longest = tmax(longest, Num<T>::from_bits(other));
+    int rounds = 0, domains = 0;
+    if (warp == kRoundsWarps - 1) {
+        for (int l = lane; l < L; l += 32) {
+            int first = l;
+            for (int q = 0; q < dp; ++q) first = min(first, (int)cuts[q][stage_of[q][l]]);
+            low[l] = (uint8_t)first;
         }
-        t_sync = t_sync + longest;
+        __syncwarp();
+        for (int l = 0; l < L; ++l) {
+            uint32_t used[4] = {0u, 0u, 0u, 0u};
+            for (int k = (int)low[l] + lane; k < l; k += 32) { const int c = colour[k]; used[c >> 5] |= 1u << (c & 31); }
+            int c = -1;
+#pragma unroll
+            for (int word = 0; word < 4; ++word) {
+                if (c >= 0) break;   // uniform
+                const uint32_t all = __reduce_or_sync(0xffffffffu, used[word]);
+                if (all != 0xffffffffu) c = word * 32 + __ffs((int)~all) - 1;
+            }
+            if (lane == 0) colour[l] = (uint8_t)c;
+            rounds = c + 1 > rounds ? c + 1 : rounds;
+            __syncwarp();
+        }
+        for (int c = 0; c < rounds; ++c) {
+            T longest = (T)0;
+            for (int l = lane; l < L; l += 32)
+                if (colour[l] == c) longest = tmax(longest, Num<T>::sync(sp.PP[l + 1] - sp.PP[l], dp, sp.bw_sync, sp.intval));
+            for (int o = 16; o > 0; o >>= 1) {
+                const uint64_t other = __shfl_xor_sync(0xffffffffu, Num<T>::bits(longest), o);
+                longest = tmax(longest, Num<T>::from_bits(other));
+            }
+            t_sync = t_sync + longest;
+        }
+        for (int base = 0; base < L; base += 32) {
+            const int l = base + lane;
+            bool fresh = l == 0;
+            if (l > 0 && l < L)
+                for (int q = 0; q < dp; ++q) fresh = fresh || stage_of[q][l] != stage_of[q][l - 1];
+            domains += __popc(__ballot_sync(0xffffffffu, fresh && l < L));
+        }
     }
-    int domains = 0;
-    for (int base = 0; base < L; base += 32) {
-        const int l = base + lane;
-        bool fresh = l == 0;
-        if (l > 0 && l < L)
-            for (int q = 0; q < dp; ++q) fresh = fresh || rw.stage_of[q][l] != rw.stage_of[q][l - 1];
-        domains += __popc(__ballot_sync(0xffffffffu, fresh && l < L));
-    }
-    if (lane == 0) {
+    __syncthreads();
+    if (threadIdx.x == (kRoundsWarps - 1) * 32) {
+        T t_pipe = (T)0;
+        for (int q = 0; q < dp; ++q) t_pipe = tmax(t_pipe, pipe_time[q]);
         od.short_step[slot * 2] = Num<T>::bits(t_pipe + t_sync);
         od.short_step[slot * 2 + 1] = Num<T>::bits(t_sync);
         od.short_rounds[slot * 2] = rounds;
@@ -550,9 +554,9 @@ __global__ void __launch_bounds__(kMatchWarps * 32) cm_plan_rounds_kernel(Tables
 cudaError_t launch_plan_rounds(const Tables &t, const BatchDev &b, const ObjDev &o, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
     const size_t slots = (size_t)b.B * o.topk;
-    const unsigned grid = (unsigned)((slots + kMatchWarps - 1) / kMatchWarps);
-    if (native_i64(b)) cm_plan_rounds_kernel<long long><<<grid, kMatchWarps * 32, 0, st>>>(t, b, o);
-    else cm_plan_rounds_kernel<double><<<grid, kMatchWarps * 32, 0, st>>>(t, b, o);
+    if (slots >= (1ull << 31)) return cudaErrorInvalidConfiguration;
+    if (native_i64(b)) cm_plan_rounds_kernel<long long><<<(unsigned)slots, kRoundsWarps * 32, 0, st>>>(t, b, o);
+    else cm_plan_rounds_kernel<double><<<(unsigned)slots, kRoundsWarps * 32, 0, st>>>(t, b, o);
     return cudaGetLastError();
 }
 

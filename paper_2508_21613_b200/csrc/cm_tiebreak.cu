@@ -101,7 +101,7 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st)
     // 131 us with 64 threads, above 400 us with 256; 290 us for the plan-per-lane kernel this replaced.
     // 1024 sets of the 256-device job: 147 us, where a plan-per-lane kernel per depth took 1300 us in all.
     const bool wide = nx <= 148 * 2;
-    const unsigned threads = wide ? 256 : 64;
+    const unsigned threads = wide ? 256 : 32;
     const int n_eval = wide ? 256 / 32 : 1;
     const uint64_t tiles = ((uint64_t)b.max_tiles_per_seg * kTile + threads - 1) / threads;
     uint64_t y = (148 * 4 + nx - 1) / nx;
@@ -109,10 +109,10 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st)
     const dim3 grid((unsigned)nx, (unsigned)std::max<uint64_t>(y, 1), 1);
     if (native_i64(b)) {
         if (wide) cm_tiebreak_kernel<long long, 256><<<grid, threads, 0, st>>>(t, b, n_eval);
-        else cm_tiebreak_kernel<long long, 64><<<grid, threads, 0, st>>>(t, b, n_eval);
+        else cm_tiebreak_kernel<long long, 32><<<grid, threads, 0, st>>>(t, b, n_eval);
     } else {
         if (wide) cm_tiebreak_kernel<double, 256><<<grid, threads, 0, st>>>(t, b, n_eval);
-        else cm_tiebreak_kernel<double, 64><<<grid, threads, 0, st>>>(t, b, n_eval);
+        else cm_tiebreak_kernel<double, 32><<<grid, threads, 0, st>>>(t, b, n_eval);
     }
     return cudaGetLastError();
 }
