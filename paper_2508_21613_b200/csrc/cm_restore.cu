@@ -112,7 +112,7 @@ struct MatchWork {
     short way[kMaxMatch];                         // class: tree column that gave its least slack
     short next_col[kMaxMatch];                    // column: next column served by the same class
     short tcol[kMaxMatch];                        // tree columns in the order they joined
-    short row_class[kMaxMatch];                   // row -> class
+    short first_row[kMaxMatch], next_row[kMaxMatch];   // class: its first row; row: the next one of its class (-1 = none)
     short match[kMaxMatch];                       // column -> class while solving; column -> row on return
     uint8_t olo[kMaxMatch], ohi[kMaxMatch], nlo[kMaxMatch], nhi[kMaxMatch];   // inputs
     uint8_t clo[kMaxMatch], chi[kMaxMatch];       // class ranges
@@ -151,10 +151,15 @@ __device__ __forceinline__ int fold_rows(MatchWork &w, int n, int lane) {
             w.clo[r] = (uint8_t)lo;
             w.chi[r] = (uint8_t)hi;
         }
-        r = __shfl_sync(0xffffffffu, r, lead);
-        if (i < n) {
-            w.row_class[i] = (short)r;
-            if (lane == lead) w.cap[r] = (short)(w.cap[r] + __popc(mates));
+        if (i < n) {   // (way: the class's last row so far)
+            const uint32_t above = mates & ~((2u << lane) - 1u);
+            w.next_row[i] = above ? (short)(base + __ffs((int)above) - 1) : (short)-1;
+            if (lane == lead) {
+                if ((fresh >> lane) & 1u) w.first_row[r] = (short)i;
+                else w.next_row[w.way[r]] = (short)i;
+                w.way[r] = (short)(base + 31 - __clz((int)mates));
+                w.cap[r] = (short)(w.cap[r] + __popc(mates));
+            }
         }
         R += __popc(fresh);
         __syncwarp();
@@ -170,23 +175,54 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int R,
     // ---- start: v[j] = cheapest class of column j (u = 0), then every column claims a class that
     // attains it and still has room, lowest class first.  Most positions find a device that
     // already holds most of their layers, so few columns are left for the augmenting phase.
-    for (int j = lane; j < n; j += 32) {
-        const int x = w.nlo[j], y = w.nhi[j];
+    // Claims are dealt out in turns, the lanes that want the same class served in order: lanes that each
+    // search on with atomics of their own drift apart and are run one after another.
+    for (int base = 0; base < n; base += 32) {
+        const int j = base + lane;
+        const int x = j < n ? (int)w.nlo[j] : 0, y = j < n ? (int)w.nhi[j] : 0;
         const long long need = y > x ? PW[y] - PW[x] : 0ll;
         long long best = INF;
-        for (int r = 0; r < R; ++r) {
-            const long long c = range_cost(PW, need, w.clo[r], w.chi[r], x, y);
-            best = c < best ? c : best;
-        }
-        w.v[j] = best;
-        for (int r = 0; r < R; ++r) {
-            if (range_cost(PW, need, w.clo[r], w.chi[r], x, y) != best) continue;
-            if (atomicAdd(&w.cnt[r], 1) < (int)w.cap[r]) {
-                w.match[j] = (short)r;
-                w.next_col[j] = (short)atomicExch(&w.head[r], j);
-                break;
+        uint32_t attain[NC];                      // classes that attain it
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            attain[c] = 0;
+#pragma unroll 4
+            for (int k = 0; k < 32; ++k) {
+                const int r = c * 32 + k;
+                if (r >= R) break;                // uniform
+                const long long cost = range_cost(PW, need, w.clo[r], w.chi[r], x, y);
+                if (cost < best) {
+                    best = cost;
+#pragma unroll
+                    for (int e = 0; e < c; ++e) attain[e] = 0;
+                    attain[c] = 1u << k;
+                } else if (cost == best) attain[c] |= 1u << k;
             }
-            atomicSub(&w.cnt[r], 1);
+        }
+        if (j < n) w.v[j] = best;
+        bool open = j < n;
+        for (int turn = 0; turn <= R; ++turn) {
+            int r = -1;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (open && r < 0 && attain[c]) r = c * 32 + __ffs((int)attain[c]) - 1;
+            if (!__any_sync(0xffffffffu, r >= 0)) break;
+            const uint32_t mates = __match_any_sync(0xffffffffu, r);
+            const uint32_t before = mates & ((1u << lane) - 1u);
+            const int room = r >= 0 ? (int)w.cap[r] - w.cnt[r] : 0, served = min(room, __popc(mates));
+            const bool mine = r >= 0 && __popc(before) < room;
+            const uint32_t taken = __ballot_sync(0xffffffffu, mine) & before;
+            if (mine) {                           // the class's list: last of the turn first
+                w.match[j] = (short)r;
+                w.next_col[j] = taken ? (short)(base + 31 - __clz((int)taken)) : (short)w.head[r];
+                open = false;
+            }
+            __syncwarp();
+            if (mine && __popc(before) == served - 1) { w.head[r] = j; w.cnt[r] += served; }
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (open && r >= c * 32 && r < c * 32 + 32) attain[c] &= ~(1u << (r & 31));
         }
     }
     __syncwarp();
@@ -202,8 +238,11 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int R,
         chi[c] = r < R ? (int)w.chi[r] : 0;
     }
     bool broken = false;
+    uint32_t left = 0;                              // unserved columns of the 32 around j0 (a flip serves j0 alone)
     for (int j0 = 0; j0 < n && !broken; ++j0) {
-        if (w.match[j0] >= 0) continue;             // uniform: served since the start or an earlier flip
+        if ((j0 & 31) == 0) left = __ballot_sync(0xffffffffu, j0 + lane < n && w.match[j0 + lane] < 0);
+        if (left == 0) { j0 |= 31; continue; }
+        if (!((left >> (j0 & 31)) & 1u)) continue;
         uint32_t tree = 0;                          // bit c: class c*32+lane belongs to the tree
         long long D = 0;                            // potential shift so far
         int nt = 1, scanned = 0, found = -1;
@@ -312,11 +351,9 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int R,
     // hand the rows of every class to the columns it serves (rows ascending, list order)
     for (int r = lane; r < R; r += 32) {
         int j = w.head[r];
-        for (int i = 0; i < n && j >= 0; ++i) {
-            if (w.row_class[i] != r) continue;
-            const int nx = w.next_col[j];
+        for (int i = w.first_row[r]; i >= 0 && j >= 0; i = w.next_row[i]) {
             w.tcol[j] = (short)i;                 // scratch: row of column j
-            j = nx;
+            j = w.next_col[j];
         }
     }
     __syncwarp();
@@ -328,7 +365,8 @@ __device__ long long warp_match(MatchWork &w, const long long *PW, int n, int R,
 __device__ __forceinline__ long long warp_match_any(MatchWork &w, const long long *PW, int n, int lane) {
     // The classes, not the rows, decide how many of them a lane owns: the survivors of a job with 32 stages
     // make 32 classes, however many pipelines it has (64 failure sets of the 256-device job, eight plans
-    // each: 586 us with eight slots per lane for 250 rows, 346 us with one and the rows folded 32 at a time).
+    // each: 586 us with eight slots per lane for 250 rows and a start
+    // of diverging atomics, 200 us now).
     const int R = fold_rows(w, n, lane);
     if (R <= 32) return warp_match<1>(w, PW, n, R, lane);
     if (R <= 64) return warp_match<2>(w, PW, n, R, lane);
@@ -464,7 +502,7 @@ cudaError_t launch_range_matching(const Tables &t, int n_problems, const int32_t
 // a layer are one run too, from the lowest start of its stages to the layer before it; the lanes
 // OR-reduce the colours taken there.  A round lasts as long as its largest all-reduce, rounds add up in
 // colour order.  512 plans of the 256-device job (eight pipelines of 32 stages, 128 micro-batches):
-// XXXX us; with one warp for all pipelines of a plan, and every pair of layers looked up in every
+// 94 us; with one warp for all pipelines of a plan, and every pair of layers looked up in every
 // pipeline, 196 us.
 // ----------------------------------------------------------------------------------
 constexpr int kRoundsWarps = 8;
@@ -510,7 +548,11 @@ __global__ void __launch_bounds__(kRoundsWarps * 32) cm_plan_rounds_kernel(Table
         __syncwarp();
         for (int l = 0; l < L; ++l) {
             uint32_t used[4] = {0u, 0u, 0u, 0u};
-            for (int k = (int)low[l] + lane; k < l; k += 32) { const int c = colour[k]; used[c >> 5] |= 1u << (c & 31); }
+            for (int k = (int)low[l] + lane; k < l; k += 32) {
+                const int taken = colour[k];
+#pragma unroll
+                for (int word = 0; word < 4; ++word) used[word] |= taken >> 5 == word ? 1u << (taken & 31) : 0u;   // (registers)
+            }
             int c = -1;
 #pragma unroll
             for (int word = 0; word < 4; ++word) {

@@ -96,10 +96,11 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st)
     const uint64_t nx = (uint64_t)b.B * b.dp_max;
     if (nx >= (1ull << 31)) return cudaErrorInvalidConfiguration;
     // A failure handled on its own: a wide CTA per pipeline, whose warps try candidates side by side.  A
-    // batch: narrow CTAs, of which an SM holds nine instead of two; the first tile nearly always holds
-    // the answer, and its first candidate nearly always is it.  2576 failure sets of the 32-device job:
-    // 131 us with 64 threads, above 400 us with 256; 290 us for the plan-per-lane kernel this replaced.
-    // 1024 sets of the 256-device job: 147 us, where a plan-per-lane kernel per depth took 1300 us in all.
+    // batch: a warp per pipeline; the first 32 compositions nearly always hold the answer, and the first
+    // that its bound leaves nearly always is it.  2576 failure sets of the 32-device job: 95 us with a
+    // warp, 170 us with two, above 400 us with eight; 290 us for the plan-per-lane kernel this replaced.
+    // 1024 sets of the 256-device job: 133 us with a warp, 172 us with two, where a plan-per-lane kernel
+    // per depth took 1300 us in all.
     const bool wide = nx <= 148 * 2;
     const unsigned threads = wide ? 256 : 32;
     const int n_eval = wide ? 256 / 32 : 1;
