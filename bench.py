@@ -2,8 +2,8 @@
 plan-search latency per failure on B200.
 
 A step is one pass of the whole hot path (descriptor tables -> min-max partitions ->
-rerouting / redundant-computation plans -> cost kernel over every pipeline-plan ->
-split reduction -> tie-break pass -> policy pick -> plans on the host) over one batch
+rerouting / redundant-computation plans -> every pipeline-plan decided by its cost (a lower bound, or
+the recurrence where that does not decide) -> split reduction -> tie-break pass -> policy pick -> plans on the host) over one batch
 of synthetic failure scenarios.  Default workload: the failure-scenario sweep, the largest
 configuration that fits one GPU (256 devices DP8 x PP32, L=96, 1024 failure sets of 1-16
 devices, every policy); the other configurations are timed as context under "workloads".
@@ -51,6 +51,10 @@ KERNEL_PROFILES = {
     ("pair", 0): {"i_cell": 6.57, "issue_active": 0.546, "fp64_pipe_active": 0.496, "dram_bytes_per_cell": 6529024 / 3.653e9,
                   "profile": "profiles/cm_cost_pair_kernel_175b-like-8.md"},
 }
+# Large batches decide most plans by a lower bound (cm_bound_kernel) and run the recurrence on the few it
+# leaves: there the unit of work is one plan bounded, with I_plan thread-instructions.
+BOUND_PROFILE = {"i_plan": 201.5, "issue_active": 0.429, "dram_bytes_per_plan": 311040 / 7.636e6,
+                 "profile": "profiles/cm_bound_kernel_256dev-64.md"}
 KERNEL_NAMES = {"regs": "cm_cost_regs_kernel", "regs_pair": "cm_cost_regs_pair_kernel", "wide": "cm_cost_wide_kernel",
                 "pair": "cm_cost_pair_kernel"}
 FP64_INSTR_PER_CELL = 3.0          # 2 DADD + 1 DSETP; an FP64 warp instruction occupies its pipe for 2 cycles
@@ -537,7 +541,33 @@ def kernel_class(w) -> str:
     return "pair" if paired else "wide"
 
 
+def bound_roofline_of(stats_sum, dev_seconds, clocks, sm_max, peak_kind):
+    prof = BOUND_PROFILE
+    f_mhz = float((clocks or {}).get("sm_mhz") or sm_max)
+    peak = N_SM * 4 * 32 * f_mhz * 1e6 / prof["i_plan"]
+    cost_s = stats_sum["cost_kernel_ns"] * 1e-9
+    achieved = stats_sum["plans_simulated"] / cost_s if cost_s > 0 else 0.0
+    launches = max(1, stats_sum["cost_kernel_launches"])
+    return {
+        "bound": "alu", "kernel": "cm_bound_kernel (search pass by bounds)",
+        "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gplan bounded/s", "frac": achieved / peak,
+        "peak_kind": f"148 SM x 4 schedulers x 32 lanes x {f_mhz:.0f} MHz (median SM clock sampled during the timed region; "
+                     f"{peak_kind} max {sm_max:.0f}) / I_plan; the time is that of the whole pass: bounds, windows, "
+                     "comparison of ties and the recurrences they leave",
+        "i_plan": prof["i_plan"],
+        "i_plan_source": f"executed thread-instructions per plan bounded, ncu capture in {prof['profile']}",
+        "issue_active_profiled": prof["issue_active"], "frac_of_fp64_pipe": None, "frac_of_dispatch_bound": None,
+        "plans_bounded": stats_sum["plans_simulated"], "plans_by_recurrence": stats_sum["plans_run"],
+        "cells_by_recurrence": stats_sum["cells_run"], "launches": launches,
+        "share_of_step": cost_s / dev_seconds if dev_seconds else None,
+        "traffic": prof["dram_bytes_per_plan"] * stats_sum["plans_simulated"],
+        "traffic_source": f"scaled by plans from the ncu capture in {prof['profile']} (not measured in this run)",
+    }
+
+
 def roofline_of(stats_sum, dev_seconds, arith, kclass, clocks, sm_max, peak_kind):
+    if stats_sum["plans_run"] < stats_sum["plans_simulated"]:
+        return bound_roofline_of(stats_sum, dev_seconds, clocks, sm_max, peak_kind)
     prof = KERNEL_PROFILES.get((kclass, arith)) or KERNEL_PROFILES[(kclass, 0)]
     f_mhz = float((clocks or {}).get("sm_mhz") or sm_max)
     lanes_per_s = N_SM * 4 * 32 * f_mhz * 1e6
@@ -640,10 +670,12 @@ def main():
                        # (strategy, pipeline, micro-batch count, layer composition), as the oracle
                        # enumerates them.  Of these: plans_reused belong to pipelines that another
                        # strategy of the same survivor count has as well and are not searched again;
-                       # plans_memory_rejected fail the memory estimator; plans_simulated ran the recurrence.
+                       # plans_memory_rejected fail the memory estimator; plans_simulated are decided by their
+                       # cost, most of them by a lower bound, plans_by_recurrence by the recurrence itself.
                        "plans_reused_per_step": (m["stats"]["plans"] - m["stats"]["plans_own"]) // args.steps,
                        "plans_memory_rejected": (m["stats"]["plans_own"] - m["stats"]["plans_simulated"]) // args.steps,
                        "plans_simulated_per_step": m["stats"]["plans_simulated"] // args.steps + 2 * len(w.scenarios),
+                       "plans_by_recurrence_per_step": m["stats"]["plans_run"] // args.steps + 2 * len(w.scenarios),
                        "policies": 3, "cost_mode": "int64ns" if args.cost_mode else "fp64",
                        "l2": "flushed between timed iterations (256 MB write)",
                        "parallelism": "replicas, scenarios independent" if world > 1 else "1 gpu"},
@@ -689,7 +721,7 @@ def main():
                     "latency_us_shared_segments_p50": em["latency_us"]["shared_segments"]["p50"],
                     "latency_us_shared_segments_p99": em["latency_us"]["shared_segments"]["p99"],
                     "latency_scenarios": em["latency_us"]["scenarios"],
-                    "search_pass_kernel": r["kernel"], "search_pass_gcell_s": r["achieved"],
+                    "search_pass_kernel": r["kernel"], "search_pass_rate": r["achieved"], "search_pass_unit": r["unit"],
                     "search_pass_frac": r["frac"], "search_pass_frac_of_fp64_pipe": r["frac_of_fp64_pipe"],
                     "clocks_sm_mhz": (em["clocks"] or {}).get("sm_mhz")}
             line["workloads"] = extra

@@ -33,6 +33,9 @@
 
 namespace cm {
 
+// Bound by issue under shared-memory and arithmetic latency at three CTAs per SM: 201 thread-instructions per
+// plan, 43 % of the issue slots (64 sets of the 256-device job, 7.6 million plans: 122 us; 1024 sets, 75
+// million: 800 us, 1233 us before the additions were packed and the walks' terms kept in registers).
 // A CTA takes kBoundThreads / W segments side by side, W compositions each (W = a power of two that
 // holds the bucket's candidates, at most all threads), and walks its group of segments with the
 // composition's terms in registers.
@@ -157,7 +160,6 @@ cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo,
 // (phase 0) or the results (phase 1).  Either then marks the segments of the strategies whose step time
 // from bounds is still within reach.
 // ----------------------------------------------------------------------------------
-// ----------------------------------------------------------------------------------
 // Phase 0 marks strategies this far above the best step time from bounds: one plan of each of their
 // segments is evaluated, so that a result that misses its bound a little still leaves phase 2 nothing to do.
 constexpr float kReach = 1.0f / (1 << 13);
@@ -244,7 +246,11 @@ __global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd,
 
 cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
-    cm_window_kernel<<<b.B, b.B <= 148 ? 1024 : 128, 0, st>>>(t, b, bo, phase, k_best, batch_inf_bits(b));
+    // A warp per strategy, latency of its dependent loads.  Up to a scenario per SM the CTA takes them all at
+    // once (64 sets of the 64-device job: 10 us with 1024 threads, 16 with 256, 25 with 128); beyond, CTAs of
+    // an SM stand in for one another (515 sets of the 32-device job: 28 us with 256 threads, 37 with 1024, 40
+    // with 128; 1024 sets of the 256-device job 16, 30 and 16 us).
+    cm_window_kernel<<<b.B, b.B <= 148 ? 1024 : 256, 0, st>>>(t, b, bo, phase, k_best, batch_inf_bits(b));
     return cudaGetLastError();
 }
 

@@ -225,7 +225,9 @@ struct BoundDev {
     int uniform_x;
 };
 constexpr int kCounters = 6;   // work counters of a search in use (BatchDev::counters)
-// Recurrence cells of a search (a shallow one counting a quarter) from which bounds pay for their extra launches.
+// Recurrence cells of a search (a shallow one counting a quarter) from which bounds pay for their extra
+// launches: 33 sets of the 32-device job with the full objective (just below) 506 us directly, 745 by bounds;
+// one failure of the 256-device job (4e8) 380 us directly, 259 by bounds when they came, 146 now.
 constexpr uint64_t kBoundMinCells = 200000000ull;
 constexpr uint32_t kBoundListMin = 65536;        // plans a list has room for, at least (if there are as many)
 constexpr size_t kBoundDynMax = 160 * 1024;      // dynamic shared memory of the bound kernels, at most
@@ -380,7 +382,9 @@ struct EvalDev {
 constexpr uint32_t kEvalMinMax = 0x80000000u, kEvalMasked = 0x40000000u;   // flags of an entry's slot
 constexpr int kEvalShallow = kRegStagesMax, kEvalRest = kWideStagesMax + 1, kEvalRegions = kEvalRest + 1;   // regions by depth: up to 16, 17 .. 48, deeper
 constexpr uint32_t kEvalSlabMax = 1u << 18, kEvalListMax = 1u << 20;
-constexpr uint64_t kEvalWarpMax = 8192;    // deep spaces: calls of up to this many candidates are evaluated a warp per candidate
+// Deep spaces: calls of up to this many candidates are evaluated a warp per candidate (about 10 us for a call
+// that the GPU holds at once, five times the instructions of a thread per candidate), larger ones binned by depth.
+constexpr uint64_t kEvalWarpMax = 8192;
 // Entries of the binned path's workspace for a space whose depths are `stages` (bit S-1), counters included; 0 = not needed.
 uint64_t eval_workspace(uint64_t stages, uint32_t *slab);
 // single_policy < 0: candidates of the dynamic-parallelism segments; otherwise the one

@@ -504,14 +504,18 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
 
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
-    // a failure handled on its own: a warp for every strategy; a batch: enough to keep the SMs busy
-    cm_best_split_kernel<<<b.B, b.B <= 148 ? 1024 : 128, 0, st>>>(t, b, batch_inf_bits(b));
+    // A warp per strategy, latency of its dependent loads: all strategies at once up to a scenario per SM (64 sets
+    // of the 64-device job: 8 us with 1024 threads, 12 with 256, 18 with 128), narrower CTAs beyond (515 sets of
+    // the 32-device job: 20 us with 256 threads, 25 with 1024, 26 with 128; 1024 of the 256-device job 16, 27, 16).
+    cm_best_split_kernel<<<b.B, b.B <= 148 ? 1024 : 256, 0, st>>>(t, b, batch_inf_bits(b));
     return cudaGetLastError();
 }
 
 // ----------------------------------------------------------------------------------
 // One scenario handled on its own: clears the result words and fetches the few bytes that say which
-// devices failed from the host's pinned memory.
+// devices failed from the host's pinned memory.  One launch of about 4 us (a read across the bus) in place
+// of two copies and a clear; with the plans stored to pinned memory by the last kernel one failure of the
+// 256-device job went from 177 to 163 us.
 // ----------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) cm_prologue_kernel(uint64_t *words, size_t n_words, const uint32_t *ids_host, uint32_t *ids, int n_ids,
                                                           const uint64_t *bits_host, uint64_t *bits, int n_bits) {
@@ -535,6 +539,7 @@ cudaError_t launch_prologue(uint64_t *words, size_t n_words, const uint32_t *ids
 // policy id (Algorithm 1 keeps the plan with the least estimated time).  Sixteen threads per plan, one
 // per pipeline; four plans per scenario, the last the winner: it goes to the front of the array, the plans
 // per policy follow scenario by scenario, so that the host hands both out in one piece each.
+// Latency of a few dependent loads: 6 us (a thread per plan walked its pipelines one by one).
 // ----------------------------------------------------------------------------------
 constexpr int kFinalThreads = 64;
 __global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, BatchDev bd, uint64_t inf) {
