@@ -492,10 +492,14 @@ __device__ __forceinline__ void sim_regs_pair(int m, const FB<T> (&st)[S], const
 // ----------------------------------------------------------------------------------
 // ANY_M = true lifts the condition on m: the rounds form of the recurrence (any m >= 1) instead
 // of the unrolled triangles -- for the few segments with fewer micro-batches than warm-up slots.
+// A pipeline without micro-batches is no plan, and has no min-max partition to look up: rejected first
+// (m >= S-1 says so by itself from two stages up).
 template <typename T, int S, bool ANY_M = false>
 __device__ __forceinline__ bool plan_cost_regs(const SProf<T> &sp, const Tables &tb, int layer_mode,
                                                const SegView &g, const Cand &cand, T &cost) {
     const int m = g.m;
+    if constexpr (ANY_M || S == 1)
+        if (m < 1) return false;
     CutWalker cw;
     bool ok = make_walker(cw, tb, layer_mode, sp.L, S, cand, g.K, tb.mm_slot(S, m));
     FB<T> st[S];
@@ -516,7 +520,6 @@ __device__ __forceinline__ bool plan_cost_regs(const SProf<T> &sp, const Tables 
     if (!ok) return false;
     T t;
     if constexpr (ANY_M) {
-        if (m < 1) return false;
         const RegStages<T, S> src{st, xts};
         t = sim_stages<T, S>(sp.sched, m, src);
     } else if (sp.sched == CM_SCHED_GPIPE) {

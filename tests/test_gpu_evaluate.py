@@ -65,6 +65,35 @@ def test_evaluate_of_a_deep_space(gpu, oracle_factory, mode, native, schedule, c
     assert (cost_ns[ok] == want_ns[ok]).all() if mode else (cost[ok] == want[ok]).all()
 
 
+@pytest.mark.parametrize("schedule", [W.SCHED_1F1B, W.SCHED_GPIPE])
+@pytest.mark.parametrize("mode,native", [(0, False), (1, False), (1, True)])
+def test_evaluate_of_pipelines_without_micro_batches(gpu, oracle_factory, mode, native, schedule):
+    """More survivors than micro-batches: some shares are zero, one stage included, and a pipeline that is
+    given no work is no plan, however well it fits.  Every candidate of the space, in one call."""
+    p = W.random_small(41, L=8, n_dp=3, n_pp=2, n_micro=1).profile
+    opts = W.SearchOptions(1, 5, 1, 5, W.LAYERS_FULL, W.BATCH_REMAINDER, 1 << 62, mode, schedule)
+    for failed in ([], [0], [1, 4]):
+        orc = oracle_factory(p, opts)
+        n, _, n_seg = orc.count(failed)
+        segs = [orc.segment(failed, s) for s in range(n_seg)]
+        idle = np.concatenate([np.arange(g["first"], g["first"] + g["K"] + 1) for g in segs if g["m"] == 0] or [np.zeros(0, int)])
+        assert len(idle) and any(g["S"] == 1 and g["m"] == 0 for g in segs)
+        want, want_ns, want_feas = orc.evaluate(failed, idx=np.arange(n))
+        assert not want_feas[idle].any() and want_feas.any()
+        ctx = gpu.cm_create(0)
+        try:
+            gpu.cm_load_profile(ctx, p)
+            gpu.cm_set_int64_arithmetic(ctx, native)
+            space, got_n = gpu.cm_enumerate(ctx, W.POLICY_DYNPAR, failed, opts)
+            assert got_n == n
+            cost, cost_ns, feas = _evaluate(gpu, ctx, space, np.arange(n))
+            gpu.cm_space_free(space)
+        finally:
+            gpu.cm_destroy(ctx)
+        assert np.array_equal(feas, want_feas)
+        assert np.array_equal(cost_ns, want_ns) if mode else np.array_equal(cost, want)
+
+
 @pytest.mark.parametrize("n_micro", [1, 2, 7])
 @pytest.mark.parametrize("batch_mode", [W.BATCH_FULL, W.BATCH_REMAINDER])
 def test_best_split(gpu, oracle_factory, batch_mode, n_micro):
