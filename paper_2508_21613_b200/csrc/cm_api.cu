@@ -355,6 +355,24 @@ public:
     }
 };
 
+// Depths (bit S-1) at which the walks along the whole order of a stage can decide a bound (cm_bound.cuh): the
+// longer half of the heaviest stage, ceil(L/S) neighbouring layers, outlasts one and a half times an average
+// stage's whole turn.  Below that line going to the top takes longer than staying for nearly every stage,
+// and looking costs 5 to 11 % (256-device job, first layer 3 times the others: 48 sets 1298 us without, 1440
+// with; 4 times: 571 and 606; 6 times: 730 and 610; 10 times: 13177, the lists full, and 645).
+template <typename V> uint64_t busy_stages(const V *fwd, const V *bwd, int L) {
+    double f[kMaxL + 1] = {0.0}, b[kMaxL + 1] = {0.0};
+    for (int l = 0; l < L; ++l) { f[l + 1] = f[l] + (double)fwd[l]; b[l + 1] = b[l] + (double)bwd[l]; }
+    uint64_t mask = 0;
+    for (int S = 1; S <= kMaxS && S <= L; ++S) {
+        const int n = (L + S - 1) / S;
+        double heavy = 0.0;
+        for (int l = 0; l + n <= L; ++l) heavy = std::max(heavy, std::max(f[l + n] - f[l], b[l + n] - b[l]));
+        if (heavy * S > 1.5 * (f[L] + b[L])) mask |= 1ull << (S - 1);
+    }
+    return mask;
+}
+
 cm_status check_opts(cm_ctx *ctx, const cm_enum_opts *o) {
     if (!o) return fail(ctx, CM_EINVAL, "opts is NULL");
     if (o->dp_lo > o->dp_hi || o->pp_lo > o->pp_hi) return fail(ctx, CM_EINVAL, "empty dp/pp window");
@@ -1763,6 +1781,8 @@ static cm_status load_profile_host(cm_ctx *ctx, const cm_profile *p) {
         h.act[l] = p->act_bytes[l]; h.par[l] = p->param_bytes[l]; h.opt[l] = p->opt_bytes[l]; h.p2p[l] = p->p2p_bytes[l];
     }
     for (int i = 0; i <= p->n_pp; ++i) h.base_cuts[i] = p->base_cuts[i];
+    h.busy[CM_COST_FP64] = busy_stages(h.fwd, h.bwd, h.L);
+    h.busy[CM_COST_INT64NS] = busy_stages(h.fwd_i, h.bwd_i, h.L);
     ctx->uniform_p2p = true;
     for (int l = 1; l < p->L; ++l) ctx->uniform_p2p = ctx->uniform_p2p && p->p2p_bytes[l] == p->p2p_bytes[0];
     {

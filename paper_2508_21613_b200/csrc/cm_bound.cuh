@@ -16,6 +16,12 @@
 // per mille, against 2-3 per cent for the slowest stage alone).  Where m is too small for a
 // stage's walk, climbing once and repeating one stage's forwards or backwards,
 // U_0 + (m-1) max(f, b), still exists.
+// A stage that outweighs those above it is busy from its first forward to its last backward, and going to
+// the top in the meantime takes less time than staying.  A walk along the whole order of a stage has the
+// value U_0 - U_a + m w_a; one that goes to the top with the first micro-batch only, U_0 + (m-1) w_a -
+// (S-1-a) f_a (the forwards before the first backward are on the way up), with the last only, the same with
+// b_a.  With one layer of twenty times the others (random pipelines of 17 to 36 stages) 95 % of the plans
+// miss their bound without these, by 16 % of their time in the mean, and 10 % by 0.5 % with them.
 // All-forward-all-backward order: climb once, (m-1) extra forwards at the slowest forward, (m-1)
 // extra backwards at the slowest backward; with identical micro-batches that is the longest path.
 //
@@ -58,7 +64,7 @@ template <int STRIDE> struct CutColumn {
 // The best walk of a plan and its value (synchronisation included), in double arithmetic for either
 // cost type; value -1 if the plan does not fit in memory (looked at only where no feasible list
 // vouches for it).
-enum { kWalkStay = 0, kWalkUp = 1, kWalkDown = 2, kWalkForward = 3, kWalkBackward = 4, kWalkAfab = 5 };
+enum { kWalkStay = 0, kWalkUp = 1, kWalkDown = 2, kWalkForward = 3, kWalkBackward = 4, kWalkAfab = 5, kWalkBusy = 6, kWalkFirst = 7, kWalkLast = 8 };
 struct Walk {
     double value;
     long long g_max;    // largest gradient bytes of a stage
@@ -67,7 +73,7 @@ struct Walk {
 
 template <typename T, typename Cuts>
 __device__ __forceinline__ Walk best_walk(const SProf<T> &s, const Cuts &c, int S, int m, uint64_t tier, int n_sync, bool check) {
-    const bool gpipe = s.sched == CM_SCHED_GPIPE;
+    const bool gpipe = s.sched == CM_SCHED_GPIPE, busy = s.heavy_stage(S);
     double U = 0.0, best = -1.0, fmax = -1.0, bmax = -1.0;
     double base_n = 0.0, w_n = 0.0, q_n = 0.0;   // stage i+1: the value of its own walk (without U_0), w, pairs of stays
     int a = 0, kind = kWalkForward, fa = 0, ba = 0;
@@ -95,6 +101,10 @@ __device__ __forceinline__ Walk best_walk(const SProf<T> &s, const Cuts &c, int 
                 if (q > 0.0) take(base + q * (w_n - wi + x), i, kWalkUp);
             }
             base_n = base; w_n = wi; q_n = q;
+            if (busy) {   // uniform
+                take((double)m * wi - U, i, kWalkBusy);
+                if (n >= -1) take((double)(m - 1) * wi - (double)(S - 1 - i) * (f < bk ? f : bk), i, f < bk ? kWalkFirst : kWalkLast);
+            }
         }
         hi = lo;
     }
@@ -157,6 +167,20 @@ __device__ __forceinline__ T walk_cost(const SProf<T> &s, const Cuts &c, int S, 
         for (; n > 0; --n) t = (t + f) + bk;
         climb(a, S);
         drop(S - 1, 0);
+    } else if (w.kind >= kWalkBusy) {
+        const int warm = S - 1 - a < m ? S - 1 - a : m;   // forwards of the stage before its first backward's pair
+        climb(0, w.kind == kWalkFirst ? S : a);
+        if (w.kind == kWalkFirst) drop(S - 1, a);
+        else
+            for (int k = warm; k > 0; --k) t = t + f;
+        for (int k = w.kind == kWalkBusy ? m - warm : m - 1 - warm; k > 0; --k) t = (t + f) + bk;
+        if (w.kind == kWalkLast) {
+            climb(a, S);
+            drop(S - 1, 0);
+        } else {
+            for (int k = warm; k > 0; --k) t = t + bk;
+            if (a > 0) drop(a - 1, 0);
+        }
     } else {
         const bool forwards = w.kind != kWalkBackward, backwards = w.kind != kWalkForward;
         climb(0, a);

@@ -152,9 +152,13 @@ __device__ __forceinline__ float stay_pairs(int i, int S, int m) {
 // The stages are a loop of four at a time whose results move up the registers: all of them in a row are
 // tens of kilobytes of code per depth that every CTA runs through once, and the warps waited for
 // instructions most of the time (1024 sets of the 256-device job: 2023 -> 1997 us a call; one: 148 -> 146 us).
+// Where a stage may outweigh the others (busy) the walks along its whole order count as well.  Their values
+// depend on the link tiers through the boundaries that they leave out; with the dearer tier there they are one
+// number per lane.
 template <typename T, int NB, bool UNI_X>
 __device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, const CutColumn<kBoundThreads> &w, int S, int m, bool check, float2 *cd) {
-    const bool gpipe = s.sched == CM_SCHED_GPIPE;
+    const bool gpipe = s.sched == CM_SCHED_GPIPE, busy = s.heavy_stage(S);
+    float busy_best = 0.0f, U_hi = 0.0f;              // U_hi: U_i with the dearer transfers, rounded up
     double U = 0.0, w_n = 0.0;                        // w_n: of stage i+1
     float base_n = kNoWalk, c_n = kNoWalk, xq_n = 0.0f, q_n = 0.0f;
     const float xm_all = __double2float_rd((double)(s.XT[0][0] < s.XT[1][0] ? s.XT[0][0] : s.XT[1][0]));
@@ -192,6 +196,14 @@ __device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, 
                     c_n = q > 0.0f && i < S - 1 ? __fmaf_rd(q, __double2float_rd(-dw), base_n) : kNoWalk;
                     cd[i * kBoundThreads] = make_float2(c_n, d);
                     w_n = wi; q_n = q; xq_n = __fmul_rd(2.0f * q, xm);
+                    if (busy) {   // uniform
+                        const int at = UNI_X ? 0 : hi - 1;
+                        const float w_lo = __double2float_rd(wi), x_hi = i < S - 1 ? __double2float_ru((double)tmax(s.XT[0][at], s.XT[1][at])) : 0.0f;
+                        U_hi = __fadd_ru(U_hi, __fmaf_ru(2.0f, x_hi, __double2float_ru(wi)));
+                        busy_best = fmaxf(busy_best, __fmaf_rd((float)m, w_lo, -U_hi));
+                        if (n >= -1)
+                            busy_best = fmaxf(busy_best, __fmaf_rd(-(float)(S - 1 - i), __double2float_ru(f < bk ? f : bk), __fmul_rd((float)(m - 1), w_lo)));
+                    }
                 }
                 hi = lo;
             }
@@ -205,7 +217,7 @@ __device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, 
     if (!gpipe) v.set(0, fmaxf(base_n, c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n)));
     const double f1 = __hiloint2double(fmax, 0), b1 = __hiloint2double(bmax, 0);
     v.u0 = __double2float_rd(U);
-    v.once = __double2float_rd((double)(m - 1) * (gpipe ? f1 + b1 : tmax(f1, b1)));
+    v.once = fmaxf(__double2float_rd((double)(m - 1) * (gpipe ? f1 + b1 : tmax(f1, b1))), busy_best);
     v.g = __ll2float_rd(g_max);
 }
 

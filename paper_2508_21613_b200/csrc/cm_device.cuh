@@ -79,6 +79,8 @@ template <typename T> struct SProf {
     long long cap, bw_sync;
     int L, n_dp, n_pp, n_micro;
     int intval, sched;   // sched: order of the computations on a stage (cm_schedule), an option carried along
+    unsigned long long busy;   // DevProfile::busy of the arithmetic's inputs
+    __device__ __forceinline__ bool heavy_stage(int S) const { return (busy >> (S - 1)) & 1ull; }
 };
 
 template <typename T>
@@ -105,6 +107,7 @@ __device__ __forceinline__ void stage_profile(SProf<T> &s, const Tables &tb) {
         s.n_micro = p->n_micro;
         s.intval = p->intval;
         s.sched = tb.sched;
+        s.busy = p->busy[std::is_same<T, long long>::value || p->intval ? CM_COST_INT64NS : CM_COST_FP64];
     }
 }
 

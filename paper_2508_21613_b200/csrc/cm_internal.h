@@ -31,6 +31,7 @@ struct DevProfile {
     double XTd[2][kMaxL];   // transfer time of the boundary after layer l: [0] intra, [1] inter
     int64_t XTi[2][kMaxL];
     int32_t base_cuts[kMaxS + 1];
+    uint64_t busy[2];       // per cost mode, bit S-1: with S stages one of them may outweigh the others (busy_stages)
     // raw inputs (kept for the prefix kernel)
     double fwd[kMaxL], bwd[kMaxL];
     int64_t fwd_i[kMaxL], bwd_i[kMaxL], act[kMaxL], par[kMaxL], opt[kMaxL], p2p[kMaxL];

@@ -40,6 +40,19 @@ CASES = {
 }
 
 
+def _heavy(layer, p2p):
+    times = np.linspace(3e6, 3.6e6, 13)
+    times[layer] *= 9
+    return _small(37, times=lambda n: times, n_micro=20, p2p=p2p)
+
+
+# a layer that outweighs a pipeline: at either end and inside, transfers equal and by layer
+for _layer in (0, 6, 12):
+    for _p2p in (None, 30_000_000):
+        CASES[f"heavy-layer-{_layer}-{'equal' if _p2p else 'layered'}"] = (
+            _heavy(_layer, _p2p), (1, 3, 2, 7, W.LAYERS_FULL, W.BATCH_REMAINDER), SETS[:12], 60)
+
+
 @pytest.mark.parametrize("schedule", [W.SCHED_1F1B, W.SCHED_GPIPE])
 @pytest.mark.parametrize("name", sorted(CASES))
 def test_bounded_search_against_the_oracle(gpu, oracle_factory, name, schedule):
@@ -138,6 +151,33 @@ def test_bounded_search_of_shared_segments_against_the_oracle(gpu, oracle_factor
         best = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets, opts)[0])
         st = gpu.cm_last_stats(ctx)
         assert st["plans_run"] < st["plans_simulated"], st
+        orc = oracle_factory(profile, opts)
+        for f, plan in zip(sets, best):
+            want = orc.search(f)[0]
+            assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (f, plan, want)
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("layer", [0, 13, 39])
+def test_bounds_decide_where_one_stage_outweighs_the_others(gpu, oracle_factory, layer, mode):
+    """A stage with a layer of twelve times the others is busy from its first forward to its last backward:
+    its bound has to say so, or thousands of plans per pipeline are left to the recurrence."""
+    rng = np.random.default_rng(71)
+    L, n_dp, n_pp = 40, 2, 20
+    fwd = rng.uniform(2.8e6, 3.2e6, L).round()
+    fwd[layer] *= 12
+    profile = W.make_profile_ns(L, n_dp, n_pp, 48, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 8_000_000,
+                                list(range(0, L + 1, 2)), 80_000_000_000, 8, 300, 20)
+    sets = [[3], [5], [20], [0, 9], [8, 30]]
+    opts = W.SearchOptions(2, 2, 17, 22, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15, mode)
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets * 12, opts)[0])
+        st = gpu.cm_last_stats(ctx)
+        assert 0 < st["plans_run"] < st["plans_simulated"] // 100, st
         orc = oracle_factory(profile, opts)
         for f, plan in zip(sets, best):
             want = orc.search(f)[0]
