@@ -96,6 +96,7 @@ struct Batch {
     DevBuf<uint64_t> d_seg_best, d_kappa_sel, d_pol_cost;
     DevBuf<Winner> d_winner;
     DevBuf<uint16_t> d_rc_stages;
+    DevBuf<uint32_t> d_open;              // pipelines that the tie-break kernel leaves open
     DevBuf<cm_plan> d_plans;
     // full objective: shortlist slots (scenario-major) and per-scenario results
     DevBuf<Winner> d_short_win;
@@ -152,7 +153,7 @@ struct Batch {
     size_t bytes() const {
         return d_arena.cap + 8 * (d_seg_best.cap + d_kappa_sel.cap + d_pol_cost.cap + d_utab.cap + d_useg.cap + d_short_kappa.cap) +
                sizeof(Winner) * (d_winner.cap + d_short_win.cap) + sizeof(cm_plan) * (d_plans.cap + d_short_plans.cap) +
-               4 * (d_urep.cap + d_slot_of.cap + d_row_rep.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
+               4 * (d_urep.cap + d_slot_of.cap + d_row_rep.cap + d_open.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
     }
     // One scenario handled on its own: its first kernel reads the failed ids and the node-crossing bits
     // from the pinned arena and its last one writes the plans to pinned memory, so that no copy sits on the
@@ -1231,6 +1232,8 @@ BatchDev dev_view(const cm_ctx *ctx, Batch &bt) {
     v.winner = bt.d_winner.p; v.kappa_sel = bt.d_kappa_sel.p; v.pol_cost = bt.d_pol_cost.p;
     v.rc_stages = bt.d_rc_stages.p; v.plans = bt.direct ? bt.plans_host.p : bt.d_plans.p;
     v.counters = reinterpret_cast<unsigned long long *>(bt.d_seg_best.p + bt.n_rows);
+    v.open = bt.d_open.p;
+    v.n_open = v.counters + 6;
     v.B = bt.B; v.mode = bt.opts.cost; v.intval = bt.intval ? 1u : 0u;
     v.n_rows = (uint32_t)bt.n_rows;
     v.n_tiles = bt.n_tiles; v.max_tiles_per_seg = bt.max_tiles_per_seg;
@@ -1268,8 +1271,7 @@ Tables tables_plain(const cm_ctx *ctx) {   // for kernels that only read the byt
     return t;
 }
 
-constexpr size_t kCounterSlots = 8;                 // kCounters of them in use
-constexpr size_t kStateExtra = kCounterSlots + 2;   // + the counts of four lists (32-bit)
+constexpr size_t kStateExtra = kCounters + 2;   // work counters and the counts of four lists (32-bit)
 
 // Room for listed plans.  Captured launch sequences carry the list's address: dropped when it moves.
 cm_status reserve_bound_list(cm_ctx *ctx, size_t want) {
@@ -1311,7 +1313,8 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
     ok = bt.d_seg_best.reserve((bt.useg ? 5 : 3) * bt.n_rows + kStateExtra) && bt.d_win.reserve(B) &&
          bt.d_winner.reserve(B) &&
          bt.d_kappa_sel.reserve(B * kMaxP) && bt.d_pol_cost.reserve(B * 2) &&
-         bt.d_rc_stages.reserve(B * kMaxP) && bt.d_plans.reserve(B * 4 + 1);   // + room for the counters
+         bt.d_rc_stages.reserve(B * kMaxP) && bt.d_open.reserve(std::max<size_t>(B * bt.dp_max, 1)) &&
+         bt.d_plans.reserve(B * 4 + 1);   // + room for the counters
     if (!ok) return fail(ctx, CM_ENOMEM, "device memory");
     if (bt.keys.size() && !bt.mm_launched) {
         CM_CUDA(ctx, launch_minmax(tables(ctx, bt), (const uint32_t *)(bt.d_arena.p + bt.off_keys),
@@ -1358,7 +1361,7 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
 cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchDev &bd, cudaStream_t st, int *launches) {
     BoundDev bo = bt.bo;
     bo.bucket = (const BBucket *)(bt.d_arena.p + bt.off_bbucket);
-    bo.count = (uint32_t *)(bt.d_seg_best.p + bt.n_rows + kCounterSlots);
+    bo.count = (uint32_t *)(bt.d_seg_best.p + bt.n_rows + kCounters);
     bo.lbarg = bt.d_seg_best.p + bt.n_rows + kStateExtra;
     bo.pick = bo.lbarg + bt.n_rows;
     bo.win = bt.d_win.p;
@@ -1448,6 +1451,13 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     return CM_OK;
 }
 
+// Depths of the batch's pipelines, bit S-1.
+uint64_t stage_mask(const Batch &bt) {
+    uint64_t mask = 0;
+    for (const TSeg &g : bt.tseg) mask |= 1ull << ((g.S - 1) & 63);
+    return mask;
+}
+
 // Work counters of a finished search (they came back behind its plans).
 const unsigned long long *search_counters(const Batch &bt) {
     return reinterpret_cast<const unsigned long long *>(bt.plans_host.p + (size_t)bt.B * 4);
@@ -1465,6 +1475,30 @@ void account_search(cm_ctx *ctx, const Batch &bt, int launches) {
     ctx->stats[5] += bt.n_rows;
     ctx->stats[6] += bt.strat.size();
     ctx->stats[7] += bt.n_split;
+}
+
+// A finished search whose tie-break has left pipelines open: the rest of it, and the plans again.
+cm_status finish_tiebreak(cm_ctx *ctx, Batch &bt, int *launches) {
+    cudaStream_t st = ctx->stream;
+    const Tables tb = tables(ctx, bt);
+    const BatchDev bd = dev_view(ctx, bt);
+    ctx->stats[22] += search_counters(bt)[6];
+    CM_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
+    CM_CUDA(ctx, launch_tie_rest(tb, bd, stage_mask(bt), true, st, launches));
+    CM_CUDA(ctx, launch_finalize(tb, bd, st));
+    ++*launches;
+    CM_CUDA(ctx, cudaEventRecord(ctx->ev[5], st));
+    if (!bt.direct) {
+        const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
+        CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, back_bytes, cudaMemcpyDeviceToHost, st));
+        ctx->stats[10] += back_bytes;
+    }
+    CM_CUDA(ctx, cudaStreamSynchronize(st));
+    float ms = 0.f;
+    CM_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]));
+    ctx->stats[4] += (uint64_t)((double)ms * 1e6);
+    ctx->stats[11] += (uint64_t)((double)ms * 1e6);
+    return CM_OK;
 }
 
 // The search over an uploaded batch; results land in bt.plans_host ([B][4]) after the stream is
@@ -1527,6 +1561,10 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
         if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
         bt.direct = direct;
         return s == CM_OK ? run_batch(ctx, bt, launches, single) : s;
+    }
+    if (search_counters(bt)[6]) {
+        cm_status s = finish_tiebreak(ctx, bt, &launches);
+        if (s != CM_OK) return s;
     }
     account_search(ctx, bt, launches);
     ctx->stats[4] += (uint64_t)((double)ms * 1e6);
@@ -1881,13 +1919,6 @@ cm_status cm_host_describe(const cm_profile *p, const uint32_t *failed_ids, int3
     CM_API_END(nullptr)
 }
 
-// Depths of the space's pipelines, bit S-1.
-static uint64_t stage_mask(const Batch &bt) {
-    uint64_t mask = 0;
-    for (const TSeg &g : bt.tseg) mask |= 1ull << ((g.S - 1) & 63);
-    return mask;
-}
-
 cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids, int32_t n_failed,
                        const cm_enum_opts *opts, cm_space **out, uint64_t *n_candidates) {
     if (!ctx) return CM_EINVAL;
@@ -2035,6 +2066,7 @@ cm_status cm_select(cm_ctx *ctx, cm_space *const *spaces, int32_t n_spaces, cm_p
             continue;
         }
         ctx->stats[10] += (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
+        if (spaces[i]->policy == CM_DYNPAR && search_counters(bt)[6] && (s = finish_tiebreak(ctx, bt, &launches)) != CM_OK) return s;
         account_search(ctx, bt, 0);
     }
     ctx->stats[3] += (uint64_t)launches;
@@ -2133,7 +2165,7 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
     // the objective pass works on what the search left on the device
     const size_t slots = (size_t)B * q.topk;
     bool ok = bt.d_short_win.reserve(slots) && bt.d_short_kappa.reserve(slots * kMaxP) && bt.d_short_bytes.reserve(slots) &&
-              bt.d_short_assign.reserve(slots * kMaxMatch) && bt.d_short_plans.reserve(slots) &&
+              bt.d_open.reserve(std::max<size_t>(slots * bt.dp_max, 1)) && bt.d_short_assign.reserve(slots * kMaxMatch) && bt.d_short_plans.reserve(slots) &&
               bt.d_short_step.reserve(slots * 2) && bt.d_short_rounds.reserve(slots * 2) &&
               bt.d_obj_best.reserve(B) && bt.d_trans.reserve(B);
     if (!ok) return fail(ctx, CM_ENOMEM, "device memory");
@@ -2163,8 +2195,11 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
         sd.winner = od.short_win;
         sd.kappa_sel = od.short_kappa;
         sd.B = (int32_t)slots;
+        sd.open = bt.d_open.p;
+        sd.n_open = bd.counters + 7;
         CM_CUDA(ctx, launch_tiebreak(tb, sd, st));
         ++obj_launches;
+        CM_CUDA(ctx, launch_tie_rest(tb, sd, stage_mask(bt), false, st, &obj_launches));
     }
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[2], st));
     CM_CUDA(ctx, launch_plan_matching(tb, bd, od, st));

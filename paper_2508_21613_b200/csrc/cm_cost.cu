@@ -10,6 +10,7 @@ template <typename T> cudaError_t launch_shallow_pair_class(const Tables &, cons
 template <typename T> cudaError_t launch_short_class(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 template <typename T, int LO, int HI> cudaError_t launch_deep_range(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 template <typename T, int LO, int HI> cudaError_t launch_evaluate_range(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t);
+template <typename T, int LO, int HI> cudaError_t launch_tie_rest_range(const Tables &, const BatchDev &, int, cudaStream_t);
 template <typename T> cudaError_t launch_solo_class(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 template <typename T> cudaError_t launch_warp_class(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 
@@ -29,7 +30,9 @@ CM_EXTERN(long long)
     extern template cudaError_t launch_deep_range<double, LO, HI>(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t); \
     extern template cudaError_t launch_deep_range<long long, LO, HI>(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t); \
     extern template cudaError_t launch_evaluate_range<double, LO, HI>(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t); \
-    extern template cudaError_t launch_evaluate_range<long long, LO, HI>(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t);
+    extern template cudaError_t launch_evaluate_range<long long, LO, HI>(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t); \
+    extern template cudaError_t launch_tie_rest_range<double, LO, HI>(const Tables &, const BatchDev &, int, cudaStream_t);         \
+    extern template cudaError_t launch_tie_rest_range<long long, LO, HI>(const Tables &, const BatchDev &, int, cudaStream_t);
 CM_DEEP_RANGES(CM_DEEP_RANGE)
 #undef CM_DEEP_RANGE
 
@@ -46,6 +49,16 @@ cudaError_t launch_evaluate_deep(const Tables &t, const BatchDev &b, const EvalD
     if (stages >= LO && stages <= HI)                                                                              \
         return native_i64(b) ? launch_evaluate_range<long long, LO, HI>(t, b, ev, stages, st)                      \
                              : launch_evaluate_range<double, LO, HI>(t, b, ev, stages, st);
+    CM_DEEP_RANGES(CM_DEEP_RANGE)
+#undef CM_DEEP_RANGE
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_tie_rest_deep(const Tables &t, const BatchDev &b, int stages, cudaStream_t st) {
+#define CM_DEEP_RANGE(LO, HI)                                                                                      \
+    if (stages >= LO && stages <= HI)                                                                              \
+        return native_i64(b) ? launch_tie_rest_range<long long, LO, HI>(t, b, stages, st)                          \
+                             : launch_tie_rest_range<double, LO, HI>(t, b, stages, st);
     CM_DEEP_RANGES(CM_DEEP_RANGE)
 #undef CM_DEEP_RANGE
     return cudaErrorInvalidValue;

@@ -11,4 +11,5 @@
 namespace cm {
 template cudaError_t launch_deep_range<CM_DEEP_T, CM_DEEP_LO, CM_DEEP_HI>(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);
 template cudaError_t launch_evaluate_range<CM_DEEP_T, CM_DEEP_LO, CM_DEEP_HI>(const Tables &, const BatchDev &, const EvalDev &, int, cudaStream_t);
+template cudaError_t launch_tie_rest_range<CM_DEEP_T, CM_DEEP_LO, CM_DEEP_HI>(const Tables &, const BatchDev &, int, cudaStream_t);
 }  // namespace cm

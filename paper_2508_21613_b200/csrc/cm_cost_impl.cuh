@@ -27,6 +27,7 @@
 #include <atomic>
 
 #include "cm_eval_out.cuh"
+#include "cm_tie_rest.cuh"
 
 namespace cm {
 
@@ -691,6 +692,63 @@ static cudaError_t evaluate_dispatch(const Tables &t, const BatchDev &b, const E
 template <typename T, int LO, int HI>
 cudaError_t launch_evaluate_range(const Tables &t, const BatchDev &b, const EvalDev &ev, int stages, cudaStream_t st) {
     return evaluate_dispatch<T, LO, HI>(t, b, ev, stages, st);
+}
+
+// ----------------------------------------------------------------------------------
+// What the tie-break has left open (cm_tiebreak.cu), pipelines of S stages: one candidate per lane as above.
+// ----------------------------------------------------------------------------------
+template <typename T, int S>
+__global__ void __launch_bounds__(kChunk, wide_ctas_per_sm<S>()) cm_tie_rest_deep_kernel(Tables tb, BatchDev bd) {
+    __shared__ SProf<T> sp;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    const uint32_t n = rest_open(bd);
+    if (n == 0) return;
+    stage_profile(sp, tb);
+    FB<T> *fcol = reinterpret_cast<FB<T> *>(dyn) + threadIdx.x;
+    T *xcol = reinterpret_cast<T *>(dyn + sizeof(FB<T>) * S * kChunk) + threadIdx.x;
+    unsigned long long evaluated = 0;
+    rest_tiles(bd, n, [](int stages) { return stages == S; }, [&](const RestTile &t) {
+        const uint64_t pos = t.base + threadIdx.x;
+        uint64_t hit = ~0ull;
+        if (pos < t.count) {
+            const Cand cand = walk_cand(bd, t.g.feas_first, pos);
+            T cost;
+            if (plan_cost_wide_lane<T, S>(sp, tb, bd.layer_mode, t.g, cand, fcol, xcol, cost) && Num<T>::bits(cost) <= t.w_bits) hit = cand.kappa;
+            ++evaluated;
+        }
+        hit = warp_min_u64(hit);
+        if ((threadIdx.x & 31) == 0 && hit != ~0ull) t.commit(hit);
+    });
+    rest_count(bd, evaluated);
+}
+
+template <typename T, int S>
+static cudaError_t launch_tie_rest_one(const Tables &t, const BatchDev &b, cudaStream_t st) {
+    constexpr size_t smem = wide_smem_bytes<S, false, T>();
+    static std::atomic<uint64_t> configured{0};   // as in launch_wide_one
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 64 || !((configured.load(std::memory_order_acquire) >> dev) & 1ull)) {
+        cudaError_t e = cudaFuncSetAttribute(cm_tie_rest_deep_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
+    }
+    constexpr int ctas = wide_ctas_per_sm<S>() == 3 ? 443 : wide_ctas_per_sm<S>() == 2 ? 293 : 139;   // primes below 148 a piece
+    cm_tie_rest_deep_kernel<T, S><<<ctas, kChunk, smem, st>>>(t, b);
+    return cudaGetLastError();
+}
+
+template <typename T, int S, int HI>
+static cudaError_t tie_rest_dispatch(const Tables &t, const BatchDev &b, int stages, cudaStream_t st) {
+    if constexpr (S <= kWideStagesMax) {
+        if (stages == S) return launch_tie_rest_one<T, S>(t, b, st);
+    }
+    if constexpr (S < HI) return tie_rest_dispatch<T, S + 1, HI>(t, b, stages, st);
+    else return cudaErrorInvalidValue;
+}
+template <typename T, int LO, int HI>
+cudaError_t launch_tie_rest_range(const Tables &t, const BatchDev &b, int stages, cudaStream_t st) {
+    return tie_rest_dispatch<T, LO, HI>(t, b, stages, st);
 }
 
 // Deep pipelines are instantiated per stage count; the stage counts LO .. HI of one cost type

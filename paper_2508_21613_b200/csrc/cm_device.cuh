@@ -401,7 +401,7 @@ __device__ __forceinline__ void decode_winner(const Tables &tb, const BatchDev &
     w.strat = 0;
     w.dp = 0;
     w.scen = scen;
-    w.pad = 0;
+    w.open = 0;
     for (int p = 0; p < kMaxP; ++p) { w.seg[p] = 0; w.micro[p] = 0; }
     if (cost_bits < inf) {
         const uint32_t si = strat_of_item(bd, tp, item);

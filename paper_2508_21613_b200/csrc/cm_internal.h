@@ -225,7 +225,7 @@ struct BoundDev {
     size_t dyn_bytes;
     int uniform_x;
 };
-constexpr int kCounters = 6;   // work counters of a search in use (BatchDev::counters)
+constexpr int kCounters = 8;   // work counters of a search (BatchDev::counters)
 // Recurrence cells of a search (a shallow one counting a quarter) from which bounds pay for their extra
 // launches: 33 sets of the 32-device job with the full objective (just below) 506 us directly, 745 by bounds;
 // one failure of the 256-device job (4e8) 380 us directly, 259 by bounds when they came, 146 now.
@@ -242,7 +242,8 @@ struct Winner {
     uint32_t strat, dp;     // global strategy row; pipelines
     uint32_t seg[kMaxP];    // global segment row of every pipeline
     uint16_t micro[kMaxP];
-    uint32_t scen, pad;     // scenario it belongs to (a shortlist holds several records per scenario)
+    uint32_t scen;          // scenario it belongs to (a shortlist holds several records per scenario)
+    uint32_t open;          // pipelines (bits) that the tie-break kernel has left to cm_tie_rest_kernel
 };
 
 struct BatchDev {
@@ -273,7 +274,10 @@ struct BatchDev {
     cm_plan *plans;         // [B] the overall best, then [B][3] per policy, then the work counters
     // [0] cells of the plans the search pass decided, [1] plans of the tie-break pass, [2] plans decided;
     // bounded pass: [3] cells and [5] plans whose recurrence ran, [4] a list was full
+    // [6], [7] pipelines left to cm_tie_rest_kernel, by the winners' tie-break and by a shortlist's
     unsigned long long *counters;
+    uint32_t *open;              // those pipelines: winner record * kMaxP + pipeline
+    unsigned long long *n_open;  // their number minus one (counters + 6 or + 7)
     int32_t B, mode;
     uint32_t n_rows;             // rows of seg_best over all scenarios
     // 1: integer-nanosecond mode evaluated in double arithmetic on integer-valued inputs; every
@@ -361,7 +365,11 @@ cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo
 cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
 cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches);   // first_list and the next
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st);
-cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);   // cm_tiebreak.cu
+// cm_tiebreak.cu; the second one, for what the first leaves open: stages, the depths there are (bit S-1); by_depth, a
+// launch for each of 17 .. kWideStagesMax
+cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);
+cudaError_t launch_tie_rest(const Tables &t, const BatchDev &b, uint64_t stages, bool by_depth, cudaStream_t st, int *launches);
+cudaError_t launch_tie_rest_deep(const Tables &t, const BatchDev &b, int stages, cudaStream_t st);
 // first kernel of a scenario handled on its own: clear n_words result words, fetch its ids and bits from host memory
 cudaError_t launch_prologue(uint64_t *words, size_t n_words, const uint32_t *ids_host, uint32_t *ids, int n_ids,
                             const uint64_t *bits_host, uint64_t *bits, int n_bits, cudaStream_t st);

@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
     Winner &w = bd.winner[b];
     uint64_t *kappa = bd.kappa_sel + (size_t)b * kMaxP;
     if (best_c >= inf) {
-        if (lane == 0) { w.cost_bits = inf; w.item = ~0ull; w.strat = 0; w.dp = 0; w.scen = b; w.pad = 0; }
+        if (lane == 0) { w.cost_bits = inf; w.item = ~0ull; w.strat = 0; w.dp = 0; w.scen = b; w.open = 0; }
         if (lane < kMaxP) { w.seg[lane] = 0; w.micro[lane] = 0; kappa[lane] = ~0ull; }
         return;
     }
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
         w.strat = tp.strat_first + best_i;
         w.dp = s.dp;
         w.scen = b;
-        w.pad = 0;
+        w.open = 0;
     }
     if (lane < kMaxP) {
         const uint32_t seg = mine ? s.seg_first + lane * s.n_m + (micro - s.m_lo[lane]) : 0u;

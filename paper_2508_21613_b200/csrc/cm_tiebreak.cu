@@ -4,8 +4,14 @@
 #include <algorithm>
 
 #include "cm_bound.cuh"
+#include "cm_tie_rest.cuh"
 
 namespace cm {
+
+// Rounds of recurrences without success after which a CTA leaves its pipeline to cm_tie_rest_kernel: bounds
+// that decide leave one or two candidates, and where they do not (transfers about as long as the stages) tens
+// of thousands are left, and a warp each, a few at a time, is the slowest way through them.
+constexpr int kTieRoundsWide = 2, kTieRoundsWarp = 6;
 
 // ----------------------------------------------------------------------------------
 // A CTA per (winner record, pipeline) walks the segment's candidates upwards, a thread per
@@ -26,17 +32,19 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
     __shared__ unsigned long long found;
     const uint32_t b = blockIdx.x / bd.dp_max, p = blockIdx.x % bd.dp_max;
     const Winner &w = bd.winner[b];
-    if (w.cost_bits >= inf_bits<T>() || p >= w.dp) return;          // uniform over the CTA
+    const uint64_t w_bits = w.cost_bits;
+    if (w_bits >= inf_bits<T>() || p >= w.dp) return;               // uniform over the CTA
     const SegView g = seg_view(bd, w.scen, w.seg[p]);
     if (g.K == 0) return;                                           // one candidate: known already
     stage_profile(sp, tb);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double goal = std::is_same<T, long long>::value ? __ll2double_ru((long long)w.cost_bits)
-                                                          : __longlong_as_double((long long)w.cost_bits);
+    const double goal = std::is_same<T, long long>::value ? __ll2double_ru((long long)w_bits)
+                                                          : __longlong_as_double((long long)w_bits);
     unsigned long long *slot = reinterpret_cast<unsigned long long *>(&bd.kappa_sel[(size_t)b * kMaxP + p]);
     const uint64_t count = walk_count(g);
     unsigned long long evaluated = 0;
-    for (uint64_t base = (uint64_t)blockIdx.y * kTieThreads; base < count; base += (uint64_t)gridDim.y * kTieThreads) {
+    int rounds = kTieThreads > 32 ? kTieRoundsWide : kTieRoundsWarp;
+    for (uint64_t base = (uint64_t)blockIdx.y * kTieThreads; rounds && base < count; base += (uint64_t)gridDim.y * kTieThreads) {
         __syncthreads();
         if (threadIdx.x == 0) found = *(volatile unsigned long long *)slot;
         __syncthreads();
@@ -50,7 +58,7 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
                 c.fill(cw, g.S);
                 const Walk walk = best_walk<T>(sp, c, g.S, g.m, g.tier, g.n_sync, g.feas_first == kNoFeasList);
                 maybe = walk.value >= 0.0 && walk.value <= goal;
-                if (maybe) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= w.cost_bits;
+                if (maybe) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= w_bits;
             }
         }
         const uint32_t vote = __ballot_sync(0xffffffffu, maybe);
@@ -73,7 +81,7 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
                 const Cand cand = walk_cand(bd, g.feas_first, base + at);
                 T cost;
                 if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, cand, cuts_s[warp], cost) && lane == 0 &&
-                    Num<T>::bits(cost) <= w.cost_bits)
+                    Num<T>::bits(cost) <= w_bits)
                     atomicMin(&found, (unsigned long long)cand.kappa);
                 if (lane == 0) ++evaluated;
             }
@@ -81,7 +89,7 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
                 for (int q = 0, n = n_eval; q < kTieThreads / 32 && n > 0; ++q)
                     while (left[q] && n > 0) { left[q] &= left[q] - 1; --n; }
             __syncthreads();
-            if (found != ~0ull) break;                              // uniform
+            if (found != ~0ull || --rounds == 0) break;             // uniform
         }
         if (found != ~0ull) {                                       // the lowest of this tile: later tiles are higher
             if (threadIdx.x == 0) atomicMin(slot, found);
@@ -89,6 +97,112 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
         }
     }
     if (lane == 0 && evaluated) atomicAdd(&bd.counters[1], evaluated);
+    if (threadIdx.x == 0 && rounds == 0 && found == ~0ull && !((atomicOr(&bd.winner[b].open, 1u << p) >> p) & 1u))
+        bd.open[atomicAdd(bd.n_open, 1ull) + 1ull] = b * kMaxP + p;   // (the count starts at -1)
+}
+
+// ----------------------------------------------------------------------------------
+// The pipelines that the kernel above has left open, from their lowest candidate on (cm_tie_rest.cuh).  Up to
+// kRegStagesMax stages a thread per candidate, its state in registers; 17 .. 48 stages the same with
+// a launch per depth (cm_cost_impl.cuh), for which the host has to know that there are any.  Deeper ones, and
+// a shortlist's, whose completion the host does not wait for, as above: bounds first and a warp for
+// each that is left, but without waiting for one another.
+// Bound by issue, as the search pass.  60 sets of a 40-device job, transfers three times the stages (620 000
+// candidates, nearly all of 19 and 20 stages): 0.85 ms by depth, 4.5 ms with a warp each, 9 ms if a
+// pipeline's tiles stay with four CTAs.  600 sets of the 32-device job over links of 1 GB/s: 9.1 ms a call with
+// the kernel above alone, 3.7 with this one.
+// ----------------------------------------------------------------------------------
+// CTAs: two and four per SM, rounded down to primes.
+constexpr int kRestShallow = 293, kRestWarps = 587;
+
+template <typename T>
+__global__ void __launch_bounds__(kRestThreads) cm_tie_rest_kernel(Tables tb, BatchDev bd) {
+    __shared__ SProf<T> sp;
+    const uint32_t n = rest_open(bd);
+    if (n == 0) return;
+    stage_profile(sp, tb);
+    unsigned long long evaluated = 0;
+    rest_tiles(bd, n, [](int S) { return S <= kRegStagesMax; }, [&](const RestTile &t) {
+        const uint64_t pos = t.base + threadIdx.x;
+        unsigned long long hit = ~0ull;
+        if (pos < t.count) {
+            const Cand cand = walk_cand(bd, t.g.feas_first, pos);
+            T cost;
+            if (plan_cost_regs_any<T, true>(sp, tb, bd.layer_mode, t.g, cand, cost) && Num<T>::bits(cost) <= t.w_bits) hit = cand.kappa;
+            ++evaluated;
+        }
+        hit = warp_min_u64(hit);
+        if ((threadIdx.x & 31) == 0 && hit != ~0ull) t.commit(hit);
+    });
+    rest_count(bd, evaluated);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRestThreads) cm_tie_rest_warp_kernel(Tables tb, BatchDev bd, int least_stages) {
+    __shared__ SProf<T> sp;
+    __shared__ uint8_t cuts_s[kRestThreads / 32][kMaxS + 8];
+    __shared__ uint8_t cut_col[kMaxS * kRestThreads];
+    __shared__ uint32_t left[kRestThreads / 32];
+    const uint32_t n = rest_open(bd);
+    if (n == 0) return;
+    stage_profile(sp, tb);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long evaluated = 0;
+    rest_tiles(bd, n, [&](int S) { return S >= least_stages; }, [&](const RestTile &t) {
+        const SegView &g = t.g;
+        const double goal = std::is_same<T, long long>::value ? __ll2double_ru((long long)t.w_bits) : __longlong_as_double((long long)t.w_bits);
+        const uint64_t pos = t.base + threadIdx.x;
+        bool maybe = false;
+        CutWalker cw;
+        if (pos < t.count && make_walker(cw, tb, bd.layer_mode, sp.L, g.S, walk_cand(bd, g.feas_first, pos), g.K, tb.mm_slot(g.S, g.m))) {
+            const CutColumn<kRestThreads> c{cut_col + threadIdx.x};
+            c.fill(cw, g.S);
+            const Walk walk = best_walk<T>(sp, c, g.S, g.m, g.tier, g.n_sync, g.feas_first == kNoFeasList);
+            maybe = walk.value >= 0.0 && walk.value <= goal;
+            if (maybe) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= t.w_bits;
+        }
+        const uint32_t vote = __ballot_sync(0xffffffffu, maybe);
+        if (lane == 0) left[warp] = vote;
+        __syncthreads();
+        // this warp's: every fourth of those left, upwards
+        bool more = true;
+        for (int q = 0, k = 0; q < kRestThreads / 32 && more; ++q)
+            for (uint32_t v = left[q]; v && more; v &= v - 1, ++k) {
+                if (k % (kRestThreads / 32) != warp) continue;
+                const Cand cand = walk_cand(bd, g.feas_first, t.base + q * 32 + __ffs((int)v) - 1);
+                const unsigned long long so_far = __shfl_sync(0xffffffffu, (unsigned long long)*t.slot, 0);
+                if (so_far <= cand.kappa) { more = false; continue; }
+                T cost;
+                if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, cand, cuts_s[warp], cost) && lane == 0 && Num<T>::bits(cost) <= t.w_bits)
+                    t.commit(cand.kappa);
+                if (lane == 0) ++evaluated;
+                __syncwarp();
+            }
+    });
+    rest_count(bd, evaluated);
+}
+
+cudaError_t launch_tie_rest(const Tables &t, const BatchDev &b, uint64_t stages, bool by_depth, cudaStream_t st, int *launches) {
+    if (b.B <= 0 || b.max_tiles_per_seg == 0 || b.dp_max == 0) return cudaSuccess;
+    const bool native = native_i64(b);
+    if (stages & ((1ull << kRegStagesMax) - 1ull)) {
+        if (native) cm_tie_rest_kernel<long long><<<kRestShallow, kRestThreads, 0, st>>>(t, b);
+        else cm_tie_rest_kernel<double><<<kRestShallow, kRestThreads, 0, st>>>(t, b);
+        ++*launches;
+    }
+    for (int S = kRegStagesMax + 1; by_depth && S <= kWideStagesMax; ++S)
+        if ((stages >> (S - 1)) & 1ull) {
+            const cudaError_t e = launch_tie_rest_deep(t, b, S, st);
+            if (e != cudaSuccess) return e;
+            ++*launches;
+        }
+    const int least = by_depth ? kWideStagesMax + 1 : kRegStagesMax + 1;
+    if (stages >> (least - 1)) {
+        if (native) cm_tie_rest_warp_kernel<long long><<<kRestWarps, kRestThreads, 0, st>>>(t, b, least);
+        else cm_tie_rest_warp_kernel<double><<<kRestWarps, kRestThreads, 0, st>>>(t, b, least);
+        ++*launches;
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st) {

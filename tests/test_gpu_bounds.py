@@ -184,3 +184,58 @@ def test_bounds_decide_where_one_stage_outweighs_the_others(gpu, oracle_factory,
             assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (f, plan, want)
     finally:
         gpu.cm_destroy(ctx)
+
+
+def _slow_links(deep, p2p, bw):
+    """Transfers about as long as the stages, on either link tier: the longest path changes between stages all
+    the time and bounds leave a part of the plans open."""
+    rng = np.random.default_rng(3 if deep else 1)
+    if deep:
+        L = 44
+        fwd = rng.uniform(5e6, 6e6, L).round()
+        profile = W.make_profile_ns(L, 2, 20, 48, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, p2p,
+                                    [0] + [round((i + 1) * L / 20) for i in range(20)], 80_000_000_000, 8, bw, bw)
+        return profile, W.SearchOptions(2, 2, 17, 22, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 16)
+    L = 32
+    fwd = (10e6 * (1 + 0.05 * rng.standard_normal(L))).round()
+    profile = W.make_profile_ns(L, 4, 8, 32, fwd, 2.0 * fwd, 16_777_216, 402_653_184, 2_415_919_104, p2p,
+                                list(range(0, 33, 4)), 80_000_000_000, 8, bw, bw)
+    return profile, W.SearchOptions(3, 5, 4, 12, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 16)
+
+
+@pytest.mark.parametrize("mode,native", [(0, False), (1, False), (1, True)])
+@pytest.mark.parametrize("deep,p2p,bw,copies", [(False, 50_000_000, 1, 0), (False, 16_777_216, 2, 40), (True, 8_000_000, 2, 0),
+                                                (True, 8_000_000, 2, 12)])
+def test_tie_break_that_bounds_do_not_decide(gpu, oracle_factory, deep, p2p, bw, copies, mode, native):
+    """Pipelines that the tie-break leaves open after a few recurrences, a failure on its own (copies 0) and a
+    batch, shallow and a launch per depth, and the shortlist's, which go on with a warp each."""
+    profile, opts = _slow_links(deep, p2p, bw)
+    opts = opts.with_cost_mode(mode)
+    sets = [[3], [5, 9], [1, 2, 20]] if not deep else [[3], [0, 9]]
+    orc = oracle_factory(profile, opts)
+    want = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_set_int64_arithmetic(ctx, native)
+        n_open = 0
+        for turn in range(3):   # (from the second on a failure on its own replays a graph)
+            for f, w in zip(sets, want) if not copies else [(sets, want)]:
+                got = gpu.plans_from_array(gpu.cm_search_batch(ctx, [f] if not copies else f * copies, opts, latency=not copies)[0])
+                n_open += gpu.cm_last_stats(ctx)["ties_open"]
+                for b, plan in enumerate(got):
+                    x = w if not copies else w[b % len(sets)]
+                    assert plan.key() == x.key() and plan.cost == x.cost and plan.cost_ns == x.cost_ns, (plan, x)
+        assert n_open > 0
+        space, _ = gpu.cm_enumerate(ctx, W.POLICY_DYNPAR, sets[0], opts)
+        dyn, one = orc.search_policy(sets[0], W.POLICY_DYNPAR), gpu.cm_select(ctx, [space])
+        assert one.key() == dyn.key() and (one.cost, one.cost_ns) == (dyn.cost, dyn.cost_ns)
+        gpu.cm_space_free(space)
+        if not native:
+            obj = W.ObjectiveOptions(topk=4)
+            best, _, short, moved, _ = gpu.cm_search_objective(ctx, sets[:1], opts, obj, shortlist=True)
+            plan, tr = orc.search_objective(sets[0], obj)
+            assert gpu.plans_from_array(best)[0].key() == plan.key()
+            assert [p.key() for r, p in enumerate(gpu.plans_from_array(short)) if moved[0, r] >= 0] == [p.key() for p in tr.shortlist]
+    finally:
+        gpu.cm_destroy(ctx)
