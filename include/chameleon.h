@@ -485,7 +485,7 @@ cm_status cm_cache_free(cm_cache *cache);
  *       on, [16] also leaves out what other scenarios' segments already covered)
  *  [20] recurrence cells that ran in the search pass  [21] pipeline-plans whose recurrence ran in it
  *  [22] pipelines of winning plans whose layer composition bounds left open (found in a second step)
- *  [23] reserved, 0. */
+ *  [23] searches that bounds left too many plans of and that were repeated without them */
 cm_status cm_last_stats(const cm_ctx *ctx, uint64_t out[24]);
 
 const char *cm_strerror(cm_status status);

@@ -145,6 +145,10 @@ struct Batch {
     // Bounded search pass (cm_bound.cu): its buckets and its device state.
     bool bounded = false;
     bool dense_only = false;              // a list was full: this batch is searched without bounds
+    // How many calls go without bounds after that: of a resident batch its own, of one that is built for a
+    // single search (one_shot) the context's (cm_ctx::overflow).
+    bool one_shot = false;
+    uint32_t dense_left = 0, dense_span = 0;
     std::vector<BBucket> bbucket;
     BoundDev bo{};
     size_t off_bbucket = 0;
@@ -206,6 +210,10 @@ struct cm_ctx {
     DevBuf<uint4> d_eval;             // cm_evaluate: candidates listed by depth
     DevBuf<uint4> d_bound_list;       // plans the bounded search pass lists for the recurrence
     bool uniform_p2p = false;         // every stage boundary moves the same bytes
+    // Searches of this profile whose lists were full (transfers about as long as the stages: bounds decide
+    // little).  The next `left` searches alike go without bounds; span is what the last refusal bought.
+    struct Overflow { cm_enum_opts opts; uint32_t form, span, left; };
+    std::vector<Overflow> overflow;
     bool screen = true;               // walk only the listed feasible compositions (cm_set_memory_screen)
     bool dedup = true;                // search a pipeline that several strategies of a survivor count share once (cm_set_pipeline_reuse)
     bool pairs = true;                // one recurrence for a pipeline's m and m+1 micro-batch variants (cm_set_micro_batch_pairs)
@@ -566,6 +574,23 @@ cm_status build_buckets(cm_ctx *ctx, Batch &bt) {
     return layout_buckets(ctx, bt, pre);
 }
 
+// Searches alike for cm_ctx::overflow: options, arithmetic, switches, size of the batch to a power of two.
+cm_ctx::Overflow *overflow_of(cm_ctx *ctx, const Batch &bt, bool add) {
+    uint32_t form = (bt.intval ? 1u : 0u) | (ctx->share ? 2u : 0u) | (ctx->screen ? 4u : 0u) | (ctx->dedup ? 8u : 0u);
+    for (int n = bt.B; n > 1; n >>= 1) form += 16;
+    for (cm_ctx::Overflow &o : ctx->overflow)
+        if (o.form == form && memcmp(&o.opts, &bt.opts, sizeof(o.opts)) == 0) return &o;
+    if (!add) return nullptr;
+    if (ctx->overflow.size() >= 64) ctx->overflow.clear();
+    ctx->overflow.push_back(cm_ctx::Overflow{bt.opts, form, 0, 0});
+    return &ctx->overflow.back();
+}
+// A search by bounds in vain costs about as much again as the direct one that follows (48 sets of the 256-device
+// job over links of 1 GB/s: 20 ms with, 11.2 without), so each doubles the number of searches until the
+// next try.
+constexpr uint32_t kDenseFirst = 4, kDenseMost = 256;
+uint32_t longer_span(uint32_t span) { return std::min(std::max(2 * span, kDenseFirst), kDenseMost); }
+
 // Work layout of the bounded search pass from the groups of segments it covers (BBucket: count, K,
 // list_first, n_seg, tmpl, feas_first, S, m, role, second filled in).  bt.bounded stays false where
 // the recurrences are too few to pay for the pass's launches.
@@ -589,6 +614,12 @@ cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups) {
         max_stages = std::max<int>(max_stages, g.S);
     }
     if (cells < (double)kBoundMinCells) return CM_OK;
+    if (cm_ctx::Overflow *o = bt.one_shot ? overflow_of(ctx, bt, false) : nullptr)
+        if (o->left) {
+            --o->left;
+            bt.dense_only = true;
+            return CM_OK;
+        }
     std::stable_sort(groups.begin(), groups.end(), [](const BBucket &a, const BBucket &b) { return a.S > b.S; });
     BoundDev bo{};
     for (int l = 0; l < 4; ++l) {
@@ -1184,6 +1215,7 @@ cm_status build_batch(cm_ctx *ctx, Batch &bt, const uint32_t *failed_ids, const 
     bt.n_tiles = bt.max_tiles_per_seg ? 1 : 0;   // only "is there anything to tie-break" matters
     bt.mm_launched = false;
     bt.bounded = bt.dense_only = false;
+    bt.dense_left = bt.dense_span = 0;
     bt.bbucket.clear();
     if (ctx->d_prof && ctx->screen) {   // (a context without a device only describes: cm_host_describe)
         const uint64_t t0 = now_ns();
@@ -1501,9 +1533,28 @@ cm_status finish_tiebreak(cm_ctx *ctx, Batch &bt, int *launches) {
     return CM_OK;
 }
 
+cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single = nullptr);
+
+// After a bounded search whose lists were full (bounds left hundreds of thousands of plans): again, every plan.
+cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *single) {
+    if (single && single->exec) { cudaGraphExecDestroy(single->exec); single->exec = nullptr; }
+    ++ctx->stats[23];
+    bt.dense_only = true;
+    bt.dense_left = bt.dense_span = longer_span(bt.dense_span);
+    if (bt.one_shot) {
+        cm_ctx::Overflow *o = overflow_of(ctx, bt, true);
+        o->left = o->span = longer_span(o->span);
+    }
+    const bool direct = bt.direct;
+    cm_status s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
+    if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
+    bt.direct = direct;
+    return s == CM_OK ? run_batch(ctx, bt, launches, single) : s;
+}
+
 // The search over an uploaded batch; results land in bt.plans_host ([B][4]) after the stream is
 // synchronised.  `single`: a resident one-scenario entry whose sequence may replay as a graph.
-cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single = nullptr) {
+cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single) {
     cudaStream_t st = ctx->stream;
     int launches = 0, cost_launches = 0;
     const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
@@ -1553,14 +1604,7 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
     }
     ctx->stats[10] += back_bytes;
     if (bt.bounded && search_counters(bt)[4]) {
-        // a list was full (plans whose bounds tie in their hundreds of thousands): search again, every plan
-        if (single && single->exec) { cudaGraphExecDestroy(single->exec); single->exec = nullptr; }
-        bt.dense_only = true;
-        const bool direct = bt.direct;
-        cm_status s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
-        if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
-        bt.direct = direct;
-        return s == CM_OK ? run_batch(ctx, bt, launches, single) : s;
+        return search_directly(ctx, bt, launches, single);
     }
     if (search_counters(bt)[6]) {
         cm_status s = finish_tiebreak(ctx, bt, &launches);
@@ -1630,6 +1674,15 @@ cm_status single_batch(cm_ctx *ctx, const uint32_t *ids, int n, const cm_enum_op
     if (ok)
         for (auto &e : ctx->single)
             if (e->n_surv == N - n && e->intval == intval && memcmp(&e->opts, &o, sizeof(o)) == 0) { hit = e.get(); break; }
+    uint32_t span = 0;
+    if (hit && hit->batch->dense_left && --hit->batch->dense_left == 0) {   // time to try bounds again
+        span = hit->batch->dense_span;
+        CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        for (auto &e : ctx->single)
+            if (e.get() == hit) { std::swap(e, ctx->single.back()); break; }
+        ctx->single.pop_back();
+        hit = nullptr;
+    }
     *entry = hit;
     if (!hit) {
         // (also the path of malformed sets: the builder produces the error)
@@ -1639,6 +1692,7 @@ cm_status single_batch(cm_ctx *ctx, const uint32_t *ids, int n, const cm_enum_op
         if (s == CM_OK) s = upload_batch(ctx, *b, launches);
         if (s != CM_OK) { cudaStreamSynchronize(ctx->stream); forget_keys(ctx, *b); return s; }
         b->direct = true;
+        b->dense_span = span;
         if (ctx->single.size() >= 64) {   // bounded: start over rather than grow without limit
             cudaStreamSynchronize(ctx->stream);
             ctx->single.clear();
@@ -1864,6 +1918,7 @@ cm_status cm_load_profile(cm_ctx *ctx, const cm_profile *p) {
     ctx->has_profile = false;
     ++ctx->profile_gen;                                  // spaces and batches of the old profile are refused from here on
     ctx->single.clear();                                 // prepared one-scenario batches describe the old profile
+    ctx->overflow.clear();
     for (auto &f : ctx->feas) f.clear();                 // so do the feasible-composition lists
     ctx->feas_used = 0;
     cm_status s = load_profile_host(ctx, p);
@@ -1942,6 +1997,7 @@ cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids
     if (!sp->own) return fail(ctx, CM_ENOMEM, "host memory");
     sp->failed.assign(failed_ids, failed_ids + n_failed);
     const int32_t offsets[2] = {0, n_failed};
+    sp->own->one_shot = true;
     s = build_batch(ctx, *sp->own, failed_ids, offsets, 1, o, 1u << policy);
     if (s == CM_OK) s = upload_batch(ctx, *sp->own, nullptr);
     if (s == CM_OK && policy != CM_DYNPAR) {
@@ -2061,7 +2117,7 @@ cm_status cm_select(cm_ctx *ctx, cm_space *const *spaces, int32_t n_spaces, cm_p
     for (int i = 0; i < n_spaces; ++i) {
         Batch &bt = *spaces[i]->own;
         if (spaces[i]->policy == CM_DYNPAR && (n_dyn > 1 || (bt.bounded && search_counters(bt)[4]))) {
-            s = run_batch(ctx, bt, 0);
+            s = n_dyn > 1 ? run_batch(ctx, bt, 0) : search_directly(ctx, bt, 0, nullptr);
             if (s != CM_OK) return s;
             continue;
         }
@@ -2102,6 +2158,7 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
     if (B == 0) return CM_OK;
     const uint32_t mask = (1u << CM_REROUTE) | (1u << CM_REDUNDANT) | (1u << CM_DYNPAR);
     Batch &bt = ctx->batch;
+    bt.one_shot = true;
     if (!latency_us) {
         int launches = 0;
         const uint64_t h0 = now_ns();
@@ -2154,6 +2211,7 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
     if (B == 0) return CM_OK;
     const uint32_t mask = (1u << CM_REROUTE) | (1u << CM_REDUNDANT) | (1u << CM_DYNPAR);
     Batch &bt = ctx->batch;
+    bt.one_shot = true;
     int launches = 0;
     const uint64_t h0 = now_ns();
     if ((s = build_batch(ctx, bt, failed_ids, offsets, B, *opts, mask)) != CM_OK) { forget_keys(ctx, bt); return s; }
@@ -2387,6 +2445,7 @@ cm_status cm_batch_prepare(cm_ctx *ctx, const uint32_t *failed_ids, const int32_
     if (!bp->own) return fail(ctx, CM_ENOMEM, "host memory");
     memset(ctx->stats, 0, sizeof(ctx->stats));
     const uint32_t mask = (1u << CM_REROUTE) | (1u << CM_REDUNDANT) | (1u << CM_DYNPAR);
+    bp->own->one_shot = false;
     s = build_batch(ctx, *bp->own, failed_ids, offsets, B, *opts, mask);
     if (s == CM_OK) s = upload_batch(ctx, *bp->own, &bp->prep_launches);
     if (s != CM_OK) {

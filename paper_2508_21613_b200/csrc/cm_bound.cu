@@ -305,7 +305,7 @@ template <typename T>
 __global__ void __launch_bounds__(kChunk) cm_list_shallow_kernel(Tables tb, BatchDev bd, BoundDev bo, int list) {
     __shared__ SProf<T> sp;
     const uint32_t n = list_length(bo, list);
-    if ((uint64_t)blockIdx.x * kChunk >= n) return;
+    if ((uint64_t)blockIdx.x * kChunk >= n || lists_full(bd)) return;
     stage_profile(sp, tb);
     __syncthreads();
     const uint4 *entries = bo.list + bo.list_first[list];
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kChunk, 5) cm_list_deep_kernel(Tables tb, Batc
     __shared__ SProf<T> sp;
     __shared__ uint8_t cuts_s[kChunk / 32][kMaxS + 8];
     const uint32_t n = list_length(bo, list);
-    if ((uint64_t)blockIdx.x * (kChunk / 32) >= n) return;
+    if ((uint64_t)blockIdx.x * (kChunk / 32) >= n || lists_full(bd)) return;
     stage_profile(sp, tb);
     __syncthreads();
     const uint4 *entries = bo.list + bo.list_first[list];

@@ -41,6 +41,10 @@ namespace cm {
 // has at most 2 (m + S) <= 8320 additions of one rounding each (2^-53), on either side.
 constexpr double kBoundSlack = 1.0 - 1.0 / (1ull << 36);
 
+// A list of the bounded search pass was full: the host repeats the search without bounds, and what is left of
+// this one need not run.
+__device__ __forceinline__ bool lists_full(const BatchDev &bd) { return *(volatile unsigned long long *)(bd.counters + 4) == 0ull; }
+
 // Layer cuts of a plan in a shared-memory column, one byte per stage, a plan per thread:
 // edge(i) = first layer of stage i, edge(S) = L.
 template <int STRIDE> struct CutColumn {

@@ -121,9 +121,10 @@ __global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, Bat
     const uint32_t tid = threadIdx.x;
     if (tid == 0) {
         bks = bo.bucket[bound_bucket(bo, blockIdx.x)];
-        n_act_s = 0;
+        n_act_s = lists_full(bd) ? -1 : 0;
     }
     __syncthreads();
+    if (n_act_s < 0) return;   // uniform (it only grows from 0)
     const BBucket &bk = bks;
     const BoundJob job = bound_job(bk, blockIdx.x);
     const BoundSmem sm = bound_smem(dyn, bo);

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
     const uint32_t b = blockIdx.x / bd.dp_max, p = blockIdx.x % bd.dp_max;
     const Winner &w = bd.winner[b];
     const uint64_t w_bits = w.cost_bits;
-    if (w_bits >= inf_bits<T>() || p >= w.dp) return;               // uniform over the CTA
+    if (w_bits >= inf_bits<T>() || p >= w.dp || lists_full(bd)) return;   // uniform over the CTA
     const SegView g = seg_view(bd, w.scen, w.seg[p]);
     if (g.K == 0) return;                                           // one candidate: known already
     stage_profile(sp, tb);

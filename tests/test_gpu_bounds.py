@@ -84,7 +84,8 @@ def test_bounded_search_against_the_oracle(gpu, oracle_factory, name, schedule):
 @pytest.mark.parametrize("mode", [0, 1])
 def test_search_with_more_ties_than_the_list_holds(gpu, oracle_factory, mode):
     """One layer holds all the time, so every composition of a pipeline ties with a quarter of a million
-    others: the list of plans left to the recurrence overflows and the search is repeated in full."""
+    others.  (Too little work for bounds: every plan is evaluated at once.  Lists that do overflow:
+    test_searches_whose_lists_overflow.)"""
     L = 24
     fwd = np.zeros(L)
     fwd[0] = 5e6
@@ -237,5 +238,56 @@ def test_tie_break_that_bounds_do_not_decide(gpu, oracle_factory, deep, p2p, bw,
             plan, tr = orc.search_objective(sets[0], obj)
             assert gpu.plans_from_array(best)[0].key() == plan.key()
             assert [p.key() for r, p in enumerate(gpu.plans_from_array(short)) if moved[0, r] >= 0] == [p.key() for p in tr.shortlist]
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_searches_whose_lists_overflow(gpu, oracle_factory, mode):
+    """Bounds that leave more plans than the lists hold: the search is repeated without them, searches alike go
+    without for a while (twice as long after every refusal), other searches are not held back, and a
+    new profile starts afresh.  Plans are the same throughout."""
+    profile, opts = _slow_links(True, 8_000_000, 1)
+    opts = opts.with_cost_mode(mode)
+    sets = [[3], [0, 9]]
+    orc = oracle_factory(profile, opts)
+    want = [orc.search(f)[0] for f in sets]
+
+    def check(arr):
+        for b, plan in enumerate(gpu.plans_from_array(arr)):
+            w = want[b % 2]
+            assert plan.key() == w.key() and plan.cost == w.cost and plan.cost_ns == w.cost_ns
+        return gpu.cm_last_stats(ctx)
+
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        tried = []
+        for call in range(1, 17):
+            st = check(gpu.cm_search_batch(ctx, sets * 20, opts)[0])
+            assert st["plans_run"] == st["plans_simulated"]
+            if st["repeated"]:
+                tried.append(call)
+        assert tried == [1, 6, 15]
+        # another size, then a failure on its own, resident: they find out for themselves
+        assert check(gpu.cm_search_batch(ctx, sets * 4, opts)[0])["repeated"] == 1
+        tried = [call for call in range(1, 15) if check(gpu.cm_search_batch(ctx, sets[:1], opts, latency=True)[0])["repeated"]]
+        assert tried == [1, 5, 13]
+        # spaces are made for one selection: the second one knows
+        for repeated in (1, 0, 0):
+            space, _ = gpu.cm_enumerate(ctx, W.POLICY_DYNPAR, sets[0], opts)
+            plan = gpu.cm_select(ctx, [space])
+            assert plan.cost == want[0].cost and plan.cost_ns == want[0].cost_ns and plan.kappa == want[0].kappa
+            assert gpu.cm_last_stats(ctx)["repeated"] == repeated
+            gpu.cm_space_free(space)
+        # a prepared batch keeps to what it found out
+        packed = gpu.PackedScenarios(sets * 20)
+        batch, _ = packed.prepare(ctx, opts)
+        for repeated in (1, 0, 0, 0, 0, 0):
+            packed.search_prepared(ctx, batch)
+            assert check(packed.best)["repeated"] == repeated
+        gpu.cm_batch_free(batch)
+        gpu.cm_load_profile(ctx, profile)
+        assert check(gpu.cm_search_batch(ctx, sets * 20, opts)[0])["repeated"] == 1
     finally:
         gpu.cm_destroy(ctx)
