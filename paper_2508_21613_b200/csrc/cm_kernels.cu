@@ -347,21 +347,27 @@ cudaError_t launch_useg_copy(const BatchDev &b, const USegDev &u, cudaStream_t s
 // Remainder rule: cm_split.cuh gives the step time; the R larger shares go where they must and then to the
 // lowest pipelines that may have them (colexicographic ranks grow with the highest element first).
 //
-// Full enumeration: a pipeline's best cost does not fall when it gets one more micro-batch, so a step time
-// t is within reach if the most micro-batches that every pipeline can take within t add up to G.  The
-// pipelines start with one each, t with the slowest of them; whoever can take one more within t does, and
-// where nobody can t moves to the least next cost.  The split of lowest rank gives the last pipelines as
-// many as they can take.  (Costs can fall only where the min-max partition is the only candidate and
-// memory forces a luckier one; such a strategy is seen and goes through its splits.)
+// Full enumeration: a step time t is within reach if shares that every pipeline can take within t add up to
+// G, and the least such t is found by halving the range between two costs.  A pipeline's best cost does not
+// fall when it gets one more micro-batch, so what it can take is all up to a largest share.  (Costs can fall
+// only where the min-max partition is the only candidate and memory forces a luckier one; such a strategy
+// is seen, and the sums within reach are kept as a set of bits.)  The split of lowest rank gives the last
+// pipelines as many as they can take.
 // ----------------------------------------------------------------------------------
+// Micro-batches from which halving takes fewer dependent loads than counting up (one failure of the 32-device job,
+// three pipelines, 8, 16, 32 and 64 micro-batches: 60, 70, 81 and 110 us a call counting, 64, 73, 79 and 95 halving).
+constexpr int kHalveFrom = 32;
 struct FullSplit {   // full enumeration, lane = pipeline
     const BatchDev &bd; const Tmpl &tp; const Scen &sc; const Strat &s;
     uint64_t inf;
-    __device__ __forceinline__ uint64_t cost(int m) const {   // of this lane's pipeline with m micro-batches
-        const int lane = threadIdx.x & 31;
-        if (lane >= (int)s.dp || m > (int)s.n_m) return inf;
-        const uint64_t v = bd.seg_best[canon_row(bd, tp, sc, s, lane, m - 1)];
+    __device__ __forceinline__ uint64_t share_cost(int p, int m) const {   // of pipeline p with m micro-batches
+        if (m < 1 || m > (int)s.n_m) return inf;
+        const uint64_t v = bd.seg_best[canon_row(bd, tp, sc, s, p, m - 1)];
         return v < inf ? v : inf;
+    }
+    __device__ __forceinline__ uint64_t cost(int m) const {                // of this lane's
+        const int lane = threadIdx.x & 31;
+        return lane < (int)s.dp ? share_cost(lane, m) : inf;
     }
     __device__ __forceinline__ bool monotone() const {
         bool ok = true;
@@ -372,34 +378,127 @@ struct FullSplit {   // full enumeration, lane = pipeline
         }
         return __all_sync(0xffffffffu, ok);
     }
-    __device__ __forceinline__ uint64_t best(int G) const {
-        const int dp = s.dp;
-        uint64_t t = ~warp_min_u64((threadIdx.x & 31) < dp ? ~cost(1) : ~0ull);
-        int m = 1, sum = dp;
-        uint64_t next = cost(2);
-        while (sum < G && t < inf) {
-            const bool more = next <= t;
-            const uint32_t who = __ballot_sync(0xffffffffu, more && next < inf);
-            if (who) {
-                sum += __popc(who);
-                if (more && next < inf) next = cost(++m + 1);
-            } else {
-                t = warp_min_u64(next);
-            }
+    // largest share of this lane's pipeline within t (0: none), costs growing
+    __device__ __forceinline__ int most(uint64_t t) const {
+        int lo = 0, hi = (threadIdx.x & 31) < (int)s.dp ? (int)s.n_m : 0;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (cost(mid) <= t) lo = mid; else hi = mid - 1;
         }
-        return t < inf ? t : inf;
+        return lo;
+    }
+    // Least step time, costs growing.
+    __device__ __forceinline__ uint64_t best(int G) const {
+        const int lane = threadIdx.x & 31, dp = s.dp;
+        // nobody does without a micro-batch, and one pipeline at least takes an equal share or more
+        const uint64_t one = ~warp_min_u64(lane < dp ? ~cost(1) : ~0ull), equal = lane < dp ? cost((G + dp - 1) / dp) : inf;
+        uint64_t lo = warp_min_u64(equal), hi = ~warp_min_u64(lane < dp ? ~equal : ~0ull);
+        lo = one > lo ? one : lo;
+        if (dp == 1 || lo >= inf) return lo;
+        if (G < kHalveFrom) {                          // everybody takes one more within t, and where nobody can t moves to the least next cost
+            uint64_t t = lo;
+            int m = most(t), sum = m;
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            uint64_t next = cost(m + 1);
+            while (sum < G && t < inf) {
+                const uint32_t who = __ballot_sync(0xffffffffu, next <= t);
+                if (who) {
+                    sum += __popc(who);
+                    if (next <= t) next = cost(++m + 1);
+                } else {
+                    t = warp_min_u64(next);
+                }
+            }
+            return t;
+        }
+        hi = hi > lo ? hi : lo;
+        if (hi >= inf) hi = inf;                       // not known to be within reach
+        for (uint64_t t = lo; lo < hi; t = lo + (hi - lo) / 2) {
+            const int m = most(t);
+            int sum = m;
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (sum >= G) hi = ~warp_min_u64(lane < dp ? ~cost(m) : ~0ull);
+            else lo = warp_min_u64(cost(m + 1));
+        }
+        return hi;
+    }
+    // The same whatever the costs.  Sums are of shares less one; `sets`: room for two of them (words bits
+    // each), `prefix` (or null) for one per pipeline: the sums of the pipelines below it.
+    // below, above: the largest cost up to t and the least one above.
+    __device__ __forceinline__ bool reach(uint64_t t, int G, int words, uint64_t *sets, uint64_t *prefix, uint64_t &below, uint64_t &above) const {
+        const int lane = threadIdx.x & 31;
+        uint64_t *now = sets, *next = sets + words, under = 0, over = inf;
+        for (int w = lane; w < words; w += 32) now[w] = w == 0 ? 1ull : 0ull;
+        __syncwarp();
+        for (int p = 0; p < (int)s.dp; ++p) {
+            if (prefix)
+                for (int w = lane; w < words; w += 32) prefix[p * words + w] = now[w];
+            for (int w = lane; w < words; w += 32) next[w] = 0ull;
+            __syncwarp();
+            for (int base = 0; base < (int)s.n_m; base += 32) {
+                const uint64_t c = share_cost(p, base + lane + 1);
+                const bool ok = c <= t && c < inf;
+                if (ok) under = c > under ? c : under;
+                else over = c < over ? c : over;
+                if (!__any_sync(0xffffffffu, ok)) continue;
+                const int skip = (base + lane) >> 6, bits = (base + lane) & 63;   // this lane's share moves the sums up by
+                for (int w = base >> 6; w < words; ++w) {
+                    uint64_t v = 0;
+                    if (ok && w >= skip) {
+                        v = now[w - skip] << bits;
+                        if (bits && w > skip) v |= now[w - skip - 1] >> (64 - bits);
+                    }
+                    const uint32_t v0 = __reduce_or_sync(0xffffffffu, (uint32_t)v), v1 = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
+                    if (lane == 0) next[w] |= ((uint64_t)v1 << 32) | v0;
+                }
+            }
+            __syncwarp();
+            uint64_t *swap = now; now = next; next = swap;
+        }
+        below = ~warp_min_u64(~under);
+        above = warp_min_u64(over);
+        const int goal = G - (int)s.dp;
+        const bool got = (now[goal >> 6] >> (goal & 63)) & 1ull;
+        __syncwarp();
+        return got;
+    }
+    __device__ __forceinline__ uint64_t best_any(int G, int words, uint64_t *sets) const {
+        uint64_t lo = 0, hi, above;
+        if (!reach(inf, G, words, sets, nullptr, hi, above)) return inf;
+        while (lo < hi) {
+            uint64_t below;
+            if (reach(lo + (hi - lo) / 2, G, words, sets, nullptr, below, above)) hi = below; else lo = above;
+        }
+        return hi;
     }
     // micro-batches of this lane's pipeline in the split of lowest rank within t, and that rank
-    __device__ __forceinline__ int micro(const uint64_t *binom, int G, uint64_t t, uint64_t &rank) const {
+    __device__ __forceinline__ int micro(const uint64_t *binom, int G, uint64_t t, bool growing, int words, uint64_t *sets, uint64_t *prefix,
+                                         uint64_t &rank) const {
         const int lane = threadIdx.x & 31, dp = s.dp;
-        int most = 1;
-        while (cost(most + 1) <= t && most < (int)s.n_m && lane < dp) ++most;
         int left = G, mine = 0, before = 0;
-        for (int p = dp - 1; p >= 0; --p) {
-            const int can = __shfl_sync(0xffffffffu, most, p), room = left - p;   // (the p pipelines below get one each at least)
-            const int take = can < room ? can : room;
-            left -= take;
-            if (lane == p) { mine = take; before = left; }                        // before: micro-batches of the pipelines below
+        if (growing) {
+            const int can_take = most(t);
+            for (int p = dp - 1; p >= 0; --p) {
+                const int can = __shfl_sync(0xffffffffu, can_take, p), room = left - p;   // (the p pipelines below get one each at least)
+                const int take = can < room ? can : room;
+                left -= take;
+                if (lane == p) { mine = take; before = left; }                            // before: micro-batches of the pipelines below
+            }
+        } else {
+            uint64_t below, above;
+            reach(t, G, words, sets, prefix, below, above);
+            left = G - dp;
+            for (int p = dp - 1; p >= 0; --p) {
+                int take = 0;
+                for (int base = ((int)s.n_m - 1) & ~31; base >= 0 && take == 0; base -= 32) {
+                    const int m = base + lane + 1, rest = left - (m - 1);
+                    const bool ok = m <= (int)s.n_m && rest >= 0 && share_cost(p, m) <= t && ((prefix[p * words + (rest >> 6)] >> (rest & 63)) & 1ull);
+                    const uint32_t who = __ballot_sync(0xffffffffu, ok);
+                    if (who) take = base + 32 - __clz((int)who);
+                }
+                left -= take - 1;
+                if (lane == p) { mine = take; before = left + p; }
+            }
         }
         rank = lane > 0 && lane < dp ? binom_at(binom, before - 1, lane) : 0ull;
         for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
@@ -407,8 +506,12 @@ struct FullSplit {   // full enumeration, lane = pipeline
     }
 };
 
-__global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev bd, uint64_t inf) {
-    __shared__ uint64_t rc[32], rx[32];
+// words: 64-bit words of a set of sums (full enumeration); dynamic shared memory: two sets per warp, then one per
+// pipeline.
+template <bool FULL>
+__global__ void __launch_bounds__(1024, 1) cm_best_split_kernel(Tables tb, BatchDev bd, uint64_t inf, int words) {
+    extern __shared__ uint64_t sum_sets[];
+    __shared__ uint64_t rc[32];
     __shared__ uint32_t ri[32];
     const uint32_t b = blockIdx.x;
     const Scen sc = bd.scen[b];
@@ -416,43 +519,30 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
     const Strat *strat = bd.strat + tp.strat_first;
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31, G = tb.prof->G;
-    const bool full = bd.batch_mode == CM_BATCH_FULL;
     auto cost_of = [&](const Strat &s) { return strat_cost(bd, tp, sc, s, inf, [&](uint32_t row) { return bd.seg_best[row]; }); };
-    uint64_t best_c = inf, best_x = ~0ull;   // best_x: the item, where the splits were gone through
+    uint64_t best_c = inf;
     uint32_t best_i = 0;
     if (sc.rep == b)   // (else it shares another scenario's search: nothing to tie-break here)
         for (uint32_t si = warp; si < tp.n_strat; si += warps) {
             const Strat &s = strat[si];
-            uint64_t v = inf, x = ~0ull;
-            if (!full) {
+            uint64_t v = inf;
+            if constexpr (!FULL) {
                 v = strat_best(cost_of(s), s, ~0ull, inf);
             } else if (s.n_m >= 1) {
                 const FullSplit fs{bd, tp, sc, s, inf};
-                if (fs.monotone()) {
-                    v = fs.best(G);
-                } else {
-                    for (uint64_t q = lane; q < s.n_split; q += 32) {
-                        const uint64_t item = s.split_first + q, t = item_step_time(tb, bd, tp, bd.seg_best + sc.seg_base, item, inf);
-                        if (pair_less(t, item, v, x)) { v = t; x = item; }
-                    }
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const uint64_t ov = __shfl_xor_sync(0xffffffffu, v, o), ox = __shfl_xor_sync(0xffffffffu, x, o);
-                        if (pair_less(ov, ox, v, x)) { v = ov; x = ox; }
-                    }
-                }
+                v = fs.monotone() ? fs.best(G) : fs.best_any(G, words, sum_sets + (size_t)warp * 2 * words);
             }
-            if (v < best_c) { best_c = v; best_i = si; best_x = x; }
+            if (v < best_c) { best_c = v; best_i = si; }
         }
-    if (lane == 0) { rc[warp] = best_c; ri[warp] = best_i; rx[warp] = best_x; }
+    if (lane == 0) { rc[warp] = best_c; ri[warp] = best_i; }
     __syncthreads();
     if (warp) return;
     best_c = lane < (int)warps ? rc[lane] : inf;
     best_i = lane < (int)warps ? ri[lane] : 0xffffffffu;
-    best_x = lane < (int)warps ? rx[lane] : ~0ull;
     for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o), ox = __shfl_xor_sync(0xffffffffu, best_x, o);
+        const uint64_t oc = __shfl_xor_sync(0xffffffffu, best_c, o);
         const uint32_t oi = __shfl_xor_sync(0xffffffffu, best_i, o);
-        if (oc < best_c || (oc == best_c && oi < best_i)) { best_c = oc; best_i = oi; best_x = ox; }
+        if (oc < best_c || (oc == best_c && oi < best_i)) { best_c = oc; best_i = oi; }
     }
     Winner &w = bd.winner[b];
     uint64_t *kappa = bd.kappa_sel + (size_t)b * kMaxP;
@@ -465,13 +555,9 @@ __global__ void __launch_bounds__(1024) cm_best_split_kernel(Tables tb, BatchDev
     const bool mine = lane < (int)s.dp;                               // lane = pipeline from here on
     int micro;
     uint64_t rank;
-    if (best_x != ~0ull) {
-        uint16_t split[kMaxP];
-        rank = best_x - s.split_first;
-        split_micro(tb.binom, bd.batch_mode, G, s, rank, split);
-        micro = mine ? split[lane & (kMaxP - 1)] : 0;
-    } else if (full) {
-        micro = FullSplit{bd, tp, sc, s, inf}.micro(tb.binom, G, best_c, rank);
+    if constexpr (FULL) {
+        const FullSplit fs{bd, tp, sc, s, inf};
+        micro = fs.micro(tb.binom, G, best_c, fs.monotone(), words, sum_sets, sum_sets + (size_t)warps * 2 * words, rank);
     } else {
         const uint64_t v = cost_of(s);
         const uint64_t lo = __shfl_sync(0xffffffffu, v, (2 * lane) & 31), hi = __shfl_sync(0xffffffffu, v, (2 * lane + 1) & 31);
@@ -507,7 +593,14 @@ cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t
     // A warp per strategy, latency of its dependent loads: all strategies at once up to a scenario per SM (64 sets
     // of the 64-device job: 8 us with 1024 threads, 12 with 256, 18 with 128), narrower CTAs beyond (515 sets of
     // the 32-device job: 20 us with 256 threads, 25 with 1024, 26 with 128; 1024 of the 256-device job 16, 27, 16).
-    cm_best_split_kernel<<<b.B, b.B <= 148 ? 1024 : 256, 0, st>>>(t, b, batch_inf_bits(b));
+    const unsigned threads = b.B <= 148 ? 1024 : 256;
+    if (b.batch_mode == CM_BATCH_FULL) {
+        const int words = t.binom_rows / 64 + 1;   // (the table has a row per micro-batch of the job at least)
+        const size_t bytes = (threads / 32 * 2 + kMaxP) * (size_t)words * sizeof(uint64_t);
+        cm_best_split_kernel<true><<<b.B, threads, bytes, st>>>(t, b, batch_inf_bits(b), words);
+    } else {
+        cm_best_split_kernel<false><<<b.B, threads, 0, st>>>(t, b, batch_inf_bits(b), 0);
+    }
     return cudaGetLastError();
 }
 

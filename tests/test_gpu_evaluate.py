@@ -117,6 +117,68 @@ def test_best_split(gpu, oracle_factory, batch_mode, n_micro):
                 gpu.cm_destroy(ctx)
 
 
+def _uneven(seed, n_dp, n_pp, n_micro, cap, act):
+    """Transfers and stashes that differ between layers: with one more micro-batch memory forces the min-max
+    partition elsewhere, at times to cheaper cuts."""
+    rng = np.random.default_rng(seed)
+    L = 12
+    fwd = rng.uniform(1e6, 3e6, L).round()
+    p2p = (rng.random(L) < 0.5) * 400_000_000 + 1_000_000
+    return W.make_profile_ns(L, n_dp, n_pp, n_micro, fwd, 2 * fwd, (rng.uniform(0.1, 1, L) * act).astype(np.int64),
+                             (rng.uniform(0.2, 1, L) * 1e8).astype(np.int64), 300_000_000, p2p,
+                             [round(i * L / n_pp) for i in range(n_pp + 1)], int(cap), 4, 30, 20)
+
+
+@pytest.mark.parametrize("seed,n_dp,n_pp,n_micro,cap,act", [(0, 3, 4, 6, 4e9, 5e8), (5, 3, 4, 6, 7e9, 1e9), (0, 2, 6, 40, 4e9, 5e8),
+                                                            (5, 2, 6, 40, 5e9, 1e9), (1, 3, 4, 6, 3e9, 1e9)])
+def test_best_split_where_costs_fall(gpu, oracle_factory, seed, n_dp, n_pp, n_micro, cap, act):
+    """A pipeline's best cost can fall when it gets one more micro-batch; the least step time over all splits
+    and the first split that has it have to be found all the same.  The last case fits nearly nowhere."""
+    p = _uneven(seed, n_dp, n_pp, n_micro, cap, act)
+    sets = [[0], [1, 7], [2, 3, 8]]
+    for mode in (0, 1):
+        opts = W.SearchOptions(1, 4, 2, 8, W.LAYERS_MINMAX, W.BATCH_FULL, 1 << 62, mode)
+        orc = oracle_factory(p, opts)
+        n, _, n_seg = orc.count(sets[0])
+        value = orc.evaluate(sets[0], idx=np.arange(n))[mode]
+        segs = [orc.segment(sets[0], s) for s in range(n_seg)]
+        by = {(g["strategy"], g["pipe"], g["m"]): value[g["first"]] for g in segs}
+        assert cap < 4e9 or any(v > by.get((s, q, m + 1), v) for (s, q, m), v in by.items())
+        ctx = gpu.cm_create(0)
+        try:
+            gpu.cm_load_profile(ctx, p)
+            best, _, _ = gpu.cm_search_batch(ctx, sets, opts)
+            for f, got in zip(sets, gpu.plans_from_array(best)):
+                want = orc.search(f)[0]
+                assert got.feasible == (want is not None and want.feasible)
+                if got.feasible:
+                    assert got.key() == want.key() and got.cost == want.cost and got.cost_ns == want.cost_ns
+        finally:
+            gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("layer_mode", [W.LAYERS_REMAINDER, W.LAYERS_MINMAX])
+@pytest.mark.parametrize("n_micro", [31, 32, 64])
+def test_best_split_of_many_micro_batches(gpu, oracle_factory, n_micro, layer_mode):
+    """62, 64 and 128 micro-batches over one to three pipelines."""
+    p = W.random_small(43, L=8, n_dp=2, n_pp=4, n_micro=n_micro).profile
+    for mode in (0, 1):
+        opts = W.SearchOptions(1, 3, 1, 8, layer_mode, W.BATCH_FULL, 1 << 62, mode)
+        orc = oracle_factory(p, opts)
+        ctx = gpu.cm_create(0)
+        try:
+            gpu.cm_load_profile(ctx, p)
+            sets = [[], [0], [0, 5], [1, 2, 3]]
+            best, _, _ = gpu.cm_search_batch(ctx, sets, opts)
+            for f, got in zip(sets, gpu.plans_from_array(best)):
+                want = orc.search(f)[0]
+                assert got.feasible == (want is not None and want.feasible)
+                if got.feasible:
+                    assert got.key() == want.key() and got.cost == want.cost and got.cost_ns == want.cost_ns
+        finally:
+            gpu.cm_destroy(ctx)
+
+
 def test_spaces_that_take_over_buffers(gpu, oracle_factory):
     """Spaces of different sizes made, freed and made again while others live: what a freed one leaves
     behind must not reach the next, and a selection over several sees each of them."""
