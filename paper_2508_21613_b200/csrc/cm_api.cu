@@ -90,6 +90,7 @@ struct Batch {
     std::vector<int> tmpl_of_nsurv;        // survivor count -> template, -1 = not built
     PinnedVec<unsigned char> arena;        // host image of the tables
     DevBuf<unsigned char> d_arena;
+    DevBuf<unsigned char> d_arena_first;   // what d_arena was before the search was repeated without bounds
     size_t off_scen = 0, off_tmpl = 0, off_strat = 0, off_tseg = 0, off_failed = 0, off_keys = 0,
            off_tmpl_scen = 0, off_bucket_tseg = 0, off_cross = 0, off_bucket = 0;
     PinnedVec<cm_plan> plans_host;
@@ -155,7 +156,7 @@ struct Batch {
     DevBuf<SearchWin> d_win;
     // device memory held (what a spare batch ties up)
     size_t bytes() const {
-        return d_arena.cap + 8 * (d_seg_best.cap + d_kappa_sel.cap + d_pol_cost.cap + d_utab.cap + d_useg.cap + d_short_kappa.cap) +
+        return d_arena.cap + d_arena_first.cap + 8 * (d_seg_best.cap + d_kappa_sel.cap + d_pol_cost.cap + d_utab.cap + d_useg.cap + d_short_kappa.cap) +
                sizeof(Winner) * (d_winner.cap + d_short_win.cap) + sizeof(cm_plan) * (d_plans.cap + d_short_plans.cap) +
                4 * (d_urep.cap + d_slot_of.cap + d_row_rep.cap + d_open.cap) + sizeof(SearchWin) * d_win.cap + sizeof(cm_transition) * d_trans.cap;
     }
@@ -1546,6 +1547,9 @@ cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *
         o->left = o->span = longer_span(o->span);
     }
     const bool direct = bt.direct;
+    // the tables are laid out anew beside the old ones: an evaluation of this space that was captured reads those
+    std::swap(bt.d_arena.p, bt.d_arena_first.p);
+    std::swap(bt.d_arena.cap, bt.d_arena_first.cap);
     cm_status s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
     if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
     bt.direct = direct;
@@ -2011,13 +2015,12 @@ cm_status cm_enumerate(cm_ctx *ctx, cm_policy policy, const uint32_t *failed_ids
         forget_keys(ctx, *sp->own);
         return s;
     }
-    // cm_evaluate only enqueues: the workspace it bins candidates in (once per context) is found here
+    // cm_evaluate only enqueues: the workspace it bins candidates in is found here, once per context and as large
+    // as any space needs (17 MB): captured evaluations carry its address, so it never moves.
     uint32_t slab = 0;
-    const uint64_t want = policy == CM_DYNPAR ? eval_workspace(stage_mask(*sp->own), &slab) : 0;
-    if (want > ctx->d_eval.cap) {
-        CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // growing frees the old block
-        if (!ctx->d_eval.reserve(want)) return fail(ctx, CM_ENOMEM, "device memory");
-    }
+    if (policy == CM_DYNPAR && !ctx->d_eval.cap && eval_workspace(stage_mask(*sp->own), &slab) &&
+        !ctx->d_eval.reserve(eval_workspace(~0ull, &slab)))
+        return fail(ctx, CM_ENOMEM, "device memory");
     sp->own->direct = true;
     if (n_candidates) *n_candidates = policy == CM_DYNPAR ? sp->own->n_cand : 1;
     *out = sp.release();

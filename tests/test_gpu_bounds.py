@@ -291,3 +291,43 @@ def test_searches_whose_lists_overflow(gpu, oracle_factory, mode):
         assert check(gpu.cm_search_batch(ctx, sets * 20, opts)[0])["repeated"] == 1
     finally:
         gpu.cm_destroy(ctx)
+
+
+def test_captured_evaluations_outlive_other_calls(gpu, oracle_factory):
+    """cm_evaluate in a CUDA graph: spaces that need more of the workspace, and a selection that lays the
+    space's own tables out again, must leave what the graph refers to in place."""
+    import torch
+    profile, opts = _slow_links(True, 8_000_000, 1)
+    few = W.SearchOptions(2, 2, 19, 20, opts.layer_mode, opts.batch_mode, opts.kappa_cap)
+    stream = torch.cuda.Stream()
+    ctx = gpu.cm_create(0, stream.cuda_stream)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        graphs = []
+        for o in (few, opts):
+            orc = oracle_factory(profile, o)
+            space, n = gpu.cm_enumerate(ctx, W.POLICY_DYNPAR, [3], o)
+            idx = np.sort(np.random.default_rng(5).integers(0, n, 20_000)).astype(np.int64)
+            want, _, want_feas = orc.evaluate([3], idx=idx)
+            dev = torch.from_numpy(idx).cuda()
+            cost, feas = torch.zeros(len(idx), dtype=torch.float64, device="cuda"), torch.zeros(len(idx), dtype=torch.uint8, device="cuda")
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.stream(stream):
+                gpu.cm_evaluate(ctx, space, 0, len(idx), dev, cost, None, feas)
+            torch.cuda.synchronize()
+            with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+                gpu.cm_evaluate(ctx, space, 0, len(idx), dev, cost, None, feas)
+            graphs.append((graph, cost, feas, want, want_feas, space, dev))
+        gpu.cm_select(ctx, [graphs[1][5]])
+        assert gpu.cm_last_stats(ctx)["repeated"] == 1
+        for graph, cost, feas, want, want_feas, _, _ in graphs:
+            with torch.cuda.stream(stream):
+                cost.zero_()
+                feas.zero_()
+                graph.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(feas.cpu().numpy(), want_feas) and np.array_equal(cost.cpu().numpy(), want)
+        del graph, graphs
+    finally:
+        gpu.cm_destroy(ctx)
