@@ -1000,15 +1000,20 @@ Tables tables(const cm_ctx *ctx, const Batch &bt);
 // captured again at their next use.
 cm_status grow_feas_pool(cm_ctx *ctx, size_t want) {
     if (want <= ctx->d_feas.cap) return CM_OK;
-    size_t nc = std::max<size_t>(want, std::max<size_t>(ctx->d_feas.cap * 2, 1u << 20));
+    size_t nc = 0;
     uint32_t *q = nullptr;
     ulonglong2 *qm = nullptr;
     CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (cudaMalloc((void **)&q, nc * sizeof(uint32_t)) != cudaSuccess || cudaMalloc((void **)&qm, nc * sizeof(ulonglong2)) != cudaSuccess) {
+    for (size_t room : {std::max<size_t>(want, std::max<size_t>(ctx->d_feas.cap * 2, 1u << 20)), want}) {   // room to grow, or just enough
+        if (cudaMalloc((void **)&q, room * sizeof(uint32_t)) == cudaSuccess && cudaMalloc((void **)&qm, room * sizeof(ulonglong2)) == cudaSuccess) {
+            nc = room;
+            break;
+        }
         cudaGetLastError();
         if (q) cudaFree(q);
-        return fail(ctx, CM_ENOMEM, "device memory");
+        q = nullptr;
     }
+    if (!nc) return fail(ctx, CM_ENOMEM, "device memory");
     if (ctx->feas_used) {
         cudaError_t e = cudaMemcpyAsync(q, ctx->d_feas.p, ctx->feas_used * sizeof(uint32_t), cudaMemcpyDeviceToDevice, ctx->stream);
         if (e == cudaSuccess)
@@ -1052,10 +1057,14 @@ cm_status ensure_feasible_lists(cm_ctx *ctx, Batch &bt) {
         new_first.push_back((uint32_t)used);
         used += g.K + 1;
     }
+    auto undo = [&]() { for (uint32_t k : new_keys) entry(k).listed = 0; };
     if (!new_keys.empty()) {
-        auto undo = [&]() { for (uint32_t k : new_keys) entry(k).listed = 0; };
-        cm_status s = grow_feas_pool(ctx, used);
-        if (s != CM_OK) { undo(); return s; }
+        const cm_status s = grow_feas_pool(ctx, used);
+        if (s != CM_OK) undo();
+        if (s == CM_ENOMEM) { new_keys.clear(); ctx->err.clear(); }   // no room for lists: these segments are walked in full
+        else if (s != CM_OK) return s;
+    }
+    if (!new_keys.empty()) {
         const size_t n = new_keys.size(), n_mm = bt.keys.size();
         // staging layout: K (8n) | keys (4n) | first (4n) | min-max keys (4 n_mm) | counts (4n, device -> host)
         const size_t off_key = 8 * n, off_first = off_key + 4 * n, off_mm = off_first + 4 * n, off_cnt = off_mm + 4 * n_mm;

@@ -331,3 +331,32 @@ def test_captured_evaluations_outlive_other_calls(gpu, oracle_factory):
         del graph, graphs
     finally:
         gpu.cm_destroy(ctx)
+
+
+def test_feasible_lists_that_find_no_room(gpu):
+    """A device whose memory others hold: compositions that cannot be listed are walked in full, with the
+    same plans."""
+    import torch
+    rng = np.random.default_rng(9)
+    L = 24
+    fwd = rng.uniform(2e6, 4e6, L).round()
+    profile = W.make_profile_ns(L, 2, 8, 16, fwd, 2.0 * fwd, 1_000_000_000, 50_000_000, 300_000_000, 8_000_000,
+                                list(range(0, 25, 3)), 40_000_000_000, 4, 300, 20)
+    opts = W.SearchOptions(2, 2, 7, 8, W.LAYERS_FULL, W.BATCH_FULL, 1 << 62)
+    sets = [[0], [9]]
+    plans = []
+    for hog in (False, True):
+        ctx = gpu.cm_create(0)
+        held = None
+        try:
+            gpu.cm_load_profile(ctx, profile)
+            gpu.cm_search_batch(ctx, sets, W.SearchOptions(2, 2, 7, 8, W.LAYERS_REMAINDER, W.BATCH_FULL, 1 << 62))
+            if hog:   # (the lists take 215 MB)
+                torch.cuda.empty_cache()
+                held = torch.empty(torch.cuda.mem_get_info()[0] - (120 << 20), dtype=torch.uint8, device="cuda")
+            plans.append(gpu.plans_from_array(gpu.cm_search_batch(ctx, sets, opts)[0]))
+        finally:
+            del held
+            torch.cuda.empty_cache()
+            gpu.cm_destroy(ctx)
+    assert plans[0] == plans[1] and plans[0][0].feasible
