@@ -360,3 +360,31 @@ def test_feasible_lists_that_find_no_room(gpu):
             torch.cuda.empty_cache()
             gpu.cm_destroy(ctx)
     assert plans[0] == plans[1] and plans[0][0].feasible
+
+
+@pytest.mark.parametrize("mode,native", [(0, False), (1, False), (1, True)])
+@pytest.mark.parametrize("per_node", [1, 2, 3])
+def test_bounds_of_pipelines_over_many_nodes(gpu, oracle_factory, per_node, mode, native):
+    """Equal transfers, nodes of one to three devices: pipelines of 17 to 22 stages cross five to twenty-one
+    node boundaries, on either side of the six that are kept in a list."""
+    rng = np.random.default_rng(81)
+    L = 40
+    fwd = rng.uniform(2.5e6, 3.5e6, L).round()
+    profile = W.make_profile_ns(L, 2, 20, 48, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 8_000_000,
+                                list(range(0, L + 1, 2)), 80_000_000_000, per_node, 300, 12)
+    sets = [[3], [20], [0, 9]]
+    opts = W.SearchOptions(2, 2, 17, 22, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15, mode)
+    orc = oracle_factory(profile, opts)
+    wants = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_set_int64_arithmetic(ctx, native)
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets * 20, opts)[0])
+        st = gpu.cm_last_stats(ctx)
+        assert 0 < st["plans_run"] < st["plans_simulated"]
+        for b, plan in enumerate(best):
+            want = wants[b % 3]
+            assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (sets[b % 3], plan, want)
+    finally:
+        gpu.cm_destroy(ctx)
