@@ -24,8 +24,8 @@
 // above ub, and the split reduction returns the same winner as with all minima exact.  For a shortlist
 // of k pairs, ub is the k-th best step time.  A segment that scenarios share goes by the least lo and the
 // largest ub of the scenarios it is marked for (1000 sets of the 256-device job, searched with sharing:
-// 1190 us; with the segment's own result for ub and nothing for lo 2380 us, or, where bounds miss and the
-// lists overflow, 8200 us).
+// 1190 us when this came, 963 now; with the segment's own result for ub and nothing for lo 2380 us, or, where
+// bounds miss and the lists overflow, 8200 us).
 #include <algorithm>
 
 #include "cm_bound_lane.cuh"

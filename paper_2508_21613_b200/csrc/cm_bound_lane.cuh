@@ -151,7 +151,8 @@ __device__ __forceinline__ float stay_pairs(int i, int S, int m) {
 // forward and backward are compared by the upper halves of their bit patterns.
 // The stages are a loop of four at a time whose results move up the registers: all of them in a row are
 // tens of kilobytes of code per depth that every CTA runs through once, and the warps waited for
-// instructions most of the time (1024 sets of the 256-device job: 2023 -> 1997 us a call; one: 148 -> 146 us).
+// instructions most of the time.  (The whole call changes by less than its runs differ: 1024 sets of the
+// 256-device job 2.0 ms either way.)
 // Where a stage may outweigh the others (busy) the walks along its whole order count as well.  Their values
 // depend on the link tiers through the boundaries that they leave out; with the dearer tier there they are one
 // number per lane.

@@ -21,7 +21,8 @@
 //       per-lane shared-memory column; for buckets with too few segments to transpose.
 //       S = 49..64 (transposed only): the pending forwards move to a per-lane shared-memory
 //       column as well; one CTA per SM.
-//   cm_cost_short_kernel<T>         S <= 16 with m < S-1: the rounds form, all in registers.
+//   cm_cost_short_kernel<T>         S <= 16 with m < S-1: the rounds form, all in registers, every depth in
+//       one launch beside the launches per depth (small batches: cm_cost_regs_any_kernel takes all m).
 #pragma once
 
 #include <atomic>
@@ -182,7 +183,8 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_pair_kernel(Tables tb, Ba
 }
 
 // Every shallow depth in one launch: for batches so small that a launch per depth would
-// cost more than the work (a single failure scenario of a 32-device job is ~250 CTAs).
+// cost more than the work (a single failure scenario of a 32-device job is ~250 CTAs).  The rounds form, any m;
+// cm_cost_short_kernel evaluates plans the same way and differs in how chunks are numbered.
 template <typename T>
 __global__ void __launch_bounds__(kChunk) cm_cost_regs_any_kernel(Tables tb, BatchDev bd, uint32_t b0, uint32_t b1) {
     __shared__ SProf<T> sp;

@@ -20,7 +20,7 @@ __device__ __forceinline__ EvalEntry eval_entry(const BatchDev &bd, const EvalDe
     const uint4 e = eval_region(ev, region)[i];
     const uint64_t word = (uint64_t)e.z | ((uint64_t)e.w << 32);
     EvalEntry x;
-    x.t = ev.base + (e.x & ~(kEvalMinMax | kEvalMasked));
+    x.t = ev.base + (e.x & ~kEvalMasked);
     x.g = seg_view(bd, 0, e.y);
     x.cand = e.x & kEvalMasked ? Cand{0, word, 0, true} : Cand{word, 0, 0, false};   // (a masked one is no min-max partition: any rank below K)
     return x;

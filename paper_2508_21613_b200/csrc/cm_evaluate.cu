@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(128) cm_evaluate_bin_kernel(Tables tb, BatchDe
             // (the mask of a remainder composition rides along, so that nobody unranks it again)
             const bool masked = ok && w.kind == 0;
             const uint64_t word = masked ? w.a : kappa;
-            const uint32_t flags = ok && w.kind == 2 ? kEvalMinMax : masked ? kEvalMasked : 0u;
+            const uint32_t flags = masked ? kEvalMasked : 0u;
             int lo = 0;
             for (int i = 0; i < g.S && ok; ++i) {
                 const int hi = w.next();

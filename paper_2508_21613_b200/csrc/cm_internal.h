@@ -228,7 +228,7 @@ struct BoundDev {
 constexpr int kCounters = 8;   // work counters of a search (BatchDev::counters)
 // Recurrence cells of a search (a shallow one counting a quarter) from which bounds pay for their extra
 // launches: 33 sets of the 32-device job with the full objective (just below) 506 us directly, 745 by bounds;
-// one failure of the 256-device job (4e8) 380 us directly, 259 by bounds when they came, 146 now.
+// one failure of the 256-device job (4e8) 380 us directly, 259 by bounds when they came, 155 now.
 constexpr uint64_t kBoundMinCells = 200000000ull;
 constexpr uint32_t kBoundListMin = 65536;        // plans a list has room for, at least (if there are as many)
 constexpr size_t kBoundDynMax = 160 * 1024;      // dynamic shared memory of the bound kernels, at most
@@ -388,7 +388,7 @@ struct EvalDev {
     uint32_t slab;            // candidates per round
     uint64_t base;            // first candidate of the round
 };
-constexpr uint32_t kEvalMinMax = 0x80000000u, kEvalMasked = 0x40000000u;   // flags of an entry's slot
+constexpr uint32_t kEvalMasked = 0x40000000u;   // flag of an entry's slot
 constexpr int kEvalShallow = kRegStagesMax, kEvalRest = kWideStagesMax + 1, kEvalRegions = kEvalRest + 1;   // regions by depth: up to 16, 17 .. 48, deeper
 constexpr uint32_t kEvalSlabMax = 1u << 18, kEvalListMax = 1u << 20;
 // Deep spaces: calls of up to this many candidates are evaluated a warp per candidate (about 10 us for a call
