@@ -151,6 +151,7 @@ struct Batch {
     bool one_shot = false;
     uint32_t dense_left = 0, dense_span = 0;
     std::vector<BBucket> bbucket;
+    uint64_t tile_mins = 0;               // entries of BoundDev::tile_min (0: none kept)
     BoundDev bo{};
     size_t off_bbucket = 0;
     DevBuf<SearchWin> d_win;
@@ -210,6 +211,8 @@ struct cm_ctx {
     DevBuf<unsigned char> d_feas_stage;
     DevBuf<uint4> d_eval;             // cm_evaluate: candidates listed by depth
     DevBuf<uint4> d_bound_list;       // plans the bounded search pass lists for the recurrence
+    DevBuf<SegRec> d_seg_rec;         // the segments of its layout
+    DevBuf<float> d_tile_min;         // its least bounds per tile of compositions and segment
     bool uniform_p2p = false;         // every stage boundary moves the same bytes
     // Searches of this profile whose lists were full (transfers about as long as the stages: bounds decide
     // little).  The next `left` searches alike go without bounds; span is what the last refusal bought.
@@ -629,37 +632,38 @@ cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups) {
         bo.list_first[l + 1] = bo.list_first[l] + (uint32_t)room;
     }
     // segments a CTA walks with one set of compositions; fewer where the grid would not fill the GPU
-    uint64_t chunks = 0, n_segs = 0;
-    int max_group = 1;
-    for (int most = bound_group(max_stages, ctx->uniform_p2p);; most = std::max(most / 2, 1)) {
-        chunks = n_segs = 0;
-        max_group = 1;
+    uint64_t chunks = 0, n_segs = 0, mins = 0;   // (mins: far below 2^64, chunks being limited)
+    for (int most = bound_group();; most /= 2) {
+        chunks = n_segs = mins = 0;
         for (BBucket &g : groups) {
-            int width = 1;   // (segments side by side: at most the group)
-            while (width < 128 && ((uint64_t)width < g.count || 128 / width > most)) width *= 2;
-            const int side = 128 / width;
-            int group = most / side * side;
-            group = (int)std::min<uint64_t>((uint64_t)group, ((uint64_t)g.n_seg + side - 1) / side * side);
+            int width = 1;
+            while (width < 128 && (uint64_t)width < g.count) width *= 2;
+            const int group = (int)std::min<uint64_t>((uint64_t)most, g.n_seg);
             g.width = (uint16_t)width;
             g.seg_group = (uint16_t)group;
             g.n_groups = (uint32_t)((g.n_seg + group - 1) / group);
             g.chunk_first = (uint32_t)chunks;
             g.seg_first = (uint32_t)n_segs;
-            chunks += (g.count + width - 1) / width * g.n_groups;
+            g.min_first = (uint32_t)mins;
+            const uint64_t tiles = (g.count + width - 1) / width;
+            chunks += tiles * g.n_groups;
+            mins += tiles * g.n_seg;
             n_segs += g.n_seg;
-            max_group = std::max(max_group, group);
             if (chunks >= 0x7fffffffull) return CM_OK;
         }
-        if (chunks >= 4 * 148 || most <= 8) break;
+        if (chunks >= 6 * 148 || most <= 32) break;
     }
+    bo.parts = 1;
+    for (const BBucket &g : groups) bo.parts = std::max<uint32_t>(bo.parts, ((uint32_t)g.seg_group + 127) / 128);
+    if (chunks * bo.parts >= 0x7fffffffull) return CM_OK;
     bo.n_buckets = (uint32_t)groups.size();
     bo.n_chunks = (uint32_t)chunks;
     bo.n_segs = (uint32_t)n_segs;
     bo.uniform_x = ctx->uniform_p2p ? 1 : 0;
-    bo.dyn_bytes = bound_dyn_bytes(bo, max_stages, max_group, ctx->uniform_p2p);
-    if (bo.dyn_bytes > kBoundDynMax) return CM_OK;
+    if (bound_dyn_bytes(bo, max_stages, ctx->uniform_p2p) > kBoundDynMax) return CM_OK;
     bt.bo = bo;
     bt.bbucket = groups;
+    bt.tile_mins = mins <= kTileMinMax ? mins : 0;
     bt.bounded = true;
     return CM_OK;
 }
@@ -1315,11 +1319,14 @@ Tables tables_plain(const cm_ctx *ctx) {   // for kernels that only read the byt
 
 constexpr size_t kStateExtra = kCounters + 2;   // work counters and the counts of four lists (32-bit)
 
-// Room for listed plans.  Captured launch sequences carry the list's address: dropped when it moves.
-cm_status reserve_bound_list(cm_ctx *ctx, size_t want) {
-    if (want <= ctx->d_bound_list.cap) return CM_OK;
+// Room for listed plans and, if there is memory for it, for the least bounds of tiles.  Captured launch sequences
+// carry the addresses: dropped when they move.
+cm_status reserve_bound_list(cm_ctx *ctx, Batch &bt) {
+    const size_t want = bt.bo.list_first[4], mins = bt.tile_mins, segs = bt.bo.n_segs;
+    if (want <= ctx->d_bound_list.cap && segs <= ctx->d_seg_rec.cap && mins <= ctx->d_tile_min.cap) return CM_OK;
     CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (!ctx->d_bound_list.reserve(want)) return fail(ctx, CM_ENOMEM, "device memory");
+    if (!ctx->d_tile_min.reserve(mins)) bt.tile_mins = 0;
+    if (!ctx->d_bound_list.reserve(want) || !ctx->d_seg_rec.reserve(segs)) return fail(ctx, CM_ENOMEM, "device memory");
     for (auto &e : ctx->single)
         if (e->exec) { cudaGraphExecDestroy(e->exec); e->exec = nullptr; }
     return CM_OK;
@@ -1395,7 +1402,7 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
             ctx->stats[9] += bt.bucket.size() * sizeof(Bucket);
         }
     }
-    if (bt.bounded) return reserve_bound_list(ctx, bt.bo.list_first[4]);
+    if (bt.bounded) return reserve_bound_list(ctx, bt);
     return CM_OK;
 }
 
@@ -1413,6 +1420,8 @@ cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchD
         bo.row_ub = bo.row_lo + bt.n_rows;
     }
     bo.list = ctx->d_bound_list.p;
+    bo.rec = ctx->d_seg_rec.p;
+    bo.tile_min = bt.tile_mins ? ctx->d_tile_min.p : nullptr;
     CM_CUDA(ctx, launch_bound(tb, bd, bo, st));
     ++*launches;
     for (int phase = 1; phase <= 2; ++phase) {

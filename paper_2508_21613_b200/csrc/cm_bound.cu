@@ -33,113 +33,108 @@
 
 namespace cm {
 
-// Bound by issue under shared-memory and arithmetic latency at three CTAs per SM: 201 thread-instructions per
-// plan, 43 % of the issue slots (64 sets of the 256-device job, 7.6 million plans: 122 us; 1024 sets, 75
-// million: 800 us, 1233 us before the additions were packed and the walks' terms kept in registers).
-// A CTA takes kBoundThreads / W segments side by side, W compositions each (W = a power of two that
-// holds the bucket's candidates, at most all threads), and walks its group of segments with the
-// composition's terms in registers.
-template <typename T, int NB, bool UNI_X>
-__device__ void bound_body(const SProf<T> &sp, const Tables &tb, const BatchDev &bd, const BBucket &bk, uint64_t tile0, int n_seg,
-                           const BoundSmem &sm) {
-    const int S = bk.S, m = bk.m, W = bk.width;
-    const uint32_t tid = threadIdx.x, lane = tid & 31;
-    const int sub = tid / W, n_sub = kBoundThreads / W;
-    if (UNI_X) fill_transfers<T, NB>(sm, sp, S, m, n_seg);
-    const uint64_t pos = tile0 + (tid & (W - 1));
-    LaneBound<NB> v;
-    v.ok = pos < bk.count;
-    if (v.ok) {
-        CutWalker w;
-        const CutColumn<kBoundThreads> cuts{sm.cut};
-        v.ok = make_walker(w, tb, bd.layer_mode, sp.L, S, walk_cand(bd, bk.feas_first, pos), bk.K, tb.mm_slot(S, m)) && cuts.fill(w, S);
-        if (v.ok) lane_setup<T, NB, UNI_X>(v, sp, cuts, S, m, bk.feas_first == kNoFeasList, sm.cd);
+// (figures below)
+// A CTA holds the terms of up to kBoundThreads compositions (a thread sets up one) and takes its group of segments
+// by them, kBoundSegs at a time, a lane per segment: the lane has the places of its segment's dear boundaries in
+// registers and goes through the compositions, one look-up, addition and maximum per dear boundary and no
+// reduction over lanes.  The warps share the compositions (or, where these are few, the segments).
+template <bool UNI_X, int NF>
+__device__ __forceinline__ unsigned long long least_bound(const float4 *comp, const unsigned char *terms, const SegHot &h, float delta, int c0, int c1) {
+    float least = __uint_as_float(0x7f800000u);
+    int at = 0;
+#pragma unroll 4
+    for (int c = c0; c < c1; ++c) {
+        const float4 v = comp[c];
+        const float value = bound_value<UNI_X, NF>(v.x, v.y, v.z, terms + c * kTermSize<UNI_X>, h, delta);
+        if (value < least) { least = value; at = c; }
     }
-    const int n_ok = __syncthreads_count(v.ok && sub == 0);
-    if (tid == 0 && n_ok) {   // what this pass decides: the plans, and the cells recurrences over them would take
-        const unsigned long long plans = (unsigned long long)n_ok * (unsigned long long)n_seg;
-        const unsigned long long cells = bk.role == 2 ? 0ull
-            : bk.role == 1 ? 2ull * S * (m + 1) + 3ull * S * (S - 1) / 2 : 2ull * S * m;
-        atomicAdd(&bd.counters[0], plans * cells);
-        atomicAdd(&bd.counters[2], plans);
-    }
-    const float slack = sp.intval || std::is_same<T, long long>::value ? 1.0f : 0.0f;
-    const int n_it = (n_seg + n_sub - 1) / n_sub;
-    const float none = __uint_as_float(0x7f800000u);
-#pragma unroll 2
-    for (int it = 0; it < n_it; ++it) {
-        const int s = it * n_sub + sub;
-        const float value = s < n_seg && v.ok ? lane_value<T, NB, UNI_X>(v, sp, S, m, s, sm) : none;
-        if (W >= 32) {   // (the lanes of a warp share the segment; one lane works on its minimum)
-            const float least = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(value)));   // (values are not negative)
-            const uint32_t who = __ballot_sync(0xffffffffu, value == least);
-            if (least < none && lane == (uint32_t)(__ffs(who) - 1))
-                sm.word[4 * s + (tid >> 5)] = ((unsigned long long)__float_as_uint(bound_of(value, slack)) << 32) | (uint32_t)pos;
-        } else {
-            unsigned long long key = value < none ? ((unsigned long long)__float_as_uint(bound_of(value, slack)) << 32) | (uint32_t)pos : ~0ull;
-            for (int o = W >> 1; o > 0; o >>= 1) {
-                const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
-                key = k2 < key ? k2 : key;
-            }
-            if (s < n_seg && (tid & (W - 1)) == 0 && key != ~0ull) sm.word[4 * s] = key;   // the only writer of its segment
-        }
-    }
+    return ((unsigned long long)__float_as_uint(least) << 32) | (uint32_t)at;
 }
 
 template <typename T, bool UNI_X>
 __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, BatchDev bd, BoundDev bo) {
     __shared__ SProf<T> sp;
     __shared__ BBucket bks;
-    extern __shared__ __align__(16) unsigned char dyn[];
-    const uint32_t tid = threadIdx.x;
-    if (tid == 0) bks = bo.bucket[bound_bucket(bo, blockIdx.x)];
+    __shared__ float4 comp[kBoundThreads];
+    __shared__ SegLite segs[kBoundSegs];
+    __shared__ unsigned long long word[kBoundThreads / 32][kBoundSegs];
+    extern __shared__ __align__(16) unsigned char terms[];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    find_bucket(bo, blockIdx.x, &bks);
     stage_profile(sp, tb);
     __syncthreads();
     const BBucket &bk = bks;
     const BoundJob job = bound_job(bk, blockIdx.x);
-    const BoundSmem sm = bound_smem(dyn, bo);
-    const int n_seg = (int)(job.s1 - job.s0);
-    for (int q = tid; q < n_seg; q += kBoundThreads) {
-        sm.segs[q] = seg_lite(tb, bound_segment(bd, bk, job.s0 + q));
-        for (int w = 0; w < 4; ++w) sm.word[4 * q + w] = ~0ull;   // a word per warp
+    const int S = bk.S, m = bk.m, W = bk.width, dear = dear_tier(tb);
+    const uint32_t tile0 = (uint32_t)job.tile0;   // (positions are 32-bit)
+    const bool any = (int)tid < W && tile0 + tid < bk.count;
+    Cand cand{0, 0, 0, false};
+    if (any) cand = walk_cand(bd, bk.feas_first, tile0 + tid);   // (on its way while the segments are looked up)
+    auto take_segments = [&](uint32_t base, int n_seg) {
+        if ((int)tid >= n_seg) return;
+        const BoundSeg g = bound_segment(bd, bk, base + tid);
+        segs[tid] = seg_lite(g.tier, g.row, g.n_sync, sp.bw_sync);
+        if (job.tile == 0) bo.rec[bk.seg_first + base + tid] = seg_record(g);
+    };
+    take_segments(job.s0, (int)min(job.s1 - job.s0, (uint32_t)kBoundSegs));
+    const LaneBound v = lane_of<T, UNI_X, false>(sp, tb, bd, bk, any, cand, dear, terms + tid * kTermSize<UNI_X>, nullptr);
+    comp[tid] = make_float4(v.best, v.u0, v.g, 0.0f);
+    const float delta = dear_extra(sp, dear), slack = sp.intval || std::is_same<T, long long>::value ? 1.0f : 0.0f;
+    const bool gpipe = sp.sched == CM_SCHED_GPIPE;
+    const int n_ok = __syncthreads_count(v.ok);
+    if (tid == 0 && n_ok) {   // what this pass decides: the plans, and the cells recurrences over them would take
+        const unsigned long long plans = (unsigned long long)n_ok * (unsigned long long)(job.s1 - job.s0);
+        const unsigned long long cells = bk.role == 2 ? 0ull
+            : bk.role == 1 ? 2ull * S * (m + 1) + 3ull * S * (S - 1) / 2 : 2ull * S * m;
+        atomicAdd(&bd.counters[0], plans * cells);
+        atomicAdd(&bd.counters[2], plans);
     }
-    __syncthreads();
-    const int nb = (bk.S + 3) >> 2;
-#define CM_NB(K) if (nb <= K) bound_body<T, K, UNI_X>(sp, tb, bd, bk, job.tile0, n_seg, sm); else
-    if constexpr (UNI_X && std::is_same<T, double>::value) { CM_NB(1) CM_NB(2) CM_NB(3) CM_NB(4) CM_NB(6) CM_NB(8) CM_NB(9) CM_NB(12) CM_NB(16) {} }
-    else { CM_NB(4) CM_NB(9) CM_NB(16) {} }
-#undef CM_NB
-    __syncthreads();
-    for (int q = tid; q < n_seg; q += kBoundThreads) {
-        unsigned long long least = sm.word[4 * q];
-        for (int w = 1; w < 4; ++w) least = sm.word[4 * q + w] < least ? sm.word[4 * q + w] : least;
-        if (least < bo.lbarg[sm.segs[q].row]) atomicMin((unsigned long long *)&bo.lbarg[sm.segs[q].row], least);
+    const int parts = W > 64 ? 4 : W > 32 ? 2 : 1, part = warp % parts;   // of the compositions
+    const int c0 = part * 32, c1 = W < 32 ? W : c0 + 32;
+    for (uint32_t base = job.s0; base < job.s1; base += kBoundSegs) {
+        const int n_seg = (int)min(job.s1 - base, (uint32_t)kBoundSegs);
+        if (base > job.s0) {
+            take_segments(base, n_seg);
+            __syncthreads();
+        }
+        for (int g = warp / parts * 32; g < n_seg; g += 128 / parts) {
+            const SegHot h = seg_hot<UNI_X>(segs[min(g + (int)lane, n_seg - 1)], S, dear, delta, gpipe);
+            unsigned long long key;
+#define CM_NF(N) case N: key = least_bound<UNI_X, N>(comp, terms, h, delta, c0, c1); break;
+            switch (__reduce_max_sync(0xffffffffu, h.n)) {
+                CM_NF(0) CM_NF(1) CM_NF(2) CM_NF(3) CM_NF(4) CM_NF(5) CM_NF(6)
+            default: key = least_bound<UNI_X, -1>(comp, terms, h, delta, c0, c1);
+            }
+#undef CM_NF
+            word[part][g + lane] = key;
+        }
+        __syncthreads();
+        if ((int)tid < n_seg) {
+            unsigned long long least = word[0][tid];
+            for (int w = 1; w < parts; ++w) least = word[w][tid] < least ? word[w][tid] : least;
+            const float value = __uint_as_float((uint32_t)(least >> 32)), lb = bound_of(value, slack);
+            if (bo.tile_min) bo.tile_min[bk.min_first + job.tile * bk.n_seg + base + tid] = lb;
+            if (value < __uint_as_float(0x7f800000u)) {
+                least = ((unsigned long long)__float_as_uint(lb) << 32) | (tile0 + (uint32_t)least);
+                unsigned long long *row = (unsigned long long *)&bo.lbarg[segs[tid].row];
+                if (least < *row) atomicMin(row, least);
+            }
+        }
+        __syncthreads();
     }
 }
+static_assert(kDearMax == 6, "the cases above");
 
-// Segments a CTA walks with one set of compositions, and the layout of its shared memory.  Three CTAs per
-// SM are wanted up to 36 stages; a deeper pipeline's columns alone take a third of an SM.
-int bound_group(int max_stages, bool uniform_x) {
-    BoundDev bo{};
-    const size_t fixed = bound_dyn_bytes(bo, max_stages, 0, uniform_x), per = (bound_dyn_bytes(bo, max_stages, 1024, uniform_x) - fixed) / 1024;
-    const size_t target = std::max<size_t>(kBoundDynTarget, fixed + 16 * 1024);
-    return (int)std::min<size_t>(255, std::max<size_t>(16, (target - fixed) / std::max<size_t>(per, 1)));
-}
-size_t bound_dyn_bytes(BoundDev &bo, int max_stages, int max_group, bool uniform_x) {
-    size_t nb = (size_t)(max_stages + 3) / 4;
-    for (size_t k : kBoundNb)
-        if (nb <= k) { nb = k; break; }
-    const size_t n = (size_t)max_group, columns = (size_t)max_stages * kBoundThreads;
-    size_t off = uniform_x ? n * 16 * nb : 0;
-    bo.dyn_far = (uint32_t)off;
-    off += uniform_x ? n * kFarMax * sizeof(FarVisit) : 0;
-    bo.dyn_cols = (uint32_t)off;
-    off += columns * sizeof(float2);
-    bo.dyn_cuts = (uint32_t)off;
-    off += columns;
-    bo.dyn_segs = (uint32_t)off;
-    bo.max_group = (uint32_t)max_group;
-    return off + n * (sizeof(SegLite) + sizeof(unsigned long long) + kRefineSegBytes);   // (cm_bound_kernel: four words, nothing else)
+// Segments that a CTA takes by one set of compositions: setting those up costs about as much as 128 segments.
+constexpr int kBoundGroup = 384;
+int bound_group() { return kBoundGroup; }
+// Dynamic shared memory: terms; cm_refine_kernel, from dyn_cuts on, cuts [stages][threads] bytes.
+size_t bound_dyn_bytes(BoundDev &bo, int max_stages, bool uniform_x) {
+    const size_t terms = (size_t)max_stages * kTermRow * (uniform_x ? kTermSize<true> : kTermSize<false>);
+    bo.dyn_cuts = (uint32_t)terms;
+    bo.dyn_bytes = terms;
+    bo.dyn_refine = terms + (size_t)max_stages * kBoundThreads;
+    return bo.dyn_refine;
 }
 
 template <typename T, bool UNI_X>
@@ -260,17 +255,13 @@ cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo
 __global__ void __launch_bounds__(128) cm_gather_kernel(Tables tb, BatchDev bd, BoundDev bo) {
     const uint32_t at = blockIdx.x * 128 + threadIdx.x;
     if (at >= bo.n_segs) return;
-    uint32_t lo = 0, hi = bo.n_buckets - 1;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1) >> 1;
-        if (bo.bucket[mid].seg_first <= at) lo = mid; else hi = mid - 1;
-    }
-    const BBucket bk = bo.bucket[lo];
-    const BoundSeg g = bound_segment(bd, bk, at - bk.seg_first);
+    const SegRec g = bo.rec[at];
     const uint64_t la = bo.lbarg[g.row], key = bo.pick[g.row];
     if (la == ~0ull || key == ~0ull) return;   // nothing fits in memory / not needed
-    const uint32_t pos = key == kPickWanted ? (uint32_t)la : (uint32_t)(key & ((1ull << pick_bits(bk.count)) - 1ull));
-    list_append(bd, bo, bk.S <= kRegStagesMax ? 0 : 1, g.scen, g.tseg, pos);
+    const TSeg &ts = bd.tseg[g.tseg];
+    const uint64_t count = ts.feas_first != kNoFeasList ? (uint64_t)ts.feas_count : ts.K ? ts.K + 1 : 1;
+    const uint32_t pos = key == kPickWanted ? (uint32_t)la : (uint32_t)(key & ((1ull << pick_bits(count)) - 1ull));
+    list_append(bd, bo, ts.S <= kRegStagesMax ? 0 : 1, g.scen, g.tseg, pos);
 }
 
 cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st) {

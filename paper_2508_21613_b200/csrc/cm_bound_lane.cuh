@@ -11,38 +11,19 @@ namespace cm {
 // issue slots).
 constexpr float kFloatSlack = 1.0f - 1.0f / (1 << 22);
 constexpr float kTieWindow = 1.0f / (1 << 18);     // bounds this close to the least one of a segment are compared bit for bit
-constexpr int kBoundThreads = 128;
+constexpr int kBoundThreads = 128;                 // compositions side by side
 constexpr float kNoWalk = -__builtin_huge_valf();   // value of a walk that does not exist
 
-// What the bound of a segment needs: its link tiers, its row, the synchronisation time per gradient byte,
-// how many of its inter-node boundaries are in the list of visits (kFarLong: too many, see lane_value).
-struct SegLite { uint64_t tier; uint32_t row; float coef; int n_sync, n_far; };
-// A visit across an inter-node boundary between stages `at` and at+1: what it adds to the lane's terms.
-struct FarVisit { float up, down; int at, pad; };
-constexpr int kFarMax = 6, kFarLong = kFarMax + 1;
-// Shared memory of a bound CTA, in this order: transfers above every stage [group][4 NB] floats (UNI_X) |
-// visits [group][kFarMax] (UNI_X) | visit terms [stages][threads] float2 | cuts [stages][threads] bytes |
-// segments [group] | a 64-bit word per segment | what else the kernel keeps per segment.
-struct BoundSmem {
-    float *xs;
-    FarVisit *far;
-    float2 *cd;       // this thread's column
-    uint8_t *cut;     // this thread's column
-    SegLite *segs;
-    unsigned long long *word;
-    unsigned char *rest;
-};
-__device__ __forceinline__ BoundSmem bound_smem(unsigned char *dyn, const BoundDev &bo) {
-    BoundSmem m;
-    m.xs = reinterpret_cast<float *>(dyn);
-    m.far = reinterpret_cast<FarVisit *>(dyn + bo.dyn_far);
-    m.cd = reinterpret_cast<float2 *>(dyn + bo.dyn_cols) + threadIdx.x;
-    m.cut = dyn + bo.dyn_cuts + threadIdx.x;
-    m.segs = reinterpret_cast<SegLite *>(dyn + bo.dyn_segs);
-    m.word = reinterpret_cast<unsigned long long *>(dyn + bo.dyn_segs + sizeof(SegLite) * bo.max_group);
-    m.rest = reinterpret_cast<unsigned char *>(m.word + bo.max_group);
-    return m;
-}
+// What a CTA keeps of a segment: its link tiers, its row, the synchronisation time per gradient byte.
+struct SegLite { uint64_t tier; uint32_t row; float coef; };
+constexpr int kDearMax = 6;    // dear boundaries (those on the slower link tier) that are looked up by a list
+// Terms of a CTA's compositions: [stages][kBoundThreads + 1] floats (UNI_X) or float2, a column per composition.
+// A row is one word longer than the threads, so that lanes with a segment each, which look at different rows of
+// one column, use different banks.
+constexpr int kTermRow = kBoundThreads + 1;
+template <bool UNI_X> constexpr uint32_t kTermSize = UNI_X ? sizeof(float) : sizeof(float2);
+constexpr int kBoundSegs = 128;   // segments whose data a CTA holds at a time
+static_assert(kBoundSegs == kBoundThreads, "a thread per segment");
 
 __device__ __forceinline__ bool native_i64_dev(const BatchDev &b) { return b.mode == CM_COST_INT64NS && !b.intval; }
 __device__ __forceinline__ float lb_of(uint64_t lbarg) { return __uint_as_float((uint32_t)(lbarg >> 32)); }
@@ -82,21 +63,17 @@ __device__ __forceinline__ BoundSeg bound_segment(const BatchDev &bd, const BBuc
     static_cast<SegView &>(v) = seg_view(bd, v.scen, v.tseg);
     return v;
 }
-__device__ __forceinline__ SegLite seg_lite(const Tables &tb, const BoundSeg &g) {
-    SegLite s{g.tier, g.row, 0.0f, g.n_sync, 0};
-    if (g.n_sync > 1) s.coef = __double2float_rd((2.0 * (double)(g.n_sync - 1)) / ((double)g.n_sync * (double)tb.prof->bw_sync));
-    return s;
-}
+// What the kernels after cm_bound_kernel need to know about a segment of the layout (its number q through all buckets).
+__device__ __forceinline__ SegRec seg_record(const BoundSeg &g) { return SegRec{g.tier, g.row, g.scen, g.tseg, g.n_sync}; }
 
 // Bucket, tile of compositions and group of segments of a CTA.
 struct BoundJob { uint32_t tile, group, s0, s1; uint64_t tile0; };
-__device__ __forceinline__ uint32_t bound_bucket(const BoundDev &bo, uint32_t cta) {
-    uint32_t lo = 0, hi = bo.n_buckets - 1;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1) >> 1;
-        if (bo.bucket[mid].chunk_first <= cta) lo = mid; else hi = mid - 1;
+// The bucket of CTA number `cta`, into shared memory (all threads; one load deep where halving takes six).
+__device__ __forceinline__ void find_bucket(const BoundDev &bo, uint32_t cta, BBucket *out) {
+    for (uint32_t t = threadIdx.x; t < bo.n_buckets; t += kBoundThreads) {
+        const uint32_t first = bo.bucket[t].chunk_first, next = t + 1 < bo.n_buckets ? bo.bucket[t + 1].chunk_first : bo.n_chunks;
+        if (first <= cta && cta < next) *out = bo.bucket[t];
     }
-    return lo;
 }
 __device__ __forceinline__ BoundJob bound_job(const BBucket &bk, uint32_t cta) {
     BoundJob j;
@@ -109,31 +86,11 @@ __device__ __forceinline__ BoundJob bound_job(const BBucket &bk, uint32_t cta) {
     return j;
 }
 
-// Maximum of three and two additions (rounded down) in one instruction each.
-__device__ __forceinline__ float max3(float a, float b, float c) {
+__device__ __forceinline__ float max3(float a, float b, float c) {   // one instruction
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ float2 add2_rd(float2 a, float2 b) {
-    uint64_t x, y, z;
-    float2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
-    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(z) : "l"(x), "l"(y));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(z));
-    return r;
-}
-
-// Everything a lane knows about its layer composition: b[i] + X_i is the best walk through stage i
-// whose visits stay on the cheaper link tier, X_i = 2 * (transfers of boundaries i .. S-2).
-template <int NB> struct LaneBound {
-    float2 b[2 * NB];
-    float u0, once, g;
-    bool ok;
-    __device__ __forceinline__ float get(int i) const { return i & 1 ? b[i >> 1].y : b[i >> 1].x; }
-    __device__ __forceinline__ void set(int i, float v) { if (i & 1) b[i >> 1].y = v; else b[i >> 1].x = v; }
-};
 
 // Stays at stage i in its own walk (negative: the walk does not exist), and the pairs of them that
 // visits can replace.
@@ -143,169 +100,198 @@ __device__ __forceinline__ float stay_pairs(int i, int S, int m) {
     return n > 1 ? (float)(n >> 1) : 0.0f;
 }
 
-// cd (shared memory, a column per thread): entry i = the walks that visit across boundary i, from stage i
-// upwards and from stage i+1 downwards, without the boundary's transfers.
-//
-// This is a third of the kernel's instructions, so double arithmetic is kept to the sums that cancel or
-// grow (six operations a stage); what is left is done in floats rounded down, and the slowest single
-// forward and backward are compared by the upper halves of their bit patterns.
-// The stages are a loop of four at a time whose results move up the registers: all of them in a row are
-// tens of kilobytes of code per depth that every CTA runs through once, and the warps waited for
-// instructions most of the time.  (The whole call changes by less than its runs differ: 1024 sets of the
-// 256-device job 2.0 ms either way.)
-// Where a stage may outweigh the others (busy) the walks along its whole order count as well.  Their values
-// depend on the link tiers through the boundaries that they leave out; with the dearer tier there they are one
-// number per lane.
-template <typename T, int NB, bool UNI_X>
-__device__ __forceinline__ void lane_setup(LaneBound<NB> &v, const SProf<T> &s, const CutColumn<kBoundThreads> &w, int S, int m, bool check, float2 *cd) {
+// Which of the two link tiers is the dearer one, and its boundaries among a segment's S-1.
+__device__ __forceinline__ int dear_tier(const Tables &tb) { return tb.prof->bw_inter <= tb.prof->bw_intra ? 1 : 0; }
+__device__ __forceinline__ uint64_t dear_bits(uint64_t tier, int dear, int S) {
+    return (dear ? tier : ~tier) & ((1ull << (S - 1)) - 1ull);
+}
+// Transfer times of the boundary after a layer, twice, over the cheaper tier and over the dearer one, rounded either way.
+struct Transfers { float lo_rd, lo_ru, hi_rd, hi_ru; };
+template <typename T> __device__ __forceinline__ Transfers transfers_at(const SProf<T> &s, int layer, int dear) {
+    const double lo = 2.0 * (double)s.XT[dear ^ 1][layer], hi = 2.0 * (double)s.XT[dear][layer];
+    return Transfers{__double2float_rd(lo), __double2float_ru(lo), __double2float_rd(hi), __double2float_ru(hi)};
+}
+
+// What a lane knows about its layer composition.  With k dear boundaries from stage i upwards (k of their extra
+// time Delta each in a transfer up and one down) and P_i the cheap transfers below stage i, the walk through
+// stage i has a value b_i - P_i + k Delta, all of it but k a matter of the composition.  As k grows downwards, the best
+// of all walks is the best of: max over every i of (b_i - P_i), and for the k-th dear boundary from the top,
+// after stage j, max over i <= j of (b_i - P_i), plus k Delta.  (Stages further down have more dear boundaries above
+// them than k, and their turn comes with the next one.)  The visits across that boundary at its dear price join
+// in: one term per (composition, boundary), and a segment costs one addition and one maximum per dear boundary
+// instead of one per stage.
+// best: the walks that need no dear boundary; u0: the climb and the drop, the cheap transfers included, and once
+// more those that best and the terms are short of.
+struct LaneBound {
+    float best, u0, g;
+    bool ok;
+};
+
+// Terms of a composition, stage after stage upwards; the boundary below stage i is complete once the stage is known.
+// Transfers that depend on the layer (!UNI_X) bring their Delta along in the terms.
+// Double arithmetic is kept to the sums that cancel or grow; what is left is done in floats rounded down,
+// and the slowest single forward and backward are compared by the upper halves of their bit patterns.
+// Where a stage may outweigh the others (busy) the walks along its whole order count as well, with the dearer
+// transfers in what they leave out: one number per lane.
+template <typename T, bool UNI_X, bool CUTS>
+__device__ __forceinline__ void lane_setup(LaneBound &v, const SProf<T> &s, CutWalker w, int S, int m, bool check, int dear,
+                                           unsigned char *term_col, uint8_t *cut_col) {
     const bool gpipe = s.sched == CM_SCHED_GPIPE, busy = s.heavy_stage(S);
-    float busy_best = 0.0f, U_hi = 0.0f;              // U_hi: U_i with the dearer transfers, rounded up
-    double U = 0.0, w_n = 0.0;                        // w_n: of stage i+1
-    float base_n = kNoWalk, c_n = kNoWalk, xq_n = 0.0f, q_n = 0.0f;
-    const float xm_all = __double2float_rd((double)(s.XT[0][0] < s.XT[1][0] ? s.XT[0][0] : s.XT[1][0]));
-    int fmax = 0, bmax = 0;
+    constexpr uint32_t row = kTermRow * kTermSize<UNI_X>;
+    const T TF = s.PF[s.L], TB = s.PB[s.L];
+    Transfers x = transfers_at(s, 0, dear);           // of the boundary below stage i
+    float best = kNoWalk, busy_rel = kNoWalk, busy_best = 0.0f;
+    float base_p = kNoWalk, down_p = kNoWalk, q_p = 0.0f;   // of stage i-1: its own walk, the best visit downwards
+    double w_p = 0.0, P = 0.0, H = 0.0;               // transfers below stage i, over the cheaper and over the dearer tier
+    float P_p = 0.0f;                                 // below stage i-1, rounded up
+    int fmax = 0, bmax = 0, lo = 0;
     long long g_max = 0;
-    int hi = s.L;
-#pragma unroll
-    for (int j = 0; j < 2 * NB; ++j) v.b[j] = make_float2(kNoWalk, kNoWalk);
-#pragma unroll 1
-    for (int k = (S - 1) >> 2; k >= 0; --k) {   // four stages a turn, topmost first
-#pragma unroll
-        for (int r = 3; r >= 0; --r) {
-            const int i = 4 * k + r;
-            if (i < S) {
-                const int lo = w.edge(i);
-                if (check && (hi <= lo || !stage_fits(s.PS[hi] - s.PS[lo], s.PA[hi] - s.PA[lo], i, S, m, s.cap, s.sched))) v.ok = false;
-                const double f = (double)(s.PF[hi] - s.PF[lo]), bk = (double)(s.PB[hi] - s.PB[lo]), wi = f + bk;
-                const long long g = s.PP[hi] - s.PP[lo];
-                g_max = g > g_max ? g : g_max;
-                fmax = max(fmax, __double2hiint(f));
-                bmax = max(bmax, __double2hiint(bk));
-                U += wi;
-                if (!gpipe) {
-                    const int n = stays(i, S, m);
-                    const float q = stay_pairs(i, S, m);
-                    float xm = xm_all, d = kNoWalk;
-                    if (!UNI_X) xm = __double2float_rd((double)(s.XT[0][hi - 1] < s.XT[1][hi - 1] ? s.XT[0][hi - 1] : s.XT[1][hi - 1]));
-                    const double dw = wi - w_n;
-                    if (i < S - 1) {   // stage i+1 is complete now that its lower neighbour is known
-                        if (q_n > 0.0f) d = __fmaf_rd(q_n, __double2float_rd(dw), base_n);
-                        const float up = c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n);
-                        v.set(r == 3 ? 0 : r + 1, max3(base_n, up, __fmaf_rd(2.0f * q_n, xm, d)));   // (r == 3: not shifted yet)
-                    }
-                    base_n = n >= 0 ? __double2float_rd(__fma_rd((double)n, wi, U)) : kNoWalk;
-                    c_n = q > 0.0f && i < S - 1 ? __fmaf_rd(q, __double2float_rd(-dw), base_n) : kNoWalk;
-                    cd[i * kBoundThreads] = make_float2(c_n, d);
-                    w_n = wi; q_n = q; xq_n = __fmul_rd(2.0f * q, xm);
-                    if (busy) {   // uniform
-                        const int at = UNI_X ? 0 : hi - 1;
-                        const float w_lo = __double2float_rd(wi), x_hi = i < S - 1 ? __double2float_ru((double)tmax(s.XT[0][at], s.XT[1][at])) : 0.0f;
-                        U_hi = __fadd_ru(U_hi, __fmaf_ru(2.0f, x_hi, __double2float_ru(wi)));
-                        busy_best = fmaxf(busy_best, __fmaf_rd((float)m, w_lo, -U_hi));
-                        if (n >= -1)
-                            busy_best = fmaxf(busy_best, __fmaf_rd(-(float)(S - 1 - i), __double2float_ru(f < bk ? f : bk), __fmul_rd((float)(m - 1), w_lo)));
-                    }
-                }
-                hi = lo;
-            }
-            if (r == 3) {   // the stages so far move up by four
-#pragma unroll
-                for (int j = 2 * NB - 1; j > 1; --j) v.b[j] = v.b[j - 2];
-                v.b[0] = v.b[1] = make_float2(kNoWalk, kNoWalk);
-            }
-        }
-    }
-    if (!gpipe) v.set(0, fmaxf(base_n, c_n == kNoWalk ? kNoWalk : __fadd_rd(c_n, xq_n)));
-    const double f1 = __hiloint2double(fmax, 0), b1 = __hiloint2double(bmax, 0);
-    v.u0 = __double2float_rd(U);
-    v.once = fmaxf(__double2float_rd((double)(m - 1) * (gpipe ? f1 + b1 : tmax(f1, b1))), busy_best);
-    v.g = __ll2float_rd(g_max);
-}
-
-// Transfers above every stage and the visits across inter-node boundaries, per segment of the CTA, where
-// the transfer times do not depend on the layer (UNI_X).
-template <typename T, int NB>
-__device__ __forceinline__ void fill_transfers(const BoundSmem &sm, const SProf<T> &sp, int S, int m, int n_seg) {
-    const float x0 = __double2float_rd((double)sp.XT[0][0]), x1 = __double2float_rd((double)sp.XT[1][0]);
-    for (int s = threadIdx.x; s < n_seg; s += kBoundThreads) {
-        const uint64_t tier = sm.segs[s].tier;
-        float X = 0.0f;
-        int n = 0;
+    bool ok = true;
 #pragma unroll 4
-        for (int i = 4 * NB - 1; i >= 0; --i) {
-            if (i < S - 1) {
-                const bool far = (tier >> i) & 1ull;
-                const float X_up = X;
-                X = __fadd_rd(X, 2.0f * (far ? x1 : x0));
-                if (far && sp.sched != CM_SCHED_GPIPE) {
-                    if (n < kFarMax)
-                        sm.far[s * kFarMax + n] = FarVisit{__fmaf_rd(2.0f * stay_pairs(i, S, m), x1, X),
-                                                           __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x1, X_up), i, 0};
-                    n = n < kFarMax ? n + 1 : kFarLong;
-                }
-            }
-            sm.xs[s * 4 * NB + i] = X;
+    for (int i = 0; i < S; ++i) {
+        const int hi = w.next();
+        if (CUTS) cut_col[i * kBoundThreads] = (uint8_t)hi;
+        ok = ok && hi > lo;
+        if (check && !stage_fits(s.PS[hi] - s.PS[lo], s.PA[hi] - s.PA[lo], i, S, m, s.cap, s.sched)) ok = false;
+        const double f = (double)(s.PF[hi] - s.PF[lo]), bk = (double)(s.PB[hi] - s.PB[lo]), wi = f + bk;
+        const long long g = s.PP[hi] - s.PP[lo];
+        g_max = g > g_max ? g : g_max;
+        fmax = max(fmax, __double2hiint(f));
+        bmax = max(bmax, __double2hiint(bk));
+        if (i > 0) {
+            if (!UNI_X) x = transfers_at(s, lo - 1, dear);
+            P += 2.0 * (double)s.XT[dear ^ 1][lo - 1];
+            H += 2.0 * (double)s.XT[dear][lo - 1];
         }
-        sm.segs[s].n_far = n;
+        const float P_i = __double2float_ru(P);
+        float term = kNoWalk;
+        if (!gpipe) {
+            const int n = stays(i, S, m);
+            const float q = stay_pairs(i, S, m);
+            const double U = (double)(TF - s.PF[lo]) + (double)(TB - s.PB[lo]), dw = wi - w_p;
+            const float base = n >= 0 ? __double2float_rd(__fma_rd((double)n, wi, U)) : kNoWalk;
+            const float up = q_p > 0.0f ? __fmaf_rd(q_p, __double2float_rd(dw), base_p) : kNoWalk;
+            const float down = q > 0.0f && i > 0 ? __fmaf_rd(q, __double2float_rd(-dw), base) : kNoWalk;
+            if (i > 0) {
+                best = fmaxf(best, __fsub_rd(max3(base_p, down_p, __fmaf_rd(q_p, x.lo_rd, up)), P_p));
+                const float d_ru = __fsub_ru(x.hi_ru, x.lo_rd);
+                term = max3(best, __fsub_rd(__fmaf_rd(q_p, x.hi_rd, up), P_p), __fsub_rd(__fsub_rd(__fmaf_rd(q, x.hi_rd, down), P_i), d_ru));
+            }
+            if (busy) {   // uniform
+                const float w_lo = __double2float_rd(wi);
+                busy_rel = fmaxf(busy_rel, __fadd_rd(__fmaf_rd((float)m, w_lo, -__double2float_ru(U)), __double2float_rd(H)));
+                if (n >= -1)
+                    busy_best = fmaxf(busy_best, __fmaf_rd(-(float)(S - 1 - i), __double2float_ru(f < bk ? f : bk), __fmul_rd((float)(m - 1), w_lo)));
+            }
+            down_p = __fmaf_rd(q, x.lo_rd, down);
+            base_p = base; w_p = wi; q_p = q; P_p = P_i;
+        }
+        if (i > 0) {
+            if (UNI_X) *reinterpret_cast<float *>(term_col + (i - 1) * row) = term;
+            else *reinterpret_cast<float2 *>(term_col + (i - 1) * row) = make_float2(term, fmaxf(__fsub_rd(x.hi_rd, x.lo_ru), 0.0f));
+        }
+        lo = hi;
     }
+    if (UNI_X) *reinterpret_cast<float *>(term_col + (S - 1) * row) = kNoWalk;   // the row that says nothing
+    else *reinterpret_cast<float2 *>(term_col + (S - 1) * row) = make_float2(kNoWalk, 0.0f);
+    best = fmaxf(best, __fsub_rd(fmaxf(base_p, down_p), P_p));
+    const double f1 = __hiloint2double(fmax, 0), b1 = __hiloint2double(bmax, 0);
+    float once = __double2float_rd((double)(m - 1) * (gpipe ? f1 + b1 : tmax(f1, b1)));
+    once = max3(once, busy_best, __fsub_rd(busy_rel, __double2float_ru(H)));
+    v.best = fmaxf(best, __fsub_rd(once, __double2float_ru(P)));
+    v.u0 = __fadd_rd(__double2float_rd((double)TF + (double)TB), __fmul_rd(2.0f, __double2float_rd(P)));
+    v.g = __ll2float_rd(g_max);
+    if (!ok) v.best = v.u0 = __uint_as_float(0x7f800000u);
+    v.ok = ok;
 }
 
-// Bound of the lane's composition in one segment, without the slack (bound_of).  What a segment adds -- the
-// transfers of its link tiers -- is prepared once per CTA (UNI_X) or worked out per plan.
-template <typename T, int NB, bool UNI_X>
-__device__ __forceinline__ float lane_value(const LaneBound<NB> &v, const SProf<T> &sp, int S, int m, int s, const BoundSmem &sm) {
-    const SegLite &sg = sm.segs[s];
-    float best = v.once, x_all;
-    if (UNI_X) {
-        const float4 *xr = reinterpret_cast<const float4 *>(sm.xs + s * 4 * NB);
-        float other = kNoWalk;
+// A composition's lane (any: there is one); one that is no plan has an infinite bound.
+template <typename T, bool UNI_X, bool CUTS>
+__device__ __forceinline__ LaneBound lane_of(const SProf<T> &sp, const Tables &tb, const BatchDev &bd, const BBucket &bk, bool any, const Cand &cand, int dear,
+                                             unsigned char *term_col, uint8_t *cut_col) {
+    const float none = __uint_as_float(0x7f800000u);
+    LaneBound v{none, none, 0.0f, false};
+    CutWalker w;
+    if (any && make_walker(w, tb, bd.layer_mode, sp.L, bk.S, cand, bk.K, tb.mm_slot(bk.S, bk.m)))
+        lane_setup<T, UNI_X, CUTS>(v, sp, w, bk.S, bk.m, bk.feas_first == kNoFeasList, dear, term_col, cut_col);
+    if (!v.ok)   // (terms of nothing could be no numbers)
+        for (int i = 0; i < bk.S; ++i) {
+            if (UNI_X) *reinterpret_cast<float *>(term_col + i * kTermRow * kTermSize<UNI_X>) = kNoWalk;
+            else *reinterpret_cast<float2 *>(term_col + i * kTermRow * kTermSize<UNI_X>) = make_float2(kNoWalk, 0.0f);
+        }
+    return v;
+}
+
+// Time that a dear boundary adds to a transfer up and one down, where it does not depend on the layer.
+template <typename T> __device__ __forceinline__ float dear_extra(const SProf<T> &s, int dear) {
+    const Transfers x = transfers_at(s, 0, dear);
+    return fmaxf(__fsub_rd(x.hi_rd, x.lo_ru), 0.0f);
+}
+
+__device__ __forceinline__ SegLite seg_lite(uint64_t tier, uint32_t row, int n_sync, long long bw_sync) {
+    SegLite s{tier, row, 0.0f};
+    if (n_sync > 1) s.coef = __double2float_rd((2.0 * (double)(n_sync - 1)) / ((double)n_sync * (double)bw_sync));
+    return s;
+}
+// What the bound of a plan in a segment takes from it: the synchronisation time per gradient byte, what its dear
+// boundaries add to a climb and a drop (UNI_X), and where their terms are in a composition's column, topmost
+// first (the rest of the list: the row that says nothing).
+struct SegHot { uint64_t bits; float coef, extra; uint32_t off[kDearMax]; int n; };
+template <bool UNI_X>
+__device__ __forceinline__ SegHot seg_hot(const SegLite &sg, int S, int dear, float delta, bool gpipe) {
+    SegHot h;
+    h.bits = dear_bits(sg.tier, dear, S);
+    h.n = __popcll(h.bits);
+    h.coef = sg.coef;
+    h.extra = UNI_X ? __fmul_rd((float)h.n, delta) : 0.0f;
+    if (UNI_X && gpipe) { h.bits = 0; h.n = 0; }   // (no stays, no visits)
+    uint64_t bits = h.bits;
 #pragma unroll
-        for (int k = 0; k < NB; ++k) {
-            const float4 x = xr[k];
-            const float2 p = add2_rd(v.b[2 * k], make_float2(x.x, x.y)), q = add2_rd(v.b[2 * k + 1], make_float2(x.z, x.w));
-            best = max3(best, p.x, p.y);
-            other = max3(other, q.x, q.y);
-            if (k == 0) x_all = x.x;
-        }
-        if (sg.n_far <= kFarMax) {
-            for (int k = 0; k < sg.n_far; ++k) {
-                const FarVisit f = sm.far[s * kFarMax + k];
-                const float2 r = add2_rd(sm.cd[f.at * kBoundThreads], make_float2(f.up, f.down));
-                best = max3(best, r.x, r.y);
-            }
-        } else {
-            const float x1 = __double2float_rd((double)sp.XT[1][0]);
-            const float *xf = sm.xs + s * 4 * NB;
-            for (uint64_t t = sg.tier; t; t &= t - 1) {
-                const int i = __ffsll((long long)t) - 1;
-                const float2 cd = sm.cd[i * kBoundThreads];
-                best = fmaxf(best, __fadd_rd(cd.x, __fmaf_rd(2.0f * stay_pairs(i, S, m), x1, xf[i])));
-                best = fmaxf(best, __fadd_rd(cd.y, __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x1, i + 1 < S - 1 ? xf[i + 1] : 0.0f)));
-            }
-        }
-        best = fmaxf(best, other);
-    } else {
-        float X = 0.0f;
-#pragma unroll
-        for (int i = 4 * NB - 1; i >= 0; --i) {
-            if (i < S) {
-                if (i < S - 1) {
-                    const bool far = (sg.tier >> i) & 1ull;
-                    const float x = __double2float_rd((double)sp.XT[far ? 1 : 0][sm.cut[i * kBoundThreads] - 1]);
-                    const float X_up = X;
-                    X = __fadd_rd(X, 2.0f * x);
-                    if (far && sp.sched != CM_SCHED_GPIPE) {
-                        const float2 cd = sm.cd[i * kBoundThreads];
-                        best = fmaxf(best, __fadd_rd(cd.x, __fmaf_rd(2.0f * stay_pairs(i, S, m), x, X)));
-                        best = fmaxf(best, __fadd_rd(cd.y, __fmaf_rd(2.0f * stay_pairs(i + 1, S, m), x, X_up)));
-                    }
-                }
-                best = fmaxf(best, __fadd_rd(v.get(i), X));
-            }
-        }
-        x_all = X;
+    for (int k = 0; k < kDearMax; ++k) {
+        const int i = bits ? 63 - __clzll((long long)bits) : S - 1;
+        h.off[k] = i * kTermRow * kTermSize<UNI_X>;
+        if (bits) bits ^= 1ull << i;
     }
-    return __fmaf_rd(v.g, sg.coef, __fadd_rd(__fadd_rd(v.u0, x_all), best));
+    return h;
+}
+
+// Bound of a composition in a segment, without the slack (bound_of).  NF: dear boundaries looked at; -1: as many as
+// there are.  (The value does not depend on NF as long as it is enough.)  A value below no zero is made of zeros only;
+// rounding down makes -0 of a difference of equals, and the least value is found by its bits.
+template <bool UNI_X, int NF>
+__device__ __forceinline__ float bound_value(float v_best, float v_u0, float v_g, const unsigned char *term_col, const SegHot &h, float delta) {
+    float best = v_best, extra = h.extra;
+    float a[NF > 0 ? NF : 1];
+    if constexpr (NF > 0) {
+#pragma unroll
+        for (int k = 0; k < NF; ++k) {
+            if constexpr (UNI_X) {
+                a[k] = __fadd_rd(*reinterpret_cast<const float *>(term_col + h.off[k]), __fmul_rd((float)(k + 1), delta));
+            } else {
+                const float2 t = *reinterpret_cast<const float2 *>(term_col + h.off[k]);
+                extra = __fadd_rd(extra, t.y);
+                a[k] = __fadd_rd(t.x, extra);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k + 1 < NF; k += 2) best = max3(best, a[k], a[k + 1]);
+        if constexpr (NF & 1) best = fmaxf(best, a[NF - 1]);
+    } else if constexpr (NF < 0) {
+        int k = 0;
+        for (uint64_t bits = h.bits; bits;) {
+            const int i = 63 - __clzll((long long)bits);
+            bits ^= 1ull << i;
+            if constexpr (UNI_X) {
+                ++k;
+                best = fmaxf(best, __fadd_rd(*reinterpret_cast<const float *>(term_col + i * kTermRow * kTermSize<UNI_X>), __fmul_rd((float)k, delta)));
+            } else {
+                const float2 t = *reinterpret_cast<const float2 *>(term_col + i * kTermRow * kTermSize<UNI_X>);
+                extra = __fadd_rd(extra, t.y);
+                best = fmaxf(best, __fadd_rd(t.x, extra));
+            }
+        }
+    }
+    return fmaxf(__fmaf_rd(v_g, h.coef, __fadd_rd(__fadd_rd(v_u0, extra), best)), 0.0f);
 }
 // slack: 1 where the synchronisation quotient floors
 __device__ __forceinline__ float bound_of(float value, float slack) {
@@ -322,8 +308,5 @@ __device__ __forceinline__ void list_append(const BatchDev &bd, const BoundDev &
     if (at < bo.list_first[list + 1] - bo.list_first[list]) bo.list[bo.list_first[list] + at] = make_uint4(scen, tseg, pos, 0u);
     else bd.counters[4] = 0ull;   // list full: the host repeats the search without bounds
 }
-
-// Instantiations of the kernel bodies by stages in fours; a depth in between takes the next one.
-constexpr int kBoundNb[] = {4, 9, 16};
 
 }  // namespace cm

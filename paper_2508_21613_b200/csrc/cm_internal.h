@@ -188,8 +188,8 @@ constexpr int kUniBatchStagesMax = 28;     // deeper transposed classes keep one
 constexpr uint64_t kUniMinChunks = 4096;   // keep at least this many CTAs (about ten waves) in a class before batching items
 
 // Bounded search pass (cm_bound.cu).  Its work layout groups segments as the buckets above do, every
-// segment on its own; a CTA of the bound kernel takes `width` compositions of a bucket side by side
-// for 128 / width segments at a time and walks a group of seg_group of them.
+// segment on its own; a CTA of the bound kernel sets up `width` compositions of a bucket and takes a group of
+// seg_group segments by them.
 struct BBucket {
     uint64_t count, K;      // candidates walked per segment; enumerated compositions
     uint32_t chunk_first;   // its first CTA
@@ -202,13 +202,18 @@ struct BBucket {
     uint16_t role;          // work accounting: 0 on its own, 1 head of a micro-batch pair, 2 the row after a head
     uint16_t second;        // distinct segments: the rows after the listed ones (m is theirs)
     uint16_t width, seg_group;
-    uint32_t pad;
+    uint32_t min_first;     // its entries of BoundDev::tile_min: by tile, then by segment
 };
 // Step times that can still be a scenario's answer: lo <= T* <= ub, lo from bounds.
 // reach: strategies whose step time from bounds is at most this had their segments marked.
 struct SearchWin { float lo, reach; uint64_t ub; };
+// A segment of the layout, for the kernels after the first.
+struct SegRec { uint64_t tier; uint32_t row, scen, tseg; int32_t n_sync; };
 struct BoundDev {
     const BBucket *bucket;
+    SegRec *rec;                  // per segment of the layout
+    uint32_t parts;               // CTAs of cm_refine_kernel for one of cm_bound_kernel
+    uint32_t pad;
     uint64_t *lbarg;              // per row: least bound (float bits) << 32 | its position in the walk; all-ones = no plan fits
     uint64_t *pick;               // per row: the plan phase 1 takes (cm_bound_lane.cuh)
     SearchWin *win;               // per scenario
@@ -221,8 +226,9 @@ struct BoundDev {
     uint32_t *count;              // per list: plans listed minus one
     uint32_t list_first[5];       // lists: phase 1 up to kRegStagesMax stages, deeper; phase 2 the same
     uint32_t n_buckets, n_chunks, n_segs;
-    uint32_t dyn_far, dyn_cols, dyn_cuts, dyn_segs, max_group;   // shared memory of a CTA (BoundSmem)
-    size_t dyn_bytes;
+    float *tile_min;              // per (tile of compositions, segment): least bound; null: too many
+    uint32_t dyn_cuts;
+    size_t dyn_bytes, dyn_refine;   // dynamic shared memory of a CTA of cm_bound_kernel, of cm_refine_kernel
     int uniform_x;
 };
 constexpr int kCounters = 8;   // work counters of a search (BatchDev::counters)
@@ -230,10 +236,9 @@ constexpr int kCounters = 8;   // work counters of a search (BatchDev::counters)
 // launches: 33 sets of the 32-device job with the full objective (just below) 506 us directly, 745 by bounds;
 // one failure of the 256-device job (4e8) 380 us directly, 259 by bounds when they came, 155 now.
 constexpr uint64_t kBoundMinCells = 200000000ull;
+constexpr uint64_t kTileMinMax = 1ull << 24;     // entries of BoundDev::tile_min, at most (64 MB)
 constexpr uint32_t kBoundListMin = 65536;        // plans a list has room for, at least (if there are as many)
 constexpr size_t kBoundDynMax = 160 * 1024;      // dynamic shared memory of the bound kernels, at most
-constexpr size_t kBoundDynTarget = 64 * 1024;    //   and wanted: three CTAs per SM
-constexpr size_t kRefineSegBytes = 32;
 
 // Per-scenario winner of the split reduction, decoded for the tie-break pass.
 struct Winner {
@@ -357,8 +362,8 @@ struct SideStreams {
 cudaError_t launch_cost_pass1(const Tables &t, const BatchDev &b, const LaunchClass *classes, int n_classes,
                               cudaStream_t st, const SideStreams *side, int *launches);
 // bounded search pass (cm_bound.cu, cm_refine.cu)
-size_t bound_dyn_bytes(BoundDev &bo, int max_stages, int max_group, bool uniform_x);   // also sets the offsets
-int bound_group(int max_stages, bool uniform_x);   // segments per CTA
+size_t bound_dyn_bytes(BoundDev &bo, int max_stages, bool uniform_x);   // sets them; the largest
+int bound_group();   // segments per CTA, at most
 cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
 cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st);
 cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st);
