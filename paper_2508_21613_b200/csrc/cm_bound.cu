@@ -228,8 +228,11 @@ __global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd,
         const int p = lane >> 1, k = lane & 1;
         if (p < s.dp && k < s.n_m) {
             uint32_t row = canon_row(bd, tp, sc, s, p, k);
+            if (bo.row_rep) row = bo.row_rep[row];
+            // a bound beyond reach: not part of the answer through this share (where results move the reach up, the
+            // second window marks again)
+            if (lb_of(bo.lbarg[row]) > reach) continue;
             if (bo.row_rep) {
-                row = bo.row_rep[row];
                 const unsigned long long l = __float_as_uint(lo), u = ~t;   // (u: of a result, phase 1)
                 if (l < bo.row_lo[row]) atomicMin((unsigned long long *)&bo.row_lo[row], l);
                 if (phase && u < bo.row_ub[row]) atomicMin((unsigned long long *)&bo.row_ub[row], u);
@@ -272,8 +275,8 @@ cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo
 
 // ----------------------------------------------------------------------------------
 // The recurrence on the listed plans.  Pipelines of at most 16 stages: a thread per plan, state in
-// registers; deeper ones: a warp per plan in lock step, 2(S+m) slots of ~45 cycles (a thread would
-// need ~100 us for its chain of 2 S m cells, and the lists are short).
+// registers; deeper ones in lock step, 2(S+m) slots (a thread would need ~100 us for its chain of 2 S m cells): a
+// warp per plan where the warps are enough for the list, three plans per warp (two beyond 40 stages) where not.
 // ----------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t list_length(const BoundDev &bo, int list) {
     const uint32_t n = bo.count[list] + 1u, room = bo.list_first[list + 1] - bo.list_first[list];
@@ -317,21 +320,43 @@ __global__ void __launch_bounds__(kChunk) cm_list_shallow_kernel(Tables tb, Batc
 template <typename T>
 __global__ void __launch_bounds__(kChunk, 5) cm_list_deep_kernel(Tables tb, BatchDev bd, BoundDev bo, int list) {
     __shared__ SProf<T> sp;
-    __shared__ uint8_t cuts_s[kChunk / 32][kMaxS + 8];
+    __shared__ uint8_t cuts_s[kChunk / 32][4][kMaxS + 8];   // (per plan; the fourth: lanes without one)
     const uint32_t n = list_length(bo, list);
     if ((uint64_t)blockIdx.x * (kChunk / 32) >= n || lists_full(bd)) return;
     stage_profile(sp, tb);
     __syncthreads();
     const uint4 *entries = bo.list + bo.list_first[list];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t n_warps = gridDim.x * (kChunk / 32), first = blockIdx.x * (kChunk / 32) + warp;
     unsigned long long work = 0;
-    for (uint32_t i = blockIdx.x * (kChunk / 32) + warp; i < n; i += gridDim.x * (kChunk / 32)) {
-        const uint4 e = entries[i];
-        const SegView g = seg_view(bd, e.x, e.y);
-        T cost;
-        if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, walk_cand(bd, g.feas_first, e.z), cuts_s[warp], cost) && lane == 0)
-            list_commit<T>(bd, g.row, cost);
-        if (lane == 0) work += 2ull * g.S * g.m + (1ull << 40);
+    if (n <= n_warps || sp.sched == CM_SCHED_GPIPE) {
+        for (uint32_t i = first; i < n; i += n_warps) {
+            const uint4 e = entries[i];
+            const SegView g = seg_view(bd, e.x, e.y);
+            T cost;
+            if (warp_plan_cost<T>(sp, tb, bd.layer_mode, g, walk_cand(bd, g.feas_first, e.z), cuts_s[warp][0], cost) && lane == 0)
+                list_commit<T>(bd, g.row, cost);
+            if (lane == 0) work += 2ull * g.S * g.m + (1ull << 40);
+        }
+    } else {
+        for (uint32_t i0 = 3 * first; i0 < n; i0 += 3 * n_warps)
+            for (uint32_t i = i0; i < i0 + 3 && i < n;) {   // those of equal depth together
+                const int S = bd.tseg[entries[i].y].S, width = (S + 3) >> 2, most = 32 / width < 3 ? 32 / width : 3;
+                const int grp = lane / width, gl = lane - grp * width;
+                const uint32_t at = i + grp;
+                const bool here = grp < most && at < i0 + 3 && at < n;
+                const uint4 e = entries[here ? at : i];
+                const uint32_t other = __ballot_sync(0xffffffffu, !here || bd.tseg[e.y].S != S);
+                const int k = other ? (__ffs((int)other) - 1) / width : most;   // (lanes without a plan come last)
+                const SegView g = seg_view(bd, entries[grp < k ? at : i].x, entries[grp < k ? at : i].y);
+                const uint4 mine = entries[grp < k ? at : i];
+                T cost;
+                if (group_plan_cost<T>(sp, tb, bd.layer_mode, g, walk_cand(bd, g.feas_first, mine.z), grp < k, gl, width, cuts_s[warp][grp < 3 ? grp : 3], cost) &&
+                    gl == 0)
+                    list_commit<T>(bd, g.row, cost);
+                if (gl == 0 && grp < k) work += 2ull * g.S * g.m + (1ull << 40);
+                i += k;
+            }
     }
     count_list_work(bd, work);
 }

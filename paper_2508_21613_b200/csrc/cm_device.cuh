@@ -438,165 +438,161 @@ __device__ __forceinline__ void init_kappa_sel(const BatchDev &bd, const Winner 
 }
 
 // ----------------------------------------------------------------------------------
-// The pipeline-time recurrence of ONE pipeline spread over a warp: PER consecutive stages
-// per lane (S <= 32 * PER), walked in lock step over time slots.  With unit durations the
-// 1F1B schedule puts forward (i,j) at slot i+j while j <= S-1-i and at slot i+2j afterwards,
-// and backward (i,j) at slot 2S-1-i+2j; taking those slots as the evaluation order is a
+// The pipeline-time recurrence of ONE pipeline spread over a warp, walked in lock step over time slots.  With
+// unit durations the 1F1B schedule puts forward (i,j) at slot i+j while j <= S-1-i and at slot i+2j afterwards,
+// and backward (i,j) at slot 2S-1-i+2j; under the all-forward-all-backward order forward (i,j) sits at slot i+j and
+// backward (i,j) at slot (S+m-1) + (S-1-i) + j.  Taking those slots as the evaluation order is a
 // valid topological order for arbitrary durations and every m >= 1.  Every stage keeps
 // its clock, its latest forward end (transfer added) and its latest backward end; inputs
 // of a slot are gathered from the neighbours' state before any stage of the slot updates.
-// F, B, xt: the lane's own stages.  Returns the pipeline time in every lane.
+// Times are non-negative, so "no dependency" (forward of stage 0, backward of the last stage) is a dependency on
+// time 0.  F, B, xt: the lane's own stages.
 // ----------------------------------------------------------------------------------
-// Under the all-forward-all-backward order forward (i,j) sits at slot i+j and backward (i,j)
-// at slot (S+m-1) + (S-1-i) + j.
-// The loop is branch-free inside a slot -- lanes that run a forward, a backward or nothing take
-// the same instructions, so the stages of a lane and the two kinds of work interleave -- and
-// the slot tests are kept short, because one warp alone issues them: times are non-negative,
-// so "no dependency" (forward of stage 0, backward of the last stage) is a dependency on time 0
-// (a stage past the end never runs and keeps its zeros), and under 1F1B the parity of s - i
-// says which kind of work a steady-state slot can hold.
+// All-forward-all-backward order, PER consecutive stages per lane (S <= 32 * PER); the time in every lane.
 template <typename T, int PER>
-__device__ __forceinline__ T sim_lockstep_n(int S, int m, const T *F, const T *B, const T *xt, int sched) {
+__device__ __forceinline__ T sim_lockstep_afab(int S, int m, const T *F, const T *B, const T *xt) {
     const int lane = threadIdx.x & 31;
     T clock[PER], last_f[PER], last_b[PER];
-    int d[PER];          // slot - stage
+    int d[PER], e[PER];  // slot - stage; slot - stage counted from the last one
     unsigned mk[PER];    // micro-batches of the stage (0: past the end)
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         clock[k] = (T)0; last_f[k] = (T)0; last_b[k] = (T)0;
         d[k] = -(lane * PER + k);
+        e[k] = -(S - 1 - (lane * PER + k));
         mk[k] = lane * PER + k < S ? (unsigned)m : 0u;
     }
-    auto slot = [&](auto only_forward, auto pick) {
+    for (int s = 0; s < S + m - 1; ++s) {
         T up = __shfl_up_sync(0xffffffffu, last_f[PER - 1], 1);
-        T down = __shfl_down_sync(0xffffffffu, last_b[0], 1);
         up = lane == 0 ? (T)0 : up;       // the end lanes get their own value back from the shuffle
-        down = lane == 31 ? (T)0 : down;
-        T f_in[PER], b_in[PER];
+        T fin[PER];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) fin[k] = tmax(clock[k], k == 0 ? up : last_f[k > 0 ? k - 1 : 0]) + F[k];
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-            f_in[k] = k == 0 ? up : last_f[k > 0 ? k - 1 : 0];
-            b_in[k] = k == PER - 1 ? down : last_b[k < PER - 1 ? k + 1 : 0];
-        }
-#pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            bool is_f, is_b;
-            pick(k, is_f, is_b);
-            if constexpr (decltype(only_forward)::value) {
-                const T fin = tmax(clock[k], f_in[k]) + F[k];
-                clock[k] = is_f ? fin : clock[k];
-                last_f[k] = is_f ? fin + xt[k] : last_f[k];
-            } else {
-                const T dep = is_f ? f_in[k] : b_in[k] + xt[k];
-                const T fin = tmax(clock[k], dep) + (is_f ? F[k] : B[k]);
-                clock[k] = (is_f || is_b) ? fin : clock[k];
-                last_f[k] = is_f ? fin + xt[k] : last_f[k];
-                last_b[k] = is_b ? fin : last_b[k];
-            }
+            if ((unsigned)d[k] < mk[k]) { clock[k] = fin[k]; last_f[k] = fin[k] + xt[k]; }
             ++d[k];
         }
-    };
-    using Yes = std::true_type;
-    using No = std::false_type;
-    if (sched == CM_SCHED_GPIPE) {
-        // forward (i,j) at slot i+j; backward (i,j) at slot (S+m-1) + (S-1-i) + j
-        for (int s = 0; s < S + m - 1; ++s)
-            slot(Yes{}, [&](int k, bool &is_f, bool &is_b) { is_f = (unsigned)d[k] < mk[k]; is_b = false; });
-        int e[PER];
+    }
+    for (int s = 0; s < S + m - 1; ++s) {
+        T down = __shfl_down_sync(0xffffffffu, last_b[0], 1);
+        down = lane == 31 ? (T)0 : down;
+        T fin[PER];
 #pragma unroll
-        for (int k = 0; k < PER; ++k) e[k] = -(S - 1 - (lane * PER + k));
-        for (int s = 0; s < S + m - 1; ++s)
-            slot(No{}, [&](int k, bool &is_f, bool &is_b) { is_f = false; is_b = (unsigned)e[k] < mk[k]; ++e[k]; });
-    } else {
-        // slots 0 .. S-1: warm-up forwards only (the first backward sits at slot S)
-        for (int s = 0; s < S; ++s)
-            slot(Yes{}, [&](int k, bool &is_f, bool &is_b) { is_f = (unsigned)d[k] < mk[k]; is_b = false; });
-        // afterwards forward j = (s-i)/2 when s-i is even and j > S-1-i; backward (s-i-(2S-1-2i))/2 when s-i is odd
-        int warm[PER], off[PER];
+        for (int k = 0; k < PER; ++k) fin[k] = tmax(clock[k], (k == PER - 1 ? down : last_b[k < PER - 1 ? k + 1 : 0]) + xt[k]) + B[k];
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-            warm[k] = S - 1 - (lane * PER + k);
-            off[k] = 2 * S - 1 - 2 * (lane * PER + k);
+            if ((unsigned)e[k] < mk[k]) { clock[k] = fin[k]; last_b[k] = fin[k]; }
+            ++e[k];
         }
-        const int n_slots = 2 * (S + m) - 2;
-        for (int s = S; s < n_slots; ++s)
-            slot(No{}, [&](int k, bool &is_f, bool &is_b) {
-                const bool even = (d[k] & 1) == 0;
-                const int j = d[k] >> 1;
-                is_f = even && j > warm[k] && (unsigned)j < mk[k];
-                is_b = !even && ((unsigned)(d[k] - off[k]) >> 1) < mk[k];
-            });
     }
     return __shfl_sync(0xffffffffu, clock[0], 0);
 }
 
-// The 1F1B order with TWO consecutive stages per lane (stage 2l and 2l+1; S <= 64).  After the
+// The 1F1B order with NP PAIRS of consecutive stages per lane (stages 2 NP l .. 2 NP l + 2 NP - 1).  After the
 // warm-up slots a stage alternates forward and backward, even stages run their forwards in even
-// slots and odd stages in odd ones, so which kind of work each of a lane's two stages can do in
+// slots and odd stages in odd ones, so which kind of work each of a lane's stages can do in
 // a slot is known at compile time once the loop takes an even and an odd slot per iteration:
-// no selects between forward and backward operands.  In the odd slot both inputs are the lane's
-// own (the forward of stage 2l feeds stage 2l+1, the backward of stage 2l+1 feeds stage 2l), so
-// only the even slot shuffles.  With h = slot / 2 and c = h + l + 1 - S the micro-batch tests are
-//   even slot: stage 2l   forward  j = h - l     runs iff 0 <= c - 1 < m - S + 2l
-//              stage 2l+1 backward j = c         runs iff 0 <= c < m
-//   odd slot:  stage 2l   backward j = c         runs iff 0 <= c < m
-//              stage 2l+1 forward  j = h - l     runs iff 0 <= c < m - S + 2l + 1
-// Same operations on the same operands as sim_lockstep_n: identical bits.
-template <typename T>
-__device__ __forceinline__ T sim_lockstep_pairs(int S, int m, const T *F, const T *B, const T *xt) {
-    const int lane = threadIdx.x & 31;
-    const bool valid0 = 2 * lane < S, valid1 = 2 * lane + 1 < S;
-    T clock0 = (T)0, clock1 = (T)0, last_f0 = (T)0, last_f1 = (T)0, last_b0 = (T)0, last_b1 = (T)0;
+// no selects between forward and backward operands.  In the odd slot all inputs are the lane's
+// own (the forward of stage 2e feeds stage 2e+1, the backward of stage 2e+1 feeds stage 2e), so
+// only the even slot shuffles.  With h = slot / 2 and c = h + e + 1 - S the micro-batch tests of pair e are
+//   even slot: stage 2e   forward  j = h - e     runs iff 0 <= c - 1 < m - S + 2e
+//              stage 2e+1 backward j = c         runs iff 0 <= c < m
+//   odd slot:  stage 2e   backward j = c         runs iff 0 <= c < m
+//              stage 2e+1 forward  j = h - e     runs iff 0 <= c < m - S + 2e + 1
+// All of them hold for S <= h < m: these rounds run without a test.  (A stage past the end, with times of
+// zero, then carries ends of the last stage's forwards up and down again, none of them later than the last stage's
+// clock: they change no maximum.)
+// Same operations on the same operands as in any other order: identical bits.
+// Several pipelines of equal S in one warp: `gl` is the lane's number within its pipeline, `last` marks its last
+// lane, m is the pipeline's own and m_lo, m_hi the least and the most of the warp's.  Returns the time in the first
+// lane of every pipeline.
+template <typename T, int NP>
+__device__ __forceinline__ T sim_lockstep_pairs(int S, int m, const T *F, const T *B, const T *xt, int gl, bool last, int m_lo, int m_hi) {
+    constexpr int PER = 2 * NP;
+    T clock[PER], last_f[PER], last_b[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) { clock[k] = (T)0; last_f[k] = (T)0; last_b[k] = (T)0; }
     {   // slots 0 .. S-1: warm-up forwards only, forward (i,j) at slot i+j
-        int d0 = -2 * lane, d1 = -2 * lane - 1;
-        const unsigned m0 = valid0 ? (unsigned)m : 0u, m1 = valid1 ? (unsigned)m : 0u;
-        for (int s = 0; s < S; ++s) {
-            T up = __shfl_up_sync(0xffffffffu, last_f1, 1);
-            up = lane == 0 ? (T)0 : up;
-            const T fin0 = tmax(clock0, up) + F[0];
-            const T fin1 = tmax(clock1, last_f0) + F[1];
-            if ((unsigned)d0 < m0) { clock0 = fin0; last_f0 = fin0 + xt[0]; }
-            if ((unsigned)d1 < m1) { clock1 = fin1; last_f1 = fin1 + xt[1]; }
-            ++d0; ++d1;
+        int d = -gl * PER;
+        for (int s = 0; s < S; ++s, ++d) {
+            T up = __shfl_up_sync(0xffffffffu, last_f[PER - 1], 1);
+            up = gl == 0 ? (T)0 : up;
+            T fin[PER];
+#pragma unroll
+            for (int k = 0; k < PER; ++k) fin[k] = tmax(clock[k], k ? last_f[k > 0 ? k - 1 : 0] : up) + F[k];
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if ((unsigned)(d - k) < (gl * PER + k < S ? (unsigned)m : 0u)) { clock[k] = fin[k]; last_f[k] = fin[k] + xt[k]; }
         }
     }
-    const int f0 = m - S + 2 * lane;
-    const unsigned lim_f0 = valid0 && f0 > 0 ? (unsigned)f0 : 0u;
-    const unsigned lim_f1 = valid1 && f0 + 1 > 0 ? (unsigned)(f0 + 1) : 0u;
-    const unsigned lim_b0 = valid0 ? (unsigned)m : 0u, lim_b1 = valid1 ? (unsigned)m : 0u;
+    unsigned lim_f0[NP], lim_f1[NP], lim_b0[NP], lim_b1[NP];
+#pragma unroll
+    for (int e = 0; e < NP; ++e) {
+        const int at = PER * gl + 2 * e, f0 = m - S + at;
+        lim_f0[e] = at < S && f0 > 0 ? (unsigned)f0 : 0u;
+        lim_f1[e] = at + 1 < S && f0 + 1 > 0 ? (unsigned)(f0 + 1) : 0u;
+        lim_b0[e] = at < S ? (unsigned)m : 0u;
+        lim_b1[e] = at + 1 < S ? (unsigned)m : 0u;
+    }
     int h = S >> 1;
-    int c = h + lane + 1 - S;
-    auto odd_slot = [&]() {
-        const T fin0 = tmax(clock0, last_b1 + xt[0]) + B[0];
-        const T fin1 = tmax(clock1, last_f0) + F[1];
-        if ((unsigned)c < lim_b0) { clock0 = fin0; last_b0 = fin0; }
-        if ((unsigned)c < lim_f1) { clock1 = fin1; last_f1 = fin1 + xt[1]; }
+    int c = h + gl * NP + 1 - S;   // of the lane's first pair
+    auto odd_slot = [&](auto tested) {
+        T fin0[NP], fin1[NP];
+#pragma unroll
+        for (int e = 0; e < NP; ++e) {
+            fin0[e] = tmax(clock[2 * e], last_b[2 * e + 1] + xt[2 * e]) + B[2 * e];
+            fin1[e] = tmax(clock[2 * e + 1], last_f[2 * e]) + F[2 * e + 1];
+        }
+#pragma unroll
+        for (int e = 0; e < NP; ++e) {
+            if (!decltype(tested)::value || (unsigned)(c + e) < lim_b0[e]) { clock[2 * e] = fin0[e]; last_b[2 * e] = fin0[e]; }
+            if (!decltype(tested)::value || (unsigned)(c + e) < lim_f1[e]) { clock[2 * e + 1] = fin1[e]; last_f[2 * e + 1] = fin1[e] + xt[2 * e + 1]; }
+        }
     };
+    auto even_slot = [&](auto tested) {
+        T up = __shfl_up_sync(0xffffffffu, last_f[PER - 1], 1);
+        T down = __shfl_down_sync(0xffffffffu, last_b[0], 1);
+        up = gl == 0 ? (T)0 : up;       // (the end lanes have no neighbour there)
+        down = last ? (T)0 : down;
+        T fin0[NP], fin1[NP];
+#pragma unroll
+        for (int e = 0; e < NP; ++e) {
+            fin0[e] = tmax(clock[2 * e], e ? last_f[e > 0 ? 2 * e - 1 : 0] : up) + F[2 * e];
+            fin1[e] = tmax(clock[2 * e + 1], (e < NP - 1 ? last_b[e < NP - 1 ? 2 * e + 2 : 0] : down) + xt[2 * e + 1]) + B[2 * e + 1];
+        }
+#pragma unroll
+        for (int e = 0; e < NP; ++e) {
+            if (!decltype(tested)::value || (unsigned)(c + e - 1) < lim_f0[e]) { clock[2 * e] = fin0[e]; last_f[2 * e] = fin0[e] + xt[2 * e]; }
+            if (!decltype(tested)::value || (unsigned)(c + e) < lim_b1[e]) { clock[2 * e + 1] = fin1[e]; last_b[2 * e + 1] = fin1[e]; }
+        }
+    };
+    using Yes = std::true_type;
+    using No = std::false_type;
     if (S & 1) {   // slot S is odd
-        odd_slot();
+        odd_slot(Yes{});
         ++h; ++c;
     }
-    for (; h <= S + m - 2; ++h, ++c) {
-        T up = __shfl_up_sync(0xffffffffu, last_f1, 1);
-        T down = __shfl_down_sync(0xffffffffu, last_b0, 1);
-        up = lane == 0 ? (T)0 : up;       // the end lanes get their own value back from the shuffle
-        down = lane == 31 ? (T)0 : down;
-        const T fin0 = tmax(clock0, up) + F[0];
-        const T fin1 = tmax(clock1, down + xt[1]) + B[1];
-        if ((unsigned)(c - 1) < lim_f0) { clock0 = fin0; last_f0 = fin0 + xt[0]; }
-        if ((unsigned)c < lim_b1) { clock1 = fin1; last_b1 = fin1; }
-        odd_slot();
-    }
-    return __shfl_sync(0xffffffffu, clock0, 0);
+    const int n_rounds = S + m_hi - 1, all_in = m_lo > S ? S : n_rounds;
+    for (; h < all_in; ++h, ++c) { even_slot(Yes{}); odd_slot(Yes{}); }
+    for (; h < m_lo; ++h, ++c) { even_slot(No{}); odd_slot(No{}); }
+    for (; h < n_rounds; ++h, ++c) { even_slot(Yes{}); odd_slot(Yes{}); }
+    return clock[0];
 }
 
-// Bare time of one pipeline (no synchronisation term), its stages spread over the warp, two per lane.
+// One pipeline over the warp, two stages per lane: its time in every lane.
 template <typename T>
-__device__ __forceinline__ T warp_pipe_time(const SProf<T> &sp, const uint8_t *cuts, int S, int m, uint64_t tier, int lane) {
-    T F[2], B[2], xt[2];
+__device__ __forceinline__ T sim_lockstep_warp(int S, int m, const T *F, const T *B, const T *xt) {
+    const int lane = threadIdx.x & 31;
+    return __shfl_sync(0xffffffffu, sim_lockstep_pairs<T, 1>(S, m, F, B, xt, lane, lane == 31, m, m), 0);
+}
+
+// Times of the stages from .. from + PER - 1 of a pipeline (zero past its end).
+template <typename T, int PER>
+__device__ __forceinline__ void lane_stages(const SProf<T> &sp, const uint8_t *cuts, int S, uint64_t tier, int from, T *F, T *B, T *xt) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int i = lane * 2 + k;
+    for (int k = 0; k < PER; ++k) {
+        const int i = from + k;
         F[k] = (T)0; B[k] = (T)0; xt[k] = (T)0;
         if (i < S) {
             const int lo = cuts[i], hi = cuts[i + 1];
@@ -605,7 +601,14 @@ __device__ __forceinline__ T warp_pipe_time(const SProf<T> &sp, const uint8_t *c
             if (i < S - 1) xt[k] = sp.XT[(tier >> i) & 1ull][hi - 1];
         }
     }
-    return sp.sched == CM_SCHED_GPIPE ? sim_lockstep_n<T, 2>(S, m, F, B, xt, sp.sched) : sim_lockstep_pairs<T>(S, m, F, B, xt);
+}
+
+// Bare time of one pipeline (no synchronisation term), its stages spread over the warp, two per lane.
+template <typename T>
+__device__ __forceinline__ T warp_pipe_time(const SProf<T> &sp, const uint8_t *cuts, int S, int m, uint64_t tier, int lane) {
+    T F[2], B[2], xt[2];
+    lane_stages<T, 2>(sp, cuts, S, tier, 2 * lane, F, B, xt);
+    return sp.sched == CM_SCHED_GPIPE ? sim_lockstep_afab<T, 2>(S, m, F, B, xt) : sim_lockstep_warp<T>(S, m, F, B, xt);
 }
 
 __device__ __forceinline__ uint64_t warp_min_u64(uint64_t v) {

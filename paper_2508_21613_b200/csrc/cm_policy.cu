@@ -18,7 +18,23 @@
 
 namespace cm {
 
-// (the lock-step recurrence with one stage per lane is sim_lockstep_n<T, 1> of cm_device.cuh)
+// The recurrence of a pipeline whose stages are a lane each (S <= 32): under 1F1B two of them move together to a
+// lane, which takes the choice between forward and backward out of the slots.
+template <typename T>
+__device__ __forceinline__ T lockstep_lanes(int S, int m, T f, T b, T xt, int sched) {
+    if (sched == CM_SCHED_GPIPE) return sim_lockstep_afab<T, 1>(S, m, &f, &b, &xt);
+    T F[2], B[2], X[2];
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int from = (2 * lane + k) & 31;
+        F[k] = __shfl_sync(0xffffffffu, f, from);
+        B[k] = __shfl_sync(0xffffffffu, b, from);
+        X[k] = __shfl_sync(0xffffffffu, xt, from);
+        if (2 * lane + k >= S) F[k] = B[k] = X[k] = (T)0;
+    }
+    return sim_lockstep_warp<T>(S, m, F, B, X);
+}
 
 template <typename T> __device__ __forceinline__ T warp_max(T v) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -69,7 +85,7 @@ __global__ void __launch_bounds__(32 * (kMaxP + 1)) cm_policy_kernel(Tables tb, 
                 }
                 ok = __all_sync(0xffffffffu, ok);
                 if (ok) {
-                    const T base = sim_lockstep_n<T, 1>(S0, m, &F, &B, &xt, sp.sched);
+                    const T base = lockstep_lanes<T>(S0, m, F, B, xt, sp.sched);
                     const T t_sync = warp_max<T>(sync_i);
                     T extra = (T)0;   // summed in stage order, affected stages only
                     for (int s = 0; s < S0; ++s) {
@@ -157,7 +173,7 @@ __global__ void __launch_bounds__(32 * (kMaxP + 1)) cm_policy_kernel(Tables tb, 
             }
             ok = __all_sync(0xffffffffu, fits);
             if (ok) {
-                const T t = sim_lockstep_n<T, 1>(S, m, &f, &bw, &xt, sp.sched);
+                const T t = lockstep_lanes<T>(S, m, f, bw, xt, sp.sched);
                 const long long g_max = warp_max<long long>(g);
                 bits = Num<T>::bits(t + Num<T>::sync(g_max, n_dp, sp.bw_sync, sp.intval));
             }
