@@ -1480,7 +1480,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
             ++launches;
         }
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
-        CM_CUDA(ctx, launch_split_reduce(tb, bd, st));
+        CM_CUDA(ctx, launch_split_reduce(tb, bd, bt.bounded ? bt.d_win.p : nullptr, st));
         ++launches;
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
         if (bt.n_tiles) {

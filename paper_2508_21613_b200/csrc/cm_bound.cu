@@ -167,9 +167,15 @@ __device__ __forceinline__ uint64_t block_min_u64(uint64_t v /* warp-uniform */,
     return v;
 }
 
+// Strategies whose step times from bounds are kept from the first look to the second.
+constexpr uint32_t kWinKept = 2048;
+
 __global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd, BoundDev bo, int phase, int k_best, uint64_t inf_cost) {
     __shared__ uint64_t red[32];
     __shared__ unsigned long long total;
+    __shared__ uint32_t kept[kWinKept];
+    __shared__ uint32_t n_listed;
+    __shared__ SearchWin was;
     const uint32_t b = blockIdx.x;
     const Scen sc = bd.scen[b];
     const Tmpl tp = bd.tmpl[sc.tmpl];
@@ -177,28 +183,58 @@ __global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd,
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint64_t inf = phase ? inf_cost : 0xffffffffull;
+    if (threadIdx.x == 0) {
+        n_listed = 0;
+        if (phase) was = bo.win[b];
+    }
+    __syncthreads();
+    // From results, only the strategies that the bounds had within reach can have any step time below infinity
+    // that counts: their segments are the ones that were evaluated.
+    const bool by_list = phase && was.n_strat <= (uint32_t)kWinStrats;
+    const uint32_t n_look = by_list ? was.n_strat : tp.n_strat;
+    auto look_at = [&](uint32_t q) -> const Strat & { return strat[by_list ? was.strat[q] : q]; };
+    auto row_of = [&](uint32_t own) { return bo.row_rep ? bo.row_rep[own] : own; };
     auto cost_of = [&](const Strat &s, int from_results, uint64_t most) {
         return strat_cost(bd, tp, sc, s, most, [&](uint32_t own) {
-            const uint32_t row = bo.row_rep ? bo.row_rep[own] : own;
+            const uint32_t row = row_of(own);
             return from_results ? bd.seg_best[row] : (uint64_t)(bo.lbarg[row] >> 32);
         });
     };
+    constexpr int kSide = 4;   // strategies side by side in a warp
     uint64_t first = ~0ull, t = ~0ull;
     bool enough = false;
     for (int r = 0; r < k_best && !enough; ++r) {
         uint64_t mine = inf;
-        for (uint32_t si = warp; si < tp.n_strat; si += warps) {
-            const uint64_t v = strat_best(cost_of(strat[si], phase, inf), strat[si], t, inf);
-            mine = v < mine ? v : mine;
+        if (!phase && r == 0) {
+            uint32_t v[kSide], least = 0xffffffffu;
+            for (uint32_t si = warp; si < tp.n_strat; si += kSide * warps) {
+                strat_bounds<kSide>(bd, tp, sc, strat, si, warps, bo.lbarg, row_of, v);
+#pragma unroll
+                for (int u = 0; u < kSide; ++u) {
+                    const uint32_t at = si + u * warps;
+                    if (at >= tp.n_strat) break;   // uniform
+                    const uint32_t best = strat_best_bound(v[u], strat[at]);
+                    if (lane == 0 && at < kWinKept) kept[at] = best;
+                    least = best < least ? best : least;
+                }
+            }
+            mine = least;
+        } else {
+            for (uint32_t q = warp; q < n_look; q += warps) {
+                const Strat &s = look_at(q);
+                const uint64_t v = strat_best(cost_of(s, phase, inf), s, t, inf);
+                mine = v < mine ? v : mine;
+            }
         }
         t = block_min_u64(mine, red);
         if (r == 0) first = t;
         if (t >= inf || k_best == 1) break;
         if (threadIdx.x == 0) total = 0;
         __syncthreads();
-        for (uint32_t si = warp; si < tp.n_strat; si += warps) {
+        for (uint32_t q = warp; q < n_look; q += warps) {
+            const Strat &s = look_at(q);
             int f, l;
-            const bool ok = splits_within(cost_of(strat[si], phase, inf), strat[si].dp, strat[si].R, t, f, l);
+            const bool ok = splits_within(cost_of(s, phase, inf), s.dp, s.R, t, f, l);
             if (ok && lane == 0) atomicAdd(&total, (unsigned long long)binom_at(tb.binom, f, l));
         }
         __syncthreads();
@@ -208,38 +244,64 @@ __global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd,
     if (k_best > 1 && !enough && t < inf) t = inf;
     float lo = 0.0f;
     float reach = -1.0f;   // step times from bounds up to here (-1: none)
+    bool relist = true;    // the strategies within reach are listed
     if (phase) {
         reach = __double2float_ru(cost_up(t, native_i64_dev(bd)));
-        const float marked = bo.win[b].reach;
-        lo = bo.win[b].lo;
-        __syncthreads();
+        lo = was.lo;
         if (threadIdx.x == 0) bo.win[b].ub = t;
         // (uniform) phase 0 has marked them all: the results came out as promised
-        if (reach <= marked && !bo.row_rep) return;
+        if (reach <= was.reach && !bo.row_rep) return;
+        relist = !(reach <= was.reach && by_list);
     } else {
         lo = first < inf ? __uint_as_float((uint32_t)first) : 0.0f;
         if (first < inf) reach = t < inf ? __fmul_ru(__uint_as_float((uint32_t)t), 1.0f + kReach) : __uint_as_float(0x7f800000u);
-        if (threadIdx.x == 0) bo.win[b] = SearchWin{lo, reach, inf_cost};
+        if (threadIdx.x == 0) { bo.win[b].lo = lo; bo.win[b].reach = reach; bo.win[b].ub = inf_cost; }
     }
-    for (uint32_t si = warp; si < tp.n_strat; si += warps) {
+    __syncthreads();   // (what was kept)
+    auto mark = [&](uint32_t si, uint32_t best) {   // a strategy and its step time from bounds, warp-uniform
+        if (best == 0xffffffffu || __uint_as_float(best) > reach) return;
         const Strat &s = strat[si];
-        const uint64_t v = strat_best(cost_of(s, 0, 0xffffffffull), s, ~0ull, 0xffffffffull);
-        if (v >= 0xffffffffull || __uint_as_float((uint32_t)v) > reach) continue;   // warp-uniform
+        if (relist && lane == 0) {
+            const uint32_t at = atomicAdd(&n_listed, 1u);
+            if (at < (uint32_t)kWinStrats) bo.win[b].strat[at] = (uint16_t)si;   // (longer lists, and numbers beyond 16 bits, go unused)
+        }
         const int p = lane >> 1, k = lane & 1;
-        if (p < s.dp && k < s.n_m) {
-            uint32_t row = canon_row(bd, tp, sc, s, p, k);
-            if (bo.row_rep) row = bo.row_rep[row];
-            // a bound beyond reach: not part of the answer through this share (where results move the reach up, the
-            // second window marks again)
-            if (lb_of(bo.lbarg[row]) > reach) continue;
-            if (bo.row_rep) {
-                const unsigned long long l = __float_as_uint(lo), u = ~t;   // (u: of a result, phase 1)
-                if (l < bo.row_lo[row]) atomicMin((unsigned long long *)&bo.row_lo[row], l);
-                if (phase && u < bo.row_ub[row]) atomicMin((unsigned long long *)&bo.row_ub[row], u);
+        if (p >= s.dp || k >= s.n_m) return;
+        const uint32_t row = row_of(canon_row(bd, tp, sc, s, p, k));
+        // a bound beyond reach: not part of the answer through this share (where results move the reach up, the
+        // second window marks again)
+        if (lb_of(bo.lbarg[row]) > reach) return;
+        if (bo.row_rep) {
+            const unsigned long long l = __float_as_uint(lo), u = ~t;   // (u: of a result, phase 1)
+            if (l < bo.row_lo[row]) atomicMin((unsigned long long *)&bo.row_lo[row], l);
+            if (phase && u < bo.row_ub[row]) atomicMin((unsigned long long *)&bo.row_ub[row], u);
+        }
+        if (bo.pick[row] == ~0ull) bo.pick[row] = kPickWanted;   // (every writer writes the same)
+    };
+    if (!phase && tp.n_strat <= kWinKept) {
+        for (uint32_t si = warp; si < tp.n_strat; si += warps) { mark(si, kept[si]); __syncwarp(); }
+    } else if (!relist) {
+        for (uint32_t q = warp; q < was.n_strat; q += warps) {
+            const Strat &s = strat[was.strat[q]];
+            mark(was.strat[q], (uint32_t)strat_best(cost_of(s, 0, 0xffffffffull), s, ~0ull, 0xffffffffull));
+            __syncwarp();
+        }
+    } else {
+        uint32_t v[kSide];
+        for (uint32_t si = warp; si < tp.n_strat; si += kSide * warps) {
+            strat_bounds<kSide>(bd, tp, sc, strat, si, warps, bo.lbarg, row_of, v);
+#pragma unroll
+            for (int u = 0; u < kSide; ++u) {
+                const uint32_t at = si + u * warps;
+                if (at >= tp.n_strat) break;   // uniform
+                mark(at, strat_best_bound(v[u], strat[at]));
+                __syncwarp();
             }
-            if (bo.pick[row] == ~0ull) bo.pick[row] = kPickWanted;   // (every writer writes the same)
         }
     }
+    if (!relist) return;
+    __syncthreads();
+    if (threadIdx.x == 0) bo.win[b].n_strat = n_listed <= (uint32_t)kWinStrats && tp.n_strat <= 0x10000u ? n_listed : kWinAll;
 }
 
 cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st) {

@@ -205,8 +205,16 @@ struct BBucket {
     uint32_t min_first;     // its entries of BoundDev::tile_min: by tile, then by segment
 };
 // Step times that can still be a scenario's answer: lo <= T* <= ub, lo from bounds.
-// reach: strategies whose step time from bounds is at most this had their segments marked.
-struct SearchWin { float lo, reach; uint64_t ub; };
+// reach: strategies whose step time from bounds is at most this had their segments marked; strat: these strategies
+// (numbers within the template, in no order) where they are few, n_strat = kWinAll where they are not.
+constexpr int kWinStrats = 14;
+constexpr uint32_t kWinAll = 0xffffffffu;
+struct SearchWin {
+    float lo, reach;
+    uint64_t ub;
+    uint32_t n_strat;
+    uint16_t strat[kWinStrats];
+};
 // A segment of the layout, for the kernels after the first.
 struct SegRec { uint64_t tier; uint32_t row, scen, tseg; int32_t n_sync; };
 struct BoundDev {
@@ -369,7 +377,7 @@ cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo
 cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st);
 cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
 cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches);   // first_list and the next
-cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st);
+cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, const SearchWin *win, cudaStream_t st);   // win: of a search by bounds
 // cm_tiebreak.cu; the second one, for what the first leaves open: stages, the depths there are (bit S-1); by_depth, a
 // launch for each of 17 .. kWideStagesMax
 cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);

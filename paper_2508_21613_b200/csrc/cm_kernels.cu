@@ -506,10 +506,11 @@ struct FullSplit {   // full enumeration, lane = pipeline
     }
 };
 
+// win (a search by bounds): the strategies whose step times from bounds are within reach, one of them the best.
 // words: 64-bit words of a set of sums (full enumeration); dynamic shared memory: two sets per warp, then one per
 // pipeline.
 template <bool FULL>
-__global__ void __launch_bounds__(1024, 1) cm_best_split_kernel(Tables tb, BatchDev bd, uint64_t inf, int words) {
+__global__ void __launch_bounds__(1024, 1) cm_best_split_kernel(Tables tb, BatchDev bd, const SearchWin *win, uint64_t inf, int words) {
     extern __shared__ uint64_t sum_sets[];
     __shared__ uint64_t rc[32];
     __shared__ uint32_t ri[32];
@@ -522,8 +523,11 @@ __global__ void __launch_bounds__(1024, 1) cm_best_split_kernel(Tables tb, Batch
     auto cost_of = [&](const Strat &s) { return strat_cost(bd, tp, sc, s, inf, [&](uint32_t row) { return bd.seg_best[row]; }); };
     uint64_t best_c = inf;
     uint32_t best_i = 0;
+    const bool by_list = win && win[b].n_strat <= (uint32_t)kWinStrats;
+    const uint32_t n_look = by_list ? win[b].n_strat : tp.n_strat;
     if (sc.rep == b)   // (else it shares another scenario's search: nothing to tie-break here)
-        for (uint32_t si = warp; si < tp.n_strat; si += warps) {
+        for (uint32_t q = warp; q < n_look; q += warps) {
+            const uint32_t si = by_list ? win[b].strat[q] : q;
             const Strat &s = strat[si];
             uint64_t v = inf;
             if constexpr (!FULL) {
@@ -532,7 +536,7 @@ __global__ void __launch_bounds__(1024, 1) cm_best_split_kernel(Tables tb, Batch
                 const FullSplit fs{bd, tp, sc, s, inf};
                 v = fs.monotone() ? fs.best(G) : fs.best_any(G, words, sum_sets + (size_t)warp * 2 * words);
             }
-            if (v < best_c) { best_c = v; best_i = si; }
+            if (v < best_c || (v == best_c && v < inf && si < best_i)) { best_c = v; best_i = si; }
         }
     if (lane == 0) { rc[warp] = best_c; ri[warp] = best_i; }
     __syncthreads();
@@ -588,7 +592,7 @@ __global__ void __launch_bounds__(1024, 1) cm_best_split_kernel(Tables tb, Batch
     }
 }
 
-cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t st) {
+cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, const SearchWin *win, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
     // A warp per strategy, latency of its dependent loads: all strategies at once up to a scenario per SM (64 sets
     // of the 64-device job: 8 us with 1024 threads, 12 with 256, 18 with 128), narrower CTAs beyond (515 sets of
@@ -597,9 +601,9 @@ cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, cudaStream_t
     if (b.batch_mode == CM_BATCH_FULL) {
         const int words = t.binom_rows / 64 + 1;   // (the table has a row per micro-batch of the job at least)
         const size_t bytes = (threads / 32 * 2 + kMaxP) * (size_t)words * sizeof(uint64_t);
-        cm_best_split_kernel<true><<<b.B, threads, bytes, st>>>(t, b, batch_inf_bits(b), words);
+        cm_best_split_kernel<true><<<b.B, threads, bytes, st>>>(t, b, win, batch_inf_bits(b), words);
     } else {
-        cm_best_split_kernel<false><<<b.B, threads, 0, st>>>(t, b, batch_inf_bits(b), 0);
+        cm_best_split_kernel<false><<<b.B, threads, 0, st>>>(t, b, win, batch_inf_bits(b), 0);
     }
     return cudaGetLastError();
 }

@@ -70,4 +70,51 @@ __device__ __forceinline__ uint64_t strat_best(uint64_t v, const Strat &s, uint6
     return warp_min_u64(ok ? v : inf);
 }
 
+// The same in 32 bits (bounds, 0xffffffff: none), for N strategies at a time: three dependent loads each, all of them
+// in flight together.  row_of(row): the row that is searched for a row.
+template <int N, typename RowOf>
+__device__ __forceinline__ void strat_bounds(const BatchDev &bd, const Tmpl &tp, const Scen &sc, const Strat *strat, uint32_t first, uint32_t step,
+                                             const uint64_t *lbarg, RowOf row_of, uint32_t (&v)[N]) {
+    const int p = (threadIdx.x & 31) >> 1, k = threadIdx.x & 1;
+    uint32_t t[N];
+    bool ok[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const uint32_t si = first + u * step;
+        const Strat &s = strat[si < tp.n_strat ? si : 0];
+        ok[u] = si < tp.n_strat && p < s.dp && k < s.n_m && s.m_lo[p] + k >= 1;
+        t[u] = ok[u] ? s.seg_first + p * s.n_m + k : tp.tseg_first;
+    }
+    if (bd.tseg_canon) {
+#pragma unroll
+        for (int u = 0; u < N; ++u) t[u] = bd.tseg_canon[t[u]];
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) t[u] = row_of(sc.seg_base + (t[u] - tp.tseg_first));
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const uint32_t w = (uint32_t)(lbarg[t[u]] >> 32);
+        v[u] = ok[u] ? w : 0xffffffffu;
+    }
+}
+// Least step time of a strategy from its bounds: strat_best, whose first case they nearly always are.
+__device__ __forceinline__ uint32_t strat_best_bound(uint32_t v, const Strat &s) {
+    const int lane = threadIdx.x & 31, dp = s.dp, R = s.R;
+    const bool mine = lane < 2 * dp;
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, v, 1);
+    if (R && !__all_sync(0xffffffffu, !mine || (lane & 1 ? v >= other : v <= other))) return (uint32_t)strat_best(v, s, ~0ull, 0xffffffffull);
+    uint32_t t = __reduce_max_sync(0xffffffffu, mine && !(lane & 1) ? v : 0u);   // largest of the smaller shares
+    if (R) {
+        int below = 0;
+        for (int p = 0; p < dp; ++p) {
+            const uint32_t h = __shfl_sync(0xffffffffu, v, 2 * p + 1);
+            below += h < v || (h == v && 2 * p + 1 < lane);
+        }
+        const uint32_t who = __ballot_sync(0xffffffffu, mine && (lane & 1) && below == R - 1);
+        const uint32_t at = who ? __shfl_sync(0xffffffffu, v, __ffs((int)who) - 1) : 0xffffffffu;
+        t = at > t ? at : t;
+    }
+    return t;
+}
+
 }  // namespace cm
