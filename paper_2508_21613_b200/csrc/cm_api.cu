@@ -1317,6 +1317,8 @@ Tables tables_plain(const cm_ctx *ctx) {   // for kernels that only read the byt
     return t;
 }
 
+uint64_t stage_mask(const Batch &bt);
+
 constexpr size_t kStateExtra = kCounters + 2;   // work counters and the counts of four lists (32-bit)
 
 // Room for listed plans and, if there is memory for it, for the least bounds of tiles.  Captured launch sequences
@@ -1484,7 +1486,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
         ++launches;
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
         if (bt.n_tiles) {
-            CM_CUDA(ctx, launch_tiebreak(tb, bd, st));
+            CM_CUDA(ctx, launch_tiebreak(tb, bd, stage_mask(bt), st));
             ++launches;
         }
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[5], st));
@@ -2276,7 +2278,7 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
         sd.B = (int32_t)slots;
         sd.open = bt.d_open.p;
         sd.n_open = bd.counters + 7;
-        CM_CUDA(ctx, launch_tiebreak(tb, sd, st));
+        CM_CUDA(ctx, launch_tiebreak(tb, sd, stage_mask(bt), st));
         ++obj_launches;
         CM_CUDA(ctx, launch_tie_rest(tb, sd, stage_mask(bt), false, st, &obj_launches));
     }

@@ -126,6 +126,10 @@ __device__ __forceinline__ Walk best_walk(const SProf<T> &s, const Cuts &c, int 
     return Walk{lb > 0.0 ? lb : 0.0, g_max, a, kind, ba};
 }
 
+// The exact cost along a walk (walk_cost) is at most `goal` for certain: a walk's value is the same sum in double
+// arithmetic, less kBoundSlack and one for quotients that floor, and either is rounded at most 2 (m + S) <= 8320 times.
+__device__ __forceinline__ bool walk_surely_within(double value, double goal) { return value + 1.0 <= goal * (1.0 - 1.0 / (1ull << 34)); }
+
 // Cost along the walk in the arithmetic and the order of the recurrence: a lower bound of the plan's
 // computed cost, bit for bit.
 template <typename T, typename Cuts>

@@ -504,26 +504,31 @@ __device__ __forceinline__ T sim_lockstep_afab(int S, int m, const T *F, const T
 // zero, then carries ends of the last stage's forwards up and down again, none of them later than the last stage's
 // clock: they change no maximum.)
 // Same operations on the same operands as in any other order: identical bits.
-// Several pipelines of equal S in one warp: `gl` is the lane's number within its pipeline, `last` marks its last
-// lane, m is the pipeline's own and m_lo, m_hi the least and the most of the warp's.  Returns the time in the first
-// lane of every pipeline.
+// Several pipelines in one warp, S and m the lane's own: `gl` is the lane's number within its pipeline, `last` marks
+// its last lane, `mine`, whether it has one (S = m = 0 and times of zero where not).  They end their warm-up
+// together (those of odd depth one slot early, for the odd slot that follows) and then take their rounds side by side.
+// Returns the time in the first lane of every pipeline.
 template <typename T, int NP>
-__device__ __forceinline__ T sim_lockstep_pairs(int S, int m, const T *F, const T *B, const T *xt, int gl, bool last, int m_lo, int m_hi) {
+__device__ __forceinline__ T sim_lockstep_pairs(bool mine, int S, int m, const T *F, const T *B, const T *xt, int gl, bool last) {
     constexpr int PER = 2 * NP;
+    constexpr int kNever = -(1 << 20);   // (no slot or round of a lane without a pipeline)
+    const int odd = S & 1, warm = __reduce_max_sync(0xffffffffu, S + odd);
     T clock[PER], last_f[PER], last_b[PER];
 #pragma unroll
     for (int k = 0; k < PER; ++k) { clock[k] = (T)0; last_f[k] = (T)0; last_b[k] = (T)0; }
     {   // slots 0 .. S-1: warm-up forwards only, forward (i,j) at slot i+j
-        int d = -gl * PER;
-        for (int s = 0; s < S; ++s, ++d) {
+        const int wait = mine ? warm - S - odd : -kNever;   // slots until this pipeline's first
+        int d = -gl * PER - wait;
+        for (int s = 0; s < warm; ++s, ++d) {
             T up = __shfl_up_sync(0xffffffffu, last_f[PER - 1], 1);
             up = gl == 0 ? (T)0 : up;
             T fin[PER];
 #pragma unroll
             for (int k = 0; k < PER; ++k) fin[k] = tmax(clock[k], k ? last_f[k > 0 ? k - 1 : 0] : up) + F[k];
+            const unsigned live = s - wait < S ? (unsigned)m : 0u;
 #pragma unroll
             for (int k = 0; k < PER; ++k)
-                if ((unsigned)(d - k) < (gl * PER + k < S ? (unsigned)m : 0u)) { clock[k] = fin[k]; last_f[k] = fin[k] + xt[k]; }
+                if ((unsigned)(d - k) < (gl * PER + k < S ? live : 0u)) { clock[k] = fin[k]; last_f[k] = fin[k] + xt[k]; }
         }
     }
     unsigned lim_f0[NP], lim_f1[NP], lim_b0[NP], lim_b1[NP];
@@ -535,8 +540,8 @@ __device__ __forceinline__ T sim_lockstep_pairs(int S, int m, const T *F, const 
         lim_b0[e] = at < S ? (unsigned)m : 0u;
         lim_b1[e] = at + 1 < S ? (unsigned)m : 0u;
     }
-    int h = S >> 1;
-    int c = h + gl * NP + 1 - S;   // of the lane's first pair
+    const int h0 = (S + 1) >> 1;           // round that follows the warm-up (and the odd slot)
+    int c = (mine && odd ? h0 - 1 : kNever) + gl * NP + 1 - S;   // of the lane's first pair; first, those of odd depth only
     auto odd_slot = [&](auto tested) {
         T fin0[NP], fin1[NP];
 #pragma unroll
@@ -569,14 +574,16 @@ __device__ __forceinline__ T sim_lockstep_pairs(int S, int m, const T *F, const 
     };
     using Yes = std::true_type;
     using No = std::false_type;
-    if (S & 1) {   // slot S is odd
-        odd_slot(Yes{});
-        ++h; ++c;
-    }
-    const int n_rounds = S + m_hi - 1, all_in = m_lo > S ? S : n_rounds;
-    for (; h < all_in; ++h, ++c) { even_slot(Yes{}); odd_slot(Yes{}); }
-    for (; h < m_lo; ++h, ++c) { even_slot(No{}); odd_slot(No{}); }
-    for (; h < n_rounds; ++h, ++c) { even_slot(Yes{}); odd_slot(Yes{}); }
+    if (__any_sync(0xffffffffu, mine && odd)) odd_slot(Yes{});   // slot S is odd
+    c = (mine ? h0 : kNever) + gl * NP + 1 - S;
+    // rounds r = h - h0: all pipelines run without tests from the last one's S on, to the first one's m
+    const int n_rounds = __reduce_max_sync(0xffffffffu, mine ? S + m - 1 - h0 : 0);
+    const int from = __reduce_max_sync(0xffffffffu, mine ? S - h0 : 0), to = __reduce_min_sync(0xffffffffu, mine ? m - h0 : n_rounds);
+    const int all_in = from < to ? from : n_rounds;
+    int r = 0;
+    for (; r < all_in; ++r, ++c) { even_slot(Yes{}); odd_slot(Yes{}); }
+    for (; r < to; ++r, ++c) { even_slot(No{}); odd_slot(No{}); }
+    for (; r < n_rounds; ++r, ++c) { even_slot(Yes{}); odd_slot(Yes{}); }
     return clock[0];
 }
 
@@ -584,7 +591,7 @@ __device__ __forceinline__ T sim_lockstep_pairs(int S, int m, const T *F, const 
 template <typename T>
 __device__ __forceinline__ T sim_lockstep_warp(int S, int m, const T *F, const T *B, const T *xt) {
     const int lane = threadIdx.x & 31;
-    return __shfl_sync(0xffffffffu, sim_lockstep_pairs<T, 1>(S, m, F, B, xt, lane, lane == 31, m, m), 0);
+    return __shfl_sync(0xffffffffu, sim_lockstep_pairs<T, 1>(true, S, m, F, B, xt, lane, lane == 31), 0);
 }
 
 // Times of the stages from .. from + PER - 1 of a pipeline (zero past its end).

@@ -378,9 +378,9 @@ cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo
 cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
 cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches);   // first_list and the next
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, const SearchWin *win, cudaStream_t st);   // win: of a search by bounds
-// cm_tiebreak.cu; the second one, for what the first leaves open: stages, the depths there are (bit S-1); by_depth, a
+// cm_tiebreak.cu; stages, the depths there are (bit S-1).  The second one, for what the first leaves open: by_depth, a
 // launch for each of 17 .. kWideStagesMax
-cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st);
+cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, uint64_t stages, cudaStream_t st);
 cudaError_t launch_tie_rest(const Tables &t, const BatchDev &b, uint64_t stages, bool by_depth, cudaStream_t st, int *launches);
 cudaError_t launch_tie_rest_deep(const Tables &t, const BatchDev &b, int stages, cudaStream_t st);
 // first kernel of a scenario handled on its own: clear n_words result words, fetch its ids and bits from host memory

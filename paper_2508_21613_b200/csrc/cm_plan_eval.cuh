@@ -677,14 +677,14 @@ __device__ __forceinline__ bool warp_plan_cost(const SProf<T> &sp, const Tables 
     return true;
 }
 
-// Costs of up to three plans of equal depth at a time, each on (S + 3) / 4 lanes with four stages per lane: half the
+// Costs of several plans at a time, each on `width` >= (S + 3) / 4 lanes with four stages per lane: half the
 // instructions per plan of warp_plan_cost where there are more plans than warps.  1F1B.  Arguments are those of
-// the lane's plan: `mine`, whether it has one, `gl`, the lane's number within it, `width` = (S + 3) / 4, `cuts`, kMaxS + 8
+// the lane's plan: `mine`, whether it has one, `gl`, the lane's number within it, `cuts`, kMaxS + 8
 // bytes of its own.  The cost is returned in the plan's first lane; false: no plan, or infeasible.
 template <typename T>
 __device__ __forceinline__ bool group_plan_cost(const SProf<T> &sp, const Tables &tb, int layer_mode, const SegView &g, const Cand &cand, bool mine,
                                                 int gl, int width, uint8_t *cuts, T &cost) {
-    const int S = g.S, m = g.m, lane = threadIdx.x & 31;   // S: the same in every lane
+    const int S = g.S, m = g.m, lane = threadIdx.x & 31;
     CutWalker cw;
     bool ok = mine && m >= 1 && make_walker(cw, tb, layer_mode, sp.L, S, cand, g.K, tb.mm_slot(S, m));
     __syncwarp();   // nobody reads the cuts of earlier plans any more
@@ -716,15 +716,18 @@ __device__ __forceinline__ bool group_plan_cost(const SProf<T> &sp, const Tables
         }
         lane_stages<T, 4>(sp, cuts, S, g.tier, 4 * gl, F, B, xt);
     }
-    const uint32_t all = ((1u << width) - 1u) << (lane - gl);   // (a plan takes at most 16 lanes)
+    const uint32_t all = ((1u << width) - 1u) << (lane - gl);   // (at most 16 lanes)
     ok = (__ballot_sync(0xffffffffu, ok) & all) == all;
     for (int o = 8; o > 0; o >>= 1) {
         const long long og = __shfl_down_sync(0xffffffffu, g_max, o);
         if (gl + o < width) g_max = og > g_max ? og : g_max;
     }
     if (!__any_sync(0xffffffffu, ok)) return false;
-    const int m_lo = __reduce_min_sync(0xffffffffu, ok ? m : 0x7fffffff), m_hi = __reduce_max_sync(0xffffffffu, ok ? m : 0);
-    const T t = sim_lockstep_pairs<T, 2>(S, ok ? m : m_lo, F, B, xt, gl, gl == width - 1, m_lo, m_hi);
+    if (!ok) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { F[k] = (T)0; B[k] = (T)0; xt[k] = (T)0; }
+    }
+    const T t = sim_lockstep_pairs<T, 2>(ok, ok ? S : 0, ok ? m : 0, F, B, xt, gl, gl == width - 1);
     cost = t + Num<T>::sync(g_max, g.n_sync, sp.bw_sync, sp.intval);
     return ok;
 }

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
                 c.fill(cw, g.S);
                 const Walk walk = best_walk<T>(sp, c, g.S, g.m, g.tier, g.n_sync, g.feas_first == kNoFeasList);
                 maybe = walk.value >= 0.0 && walk.value <= goal;
-                if (maybe) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= w_bits;
+                if (maybe && !walk_surely_within(walk.value, goal)) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= w_bits;
             }
         }
         const uint32_t vote = __ballot_sync(0xffffffffu, maybe);
@@ -99,6 +99,100 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
     if (lane == 0 && evaluated) atomicAdd(&bd.counters[1], evaluated);
     if (threadIdx.x == 0 && rounds == 0 && found == ~0ull && !((atomicOr(&bd.winner[b].open, 1u << p) >> p) & 1u))
         bd.open[atomicAdd(bd.n_open, 1ull) + 1ull] = b * kMaxP + p;   // (the count starts at -1)
+}
+
+// ----------------------------------------------------------------------------------
+// The same for a batch of shallow pipelines under 1F1B, eight to a warp: the bounds of 32 candidates of one pipeline
+// after the other, then the lowest candidate that each has left, all of them at a time in lock step, four lanes each
+// (group_plan_cost), until every pipeline has its composition.  A warp of its own keeps six lanes of 32 busy with a pipeline
+// of twelve stages: 2576 sets of the 32-device job 57 us, 106 with the kernel above.  Deeper pipelines stay with that
+// one: three to a warp wait for the one that needs most attempts (1024 sets of the 256-device job 240 us, 160 above).
+// ----------------------------------------------------------------------------------
+constexpr int kTieWarps = 2, kTieMost = 8;
+constexpr uint32_t kTieTiles = 64;   // of kTile candidates
+
+template <typename T>
+__global__ void __launch_bounds__(kTieWarps * 32) cm_tie_batch_kernel(Tables tb, BatchDev bd, uint32_t n_items) {
+    __shared__ SProf<T> sp;
+    __shared__ uint8_t cuts_s[kTieWarps][kTieMost][kRegStagesMax + 8];   // (per pipeline)
+    __shared__ uint8_t cut_col[kTieWarps][kRegStagesMax * 32];
+    if (lists_full(bd)) return;   // uniform
+    stage_profile(sp, tb);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int width = 32 / kTieMost;
+    const int grp = lane / width, gl = lane - grp * width;
+    const uint32_t item0 = (blockIdx.x * kTieWarps + warp) * kTieMost, item = item0 + grp;
+    if (item0 >= n_items) return;   // warp-uniform from here on
+    // the lane's own pipeline
+    bool open = item < n_items;
+    const uint32_t b = open ? item / bd.dp_max : 0, p = open ? item % bd.dp_max : 0;
+    const Winner &w = bd.winner[b];
+    const uint64_t w_bits = w.cost_bits;
+    open = open && w_bits < inf_bits<T>() && p < w.dp;
+    SegView g{};
+    if (open) g = seg_view(bd, w.scen, w.seg[p]);
+    open = open && g.K != 0;            // (one candidate: known already)
+    const uint32_t count = open ? (uint32_t)walk_count(g) : 0u;   // (launch_tiebreak: few)
+    uint32_t base = 0, tile = 0, left = 0, evaluated = 0;
+    int rounds = kTieRoundsWarp;
+    for (;;) {
+        // candidates that its bound does not rule out, for the pipelines that have none left
+        uint32_t want;
+        while ((want = __ballot_sync(0xffffffffu, open && left == 0)) != 0) {
+            const int k = (__ffs((int)want) - 1) / width, from = k * width;
+            SegView q;
+            q.tier = __shfl_sync(0xffffffffu, g.tier, from);
+            q.K = __shfl_sync(0xffffffffu, g.K, from);
+            q.feas_first = __shfl_sync(0xffffffffu, g.feas_first, from);
+            q.S = __shfl_sync(0xffffffffu, g.S, from);
+            q.m = __shfl_sync(0xffffffffu, g.m, from);
+            q.n_sync = __shfl_sync(0xffffffffu, g.n_sync, from);
+            const uint64_t most = __shfl_sync(0xffffffffu, w_bits, from);
+            const uint32_t n = __shfl_sync(0xffffffffu, count, from), first = __shfl_sync(0xffffffffu, base, from);
+            const double goal = std::is_same<T, long long>::value ? __ll2double_ru((long long)most) : __longlong_as_double((long long)most);
+            bool maybe = false;
+            CutWalker cw;
+            if (first + lane < n && make_walker(cw, tb, bd.layer_mode, sp.L, q.S, walk_cand(bd, q.feas_first, first + lane), q.K, tb.mm_slot(q.S, q.m))) {
+                const CutColumn<32> c{cut_col[warp] + lane};
+                c.fill(cw, q.S);
+                const Walk walk = best_walk<T>(sp, c, q.S, q.m, q.tier, q.n_sync, q.feas_first == kNoFeasList);
+                maybe = walk.value >= 0.0 && walk.value <= goal;
+                if (maybe && !walk_surely_within(walk.value, goal))
+                    maybe = Num<T>::bits(walk_cost<T>(sp, c, q.S, q.m, q.tier, q.n_sync, walk)) <= most;
+            }
+            const uint32_t vote = __ballot_sync(0xffffffffu, maybe);
+            if (grp == k) {
+                left = vote;
+                tile = base;
+                base += 32;
+                if (left == 0 && base >= count) open = false;   // (no candidate within the winning cost: not so for a winner)
+            }
+        }
+        if (!__any_sync(0xffffffffu, open)) break;
+        const uint32_t pos = tile + (open ? __ffs((int)left) - 1 : 0);
+        left &= left - 1;
+        Cand cand{0, 0, 0, false};
+        if (open) cand = walk_cand(bd, g.feas_first, pos);
+        T cost;
+        const bool ok = group_plan_cost<T>(sp, tb, bd.layer_mode, g, cand, open, gl, width, cuts_s[warp][grp], cost);
+        const uint32_t hits = __ballot_sync(0xffffffffu, ok && gl == 0 && Num<T>::bits(cost) <= w_bits);
+        if (open) {
+            if (gl == 0) ++evaluated;
+            if ((hits >> (lane - gl)) & 1u) {
+                if (gl == 0) bd.kappa_sel[(size_t)b * kMaxP + p] = cand.kappa;   // (the lowest: this warp alone looks, upwards)
+                open = false;
+            } else if (--rounds == 0) {
+                if (gl == 0 && !((atomicOr(&bd.winner[b].open, 1u << p) >> p) & 1u))
+                    bd.open[atomicAdd(bd.n_open, 1ull) + 1ull] = b * kMaxP + p;   // (the count starts at -1)
+                open = false;
+            }
+            if (!open) left = 0;
+            else if (left == 0 && base >= count) open = false;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) evaluated += __shfl_xor_sync(0xffffffffu, evaluated, o);
+    if (lane == 0 && evaluated) atomicAdd(&bd.counters[1], (unsigned long long)evaluated);
 }
 
 // ----------------------------------------------------------------------------------
@@ -159,7 +253,7 @@ __global__ void __launch_bounds__(kRestThreads) cm_tie_rest_warp_kernel(Tables t
             c.fill(cw, g.S);
             const Walk walk = best_walk<T>(sp, c, g.S, g.m, g.tier, g.n_sync, g.feas_first == kNoFeasList);
             maybe = walk.value >= 0.0 && walk.value <= goal;
-            if (maybe) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= t.w_bits;
+            if (maybe && !walk_surely_within(walk.value, goal)) maybe = Num<T>::bits(walk_cost<T>(sp, c, g.S, g.m, g.tier, g.n_sync, walk)) <= t.w_bits;
         }
         const uint32_t vote = __ballot_sync(0xffffffffu, maybe);
         if (lane == 0) left[warp] = vote;
@@ -205,7 +299,7 @@ cudaError_t launch_tie_rest(const Tables &t, const BatchDev &b, uint64_t stages,
     return cudaGetLastError();
 }
 
-cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st) {
+cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, uint64_t stages, cudaStream_t st) {
     if (b.B <= 0 || b.max_tiles_per_seg == 0 || b.dp_max == 0) return cudaSuccess;
     const uint64_t nx = (uint64_t)b.B * b.dp_max;
     if (nx >= (1ull << 31)) return cudaErrorInvalidConfiguration;
@@ -216,6 +310,13 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, cudaStream_t st)
     // 1024 sets of the 256-device job: 133 us with a warp, 172 us with two, where a plan-per-lane kernel
     // per depth took 1300 us in all.
     const bool wide = nx <= 148 * 2;
+    // Several pipelines to a warp where they have few tiles each (a long walk would hold up the others).
+    if (!wide && t.sched != CM_SCHED_GPIPE && b.max_tiles_per_seg <= kTieTiles && !(stages >> kRegStagesMax)) {
+        const unsigned ctas = (unsigned)((nx + kTieMost * kTieWarps - 1) / (kTieMost * kTieWarps));
+        if (native_i64(b)) cm_tie_batch_kernel<long long><<<ctas, kTieWarps * 32, 0, st>>>(t, b, (uint32_t)nx);
+        else cm_tie_batch_kernel<double><<<ctas, kTieWarps * 32, 0, st>>>(t, b, (uint32_t)nx);
+        return cudaGetLastError();
+    }
     const unsigned threads = wide ? 256 : 32;
     const int n_eval = wide ? 256 / 32 : 1;
     const uint64_t tiles = ((uint64_t)b.max_tiles_per_seg * kTile + threads - 1) / threads;

@@ -1,0 +1,73 @@
+"""Batches whose plans and pipelines are taken several to a warp, bounds where the dearer links are the other
+ones -- against the CPU oracle or the search of one failure at a
+time: plan tuples bit-exact, costs equal."""
+import numpy as np
+import pytest
+
+from paper_2508_21613_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    import torch
+    from paper_2508_21613_b200 import binding, build
+    build.build()
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device; there is no CPU path")
+    return binding
+
+
+def _job(L, pp, micro, seed=5, per_node=8, intra=300, inter=20):
+    rng = np.random.default_rng(seed)
+    fwd = rng.uniform(2.5e6, 3.5e6, L).round()
+    cuts = [round(i * L / pp) for i in range(pp + 1)]
+    return W.make_profile_ns(L, 2, pp, micro, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 8_000_000, cuts,
+                             80_000_000_000, per_node, intra, inter)
+
+
+# depths on either side of 16 and 40 stages, where the pipelines that share a warp go from eight to three to two;
+# odd and even ones side by side; fewer micro-batches than stages as well
+DEPTHS = {"15-18": (36, 16, 24, (2, 2, 15, 18)), "39-42": (84, 41, 48, (2, 2, 39, 42)), "few-micro-batches": (40, 18, 12, (2, 2, 16, 20))}
+
+
+@pytest.mark.parametrize("mode,native", [(0, False), (1, False), (1, True)])
+@pytest.mark.parametrize("name", sorted(DEPTHS))
+def test_batches_of_pipelines_that_share_warps(gpu, oracle_factory, name, mode, native):
+    """800 failure sets: more listed plans than warps, and more pipelines to complete."""
+    L, pp, micro, window = DEPTHS[name]
+    profile = _job(L, pp, micro)
+    opts = W.SearchOptions(*window, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 4000, mode)
+    sets = [[3], [0, pp + 1], [5, 6, pp]]
+    orc = oracle_factory(profile, opts)
+    wants = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_set_int64_arithmetic(ctx, native)
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, [sets[b % 3] for b in range(800)], opts)[0])
+        for b, plan in enumerate(best):
+            want = wants[b % 3]
+            assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (sets[b % 3], plan, want)
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("per_node", [3, 8])
+def test_bounds_where_links_inside_nodes_are_the_dearer(gpu, oracle_factory, per_node):
+    profile = _job(36, 16, 24, per_node=per_node, intra=15, inter=200)
+    opts = W.SearchOptions(2, 2, 13, 18, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15)
+    sets = [[3], [0, 17]]
+    orc = oracle_factory(profile, opts)
+    wants = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets * 60, opts)[0])
+        st = gpu.cm_last_stats(ctx)
+        assert 0 < st["plans_run"] < st["plans_simulated"]
+        for b, plan in enumerate(best):
+            assert plan.key() == wants[b % 2].key() and plan.cost == wants[b % 2].cost, (sets[b % 2], plan, wants[b % 2])
+    finally:
+        gpu.cm_destroy(ctx)
