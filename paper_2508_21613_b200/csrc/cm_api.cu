@@ -2112,10 +2112,10 @@ cm_status cm_select(cm_ctx *ctx, cm_space *const *spaces, int32_t n_spaces, cm_p
         CM_CUDA(ctx, cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0));
     }
     cm_status s = CM_OK;
+    for (int i = 0; i < n_spaces && n_dyn == 1 && s == CM_OK; ++i)   // first what takes longest
+        if (spaces[i]->policy == CM_DYNPAR) s = enqueue_search(ctx, *spaces[i]->own, st, true, &launches, &cost_launches);
     for (int i = 0; i < n_spaces && s == CM_OK; ++i)
-        if (spaces[i]->policy != CM_DYNPAR || n_dyn == 1)
-            s = enqueue_search(ctx, *spaces[i]->own, spaces[i]->policy != CM_DYNPAR && beside ? ctx->pol_stream : st,
-                               spaces[i]->policy == CM_DYNPAR, &launches, &cost_launches);
+        if (spaces[i]->policy != CM_DYNPAR) s = enqueue_search(ctx, *spaces[i]->own, beside ? ctx->pol_stream : st, false, &launches, &cost_launches);
     if (beside) {   // joined even after a failure, so that no side stream runs ahead unobserved
         const cudaError_t e1 = cudaEventRecord(ctx->pol_join, ctx->pol_stream), e2 = cudaStreamWaitEvent(st, ctx->pol_join, 0);
         if (s == CM_OK) { CM_CUDA(ctx, e1); CM_CUDA(ctx, e2); }
@@ -2283,11 +2283,21 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
         CM_CUDA(ctx, launch_tie_rest(tb, sd, stage_mask(bt), false, st, &obj_launches));
     }
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[2], st));
+    // (a matching is a chain in one warp, a plan's rounds are chains in eight: neither fills the GPU, neither needs the other)
+    const bool beside = q.sync_rounds && ctx->pol_stream;
+    if (beside) {
+        CM_CUDA(ctx, cudaEventRecord(ctx->pol_fork, st));
+        CM_CUDA(ctx, cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0));
+    }
     CM_CUDA(ctx, launch_plan_matching(tb, bd, od, st));
     ++obj_launches;
     if (q.sync_rounds) {
-        CM_CUDA(ctx, launch_plan_rounds(tb, bd, od, st));
+        CM_CUDA(ctx, launch_plan_rounds(tb, bd, od, beside ? ctx->pol_stream : st));
         ++obj_launches;
+    }
+    if (beside) {
+        CM_CUDA(ctx, cudaEventRecord(ctx->pol_join, ctx->pol_stream));
+        CM_CUDA(ctx, cudaStreamWaitEvent(st, ctx->pol_join, 0));
     }
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[3], st));
     CM_CUDA(ctx, launch_objective(tb, bd, od, st));

@@ -84,16 +84,9 @@ cudaError_t launch_cost_pass1(const Tables &t, const BatchDev &b, const LaunchCl
     int n_regs = 0;
     uint64_t regs_chunks = 0;
     while (n_regs < n_classes && classes[n_regs].kind == CM_CLASS_REGS) regs_chunks += classes[n_regs++].n_chunks;
-    int first = 0;
-    if (n_regs > 1 && regs_chunks > 0 && regs_chunks <= (uint64_t)kAnyMaxChunks) {
-        const uint32_t b0 = classes[0].bucket_begin, b1 = classes[n_regs - 1].bucket_end;
-        cudaError_t e = native_i64(b) ? launch_shallow_any<long long>(t, b, b0, b1, regs_chunks, st)
-                                                  : launch_shallow_any<double>(t, b, b0, b1, regs_chunks, st);
-        if (e != cudaSuccess) return e;
-        if (launches) ++*launches;
-        first = n_regs;
-    }
-    int n_launch = 0;
+    const bool any = n_regs > 1 && regs_chunks > 0 && regs_chunks <= (uint64_t)kAnyMaxChunks;   // every shallow depth in one launch
+    const int first = any ? n_regs : 0;
+    int n_launch = any ? 1 : 0;
     for (int i = first; i < n_classes; ++i) n_launch += classes[i].n_chunks ? 1 : 0;
     // classes only share the per-segment minima they atomically lower: run them side by side
     const int n_side = (side && n_launch > 1) ? (side->n < n_launch - 1 ? side->n : n_launch - 1) : 0;
@@ -104,11 +97,17 @@ cudaError_t launch_cost_pass1(const Tables &t, const BatchDev &b, const LaunchCl
     }
     cudaError_t err = cudaSuccess;
     int slot = 0;
-    for (int i = first; i < n_classes && err == cudaSuccess; ++i) {
-        if (classes[i].n_chunks == 0) continue;
+    for (int i = any ? first - 1 : first; i < n_classes && err == cudaSuccess; ++i) {
+        const bool all_shallow = any && i == first - 1;
+        if (!all_shallow && classes[i].n_chunks == 0) continue;
         cudaStream_t s = (n_side && slot % (n_side + 1)) ? side->stream[slot % (n_side + 1) - 1] : st;
         ++slot;
-        err = native_i64(b) ? launch_class<long long>(t, b, classes[i], s) : launch_class<double>(t, b, classes[i], s);
+        if (all_shallow) {
+            const uint32_t b0 = classes[0].bucket_begin, b1 = classes[n_regs - 1].bucket_end;
+            err = native_i64(b) ? launch_shallow_any<long long>(t, b, b0, b1, regs_chunks, s) : launch_shallow_any<double>(t, b, b0, b1, regs_chunks, s);
+        } else {
+            err = native_i64(b) ? launch_class<long long>(t, b, classes[i], s) : launch_class<double>(t, b, classes[i], s);
+        }
         if (err == cudaSuccess && launches) ++*launches;
     }
     // always join, even after a failed launch, so that the side streams never run ahead unobserved

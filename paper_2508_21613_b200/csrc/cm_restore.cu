@@ -25,13 +25,13 @@ namespace cm {
 // ----------------------------------------------------------------------------------
 // Shortlist: topk rounds of a block-wide argmin over the scenario's (strategy, split)
 // items; round r takes the least (step time, item) pair that comes after round r-1's.  Step times are
-// worked out once and kept in shared memory where they fit (kShortKept); the rounds are what is left: 64
-// sets of the 256-device job 57 us, 217 us when every round worked them out again.
+// worked out once and kept in shared memory where they fit (kShortKept), and the records of the pairs found are
+// written by a warp each once all are known.
 // ----------------------------------------------------------------------------------
 constexpr uint64_t kShortKept = 4096;
 __global__ void __launch_bounds__(256) cm_shortlist_kernel(Tables tb, BatchDev bd, ObjDev od, uint64_t inf) {
     __shared__ uint64_t rc[8], ri[8];
-    __shared__ uint64_t last_c, last_i;
+    __shared__ uint64_t found_c[kMaxShort], found_i[kMaxShort];
     const uint32_t b = blockIdx.x;
     const Scen sc = bd.scen[b];
     const Tmpl tp = bd.tmpl[sc.tmpl];
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) cm_shortlist_kernel(Tables tb, BatchDev b
     for (int r = 0; r < od.topk; ++r) {
         uint64_t best_c = inf, best_i = ~0ull;
         if (!exhausted) {
-            const uint64_t lc = r ? last_c : 0, li = r ? last_i : 0;
+            const uint64_t lc = r ? found_c[r - 1] : 0, li = r ? found_i[r - 1] : 0;
             for (uint64_t item = threadIdx.x; item < tp.n_split_total; item += blockDim.x) {
                 const uint64_t T = item < n_kept ? kept[item] : item_step_time(tb, bd, tp, best, item, inf);
                 if (T >= inf) continue;
@@ -59,24 +59,28 @@ __global__ void __launch_bounds__(256) cm_shortlist_kernel(Tables tb, BatchDev b
             uint64_t oi = __shfl_xor_sync(0xffffffffu, best_i, o);
             if (pair_less(oc, oi, best_c, best_i)) { best_c = oc; best_i = oi; }
         }
-        __syncthreads();   // everybody has read last_c / last_i of the previous round
+        __syncthreads();   // everybody has read the partial results of the previous round
         if ((threadIdx.x & 31) == 0) { rc[threadIdx.x >> 5] = best_c; ri[threadIdx.x >> 5] = best_i; }
         __syncthreads();
-        const size_t slot = (size_t)b * od.topk + r;
         if (threadIdx.x == 0) {
             for (int w = 1; w < 8; ++w)
                 if (pair_less(rc[w], ri[w], best_c, best_i)) { best_c = rc[w]; best_i = ri[w]; }
-            last_c = best_c;
-            last_i = best_i;
+            found_c[r] = best_c;
+            found_i[r] = best_i;
+        }
+        __syncthreads();
+        if (found_c[r] >= inf) exhausted = true;   // uniform: nothing is left for later rounds either
+    }
+    for (int r = threadIdx.x >> 5; r < od.topk; r += 8) {
+        const size_t slot = (size_t)b * od.topk + r;
+        if ((threadIdx.x & 31) == 0) {
             Winner w;
-            decode_winner(tb, bd, tp, b, best_c, best_i, inf, w);
+            decode_winner(tb, bd, tp, b, found_c[r], found_i[r], inf, w);
             od.short_win[slot] = w;
             od.short_bytes[slot] = -1;
         }
-        __syncthreads();   // last_c / last_i and the record are written
-        if (threadIdx.x < kMaxP) init_kappa_sel(bd, od.short_win[slot], od.short_kappa + slot * kMaxP, (int)threadIdx.x);
-        __syncthreads();
-        if (last_c >= inf) exhausted = true;   // uniform: nothing is left for later rounds either
+        __syncwarp();      // the record is written
+        if ((threadIdx.x & 31) < kMaxP) init_kappa_sel(bd, od.short_win[slot], od.short_kappa + slot * kMaxP, (int)(threadIdx.x & 31));
     }
 }
 
