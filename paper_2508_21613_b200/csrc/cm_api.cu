@@ -165,6 +165,10 @@ struct Batch {
     // from the pinned arena and its last one writes the plans to pinned memory, so that no copy sits on the
     // path (two copies in, one out: ~8 us of a 95 us call).
     bool direct = false;
+    // Plans in two parts (FinalPart), as the last enqueued search lays them out; policy_out: where the caller wants those
+    // of the one-plan policies (three plans per scenario), handed: they are there.
+    bool parted = false, handed = false;
+    cm_plan *policy_out = nullptr;
     int k_best = 1;                       // (strategy, split) pairs whose step times have to be exact
 };
 
@@ -1439,6 +1443,12 @@ cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchD
     return CM_OK;
 }
 
+// What comes back when a search is done (of parted plans, the second part): from the front of the plans.
+size_t last_bytes(const Batch &bt) {
+    const size_t tail = kCounters * sizeof(unsigned long long) + (bt.parted ? (size_t)bt.B : 0);
+    return (size_t)bt.B * (bt.parted ? 1 : 4) * sizeof(cm_plan) + tail;
+}
+
 // Enqueue the launch sequence of a search on `st`: clear, the two one-plan policies, search
 // pass, split reduction, tie-break pass, finalize, plans back to the host.  phase_events: record
 // the events between the phases (not while the sequence is being captured into a graph).
@@ -1459,12 +1469,19 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     }
     const bool policies = (bt.policy_mask & ((1u << CM_REROUTE) | (1u << CM_REDUNDANT))) != 0;
     const bool beside = policies && (bt.policy_mask & (1u << CM_DYNPAR)) && ctx->pol_stream;
+    bt.parted = beside && !bt.direct;
     if (policies) {
         if (beside) {
             CM_CUDA(ctx, cudaEventRecord(ctx->pol_fork, st));
             CM_CUDA(ctx, cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0));
         }
         CM_CUDA(ctx, launch_policies(tb, bd, ctx->hp.n_dp, beside ? ctx->pol_stream : st));
+        if (bt.parted) {   // their plans go home while the search runs
+            CM_CUDA(ctx, launch_finalize(tb, bd, kFinalFixed, ctx->pol_stream));
+            CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p + 2 * (size_t)bt.B, bt.d_plans.p + 2 * (size_t)bt.B, 2 * (size_t)bt.B * sizeof(cm_plan),
+                                         cudaMemcpyDeviceToHost, ctx->pol_stream));
+            ++launches;
+        }
         if (beside) CM_CUDA(ctx, cudaEventRecord(ctx->pol_join, ctx->pol_stream));
         ++launches;
     }
@@ -1492,13 +1509,10 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[5], st));
     }
     if (beside) CM_CUDA(ctx, cudaStreamWaitEvent(st, ctx->pol_join, 0));
-    CM_CUDA(ctx, launch_finalize(tb, bd, st));
+    CM_CUDA(ctx, launch_finalize(tb, bd, bt.parted ? kFinalDyn : kFinalAll, st));
     ++launches;
     if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
-    if (!bt.direct) {
-        const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
-        CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, back_bytes, cudaMemcpyDeviceToHost, st));
-    }
+    if (!bt.direct) CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, last_bytes(bt), cudaMemcpyDeviceToHost, st));
     *launches_out += launches;
     *cost_launches_out += cost_launches;
     return CM_OK;
@@ -1513,7 +1527,7 @@ uint64_t stage_mask(const Batch &bt) {
 
 // Work counters of a finished search (they came back behind its plans).
 const unsigned long long *search_counters(const Batch &bt) {
-    return reinterpret_cast<const unsigned long long *>(bt.plans_host.p + (size_t)bt.B * 4);
+    return reinterpret_cast<const unsigned long long *>(bt.plans_host.p + (size_t)bt.B * (bt.parted ? 1 : 4));
 }
 void account_search(cm_ctx *ctx, const Batch &bt, int launches) {
     const unsigned long long *counters_host = search_counters(bt);
@@ -1538,13 +1552,12 @@ cm_status finish_tiebreak(cm_ctx *ctx, Batch &bt, int *launches) {
     ctx->stats[22] += search_counters(bt)[6];
     CM_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
     CM_CUDA(ctx, launch_tie_rest(tb, bd, stage_mask(bt), true, st, launches));
-    CM_CUDA(ctx, launch_finalize(tb, bd, st));
+    CM_CUDA(ctx, launch_finalize(tb, bd, bt.parted ? kFinalDyn : kFinalAll, st));
     ++*launches;
     CM_CUDA(ctx, cudaEventRecord(ctx->ev[5], st));
     if (!bt.direct) {
-        const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
-        CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, back_bytes, cudaMemcpyDeviceToHost, st));
-        ctx->stats[10] += back_bytes;
+        CM_CUDA(ctx, cudaMemcpyAsync(bt.plans_host.p, bt.d_plans.p, last_bytes(bt), cudaMemcpyDeviceToHost, st));
+        ctx->stats[10] += last_bytes(bt);
     }
     CM_CUDA(ctx, cudaStreamSynchronize(st));
     float ms = 0.f;
@@ -1555,6 +1568,14 @@ cm_status finish_tiebreak(cm_ctx *ctx, Batch &bt, int *launches) {
 }
 
 cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single = nullptr);
+
+// The first part of parted plans to the caller (2576 scenarios: 1.2 of 2.4 MB, which the host would otherwise wait for
+// and copy when the search is done).
+void hand_out_fixed(Batch &bt, cm_plan *per_policy) {
+    const cm_plan *from = bt.plans_host.p + 2 * (size_t)bt.B;
+    for (int b = 0; b < bt.B; ++b) memcpy(per_policy + 3 * (size_t)b, from + 2 * (size_t)b, 2 * sizeof(cm_plan));
+    bt.handed = true;
+}
 
 // After a bounded search whose lists were full (bounds left hundreds of thousands of plans): again, every plan.
 cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *single) {
@@ -1581,8 +1602,8 @@ cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *
 cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single) {
     cudaStream_t st = ctx->stream;
     int launches = 0, cost_launches = 0;
-    const size_t back_bytes = (size_t)bt.B * 4 * sizeof(cm_plan) + kCounters * sizeof(unsigned long long);
     if (!bt.plans_host.resize((size_t)bt.B * 4 + 1)) return fail(ctx, CM_ENOMEM, "host memory");
+    bt.handed = false;
     const uint64_t h_enqueue = now_ns();
     bool replay = false;
     if (single && ctx->use_graphs && ctx->graph_stream && !single->graph_failed) {
@@ -1613,6 +1634,10 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
     }
     launches += launches_so_far;
     const uint64_t h_wait = now_ns();
+    if (bt.parted && bt.policy_out) {
+        CM_CUDA(ctx, cudaEventSynchronize(ctx->pol_join));
+        hand_out_fixed(bt, bt.policy_out);
+    }
     CM_CUDA(ctx, cudaStreamSynchronize(st));
     ctx->stats[14] += h_wait - h_enqueue;
     ctx->stats[15] += now_ns() - h_wait;
@@ -1626,7 +1651,7 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
         ctx->stats[11] += (uint64_t)((double)ms_tie * 1e6);
         ctx->stats[12] += (uint64_t)cost_launches;
     }
-    ctx->stats[10] += back_bytes;
+    ctx->stats[10] += last_bytes(bt) + (bt.parted ? 2 * (size_t)bt.B * sizeof(cm_plan) : 0);
     if (bt.bounded && search_counters(bt)[4]) {
         return search_directly(ctx, bt, launches, single);
     }
@@ -1658,7 +1683,19 @@ void scrub(cm_plan &pl) {
 }
 
 // Plans of a finished search to the caller's arrays (per_policy may be NULL).
-void hand_out(const Batch &bt, cm_plan *best, cm_plan *per_policy) {
+void hand_out(Batch &bt, cm_plan *best, cm_plan *per_policy) {
+    if (bt.parted) {
+        const cm_plan *dyn = bt.plans_host.p, *fixed = bt.plans_host.p + 2 * (size_t)bt.B;
+        const uint8_t *choice = reinterpret_cast<const uint8_t *>(search_counters(bt) + kCounters);
+        if (per_policy && !bt.handed) hand_out_fixed(bt, per_policy);
+        for (int b = 0; b < bt.B; ++b) {
+            if (per_policy) per_policy[3 * (size_t)b + CM_DYNPAR] = dyn[b];
+            if (choice[b] == kNoPolicy) memset(&best[b], 0, sizeof(cm_plan));
+            else if (per_policy) best[b] = per_policy[3 * (size_t)b + choice[b]];
+            else best[b] = choice[b] == CM_DYNPAR ? dyn[b] : fixed[2 * (size_t)b + choice[b]];
+        }
+        return;
+    }
     memcpy(best, bt.plans_host.p, sizeof(cm_plan) * bt.B);
     if (per_policy) memcpy(per_policy, bt.plans_host.p + bt.B, sizeof(cm_plan) * 3 * (size_t)bt.B);
 }
@@ -2188,7 +2225,10 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
         if ((s = build_batch(ctx, bt, failed_ids, offsets, B, *opts, mask)) != CM_OK) { forget_keys(ctx, bt); return s; }
         ctx->stats[13] += now_ns() - h0;
         if ((s = upload_batch(ctx, bt, &launches)) != CM_OK) { forget_keys(ctx, bt); return s; }
-        if ((s = run_batch(ctx, bt, launches)) != CM_OK) return s;
+        bt.policy_out = best_per_policy;
+        s = run_batch(ctx, bt, launches);
+        bt.policy_out = nullptr;
+        if (s != CM_OK) return s;
         hand_out(bt, best_per_scenario, best_per_policy);
         return CM_OK;
     }
@@ -2264,6 +2304,7 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
     od.short_win = bt.d_short_win.p; od.short_kappa = bt.d_short_kappa.p; od.short_bytes = bt.d_short_bytes.p;
     od.short_assign = bt.d_short_assign.p; od.short_plans = shortlist ? bt.d_short_plans.p : nullptr;
     od.best = bt.d_obj_best.p; od.trans = bt.d_trans.p;
+    od.fixed = bd.plans + (bt.parted ? 2 * (size_t)B : (size_t)B); od.fixed_stride = bt.parted ? 2 : 3;
     cudaStream_t st = ctx->stream;
     int obj_launches = 0;
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[0], st));
@@ -2501,7 +2542,9 @@ cm_status cm_batch_search(cm_ctx *ctx, cm_batch *bp, cm_plan *best_per_scenario,
     memset(ctx->stats, 0, sizeof(ctx->stats));
     Batch &bt = *bp->own;
     if (bt.B == 0) return CM_OK;
+    bt.policy_out = best_per_policy;
     cm_status s = run_batch(ctx, bt, 0);
+    bt.policy_out = nullptr;
     if (s != CM_OK) return s;
     hand_out(bt, best_per_scenario, best_per_policy);
     return CM_OK;

@@ -330,6 +330,8 @@ struct ObjDev {
     cm_plan *short_plans;     // [B*topk] or NULL
     cm_plan *best;            // [B]
     cm_transition *trans;     // [B]
+    const cm_plan *fixed;     // plans of the one-plan policies: two of every fixed_stride
+    int32_t fixed_stride, pad;
 };
 
 // Transition time of a reconstruction that moves `bytes` of model state (Section "Estimator",
@@ -386,7 +388,13 @@ cudaError_t launch_tie_rest_deep(const Tables &t, const BatchDev &b, int stages,
 // first kernel of a scenario handled on its own: clear n_words result words, fetch its ids and bits from host memory
 cudaError_t launch_prologue(uint64_t *words, size_t n_words, const uint32_t *ids_host, uint32_t *ids, int n_ids,
                             const uint64_t *bits_host, uint64_t *bits, int n_bits, cudaStream_t st);
-cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st);
+// What cm_finalize_kernel writes.  All: the best plan of every scenario, then the three per policy.  A batch gets its plans in
+// two parts, so that the first is with the caller before the search is done: the one-plan policies' (from entry 2 B of
+// the plans on, two per scenario), then the DYNPAR plans (from entry 0) and, from entry B, the work
+// counters and a byte per scenario: the policy of its best plan, kNoPolicy if there is none.
+enum FinalPart { kFinalAll = 0, kFinalFixed = 1, kFinalDyn = 2 };
+constexpr uint8_t kNoPolicy = 255;
+cudaError_t launch_finalize(const Tables &t, const BatchDev &b, FinalPart part, cudaStream_t st);
 // Candidates of a space one by one (cm_evaluate.cu).  EvalDev: outputs (any may be NULL) and, for the
 // binned path, the lists of candidates by depth.
 struct EvalDev {

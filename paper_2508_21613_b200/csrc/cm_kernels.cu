@@ -638,13 +638,13 @@ cudaError_t launch_prologue(uint64_t *words, size_t n_words, const uint32_t *ids
 // per policy follow scenario by scenario, so that the host hands both out in one piece each.
 // Latency of a few dependent loads: 6 us (a thread per plan walked its pipelines one by one).
 // ----------------------------------------------------------------------------------
-constexpr int kFinalThreads = 64;
-__global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, BatchDev bd, uint64_t inf) {
+constexpr int kFinalThreads = 64;   // half of them write a part (FinalPart)
+__global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, BatchDev bd, FinalPart part, uint64_t inf) {
     const uint32_t b = blockIdx.x;
-    const int slot = threadIdx.x >> 4, k = threadIdx.x & 15;
-    if (b == 0 && threadIdx.x < kCounters) {
+    const int slot = (threadIdx.x >> 4) + (part == kFinalDyn ? 2 : 0), k = threadIdx.x & 15;
+    unsigned long long *tail = reinterpret_cast<unsigned long long *>(bd.plans + (size_t)bd.B * (part == kFinalDyn ? 1 : 4));
+    if (b == 0 && threadIdx.x < kCounters && part != kFinalFixed) {
         // work counters ride home behind the plans (they start at all-ones, i.e. -1)
-        unsigned long long *tail = reinterpret_cast<unsigned long long *>(bd.plans + (size_t)bd.B * 4);
         tail[threadIdx.x] = bd.counters[threadIdx.x] + 1ull;
     }
     const DevProfile *p = tb.prof;
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, B
     const Winner &w = bd.winner[sc.rep];   // its own search, or the one it shares
     uint64_t cost[3];
     for (int pol = 0; pol < 3; ++pol) {
-        const uint64_t c = !(sc.policy_mask & (1u << pol)) ? inf : pol < 2 ? bd.pol_cost[2 * b + pol] : w.cost_bits;
+        const uint64_t c = !(sc.policy_mask & (1u << pol)) || (pol == 2 && part == kFinalFixed) ? inf : pol < 2 ? bd.pol_cost[2 * b + pol] : w.cost_bits;
         cost[pol] = c < inf ? c : inf;
     }
     int pol = slot;
@@ -663,13 +663,17 @@ __global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, B
             if (cost[q] < cost[pol]) pol = q;
         any = cost[pol] < inf;             // (else an empty plan)
     }
+    if (part == kFinalDyn && slot == 3) {   // the caller has the plan
+        if (k == 0) reinterpret_cast<uint8_t *>(tail + kCounters)[b] = any ? (uint8_t)pol : kNoPolicy;
+        return;                             // (its half of the warp)
+    }
     const bool dyn = pol == CM_DYNPAR, feasible = cost[pol] < inf, filled = any && (!dyn || feasible);
     const int n = !filled ? 0 : dyn ? (int)w.dp : p->n_dp < kMaxP ? p->n_dp : kMaxP;
     uint64_t kappa = k < n && dyn ? bd.kappa_sel[(size_t)sc.rep * kMaxP + k] : 0ull;
     // (a composition that was not found cannot happen for a feasible winner, but is never handed out as a rank)
-    const uint32_t lost = __ballot_sync(0xffffffffu, kappa == ~0ull) >> (threadIdx.x & 16) & 0xffffu;
+    const uint32_t lost = __ballot_sync(part == kFinalDyn ? 0xffffu : 0xffffffffu, kappa == ~0ull) >> (threadIdx.x & 16) & 0xffffu;
     if (kappa == ~0ull) kappa = 0ull;
-    cm_plan &out = bd.plans[slot == 3 ? (size_t)b : (size_t)bd.B + 3 * (size_t)b + slot];
+    cm_plan &out = bd.plans[part == kFinalFixed ? 2 * ((size_t)bd.B + b) + slot : part == kFinalDyn || slot == 3 ? (size_t)b : (size_t)bd.B + 3 * (size_t)b + slot];
     if (k == 0) {
         out.policy = any ? pol : 0;
         out.feasible = feasible && !lost ? 1 : 0;
@@ -686,10 +690,10 @@ __global__ void __launch_bounds__(kFinalThreads) cm_finalize_kernel(Tables tb, B
     out.kappa[k] = kappa;
 }
 
-cudaError_t launch_finalize(const Tables &t, const BatchDev &b, cudaStream_t st) {
+cudaError_t launch_finalize(const Tables &t, const BatchDev &b, FinalPart part, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
     const uint64_t inf = batch_inf_bits(b);
-    cm_finalize_kernel<<<b.B, kFinalThreads, 0, st>>>(t, b, inf);
+    cm_finalize_kernel<<<b.B, part == kFinalAll ? kFinalThreads : kFinalThreads / 2, 0, st>>>(t, b, part, inf);
     return cudaGetLastError();
 }
 

@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(32) cm_objective_kernel(Tables tb, BatchDev bd
     __shared__ int win_slot;
     const uint32_t b = blockIdx.x;
     const int mode = bd.mode;
-    const cm_plan *pol = bd.plans + bd.B + 3 * (size_t)b;
+    const cm_plan *pol = od.fixed + (size_t)od.fixed_stride * b;
     if (threadIdx.x == 0) {
         cm_transition tr;
         tr.rounds = 0; tr.domains = 0; tr.t_sync = 0.0; tr.t_sync_ns = 0;

@@ -1,5 +1,5 @@
 """Batches whose plans and pipelines are taken several to a warp, bounds where the dearer links are the other
-ones -- against the CPU oracle or the search of one failure at a
+ones, and plans that come home in two parts -- against the CPU oracle or the search of one failure at a
 time: plan tuples bit-exact, costs equal."""
 import numpy as np
 import pytest
@@ -69,5 +69,27 @@ def test_bounds_where_links_inside_nodes_are_the_dearer(gpu, oracle_factory, per
         assert 0 < st["plans_run"] < st["plans_simulated"]
         for b, plan in enumerate(best):
             assert plan.key() == wants[b % 2].key() and plan.cost == wants[b % 2].cost, (sets[b % 2], plan, wants[b % 2])
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_plans_of_a_batch_come_in_two_parts(gpu, mode):
+    """Sets that every policy survives, that rerouting does not (a stage lost in every pipeline), and that nothing
+    does (no strategy for the survivors): the same plans as one failure at a time, with and without those per policy."""
+    profile = _job(12, 4, 8, per_node=4)
+    opts = W.SearchOptions(2, 2, 3, 4, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15, mode)
+    sets = [[1], [1, 5], [0, 4], [0, 4, 1], [], [7]] * 9
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        want, want_pol, _ = gpu.cm_search_batch(ctx, sets, opts, per_policy=True, latency=True)
+        for per_policy in (True, False):
+            best, pol, _ = gpu.cm_search_batch(ctx, sets, opts, per_policy=per_policy)
+            assert bytes(best) == bytes(want)
+            if per_policy:
+                assert bytes(pol) == bytes(want_pol)
+        feasible = [p.feasible for p in gpu.plans_from_array(want)]
+        assert any(feasible) and not all(feasible)
     finally:
         gpu.cm_destroy(ctx)
