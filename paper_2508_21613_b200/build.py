@@ -16,7 +16,7 @@ SOURCES = ["cm_cost_shallow_f64.cu", "cm_cost_shallow_i64.cu",
 DEEP_RANGES = [(17, 28), (29, 34), (35, 41), (42, 48), (49, 56), (57, 64)]
 DEEP_UNITS = [(f"{tag}_{lo}_{hi}", [f"-DCM_DEEP_T={ctype}", f"-DCM_DEEP_LO={lo}", f"-DCM_DEEP_HI={hi}"])
               for lo, hi in DEEP_RANGES for tag, ctype in (("f64", "double"), ("i64", "long long"))]
-HEADERS = ["cm_internal.h", "cm_device.cuh", "cm_plan_eval.cuh", "cm_bound.cuh", "cm_bound_lane.cuh", "cm_eval_out.cuh", "cm_split.cuh", "cm_tie_rest.cuh", "cm_cost_impl.cuh"]
+HEADERS = ["cm_internal.h", "cm_device.cuh", "cm_plan_eval.cuh", "cm_bound.cuh", "cm_bound_lane.cuh", "cm_eval_out.cuh", "cm_split.cuh", "cm_tie_rest.cuh", "cm_cost_impl.cuh", "cm_launch.cuh"]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",

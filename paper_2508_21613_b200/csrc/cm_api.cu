@@ -215,6 +215,7 @@ struct cm_ctx {
     DevBuf<unsigned char> d_feas_stage;
     DevBuf<uint4> d_eval;             // cm_evaluate: candidates listed by depth
     DevBuf<uint4> d_bound_list;       // plans the bounded search pass lists for the recurrence
+    DevBuf<uint32_t> d_open_parts;    // parts of its layout with something to compare
     DevBuf<SegRec> d_seg_rec;         // the segments of its layout
     DevBuf<float> d_tile_min;         // its least bounds per tile of compositions and segment
     bool uniform_p2p = false;         // every stage boundary moves the same bytes
@@ -660,6 +661,7 @@ cm_status layout_bound(cm_ctx *ctx, Batch &bt, std::vector<BBucket> &groups) {
     bo.parts = 1;
     for (const BBucket &g : groups) bo.parts = std::max<uint32_t>(bo.parts, ((uint32_t)g.seg_group + 127) / 128);
     if (chunks * bo.parts >= 0x7fffffffull) return CM_OK;
+    bo.few = chunks * bo.parts <= 4 * 148;
     bo.n_buckets = (uint32_t)groups.size();
     bo.n_chunks = (uint32_t)chunks;
     bo.n_segs = (uint32_t)n_segs;
@@ -1323,16 +1325,17 @@ Tables tables_plain(const cm_ctx *ctx) {   // for kernels that only read the byt
 
 uint64_t stage_mask(const Batch &bt);
 
-constexpr size_t kStateExtra = kCounters + 2;   // work counters and the counts of four lists (32-bit)
+constexpr size_t kStateExtra = kCounters + 3;   // work counters and the counts of six lists (32-bit)
 
 // Room for listed plans and, if there is memory for it, for the least bounds of tiles.  Captured launch sequences
 // carry the addresses: dropped when they move.
 cm_status reserve_bound_list(cm_ctx *ctx, Batch &bt) {
     const size_t want = bt.bo.list_first[4], mins = bt.tile_mins, segs = bt.bo.n_segs;
-    if (want <= ctx->d_bound_list.cap && segs <= ctx->d_seg_rec.cap && mins <= ctx->d_tile_min.cap) return CM_OK;
+    const size_t parts = bt.bo.few || (uint64_t)bt.bo.n_chunks * bt.bo.parts > kTileMinMax ? 0 : (size_t)bt.bo.n_chunks * bt.bo.parts;
+    if (want <= ctx->d_bound_list.cap && segs <= ctx->d_seg_rec.cap && parts <= ctx->d_open_parts.cap && mins <= ctx->d_tile_min.cap) return CM_OK;
     CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (!ctx->d_tile_min.reserve(mins)) bt.tile_mins = 0;
-    if (!ctx->d_bound_list.reserve(want) || !ctx->d_seg_rec.reserve(segs)) return fail(ctx, CM_ENOMEM, "device memory");
+    if (!ctx->d_bound_list.reserve(want) || !ctx->d_seg_rec.reserve(segs) || !ctx->d_open_parts.reserve(parts)) return fail(ctx, CM_ENOMEM, "device memory");
     for (auto &e : ctx->single)
         if (e->exec) { cudaGraphExecDestroy(e->exec); e->exec = nullptr; }
     return CM_OK;
@@ -1427,17 +1430,18 @@ cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchD
     }
     bo.list = ctx->d_bound_list.p;
     bo.rec = ctx->d_seg_rec.p;
+    bo.work = (uint64_t)bo.n_chunks * bo.parts <= kTileMinMax ? ctx->d_open_parts.p : nullptr;
     bo.tile_min = bt.tile_mins ? ctx->d_tile_min.p : nullptr;
     CM_CUDA(ctx, launch_bound(tb, bd, bo, st));
     ++*launches;
     for (int phase = 1; phase <= 2; ++phase) {
         CM_CUDA(ctx, launch_window(tb, bd, bo, phase - 1, bt.k_best, st));
-        CM_CUDA(ctx, launch_refine(tb, bd, bo, phase, st));
+        CM_CUDA(ctx, launch_refine(tb, bd, bo, phase, st, launches));
         if (phase == 1) {
             CM_CUDA(ctx, launch_gather(tb, bd, bo, st));
             ++*launches;
         }
-        *launches += 2;
+        ++*launches;
         CM_CUDA(ctx, launch_lists(tb, bd, bo, 2 * phase - 2, st, launches));
     }
     return CM_OK;

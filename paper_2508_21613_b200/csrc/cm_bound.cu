@@ -76,8 +76,15 @@ __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, Batc
         segs[tid] = seg_lite(g.tier, g.row, g.n_sync, sp.bw_sync);
         if (job.tile == 0) bo.rec[bk.seg_first + base + tid] = seg_record(g);
     };
+    LaneBound v;
+    if (bo.few) {   // the compositions while the kernel before this one ends
+        v = lane_of<T, UNI_X, false>(sp, tb, bd, bk, any, cand, dear, terms + tid * kTermSize<UNI_X>, nullptr);
+        after_previous();
+    } else {
+        after_previous();
+    }
     take_segments(job.s0, (int)min(job.s1 - job.s0, (uint32_t)kBoundSegs));
-    const LaneBound v = lane_of<T, UNI_X, false>(sp, tb, bd, bk, any, cand, dear, terms + tid * kTermSize<UNI_X>, nullptr);
+    if (!bo.few) v = lane_of<T, UNI_X, false>(sp, tb, bd, bk, any, cand, dear, terms + tid * kTermSize<UNI_X>, nullptr);
     comp[tid] = make_float4(v.best, v.u0, v.g, 0.0f);
     const float delta = dear_extra(sp, dear), slack = sp.intval || std::is_same<T, long long>::value ? 1.0f : 0.0f;
     const bool gpipe = sp.sched == CM_SCHED_GPIPE;
@@ -141,8 +148,7 @@ template <typename T, bool UNI_X>
 static cudaError_t launch_bound_one(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(cm_bound_kernel<T, UNI_X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBoundDynMax);
     if (e != cudaSuccess) return e;
-    cm_bound_kernel<T, UNI_X><<<bo.n_chunks, kBoundThreads, bo.dyn_bytes, st>>>(t, b, bo);
-    return cudaGetLastError();
+    return launch_next(cm_bound_kernel<T, UNI_X>, bo.n_chunks, kBoundThreads, bo.dyn_bytes, st, t, b, bo);
 }
 cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st) {
     if (bo.n_chunks == 0) return cudaSuccess;
@@ -182,6 +188,7 @@ __global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd,
     const Strat *strat = bd.strat + tp.strat_first;
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31;
+    after_previous();
     const uint64_t inf = phase ? inf_cost : 0xffffffffull;
     if (threadIdx.x == 0) {
         n_listed = 0;
@@ -310,8 +317,7 @@ cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo
     // once (64 sets of the 64-device job: 10 us with 1024 threads, 16 with 256, 25 with 128); beyond, CTAs of
     // an SM stand in for one another (515 sets of the 32-device job: 28 us with 256 threads, 37 with 1024, 40
     // with 128; 1024 sets of the 256-device job 16, 30 and 16 us).
-    cm_window_kernel<<<b.B, b.B <= 148 ? 1024 : 256, 0, st>>>(t, b, bo, phase, k_best, batch_inf_bits(b));
-    return cudaGetLastError();
+    return launch_next(cm_window_kernel, b.B, b.B <= 148 ? 1024 : 256, 0, st, t, b, bo, phase, k_best, batch_inf_bits(b));
 }
 
 // ----------------------------------------------------------------------------------
@@ -319,6 +325,7 @@ cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo
 // ----------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) cm_gather_kernel(Tables tb, BatchDev bd, BoundDev bo) {
     const uint32_t at = blockIdx.x * 128 + threadIdx.x;
+    after_previous();
     if (at >= bo.n_segs) return;
     const SegRec g = bo.rec[at];
     const uint64_t la = bo.lbarg[g.row], key = bo.pick[g.row];
@@ -331,8 +338,7 @@ __global__ void __launch_bounds__(128) cm_gather_kernel(Tables tb, BatchDev bd, 
 
 cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st) {
     if (bo.n_segs == 0) return cudaSuccess;
-    cm_gather_kernel<<<(bo.n_segs + 127) / 128, 128, 0, st>>>(t, b, bo);
-    return cudaGetLastError();
+    return launch_next(cm_gather_kernel, (bo.n_segs + 127) / 128, 128, 0, st, t, b, bo);
 }
 
 // ----------------------------------------------------------------------------------
@@ -357,12 +363,15 @@ __device__ __forceinline__ void count_list_work(const BatchDev &bd, unsigned lon
     }
 }
 
+constexpr uint32_t kListAhead = 148;   // CTAs that fetch the profile before they know whether the list is long enough for them
 template <typename T>
 __global__ void __launch_bounds__(kChunk) cm_list_shallow_kernel(Tables tb, BatchDev bd, BoundDev bo, int list) {
     __shared__ SProf<T> sp;
+    if (blockIdx.x < kListAhead) stage_profile(sp, tb);
+    after_previous();
     const uint32_t n = list_length(bo, list);
     if ((uint64_t)blockIdx.x * kChunk >= n || lists_full(bd)) return;
-    stage_profile(sp, tb);
+    if (blockIdx.x >= kListAhead) stage_profile(sp, tb);
     __syncthreads();
     const uint4 *entries = bo.list + bo.list_first[list];
     unsigned long long work = 0;
@@ -383,9 +392,11 @@ template <typename T>
 __global__ void __launch_bounds__(kChunk, 5) cm_list_deep_kernel(Tables tb, BatchDev bd, BoundDev bo, int list) {
     __shared__ SProf<T> sp;
     __shared__ uint8_t cuts_s[kChunk / 32][4][kMaxS + 8];   // (per plan; the fourth: lanes without one)
+    if (blockIdx.x < kListAhead) stage_profile(sp, tb);
+    after_previous();
     const uint32_t n = list_length(bo, list);
     if ((uint64_t)blockIdx.x * (kChunk / 32) >= n || lists_full(bd)) return;
-    stage_profile(sp, tb);
+    if (blockIdx.x >= kListAhead) stage_profile(sp, tb);
     __syncthreads();
     const uint4 *entries = bo.list + bo.list_first[list];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -426,19 +437,20 @@ __global__ void __launch_bounds__(kChunk, 5) cm_list_deep_kernel(Tables tb, Batc
 cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches) {
     const uint64_t shallow = bo.list_first[first_list + 1] - bo.list_first[first_list];
     const uint64_t deep = bo.list_first[first_list + 2] - bo.list_first[first_list + 1];
+    cudaError_t e = cudaSuccess;
     if (shallow) {
         const unsigned grid = (unsigned)std::min<uint64_t>((shallow + kChunk - 1) / kChunk, 148 * 4);
-        if (native_i64(b)) cm_list_shallow_kernel<long long><<<grid, kChunk, 0, st>>>(t, b, bo, first_list);
-        else cm_list_shallow_kernel<double><<<grid, kChunk, 0, st>>>(t, b, bo, first_list);
+        e = native_i64(b) ? launch_next(cm_list_shallow_kernel<long long>, grid, kChunk, 0, st, t, b, bo, first_list)
+                          : launch_next(cm_list_shallow_kernel<double>, grid, kChunk, 0, st, t, b, bo, first_list);
         ++*launches;
     }
-    if (deep) {
+    if (deep && e == cudaSuccess) {
         const unsigned grid = (unsigned)std::min<uint64_t>((deep + kChunk / 32 - 1) / (kChunk / 32), 148 * 5);
-        if (native_i64(b)) cm_list_deep_kernel<long long><<<grid, kChunk, 0, st>>>(t, b, bo, first_list + 1);
-        else cm_list_deep_kernel<double><<<grid, kChunk, 0, st>>>(t, b, bo, first_list + 1);
+        e = native_i64(b) ? launch_next(cm_list_deep_kernel<long long>, grid, kChunk, 0, st, t, b, bo, first_list + 1)
+                          : launch_next(cm_list_deep_kernel<double>, grid, kChunk, 0, st, t, b, bo, first_list + 1);
         ++*launches;
     }
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace cm

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "cm_bound.cuh"
+#include "cm_launch.cuh"
 
 namespace cm {
 

@@ -28,6 +28,7 @@
 #include <atomic>
 
 #include "cm_eval_out.cuh"
+#include "cm_launch.cuh"
 #include "cm_tie_rest.cuh"
 
 namespace cm {
@@ -198,6 +199,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_regs_any_kernel(Tables tb, Bat
     plan_of_thread(base, bk.count, threadIdx.x, seg_local, kappa);
     Cand cand{};
     if (seg_local < bk.n_seg) cand = walk_cand(bd, bk.feas_first, kappa);
+    after_previous();
     uint32_t row = 0xffffffffu;
     uint64_t bits = inf_bits<T>();
     unsigned long long my_cells = 0;
@@ -634,8 +636,7 @@ cudaError_t launch_shallow_pair_class(const Tables &t, const BatchDev &b, const 
 
 template <typename T>
 cudaError_t launch_shallow_any(const Tables &t, const BatchDev &b, uint32_t b0, uint32_t b1, uint64_t chunks, cudaStream_t st) {
-    cm_cost_regs_any_kernel<T><<<(unsigned)chunks, kChunk, 0, st>>>(t, b, b0, b1);
-    return cudaGetLastError();
+    return launch_next(cm_cost_regs_any_kernel<T>, (unsigned)chunks, kChunk, 0, st, t, b, b0, b1);
 }
 
 template <typename T>

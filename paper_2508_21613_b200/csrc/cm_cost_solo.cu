@@ -17,6 +17,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_solo_kernel(Tables tb, BatchDe
     stage_profile(sp, tb);
     const Bucket bk = bd.bucket[find_bucket(bd.bucket, b0, b1, chunk)];
     __syncthreads();
+    after_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = bk.S, m = bk.m;
     const uint64_t seg_local = (chunk - bk.chunk_first) * (kChunk / 32) + warp;
@@ -52,8 +53,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_solo_kernel(Tables tb, BatchDe
 
 template <typename T>
 cudaError_t launch_solo_class(const Tables &t, const BatchDev &b, const LaunchClass &c, cudaStream_t st) {
-    cm_cost_solo_kernel<T><<<chunk_grid(c.n_chunks), kChunk, 0, st>>>(t, b, c.bucket_begin, c.bucket_end, c.chunk_begin);
-    return cudaGetLastError();
+    return launch_next(cm_cost_solo_kernel<T>, chunk_grid(c.n_chunks), kChunk, 0, st, t, b, c.bucket_begin, c.bucket_end, c.chunk_begin);
 }
 
 // A warp per plan for buckets of few plans (what the memory screen leaves of a workload that
@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_warp_kernel(Tables tb, BatchDe
     stage_profile(sp, tb);
     const Bucket bk = bd.bucket[find_bucket(bd.bucket, b0, b1, chunk)];
     __syncthreads();
+    after_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = bk.S, m = bk.m;
     const uint64_t plan = (chunk - bk.chunk_first) * (kChunk / 32) + warp;
@@ -89,8 +90,7 @@ __global__ void __launch_bounds__(kChunk) cm_cost_warp_kernel(Tables tb, BatchDe
 
 template <typename T>
 cudaError_t launch_warp_class(const Tables &t, const BatchDev &b, const LaunchClass &c, cudaStream_t st) {
-    cm_cost_warp_kernel<T><<<chunk_grid(c.n_chunks), kChunk, 0, st>>>(t, b, c.bucket_begin, c.bucket_end, c.chunk_begin);
-    return cudaGetLastError();
+    return launch_next(cm_cost_warp_kernel<T>, chunk_grid(c.n_chunks), kChunk, 0, st, t, b, c.bucket_begin, c.bucket_end, c.chunk_begin);
 }
 
 template cudaError_t launch_warp_class<double>(const Tables &, const BatchDev &, const LaunchClass &, cudaStream_t);

@@ -221,7 +221,7 @@ struct BoundDev {
     const BBucket *bucket;
     SegRec *rec;                  // per segment of the layout
     uint32_t parts;               // CTAs of cm_refine_kernel for one of cm_bound_kernel
-    uint32_t pad;
+    uint32_t few;                 // 1: the CTAs are all there at once; compositions are set up ahead (cm_launch.cuh)
     uint64_t *lbarg;              // per row: least bound (float bits) << 32 | its position in the walk; all-ones = no plan fits
     uint64_t *pick;               // per row: the plan phase 1 takes (cm_bound_lane.cuh)
     SearchWin *win;               // per scenario
@@ -231,7 +231,8 @@ struct BoundDev {
     const uint32_t *row_rep;
     uint64_t *row_lo, *row_ub;
     uint4 *list;                  // plans for the recurrence: scenario, template segment, position
-    uint32_t *count;              // per list: plans listed minus one
+    uint32_t *count;              // per list: plans listed minus one; then parts listed in `work`, by phase, minus one
+    uint32_t *work;               // parts of the layout that the compare pass has something to do in (not few)
     uint32_t list_first[5];       // lists: phase 1 up to kRegStagesMax stages, deeper; phase 2 the same
     uint32_t n_buckets, n_chunks, n_segs;
     float *tile_min;              // per (tile of compositions, segment): least bound; null: too many
@@ -376,7 +377,7 @@ size_t bound_dyn_bytes(BoundDev &bo, int max_stages, bool uniform_x);   // sets 
 int bound_group();   // segments per CTA, at most
 cudaError_t launch_bound(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
 cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st);
-cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st);
+cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st, int *launches);
 cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo, cudaStream_t st);
 cudaError_t launch_lists(const Tables &t, const BatchDev &b, const BoundDev &bo, int first_list, cudaStream_t st, int *launches);   // first_list and the next
 cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, const SearchWin *win, cudaStream_t st);   // win: of a search by bounds

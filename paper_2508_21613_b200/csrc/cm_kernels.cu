@@ -13,6 +13,7 @@
 #include <atomic>
 
 #include "cm_plan_eval.cuh"
+#include "cm_launch.cuh"
 #include "cm_split.cuh"
 
 namespace cm {
@@ -520,6 +521,7 @@ __global__ void __launch_bounds__(1024, 1) cm_best_split_kernel(Tables tb, Batch
     const Strat *strat = bd.strat + tp.strat_first;
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31, G = tb.prof->G;
+    after_previous();
     auto cost_of = [&](const Strat &s) { return strat_cost(bd, tp, sc, s, inf, [&](uint32_t row) { return bd.seg_best[row]; }); };
     uint64_t best_c = inf;
     uint32_t best_i = 0;
@@ -601,11 +603,9 @@ cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, const Search
     if (b.batch_mode == CM_BATCH_FULL) {
         const int words = t.binom_rows / 64 + 1;   // (the table has a row per micro-batch of the job at least)
         const size_t bytes = (threads / 32 * 2 + kMaxP) * (size_t)words * sizeof(uint64_t);
-        cm_best_split_kernel<true><<<b.B, threads, bytes, st>>>(t, b, win, batch_inf_bits(b), words);
-    } else {
-        cm_best_split_kernel<false><<<b.B, threads, 0, st>>>(t, b, win, batch_inf_bits(b), 0);
+        return launch_next(cm_best_split_kernel<true>, b.B, threads, bytes, st, t, b, win, batch_inf_bits(b), words);
     }
-    return cudaGetLastError();
+    return launch_next(cm_best_split_kernel<false>, b.B, threads, 0, st, t, b, win, batch_inf_bits(b), 0);
 }
 
 // ----------------------------------------------------------------------------------
@@ -617,6 +617,7 @@ cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, const Search
 __global__ void __launch_bounds__(256) cm_prologue_kernel(uint64_t *words, size_t n_words, const uint32_t *ids_host, uint32_t *ids, int n_ids,
                                                           const uint64_t *bits_host, uint64_t *bits, int n_bits) {
     const size_t at = (size_t)blockIdx.x * 256 + threadIdx.x;
+    after_previous();
     if (blockIdx.x == 0) {
         for (int i = threadIdx.x; i < n_ids; i += 256) ids[i] = ids_host[i];
         for (int i = threadIdx.x; i < n_bits; i += 256) bits[i] = bits_host[i];

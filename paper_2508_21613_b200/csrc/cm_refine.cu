@@ -8,6 +8,8 @@
 // and one turn of walks, its lanes side by side, 12 us.
 //   phase 1: the least of them per segment goes to pick[row]
 //   phase 2: those that could still improve on their segment's result go to the list
+#include <algorithm>
+
 #include "cm_bound_lane.cuh"
 
 namespace cm {
@@ -79,51 +81,85 @@ __device__ __noinline__ void refine_flush(const SProf<T> &sp, const BatchDev &bd
     __syncwarp();
 }
 
-// Few segments are open: here the lanes keep a composition each.
-template <typename T, bool UNI_X>
-__global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, BatchDev bd, BoundDev bo, int phase) {
-    __shared__ SProf<T> sp;
+// A part of kBoundSegs of the segments that CTA `cta` of cm_bound_kernel took.
+struct RefineJob : BoundJob { uint32_t base; };
+__device__ __forceinline__ RefineJob refine_job(const BBucket &bk, uint32_t cta, uint32_t part) {
+    RefineJob j;
+    static_cast<BoundJob &>(j) = bound_job(bk, cta);
+    j.base = j.s0 + part * kBoundSegs;
+    return j;
+}
+template <typename T>
+__device__ __forceinline__ bool thread_open(const BatchDev &bd, const BoundDev &bo, const BBucket &bk, const RefineJob &job, int phase, SegRec &g, RefineSeg &s) {
+    const uint32_t q = job.base + threadIdx.x;
+    if (q >= job.s1) return false;
+    const float least = bo.tile_min ? bo.tile_min[bk.min_first + job.tile * bk.n_seg + q] : 0.0f;
+    g = bo.rec[bk.seg_first + q];
+    s.scen = g.scen; s.tseg = g.tseg; s.n_sync = g.n_sync;
+    return seg_open<T>(bd, bo, bk, phase, g.row, least, s);
+}
+
+// The parts that have open segments, listed: most have none, and a CTA of the kernel below takes a quarter of an SM
+// whether it has or not (1024 sets of the 256-device job, phase 2: 64 us for its 7368 CTAs, most of them empty).
+template <typename T>
+__global__ void __launch_bounds__(kBoundThreads) cm_open_kernel(Tables tb, BatchDev bd, BoundDev bo, int phase) {
     __shared__ BBucket bks;
-    __shared__ RefineSmem sm;
-    __shared__ int n_open;
-    extern __shared__ __align__(16) unsigned char dyn[];
-    const uint32_t tid = threadIdx.x, lane = tid & 31;
-    const uint32_t cta = blockIdx.x / bo.parts, part = blockIdx.x - cta * bo.parts;   // a part of kBoundSegs of a CTA's segments there
+    const uint32_t cta = blockIdx.x / bo.parts, part = blockIdx.x - cta * bo.parts;
     find_bucket(bo, cta, &bks);
-    if (tid == 0) n_open = lists_full(bd) ? -1 : 0;
     __syncthreads();
-    if (n_open < 0) return;   // uniform
+    after_previous();
+    if (lists_full(bd)) return;   // uniform
+    SegRec g;
+    RefineSeg s;
+    const bool open = thread_open<T>(bd, bo, bks, refine_job(bks, cta, part), phase, g, s);
+    if (__syncthreads_or(open) && threadIdx.x == 0) bo.work[atomicAdd(&bo.count[3 + phase], 1u) + 1u] = blockIdx.x;   // (counts start at -1)
+}
+
+// Few segments are open: here the lanes keep a composition each.
+// ahead: the composition while the kernel before this one ends.
+template <typename T, bool UNI_X>
+__device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd, const BoundDev &bo, int phase, uint32_t item, bool ahead,
+                                            SProf<T> &sp, BBucket &bks, RefineSmem &sm, int &n_open, unsigned char *dyn) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t cta = item / bo.parts, part = item - cta * bo.parts;
+    find_bucket(bo, cta, &bks);
+    if (ahead) stage_profile(sp, tb);
+    if (tid == 0) n_open = 0;
+    __syncthreads();
     const BBucket &bk = bks;
-    const BoundJob job = bound_job(bk, cta);
+    const RefineJob job = refine_job(bk, cta, part);
+    if (!ahead) after_previous();
     const int S = bk.S, W = bk.width, dear = dear_tier(tb);
-    const uint32_t base = job.s0 + part * kBoundSegs;
-    if (base >= job.s1) return;   // uniform
+    unsigned char *term_col = dyn + tid * kTermSize<UNI_X>;
+    uint8_t *cuts = dyn + bo.dyn_cuts;
     const bool any = (int)tid < W && job.tile0 + tid < bk.count;
     Cand cand{0, 0, 0, false};
     if (any) cand = walk_cand(bd, bk.feas_first, job.tile0 + tid);   // (on its way while the segments are looked at)
-    if (base + tid < job.s1) {
-        const SegRec g = bo.rec[bk.seg_first + base + tid];
-        const float least = bo.tile_min ? bo.tile_min[bk.min_first + job.tile * bk.n_seg + base + tid] : 0.0f;
-        RefineSeg s;
-        s.scen = g.scen; s.tseg = g.tseg; s.n_sync = g.n_sync;
-        if (seg_open<T>(bd, bo, bk, phase, g.row, least, s)) {
-            const int at = atomicAdd(&n_open, 1);
-            sm.segs[at] = seg_lite(g.tier, g.row, g.n_sync, tb.prof->bw_sync);
-            sm.open[at] = s;
-            sm.word[at] = ~0ull;
-        }
+    LaneBound v;
+    if (ahead) {
+        v = lane_of<T, UNI_X, true>(sp, tb, bd, bk, any, cand, dear, term_col, cuts + tid);
+        after_previous();
+    }
+    if (lists_full(bd)) return;   // uniform
+    SegRec g;
+    RefineSeg rs;
+    if (thread_open<T>(bd, bo, bk, job, phase, g, rs)) {
+        const int at = atomicAdd(&n_open, 1);
+        sm.segs[at] = seg_lite(g.tier, g.row, g.n_sync, tb.prof->bw_sync);
+        sm.open[at] = rs;
+        sm.word[at] = ~0ull;
     }
     __syncthreads();
     const int n_act = n_open;
     if (n_act == 0) return;   // uniform
-    unsigned char *term_col = dyn + tid * kTermSize<UNI_X>;
-    uint8_t *cuts = dyn + bo.dyn_cuts;
     uint32_t *buf = sm.buf[tid >> 5];
-    stage_profile(sp, tb);
-    __syncthreads();
+    if (!ahead) {
+        stage_profile(sp, tb);
+        __syncthreads();
+        v = lane_of<T, UNI_X, true>(sp, tb, bd, bk, any, cand, dear, term_col, cuts + tid);
+    }
     const float delta = dear_extra(sp, dear), slack = sp.intval || std::is_same<T, long long>::value ? 1.0f : 0.0f;
     if ((int)tid < n_act) sm.hot[tid] = seg_hot<UNI_X>(sm.segs[tid], S, dear, delta, sp.sched == CM_SCHED_GPIPE);
-    const LaneBound v = lane_of<T, UNI_X, true>(sp, tb, bd, bk, any, cand, dear, term_col, cuts + tid);
     __syncthreads();
     int n_buf = 0;
     for (int s = 0; s < n_act; ++s) {
@@ -153,16 +189,48 @@ __global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, Bat
 }
 
 template <typename T, bool UNI_X>
-static cudaError_t launch_refine_one(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st) {
+__global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, BatchDev bd, BoundDev bo, int phase) {
+    __shared__ SProf<T> sp;
+    __shared__ BBucket bks;
+    __shared__ RefineSmem sm;
+    __shared__ int n_open;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    if (bo.few) {
+        // (there is nearly always something to compare in phase 1, and nearly never in phase 2)
+        refine_part<T, UNI_X>(tb, bd, bo, phase, blockIdx.x, phase == 1, sp, bks, sm, n_open, dyn);
+        return;
+    }
+    after_previous();
+    if (lists_full(bd)) return;   // uniform
+    if (!bo.work) {
+        refine_part<T, UNI_X>(tb, bd, bo, phase, blockIdx.x, false, sp, bks, sm, n_open, dyn);
+        return;
+    }
+    const uint32_t n = bo.count[3 + phase] + 1u;
+    for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
+        refine_part<T, UNI_X>(tb, bd, bo, phase, bo.work[k], false, sp, bks, sm, n_open, dyn);
+        __syncthreads();
+    }
+}
+
+template <typename T, bool UNI_X>
+static cudaError_t launch_refine_one(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st, int *launches) {
     cudaError_t e = cudaFuncSetAttribute(cm_refine_kernel<T, UNI_X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBoundDynMax);
     if (e != cudaSuccess) return e;
-    cm_refine_kernel<T, UNI_X><<<bo.n_chunks * bo.parts, kBoundThreads, bo.dyn_refine, st>>>(t, b, bo, phase);
-    return cudaGetLastError();
+    const unsigned items = bo.n_chunks * bo.parts;
+    const bool listed = !bo.few && bo.work;
+    if (listed) {
+        e = launch_next(cm_open_kernel<T>, items, kBoundThreads, 0, st, t, b, bo, phase);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    ++*launches;
+    return launch_next(cm_refine_kernel<T, UNI_X>, listed ? std::min(items, 148u * 4) : items, kBoundThreads, bo.dyn_refine, st, t, b, bo, phase);
 }
-cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st) {
+cudaError_t launch_refine(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, cudaStream_t st, int *launches) {
     if (bo.n_chunks == 0) return cudaSuccess;
-    if (native_i64(b)) return bo.uniform_x ? launch_refine_one<long long, true>(t, b, bo, phase, st) : launch_refine_one<long long, false>(t, b, bo, phase, st);
-    return bo.uniform_x ? launch_refine_one<double, true>(t, b, bo, phase, st) : launch_refine_one<double, false>(t, b, bo, phase, st);
+    if (native_i64(b)) return bo.uniform_x ? launch_refine_one<long long, true>(t, b, bo, phase, st, launches) : launch_refine_one<long long, false>(t, b, bo, phase, st, launches);
+    return bo.uniform_x ? launch_refine_one<double, true>(t, b, bo, phase, st, launches) : launch_refine_one<double, false>(t, b, bo, phase, st, launches);
 }
 
 }  // namespace cm

@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "cm_bound.cuh"
+#include "cm_launch.cuh"
 #include "cm_tie_rest.cuh"
 
 namespace cm {
@@ -31,12 +32,14 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
     __shared__ uint32_t left[kTieThreads / 32];
     __shared__ unsigned long long found;
     const uint32_t b = blockIdx.x / bd.dp_max, p = blockIdx.x % bd.dp_max;
+    if (kTieThreads > 32) stage_profile(sp, tb);
+    after_previous();
     const Winner &w = bd.winner[b];
     const uint64_t w_bits = w.cost_bits;
     if (w_bits >= inf_bits<T>() || p >= w.dp || lists_full(bd)) return;   // uniform over the CTA
     const SegView g = seg_view(bd, w.scen, w.seg[p]);
     if (g.K == 0) return;                                           // one candidate: known already
-    stage_profile(sp, tb);
+    if (kTieThreads <= 32) stage_profile(sp, tb);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double goal = std::is_same<T, long long>::value ? __ll2double_ru((long long)w_bits)
                                                           : __longlong_as_double((long long)w_bits);
@@ -116,8 +119,9 @@ __global__ void __launch_bounds__(kTieWarps * 32) cm_tie_batch_kernel(Tables tb,
     __shared__ SProf<T> sp;
     __shared__ uint8_t cuts_s[kTieWarps][kTieMost][kRegStagesMax + 8];   // (per pipeline)
     __shared__ uint8_t cut_col[kTieWarps][kRegStagesMax * 32];
-    if (lists_full(bd)) return;   // uniform
     stage_profile(sp, tb);
+    after_previous();
+    if (lists_full(bd)) return;   // uniform
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int width = 32 / kTieMost;
@@ -313,9 +317,8 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, uint64_t stages,
     // Several pipelines to a warp where they have few tiles each (a long walk would hold up the others).
     if (!wide && t.sched != CM_SCHED_GPIPE && b.max_tiles_per_seg <= kTieTiles && !(stages >> kRegStagesMax)) {
         const unsigned ctas = (unsigned)((nx + kTieMost * kTieWarps - 1) / (kTieMost * kTieWarps));
-        if (native_i64(b)) cm_tie_batch_kernel<long long><<<ctas, kTieWarps * 32, 0, st>>>(t, b, (uint32_t)nx);
-        else cm_tie_batch_kernel<double><<<ctas, kTieWarps * 32, 0, st>>>(t, b, (uint32_t)nx);
-        return cudaGetLastError();
+        return native_i64(b) ? launch_next(cm_tie_batch_kernel<long long>, ctas, kTieWarps * 32, 0, st, t, b, (uint32_t)nx)
+                             : launch_next(cm_tie_batch_kernel<double>, ctas, kTieWarps * 32, 0, st, t, b, (uint32_t)nx);
     }
     const unsigned threads = wide ? 256 : 32;
     const int n_eval = wide ? 256 / 32 : 1;
@@ -323,14 +326,11 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, uint64_t stages,
     uint64_t y = (148 * 4 + nx - 1) / nx;
     y = std::min<uint64_t>(std::min(y, tiles), 65535);
     const dim3 grid((unsigned)nx, (unsigned)std::max<uint64_t>(y, 1), 1);
-    if (native_i64(b)) {
-        if (wide) cm_tiebreak_kernel<long long, 256><<<grid, threads, 0, st>>>(t, b, n_eval);
-        else cm_tiebreak_kernel<long long, 32><<<grid, threads, 0, st>>>(t, b, n_eval);
-    } else {
-        if (wide) cm_tiebreak_kernel<double, 256><<<grid, threads, 0, st>>>(t, b, n_eval);
-        else cm_tiebreak_kernel<double, 32><<<grid, threads, 0, st>>>(t, b, n_eval);
-    }
-    return cudaGetLastError();
+    if (native_i64(b))
+        return wide ? launch_next(cm_tiebreak_kernel<long long, 256>, grid, threads, 0, st, t, b, n_eval)
+                    : launch_next(cm_tiebreak_kernel<long long, 32>, grid, threads, 0, st, t, b, n_eval);
+    return wide ? launch_next(cm_tiebreak_kernel<double, 256>, grid, threads, 0, st, t, b, n_eval)
+                : launch_next(cm_tiebreak_kernel<double, 32>, grid, threads, 0, st, t, b, n_eval);
 }
 
 }  // namespace cm
