@@ -1331,7 +1331,7 @@ constexpr size_t kStateExtra = kCounters + 3;   // work counters and the counts 
 // carry the addresses: dropped when they move.
 cm_status reserve_bound_list(cm_ctx *ctx, Batch &bt) {
     const size_t want = bt.bo.list_first[4], mins = bt.tile_mins, segs = bt.bo.n_segs;
-    const size_t parts = bt.bo.few || (uint64_t)bt.bo.n_chunks * bt.bo.parts > kTileMinMax ? 0 : (size_t)bt.bo.n_chunks * bt.bo.parts;
+    const size_t parts = bt.bo.few || (uint64_t)bt.bo.n_chunks * bt.bo.parts > kTileMinMax / 4 ? 0 : (size_t)bt.bo.n_chunks * bt.bo.parts * 4;
     if (want <= ctx->d_bound_list.cap && segs <= ctx->d_seg_rec.cap && parts <= ctx->d_open_parts.cap && mins <= ctx->d_tile_min.cap) return CM_OK;
     CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (!ctx->d_tile_min.reserve(mins)) bt.tile_mins = 0;
@@ -1430,7 +1430,7 @@ cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchD
     }
     bo.list = ctx->d_bound_list.p;
     bo.rec = ctx->d_seg_rec.p;
-    bo.work = (uint64_t)bo.n_chunks * bo.parts <= kTileMinMax ? ctx->d_open_parts.p : nullptr;
+    bo.work = (uint64_t)bo.n_chunks * bo.parts <= kTileMinMax / 4 ? ctx->d_open_parts.p : nullptr;
     bo.tile_min = bt.tile_mins ? ctx->d_tile_min.p : nullptr;
     CM_CUDA(ctx, launch_bound(tb, bd, bo, st));
     ++*launches;

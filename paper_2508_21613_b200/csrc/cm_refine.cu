@@ -48,45 +48,46 @@ __device__ __forceinline__ bool seg_open(const BatchDev &bd, const BoundDev &bo,
     return least <= s.lim && s.lim > s.ev;
 }
 
+// Segments that are gone through at a time, and, where parts with open segments are listed, the size of a part: plans tie by
+// the hundred in some parts while most are empty, so small parts spread them over the CTAs.
+constexpr int kRefineSegs = 32;
+static_assert(kBoundThreads == 128, "queue entries");
+
 // Shared memory of a CTA: the segments that are open, and the cuts of its compositions.
 struct RefineSmem {
     SegLite segs[kBoundSegs];
     SegHot hot[kBoundSegs];
     RefineSeg open[kBoundSegs];
     unsigned long long word[kBoundSegs];   // phase 1: least walk cost
-    uint32_t buf[kBoundThreads / 32][64];
+    int n_queue;
+    uint16_t queue[kRefineSegs * kBoundThreads];   // plans to walk: segment << 7 | thread whose composition it is
 };
 
-// Lanes 0 .. n-1 take one collected plan each: entry = segment << 8 | thread whose composition it is.
+// A plan's walk, added up in the recurrence's own arithmetic: segment s, composition of thread c.
 template <typename T>
-__device__ __noinline__ void refine_flush(const SProf<T> &sp, const BatchDev &bd, const BoundDev &bo, const BBucket &bk,
-                                          int phase, uint64_t tile0, RefineSmem &sm, uint8_t *cuts, const uint32_t *ent, int n) {
-    const int lane = threadIdx.x & 31;
-    if (lane < n) {
-        const uint32_t e = ent[lane], t = e & 0xffu;
-        const SegLite &sg = sm.segs[e >> 8];
-        const RefineSeg &rg = sm.open[e >> 8];
-        const int n_sync = rg.n_sync;
-        const uint64_t pos = tile0 + t;
-        const CutColumn<kBoundThreads> c{cuts + t};
-        const Walk w = best_walk<T>(sp, c, bk.S, bk.m, sg.tier, n_sync, false);
-        const uint64_t bits = Num<T>::bits(walk_cost<T>(sp, c, bk.S, bk.m, sg.tier, n_sync, w));
-        if (phase == 1) {
-            const float lb = lb_of(bo.lbarg[sg.row]);
-            atomicMin(&sm.word[e >> 8], (unsigned long long)pick_key(bits, pick_base(lb, std::is_same<T, long long>::value), pos, pick_bits(bk.count)));
-        } else if (bits <= rg.lim_bits) {
-            list_append(bd, bo, bk.S <= kRegStagesMax ? 2 : 3, rg.scen, rg.tseg, (uint32_t)pos);
-        }
+__device__ __noinline__ void refine_walk(const SProf<T> &sp, const BatchDev &bd, const BoundDev &bo, const BBucket &bk,
+                                         int phase, uint64_t tile0, RefineSmem &sm, uint8_t *cuts, int s, int c) {
+    const SegLite &sg = sm.segs[s];
+    const RefineSeg &rg = sm.open[s];
+    const uint64_t pos = tile0 + c;
+    const CutColumn<kBoundThreads> cc{cuts + c};
+    const Walk w = best_walk<T>(sp, cc, bk.S, bk.m, sg.tier, rg.n_sync, false);
+    const uint64_t bits = Num<T>::bits(walk_cost<T>(sp, cc, bk.S, bk.m, sg.tier, rg.n_sync, w));
+    if (phase == 1) {
+        const float lb = lb_of(bo.lbarg[sg.row]);
+        atomicMin(&sm.word[s], (unsigned long long)pick_key(bits, pick_base(lb, std::is_same<T, long long>::value), pos, pick_bits(bk.count)));
+    } else if (bits <= rg.lim_bits) {
+        list_append(bd, bo, bk.S <= kRegStagesMax ? 2 : 3, rg.scen, rg.tseg, (uint32_t)pos);
     }
-    __syncwarp();
 }
 
-// A part of kBoundSegs of the segments that CTA `cta` of cm_bound_kernel took.
+// A part of the segments that CTA `cta` of cm_bound_kernel took, `size` of them.
 struct RefineJob : BoundJob { uint32_t base; };
-__device__ __forceinline__ RefineJob refine_job(const BBucket &bk, uint32_t cta, uint32_t part) {
+__device__ __forceinline__ RefineJob refine_job(const BBucket &bk, uint32_t cta, uint32_t part, uint32_t size) {
     RefineJob j;
     static_cast<BoundJob &>(j) = bound_job(bk, cta);
-    j.base = j.s0 + part * kBoundSegs;
+    j.base = j.s0 + part * size;
+    j.s1 = min(j.s1, j.base + size);
     return j;
 }
 template <typename T>
@@ -111,23 +112,24 @@ __global__ void __launch_bounds__(kBoundThreads) cm_open_kernel(Tables tb, Batch
     if (lists_full(bd)) return;   // uniform
     SegRec g;
     RefineSeg s;
-    const bool open = thread_open<T>(bd, bo, bks, refine_job(bks, cta, part), phase, g, s);
-    if (__syncthreads_or(open) && threadIdx.x == 0) bo.work[atomicAdd(&bo.count[3 + phase], 1u) + 1u] = blockIdx.x;   // (counts start at -1)
+    const bool open = thread_open<T>(bd, bo, bks, refine_job(bks, cta, part, kBoundSegs), phase, g, s);
+    if (__any_sync(0xffffffffu, open) && (threadIdx.x & 31) == 0)   // (a warp's segments are a part; counts start at -1)
+        bo.work[atomicAdd(&bo.count[3 + phase], 1u) + 1u] = blockIdx.x * (kBoundSegs / kRefineSegs) + (threadIdx.x >> 5);
 }
 
 // Few segments are open: here the lanes keep a composition each.
 // ahead: the composition while the kernel before this one ends.
 template <typename T, bool UNI_X>
-__device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd, const BoundDev &bo, int phase, uint32_t item, bool ahead,
+__device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd, const BoundDev &bo, int phase, uint32_t item, uint32_t size, bool ahead,
                                             SProf<T> &sp, BBucket &bks, RefineSmem &sm, int &n_open, unsigned char *dyn) {
     const uint32_t tid = threadIdx.x, lane = tid & 31;
-    const uint32_t cta = item / bo.parts, part = item - cta * bo.parts;
+    const uint32_t per_cta = bo.parts * (kBoundSegs / size), cta = item / per_cta, part = item - cta * per_cta;
     find_bucket(bo, cta, &bks);
     if (ahead) stage_profile(sp, tb);
     if (tid == 0) n_open = 0;
     __syncthreads();
     const BBucket &bk = bks;
-    const RefineJob job = refine_job(bk, cta, part);
+    const RefineJob job = refine_job(bk, cta, part, size);
     if (!ahead) after_previous();
     const int S = bk.S, W = bk.width, dear = dear_tier(tb);
     unsigned char *term_col = dyn + tid * kTermSize<UNI_X>;
@@ -152,7 +154,6 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
     __syncthreads();
     const int n_act = n_open;
     if (n_act == 0) return;   // uniform
-    uint32_t *buf = sm.buf[tid >> 5];
     if (!ahead) {
         stage_profile(sp, tb);
         __syncthreads();
@@ -160,29 +161,32 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
     }
     const float delta = dear_extra(sp, dear), slack = sp.intval || std::is_same<T, long long>::value ? 1.0f : 0.0f;
     if ((int)tid < n_act) sm.hot[tid] = seg_hot<UNI_X>(sm.segs[tid], S, dear, delta, sp.sched == CM_SCHED_GPIPE);
-    __syncthreads();
-    int n_buf = 0;
-    for (int s = 0; s < n_act; ++s) {
-        bool take = false;
-        if (v.ok) {
-            const SegHot &h = sm.hot[s];
-            const float value = h.n <= 2 ? bound_value<UNI_X, 2>(v.best, v.u0, v.g, term_col, h, delta)
-                              : h.n <= kDearMax ? bound_value<UNI_X, kDearMax>(v.best, v.u0, v.g, term_col, h, delta)
-                                                : bound_value<UNI_X, -1>(v.best, v.u0, v.g, term_col, h, delta);
-            const float lb = bound_of(value, slack);
-            take = lb <= sm.open[s].lim && lb > sm.open[s].ev;
+    // plans within their segment's limits are collected, then walked, a thread each
+    for (int s0 = 0; s0 < n_act; s0 += kRefineSegs) {
+        __syncthreads();   // (the segments' data; nobody reads an earlier queue any more)
+        if (tid == 0) sm.n_queue = 0;
+        __syncthreads();
+        for (int s = s0; s < n_act && s < s0 + kRefineSegs; ++s) {
+            bool take = false;
+            if (v.ok) {
+                const SegHot &h = sm.hot[s];
+                const float value = h.n <= 2 ? bound_value<UNI_X, 2>(v.best, v.u0, v.g, term_col, h, delta)
+                                  : h.n <= kDearMax ? bound_value<UNI_X, kDearMax>(v.best, v.u0, v.g, term_col, h, delta)
+                                                    : bound_value<UNI_X, -1>(v.best, v.u0, v.g, term_col, h, delta);
+                const float lb = bound_of(value, slack);
+                take = lb <= sm.open[s].lim && lb > sm.open[s].ev;
+            }
+            const uint32_t who = __ballot_sync(0xffffffffu, take);
+            if (!who) continue;
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&sm.n_queue, __popc(who));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(who & ((1u << lane) - 1u));
+            if (take) sm.queue[at] = (uint16_t)(((s - s0) << 7) | tid);
         }
-        const uint32_t who = __ballot_sync(0xffffffffu, take);
-        if (!who) continue;
-        if (take) buf[n_buf + __popc(who & ((1u << lane) - 1u))] = ((uint32_t)s << 8) | tid;
-        n_buf += __popc(who);
-        __syncwarp();
-        if (n_buf >= 32) {
-            n_buf -= 32;
-            refine_flush<T>(sp, bd, bo, bk, phase, job.tile0, sm, cuts, buf + n_buf, 32);
-        }
+        __syncthreads();
+        for (int k = tid; k < sm.n_queue; k += kBoundThreads)
+            refine_walk<T>(sp, bd, bo, bk, phase, job.tile0, sm, cuts, s0 + (sm.queue[k] >> 7), sm.queue[k] & 127);
     }
-    if (n_buf) refine_flush<T>(sp, bd, bo, bk, phase, job.tile0, sm, cuts, buf, n_buf);
     if (phase != 1) return;
     __syncthreads();
     if ((int)tid < n_act && sm.word[tid] < bo.pick[sm.segs[tid].row]) atomicMin((unsigned long long *)&bo.pick[sm.segs[tid].row], sm.word[tid]);
@@ -197,18 +201,18 @@ __global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, Bat
     extern __shared__ __align__(16) unsigned char dyn[];
     if (bo.few) {
         // (there is nearly always something to compare in phase 1, and nearly never in phase 2)
-        refine_part<T, UNI_X>(tb, bd, bo, phase, blockIdx.x, phase == 1, sp, bks, sm, n_open, dyn);
+        refine_part<T, UNI_X>(tb, bd, bo, phase, blockIdx.x, kBoundSegs, phase == 1, sp, bks, sm, n_open, dyn);
         return;
     }
     after_previous();
     if (lists_full(bd)) return;   // uniform
     if (!bo.work) {
-        refine_part<T, UNI_X>(tb, bd, bo, phase, blockIdx.x, false, sp, bks, sm, n_open, dyn);
+        refine_part<T, UNI_X>(tb, bd, bo, phase, blockIdx.x, kBoundSegs, false, sp, bks, sm, n_open, dyn);
         return;
     }
     const uint32_t n = bo.count[3 + phase] + 1u;
     for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
-        refine_part<T, UNI_X>(tb, bd, bo, phase, bo.work[k], false, sp, bks, sm, n_open, dyn);
+        refine_part<T, UNI_X>(tb, bd, bo, phase, bo.work[k], kRefineSegs, false, sp, bks, sm, n_open, dyn);
         __syncthreads();
     }
 }
