@@ -4,7 +4,8 @@
 //   cm_bound_kernel    lower bound of every plan of every segment, the least one per segment
 //   cm_window_kernel   per scenario: the step times that can still be the answer, and the segments of
 //                      the strategies that can reach them
-//   cm_refine_kernel   compares plans whose bounds tie, bit for bit (cm_refine.cu)
+//   cm_refine_kernel   compares plans whose bounds tie, bit for bit (cm_refine.cu; cm_open_kernel lists the
+//                      parts of a large layout that have any)
 //   cm_gather_kernel   lists the most promising plan of every segment needed
 //   cm_list_*_kernel   the recurrence on the listed plans
 //
@@ -33,7 +34,9 @@
 
 namespace cm {
 
-// (figures below)
+// Bound by look-ups in shared memory and by set-up: 1024 sets of the 256-device job (75 million plans) 140 us, 795
+// with a term per stage and a reduction over lanes per segment (201 thread-instructions a plan), 270 with a term per
+// dear boundary and the lanes still a composition each; 2576 sets of the 32-device job (24 million) 56 us, 210 before.
 // A CTA holds the terms of up to kBoundThreads compositions (a thread sets up one) and takes its group of segments
 // by them, kBoundSegs at a time, a lane per segment: the lane has the places of its segment's dear boundaries in
 // registers and goes through the compositions, one look-up, addition and maximum per dear boundary and no
@@ -313,10 +316,11 @@ __global__ void __launch_bounds__(1024) cm_window_kernel(Tables tb, BatchDev bd,
 
 cudaError_t launch_window(const Tables &t, const BatchDev &b, const BoundDev &bo, int phase, int k_best, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
-    // A warp per strategy, latency of its dependent loads.  Up to a scenario per SM the CTA takes them all at
-    // once (64 sets of the 64-device job: 10 us with 1024 threads, 16 with 256, 25 with 128); beyond, CTAs of
-    // an SM stand in for one another (515 sets of the 32-device job: 28 us with 256 threads, 37 with 1024, 40
-    // with 128; 1024 sets of the 256-device job 16, 30 and 16 us).
+    // A warp per four strategies, latency of their dependent loads.  Up to a scenario per SM the CTA takes them all at
+    // once; beyond, CTAs of an SM stand in for one another (with one strategy at a time: 64 sets of the 64-device job
+    // 10 us with 1024 threads, 16 with 256; 515 sets of the 32-device job 28 us with 256 threads, 37 with 1024).
+    // Four at a time, kept for the marking and listed for later: 2576 sets of the 32-device job 95 -> 54 us from
+    // bounds, 88 -> 52 from results (where most have to be marked again), 515 sets 26 -> 16 and 17 -> 4.
     return launch_next(cm_window_kernel, b.B, b.B <= 148 ? 1024 : 256, 0, st, t, b, bo, phase, k_best, batch_inf_bits(b));
 }
 

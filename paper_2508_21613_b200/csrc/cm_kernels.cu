@@ -598,7 +598,8 @@ cudaError_t launch_split_reduce(const Tables &t, const BatchDev &b, const Search
     if (b.B <= 0) return cudaSuccess;
     // A warp per strategy, latency of its dependent loads: all strategies at once up to a scenario per SM (64 sets
     // of the 64-device job: 8 us with 1024 threads, 12 with 256, 18 with 128), narrower CTAs beyond (515 sets of
-    // the 32-device job: 20 us with 256 threads, 25 with 1024, 26 with 128; 1024 of the 256-device job 16, 27, 16).
+    // the 32-device job: 20 us with 256 threads, 25 with 1024, 26 with 128).  By the list of a search by bounds: 515 sets
+    // 17 -> 4 us, 2576 sets 47 -> 13.
     const unsigned threads = b.B <= 148 ? 1024 : 256;
     if (b.batch_mode == CM_BATCH_FULL) {
         const int words = t.binom_rows / 64 + 1;   // (the table has a row per micro-batch of the job at least)

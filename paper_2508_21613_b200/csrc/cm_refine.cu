@@ -1,11 +1,11 @@
 // Bounded search pass, plans whose bounds tie (sm_100a).  The float bounds are computed again for the
 // segments that need it (they cost less than storing them would: one addition and one maximum per
-// stage), plans within the segment's window are collected per warp, and whenever 32 of them are
-// together each lane adds up one walk in the recurrence's own arithmetic (cm_bound.cuh).
+// dear boundary), plans within the segment's window are collected per CTA, and its threads add up one walk
+// each in the recurrence's own arithmetic (cm_bound.cuh).
 // Bound by the chain of a walk's O(S+m) dependent additions wherever plans tie, else by launch and set-up:
-// 64 sets of the 64-device job 34 us a phase (most of their layers are equal), 64 of the 256-device job 42
-// and 16 us.  Of a CTA's time with ties at 30 stages, the set-up is 11 us, the loop over its segments 1 us
-// and one turn of walks, its lanes side by side, 12 us.
+// 64 sets of the 64-device job 30 and 25 us (most of their layers are equal), 1024 of the 256-device job 37 and 31,
+// 2576 of the 32-device job 30 and 29.  Of a CTA's time with ties at 30 stages, the set-up is 11 us, the loop over its
+// segments 1 us and one turn of walks, its threads side by side, 12 us.
 //   phase 1: the least of them per segment goes to pick[row]
 //   phase 2: those that could still improve on their segment's result go to the list
 #include <algorithm>

@@ -309,10 +309,8 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, uint64_t stages,
     if (nx >= (1ull << 31)) return cudaErrorInvalidConfiguration;
     // A failure handled on its own: a wide CTA per pipeline, whose warps try candidates side by side.  A
     // batch: a warp per pipeline; the first 32 compositions nearly always hold the answer, and the first
-    // that its bound leaves nearly always is it.  2576 failure sets of the 32-device job: 95 us with a
-    // warp, 170 us with two, above 400 us with eight; 290 us for the plan-per-lane kernel this replaced.
-    // 1024 sets of the 256-device job: 133 us with a warp, 172 us with two, where a plan-per-lane kernel
-    // per depth took 1300 us in all.
+    // that its bound leaves nearly always is it.  1024 sets of the 256-device job: 133 us with a warp, 172 us with
+    // two, where a plan-per-lane kernel per depth took 1300 us in all.
     const bool wide = nx <= 148 * 2;
     // Several pipelines to a warp where they have few tiles each (a long walk would hold up the others).
     if (!wide && t.sched != CM_SCHED_GPIPE && b.max_tiles_per_seg <= kTieTiles && !(stages >> kRegStagesMax)) {
