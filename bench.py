@@ -53,7 +53,7 @@ KERNEL_PROFILES = {
 }
 # Large batches decide most plans by a lower bound (cm_bound_kernel) and run the recurrence on the few it
 # leaves: there the unit of work is one plan bounded, with I_plan thread-instructions.
-BOUND_PROFILE = {"i_plan": 201.5, "issue_active": 0.429, "dram_bytes_per_plan": 311040 / 7.636e6,
+BOUND_PROFILE = {"i_plan": 87.0, "issue_active": 0.540, "dram_bytes_per_plan": 1044736 / 7.289e6,
                  "profile": "profiles/cm_bound_kernel_256dev-64.md"}
 KERNEL_NAMES = {"regs": "cm_cost_regs_kernel", "regs_pair": "cm_cost_regs_pair_kernel", "wide": "cm_cost_wide_kernel",
                 "pair": "cm_cost_pair_kernel"}
