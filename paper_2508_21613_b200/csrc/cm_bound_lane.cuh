@@ -279,17 +279,24 @@ __device__ __forceinline__ float bound_value(float v_best, float v_u0, float v_g
         if constexpr (NF & 1) best = fmaxf(best, a[NF - 1]);
     } else if constexpr (NF < 0) {
         int k = 0;
-        for (uint64_t bits = h.bits; bits;) {
-            const int i = 63 - __clzll((long long)bits);
-            bits ^= 1ull << i;
-            if constexpr (UNI_X) {
-                ++k;
-                best = fmaxf(best, __fadd_rd(*reinterpret_cast<const float *>(term_col + i * kTermRow * kTermSize<UNI_X>), __fmul_rd((float)k, delta)));
-            } else {
-                const float2 t = *reinterpret_cast<const float2 *>(term_col + i * kTermRow * kTermSize<UNI_X>);
-                extra = __fadd_rd(extra, t.y);
-                best = fmaxf(best, __fadd_rd(t.x, extra));
+        for (uint64_t bits = h.bits; bits;) {   // four at a time, so that their look-ups are under way together
+            float a4[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool on = bits != 0;
+                const int i = on ? 63 - __clzll((long long)bits) : 0;
+                if (on) bits ^= 1ull << i;
+                if constexpr (UNI_X) {
+                    ++k;
+                    a4[u] = __fadd_rd(*reinterpret_cast<const float *>(term_col + i * kTermRow * kTermSize<UNI_X>), __fmul_rd((float)k, delta));
+                } else {
+                    const float2 t = *reinterpret_cast<const float2 *>(term_col + i * kTermRow * kTermSize<UNI_X>);
+                    extra = __fadd_rd(extra, on ? t.y : 0.0f);
+                    a4[u] = __fadd_rd(t.x, extra);
+                }
+                if (!on) a4[u] = kNoWalk;
             }
+            best = max3(max3(best, a4[0], a4[1]), a4[2], a4[3]);
         }
     }
     return fmaxf(__fmaf_rd(v_g, h.coef, __fadd_rd(__fadd_rd(v_u0, extra), best)), 0.0f);
