@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kBoundThreads) cm_open_kernel(Tables tb, Batch
     find_bucket(bo, cta, &bks);
     __syncthreads();
     after_previous();
-    if (lists_full(bd)) return;   // uniform
+    if (lists_full(bd)) return;   // uniform: no kernel that may run beside this one writes the flag
     SegRec g;
     RefineSeg s;
     const bool open = thread_open<T>(bd, bo, bks, refine_job(bks, cta, part, kBoundSegs), phase, g, s);
@@ -118,7 +118,10 @@ __global__ void __launch_bounds__(kBoundThreads) cm_open_kernel(Tables tb, Batch
 }
 
 // Few segments are open: here the lanes keep a composition each.
-// ahead: the composition while the kernel before this one ends.
+// ahead: the composition while the kernel before this one ends (phase 1 only).
+// Whether the lists are full is ONE thread's look, which the CTA acts on together: in phase 2 the CTAs of this
+// very kernel set the flag, and warps that each looked for themselves could part ways at the barriers below.  (In phase
+// 1 nothing has been listed yet.)
 template <typename T, bool UNI_X>
 __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd, const BoundDev &bo, int phase, uint32_t item, uint32_t size, bool ahead,
                                             SProf<T> &sp, BBucket &bks, RefineSmem &sm, int &n_open, unsigned char *dyn) {
@@ -126,11 +129,12 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
     const uint32_t per_cta = bo.parts * (kBoundSegs / size), cta = item / per_cta, part = item - cta * per_cta;
     find_bucket(bo, cta, &bks);
     if (ahead) stage_profile(sp, tb);
-    if (tid == 0) n_open = 0;
+    else after_previous();
+    if (tid == 0) n_open = phase == 2 && lists_full(bd) ? -1 : 0;
     __syncthreads();
+    if (n_open < 0) return;   // uniform (it only grows from 0)
     const BBucket &bk = bks;
     const RefineJob job = refine_job(bk, cta, part, size);
-    if (!ahead) after_previous();
     const int S = bk.S, W = bk.width, dear = dear_tier(tb);
     unsigned char *term_col = dyn + tid * kTermSize<UNI_X>;
     uint8_t *cuts = dyn + bo.dyn_cuts;
@@ -142,7 +146,6 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
         v = lane_of<T, UNI_X, true>(sp, tb, bd, bk, any, cand, dear, term_col, cuts + tid);
         after_previous();
     }
-    if (lists_full(bd)) return;   // uniform
     SegRec g;
     RefineSeg rs;
     if (thread_open<T>(bd, bo, bk, job, phase, g, rs)) {
@@ -205,7 +208,6 @@ __global__ void __launch_bounds__(kBoundThreads) cm_refine_kernel(Tables tb, Bat
         return;
     }
     after_previous();
-    if (lists_full(bd)) return;   // uniform
     if (!bo.work) {
         refine_part<T, UNI_X>(tb, bd, bo, phase, blockIdx.x, kBoundSegs, false, sp, bks, sm, n_open, dyn);
         return;
