@@ -1327,23 +1327,29 @@ uint64_t stage_mask(const Batch &bt);
 
 constexpr size_t kStateExtra = kCounters + 3;   // work counters and the counts of six lists (32-bit)
 
-// Room for listed plans and, if there is memory for it, for the least bounds of tiles.  Captured launch sequences
-// carry the addresses: dropped when they move.
-cm_status reserve_bound_list(cm_ctx *ctx, Batch &bt) {
-    const size_t want = bt.bo.list_first[4], mins = bt.tile_mins, segs = bt.bo.n_segs;
-    const size_t parts = bt.bo.few || (uint64_t)bt.bo.n_chunks * bt.bo.parts > kTileMinMax / 4 ? 0 : (size_t)bt.bo.n_chunks * bt.bo.parts * 4;
+// Entries of the list of parts to compare (0: none kept).
+size_t open_parts(const BoundDev &bo) {
+    const uint64_t n = (uint64_t)bo.n_chunks * bo.parts;
+    return bo.few || n > kTileMinMax / 4 ? 0 : (size_t)n * 4;
+}
+
+// Workspaces of the search by bounds, which all searches of the context share.  Captured launch sequences carry their
+// addresses and are dropped before any of them can move.  The list of parts and the least bounds of tiles are kept if there
+// is memory for them; *room: so much for the others.
+cm_status reserve_bound(cm_ctx *ctx, const Batch &bt, bool *room) {
+    const size_t want = bt.bo.list_first[4], mins = bt.tile_mins, segs = bt.bo.n_segs, parts = open_parts(bt.bo);
+    *room = true;
     if (want <= ctx->d_bound_list.cap && segs <= ctx->d_seg_rec.cap && parts <= ctx->d_open_parts.cap && mins <= ctx->d_tile_min.cap) return CM_OK;
     CM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (!ctx->d_tile_min.reserve(mins)) bt.tile_mins = 0;
-    if (!ctx->d_bound_list.reserve(want) || !ctx->d_seg_rec.reserve(segs) || !ctx->d_open_parts.reserve(parts)) return fail(ctx, CM_ENOMEM, "device memory");
     for (auto &e : ctx->single)
         if (e->exec) { cudaGraphExecDestroy(e->exec); e->exec = nullptr; }
+    *room = ctx->d_bound_list.reserve(want) && ctx->d_seg_rec.reserve(segs);
+    if (*room) { ctx->d_open_parts.reserve(parts); ctx->d_tile_min.reserve(mins); }
     return CM_OK;
 }
 
 // Copy the tables of a batch to the device (one copy) and run the min-max partitions it needs.
-cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
-    struct Timer { cm_ctx *c; uint64_t t0; ~Timer() { c->stats[18] += now_ns() - t0; } } timer{ctx, now_ns()};
+cm_status upload_tables(cm_ctx *ctx, Batch &bt, int *launches) {
     bool ok = true;
     bt.arena.clear();
     bt.off_scen = arena_put(bt.arena, bt.scen, ok);
@@ -1411,8 +1417,20 @@ cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
             ctx->stats[9] += bt.bucket.size() * sizeof(Bucket);
         }
     }
-    if (bt.bounded) return reserve_bound_list(ctx, bt);
     return CM_OK;
+}
+
+// The same, and the workspaces; a search by bounds whose workspaces find no room becomes one of every plan.
+cm_status upload_batch(cm_ctx *ctx, Batch &bt, int *launches) {
+    struct Timer { cm_ctx *c; uint64_t t0; ~Timer() { c->stats[18] += now_ns() - t0; } } timer{ctx, now_ns()};
+    cm_status s = upload_tables(ctx, bt, launches);
+    bool room = true;
+    if (s == CM_OK && bt.bounded) s = reserve_bound(ctx, bt, &room);   // (without room: the stream is idle)
+    if (s != CM_OK || room) return s;
+    bt.dense_only = true;
+    bt.dense_left = bt.dense_span = longer_span(bt.dense_span);
+    s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
+    return s == CM_OK ? upload_tables(ctx, bt, launches) : s;
 }
 
 // Search pass with bounds: see cm_bound.cu.
@@ -1430,8 +1448,9 @@ cm_status enqueue_bounded(cm_ctx *ctx, Batch &bt, const Tables &tb, const BatchD
     }
     bo.list = ctx->d_bound_list.p;
     bo.rec = ctx->d_seg_rec.p;
-    bo.work = (uint64_t)bo.n_chunks * bo.parts <= kTileMinMax / 4 ? ctx->d_open_parts.p : nullptr;
-    bo.tile_min = bt.tile_mins ? ctx->d_tile_min.p : nullptr;
+    const size_t parts = open_parts(bo);
+    bo.work = parts && parts <= ctx->d_open_parts.cap ? ctx->d_open_parts.p : nullptr;
+    bo.tile_min = bt.tile_mins && bt.tile_mins <= ctx->d_tile_min.cap ? ctx->d_tile_min.p : nullptr;
     CM_CUDA(ctx, launch_bound(tb, bd, bo, st));
     ++*launches;
     for (int phase = 1; phase <= 2; ++phase) {

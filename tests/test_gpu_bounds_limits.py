@@ -1,6 +1,7 @@
 """The search by bounds where its work lists, its workspaces or the device memory run out -- against the CPU
 oracle: plan tuples bit-exact, costs equal."""
 import copy
+import ctypes as C
 
 import pytest
 
@@ -48,5 +49,81 @@ def test_lists_that_fill_while_other_blocks_look(gpu, oracle_factory, mode, nati
                 for b, plan in enumerate(best):
                     _same(plan, want[b % 2])
         assert launches[1] == launches[0] + 2
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+class _Hog:
+    """Holds the device's memory but for `leave` bytes, in blocks of 2 MB and more (what a process allocates in)."""
+
+    def __init__(self, leave):
+        import torch
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        self.lib = C.CDLL("libcudart.so.12")
+        self.lib.cudaMalloc.argtypes, self.lib.cudaFree.argtypes = [C.POINTER(C.c_void_p), C.c_size_t], [C.c_void_p]
+        self.blocks = []
+        for size in (1 << 30, 64 << 20, 2 << 20):
+            while len(self.blocks) < 1024:   # (183 GB: 183 + 16 + 32 at most)
+                p = C.c_void_p()
+                if self.lib.cudaMalloc(C.byref(p), size):
+                    self.lib.cudaGetLastError()
+                    break
+                self.blocks.append(p)
+        for _ in range(leave >> 21):
+            self.lib.cudaFree(self.blocks.pop())
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *_):
+        for p in self.blocks:
+            self.lib.cudaFree(p)
+
+
+def _warm_up(gpu, profile, opts, sets):
+    """Every kernel of the search by bounds and of the one that follows full lists, loaded while there is memory."""
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_search_batch(ctx, sets * 20, opts)
+        assert gpu.cm_last_stats(ctx)["repeated"] == 1
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("leave,bounded", [(0, False), (4 << 20, False), (32 << 20, True)])
+def test_workspaces_that_find_no_room(gpu, oracle_factory, leave, bounded):
+    """A batch on a device that others have filled: all of the workspaces of the search by bounds find no room, all
+    but the first, only the optional 57 MB of tiles' bounds.  The plans are the same, and a failure whose captured
+    sequence was made before the workspaces moved still gets its own."""
+    slow, opts = _slow_links(True, 8_000_000, 1)
+    opts = W.SearchOptions(2, 2, 18, 21, opts.layer_mode, opts.batch_mode, opts.kappa_cap)
+    only_minmax = W.SearchOptions(2, 2, 18, 21, opts.layer_mode, opts.batch_mode, 1)
+    profile = _fast_links(slow)
+    sets = [[3], [9]]
+    orc = oracle_factory(profile, opts)
+    want = [orc.search(f)[0] for f in sets]
+    _warm_up(gpu, slow, opts, sets)
+    ctx = gpu.cm_create(0)
+
+    def search(many, **kw):
+        for b, plan in enumerate(gpu.plans_from_array(gpu.cm_search_batch(ctx, many, opts, **kw)[0])):
+            _same(plan, want[b % 2])
+        return gpu.cm_last_stats(ctx)
+
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        for _ in range(3):   # (from the second on a replayed graph)
+            st = search(sets, latency=True)
+            assert st["plans_run"] < st["plans_simulated"]
+        gpu.cm_search_batch(ctx, sets * 6500, only_minmax)   # the batch's own tables find their room here
+        with _Hog(leave):
+            st = search(sets * 6000)
+            assert (st["plans_run"] < st["plans_simulated"]) == bounded and st["repeated"] == 0
+        for _ in range(2):
+            search(sets, latency=True)
+        st = search(sets * 6000)
+        assert st["plans_run"] < st["plans_simulated"]
     finally:
         gpu.cm_destroy(ctx)
