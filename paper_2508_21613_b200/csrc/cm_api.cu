@@ -1601,23 +1601,44 @@ void hand_out_fixed(Batch &bt, cm_plan *per_policy) {
 }
 
 // After a bounded search whose lists were full (bounds left hundreds of thousands of plans): again, every plan.
+// Where that finds no room for its tables, the batch is left as it was, to be searched again.
 cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *single) {
     if (single && single->exec) { cudaGraphExecDestroy(single->exec); single->exec = nullptr; }
     ++ctx->stats[23];
+    const bool direct = bt.direct, one_shot = bt.one_shot;
+    const uint32_t left = bt.dense_left, span = bt.dense_span;
     bt.dense_only = true;
     bt.dense_left = bt.dense_span = longer_span(bt.dense_span);
-    if (bt.one_shot) {
-        cm_ctx::Overflow *o = overflow_of(ctx, bt, true);
-        o->left = o->span = longer_span(o->span);
-    }
-    const bool direct = bt.direct;
     // the tables are laid out anew beside the old ones: an evaluation of this space that was captured reads those
-    std::swap(bt.d_arena.p, bt.d_arena_first.p);
-    std::swap(bt.d_arena.cap, bt.d_arena_first.cap);
-    cm_status s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
-    if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
-    bt.direct = direct;
-    return s == CM_OK ? run_batch(ctx, bt, launches, single) : s;
+    auto swap_tables = [&] {
+        std::swap(bt.d_arena.p, bt.d_arena_first.p);
+        std::swap(bt.d_arena.cap, bt.d_arena_first.cap);
+    };
+    auto lay_out = [&] {
+        cm_status s = bt.useg ? build_segment_classes(ctx, bt) : build_buckets(ctx, bt);
+        if (s == CM_OK) s = upload_batch(ctx, bt, &launches);
+        bt.direct = direct;
+        return s;
+    };
+    swap_tables();
+    const cm_status s = lay_out();
+    if (s == CM_OK) {
+        if (one_shot) {
+            cm_ctx::Overflow *o = overflow_of(ctx, bt, true);
+            o->left = o->span = longer_span(o->span);
+        }
+        return run_batch(ctx, bt, launches, single);
+    }
+    const std::string why = ctx->err;
+    cudaStreamSynchronize(ctx->stream);   // (queued copies read the host image of the tables)
+    swap_tables();
+    bt.dense_only = bt.one_shot = false;   // (not one_shot: bounds again, whatever searches alike do)
+    bt.dense_left = left;
+    bt.dense_span = span;
+    if (lay_out() != CM_OK || !bt.bounded) bt.profile_gen = 0;   // (a lost device: refused from here on)
+    bt.one_shot = one_shot;
+    ctx->err = why;
+    return s;
 }
 
 // The search over an uploaded batch; results land in bt.plans_host ([B][4]) after the stream is
@@ -2263,7 +2284,12 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
         cm_ctx::Single *entry = nullptr;
         if ((s = single_batch(ctx, failed_ids + offsets[b], offsets[b + 1] - offsets[b], *opts, mask, &sb, &launches, &entry)) != CM_OK) return s;
         ctx->stats[13] += now_ns() - h0;
-        if ((s = run_batch(ctx, *sb, launches, entry)) != CM_OK) return s;
+        if ((s = run_batch(ctx, *sb, launches, entry)) != CM_OK) {   // (the next search of its kind builds it anew)
+            cudaStreamSynchronize(ctx->stream);
+            for (auto &e : ctx->single)
+                if (e->batch.get() == sb) { std::swap(e, ctx->single.back()); ctx->single.pop_back(); break; }
+            return s;
+        }
         hand_out(*sb, best_per_scenario + b, best_per_policy ? best_per_policy + (size_t)b * 3 : nullptr);
         const auto t1 = std::chrono::steady_clock::now();
         latency_us[b] = (float)std::chrono::duration<double, std::micro>(t1 - t0).count();

@@ -3,6 +3,7 @@ oracle: plan tuples bit-exact, costs equal."""
 import copy
 import ctypes as C
 
+import numpy as np
 import pytest
 
 from paper_2508_21613_b200 import workloads as W
@@ -125,5 +126,46 @@ def test_workspaces_that_find_no_room(gpu, oracle_factory, leave, bounded):
             search(sets, latency=True)
         st = search(sets * 6000)
         assert st["plans_run"] < st["plans_simulated"]
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+def _many_sets(share):
+    """Two pipelines of 20 and 21 stages over links about as slow as the stages: 10 k plans a set, so that the tables of
+    tens of thousands of sets, and not their search, are what is large.  To be shared: small nodes and seven failures a
+    set, which leave hardly two sets with the same boundaries."""
+    L, pp, per_node = 44, 24 if share else 21, 2 if share else 8
+    rng = np.random.default_rng(3)
+    fwd = rng.uniform(5e6, 6e6, L).round()
+    profile = W.make_profile_ns(L, 2, pp, 48, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 8_000_000,
+                                [round(i * L / pp) for i in range(pp + 1)], 80_000_000_000, per_node, 1, 1)
+    sets = [[b % (2 * pp)] if not share else sorted(rng.choice(2 * pp, 7, replace=False).tolist()) for b in range(60000)]
+    return profile, W.SearchOptions(2, 2, 20, 21, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 16), sets
+
+
+@pytest.mark.parametrize("share", [False, True])
+def test_repeated_search_that_finds_no_room(gpu, oracle_factory, share):
+    """A prepared batch whose lists are full and whose second set of tables, for the search of every plan, finds no
+    room: an error, and with room again the same batch can be searched."""
+    profile, opts, sets = _many_sets(share)
+    orc = oracle_factory(profile, opts)
+    want = [orc.search(f)[0] for f in sets[:8]]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_set_sharing(ctx, share)
+        gpu.cm_search_batch(ctx, sets[:600], opts)   # (loads the kernels)
+        packed = gpu.PackedScenarios(sets)
+        batch, _ = packed.prepare(ctx, opts)
+        with _Hog(0):
+            for _ in range(2):
+                with pytest.raises(gpu.ChameleonError) as e:
+                    packed.search_prepared(ctx, batch)
+                assert e.value.status == gpu.CM_ENOMEM
+        packed.search_prepared(ctx, batch)
+        assert gpu.cm_last_stats(ctx)["repeated"] == 1
+        for plan, w in zip(gpu.plans_from_array(packed.best), want):
+            _same(plan, w)
+        gpu.cm_batch_free(batch)
     finally:
         gpu.cm_destroy(ctx)
