@@ -165,10 +165,8 @@ struct Batch {
     // from the pinned arena and its last one writes the plans to pinned memory, so that no copy sits on the
     // path (two copies in, one out: ~8 us of a 95 us call).
     bool direct = false;
-    // Plans in two parts (FinalPart), as the last enqueued search lays them out; policy_out: where the caller wants those
-    // of the one-plan policies (three plans per scenario), handed: they are there.
-    bool parted = false, handed = false;
-    cm_plan *policy_out = nullptr;
+    bool parted = false;                  // plans in two parts (FinalPart), as the last enqueued search lays them out
+    std::vector<cm_plan> replaced;        // EarlyPlans: what the caller's array held
     int k_best = 1;                       // (strategy, split) pairs whose step times have to be exact
 };
 
@@ -1590,19 +1588,35 @@ cm_status finish_tiebreak(cm_ctx *ctx, Batch &bt, int *launches) {
     return CM_OK;
 }
 
-cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single = nullptr);
+// The first part of parted plans goes to the caller's array (three plans per scenario; null: not wanted) while the search
+// runs (2576 scenarios: 1.2 of 2.4 MB, which the host would otherwise wait for and copy when it is done).  An error leaves
+// the array as it was: what it held is kept aside, in that time too, and put back unless the search ends well.
+struct EarlyPlans {
+    Batch &bt;
+    cm_plan *per_policy;
+    bool kept = false, handed = false, ended_well = false;
+    void keep() {
+        if (kept) return;
+        if (bt.replaced.size() < 2 * (size_t)bt.B) bt.replaced.resize(2 * (size_t)bt.B);
+        for (int b = 0; b < bt.B; ++b) memcpy(&bt.replaced[2 * (size_t)b], per_policy + 3 * (size_t)b, 2 * sizeof(cm_plan));
+        kept = true;
+    }
+    void hand_out() {
+        const cm_plan *from = bt.plans_host.p + 2 * (size_t)bt.B;
+        for (int b = 0; b < bt.B; ++b) memcpy(per_policy + 3 * (size_t)b, from + 2 * (size_t)b, 2 * sizeof(cm_plan));
+        handed = true;
+    }
+    ~EarlyPlans() {
+        for (int b = 0; b < bt.B && handed && !ended_well; ++b)
+            memcpy(per_policy + 3 * (size_t)b, &bt.replaced[2 * (size_t)b], 2 * sizeof(cm_plan));
+    }
+};
 
-// The first part of parted plans to the caller (2576 scenarios: 1.2 of 2.4 MB, which the host would otherwise wait for
-// and copy when the search is done).
-void hand_out_fixed(Batch &bt, cm_plan *per_policy) {
-    const cm_plan *from = bt.plans_host.p + 2 * (size_t)bt.B;
-    for (int b = 0; b < bt.B; ++b) memcpy(per_policy + 3 * (size_t)b, from + 2 * (size_t)b, 2 * sizeof(cm_plan));
-    bt.handed = true;
-}
+cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single = nullptr, EarlyPlans *early = nullptr);
 
 // After a bounded search whose lists were full (bounds left hundreds of thousands of plans): again, every plan.
 // Where that finds no room for its tables, the batch is left as it was, to be searched again.
-cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *single) {
+cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *single, EarlyPlans *early = nullptr) {
     if (single && single->exec) { cudaGraphExecDestroy(single->exec); single->exec = nullptr; }
     ++ctx->stats[23];
     const bool direct = bt.direct, one_shot = bt.one_shot;
@@ -1627,7 +1641,7 @@ cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *
             cm_ctx::Overflow *o = overflow_of(ctx, bt, true);
             o->left = o->span = longer_span(o->span);
         }
-        return run_batch(ctx, bt, launches, single);
+        return run_batch(ctx, bt, launches, single, early);
     }
     const std::string why = ctx->err;
     cudaStreamSynchronize(ctx->stream);   // (queued copies read the host image of the tables)
@@ -1643,11 +1657,10 @@ cm_status search_directly(cm_ctx *ctx, Batch &bt, int launches, cm_ctx::Single *
 
 // The search over an uploaded batch; results land in bt.plans_host ([B][4]) after the stream is
 // synchronised.  `single`: a resident one-scenario entry whose sequence may replay as a graph.
-cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single) {
+cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single *single, EarlyPlans *early) {
     cudaStream_t st = ctx->stream;
     int launches = 0, cost_launches = 0;
     if (!bt.plans_host.resize((size_t)bt.B * 4 + 1)) return fail(ctx, CM_ENOMEM, "host memory");
-    bt.handed = false;
     const uint64_t h_enqueue = now_ns();
     bool replay = false;
     if (single && ctx->use_graphs && ctx->graph_stream && !single->graph_failed) {
@@ -1678,9 +1691,10 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
     }
     launches += launches_so_far;
     const uint64_t h_wait = now_ns();
-    if (bt.parted && bt.policy_out) {
+    if (bt.parted && early && early->per_policy) {
+        early->keep();
         CM_CUDA(ctx, cudaEventSynchronize(ctx->pol_join));
-        hand_out_fixed(bt, bt.policy_out);
+        early->hand_out();
     }
     CM_CUDA(ctx, cudaStreamSynchronize(st));
     ctx->stats[14] += h_wait - h_enqueue;
@@ -1697,7 +1711,7 @@ cm_status run_batch(cm_ctx *ctx, Batch &bt, int launches_so_far, cm_ctx::Single 
     }
     ctx->stats[10] += last_bytes(bt) + (bt.parted ? 2 * (size_t)bt.B * sizeof(cm_plan) : 0);
     if (bt.bounded && search_counters(bt)[4]) {
-        return search_directly(ctx, bt, launches, single);
+        return search_directly(ctx, bt, launches, single, early);
     }
     if (search_counters(bt)[6]) {
         cm_status s = finish_tiebreak(ctx, bt, &launches);
@@ -1726,12 +1740,11 @@ void scrub(cm_plan &pl) {
         if (pl.kappa[p] == ~0ull) { pl.kappa[p] = 0; pl.feasible = 0; }
 }
 
-// Plans of a finished search to the caller's arrays (per_policy may be NULL).
-void hand_out(Batch &bt, cm_plan *best, cm_plan *per_policy) {
+// Plans of a finished search to the caller's arrays (per_policy may be NULL; of parted plans its first part is there).
+void hand_out(const Batch &bt, cm_plan *best, cm_plan *per_policy) {
     if (bt.parted) {
         const cm_plan *dyn = bt.plans_host.p, *fixed = bt.plans_host.p + 2 * (size_t)bt.B;
         const uint8_t *choice = reinterpret_cast<const uint8_t *>(search_counters(bt) + kCounters);
-        if (per_policy && !bt.handed) hand_out_fixed(bt, per_policy);
         for (int b = 0; b < bt.B; ++b) {
             if (per_policy) per_policy[3 * (size_t)b + CM_DYNPAR] = dyn[b];
             if (choice[b] == kNoPolicy) memset(&best[b], 0, sizeof(cm_plan));
@@ -1742,6 +1755,16 @@ void hand_out(Batch &bt, cm_plan *best, cm_plan *per_policy) {
     }
     memcpy(best, bt.plans_host.p, sizeof(cm_plan) * bt.B);
     if (per_policy) memcpy(per_policy, bt.plans_host.p + bt.B, sizeof(cm_plan) * 3 * (size_t)bt.B);
+}
+
+// The search over an uploaded batch, its plans to the caller's arrays.
+cm_status run_and_hand_out(cm_ctx *ctx, Batch &bt, int launches, cm_plan *best, cm_plan *per_policy) {
+    EarlyPlans early{bt, per_policy};
+    const cm_status s = run_batch(ctx, bt, launches, nullptr, &early);
+    if (s != CM_OK) return s;
+    early.ended_well = true;
+    hand_out(bt, best, per_policy);
+    return CM_OK;
 }
 
 // Node boundaries among the survivors, ascending (bit j: survivors j and j+1 sit on different nodes), from
@@ -2269,12 +2292,7 @@ cm_status cm_search_batch(cm_ctx *ctx, const uint32_t *failed_ids, const int32_t
         if ((s = build_batch(ctx, bt, failed_ids, offsets, B, *opts, mask)) != CM_OK) { forget_keys(ctx, bt); return s; }
         ctx->stats[13] += now_ns() - h0;
         if ((s = upload_batch(ctx, bt, &launches)) != CM_OK) { forget_keys(ctx, bt); return s; }
-        bt.policy_out = best_per_policy;
-        s = run_batch(ctx, bt, launches);
-        bt.policy_out = nullptr;
-        if (s != CM_OK) return s;
-        hand_out(bt, best_per_scenario, best_per_policy);
-        return CM_OK;
+        return run_and_hand_out(ctx, bt, launches, best_per_scenario, best_per_policy);
     }
     for (int b = 0; b < B; ++b) {
         const auto t0 = std::chrono::steady_clock::now();
@@ -2591,12 +2609,7 @@ cm_status cm_batch_search(cm_ctx *ctx, cm_batch *bp, cm_plan *best_per_scenario,
     memset(ctx->stats, 0, sizeof(ctx->stats));
     Batch &bt = *bp->own;
     if (bt.B == 0) return CM_OK;
-    bt.policy_out = best_per_policy;
-    cm_status s = run_batch(ctx, bt, 0);
-    bt.policy_out = nullptr;
-    if (s != CM_OK) return s;
-    hand_out(bt, best_per_scenario, best_per_policy);
-    return CM_OK;
+    return run_and_hand_out(ctx, bt, 0, best_per_scenario, best_per_policy);
     CM_API_END(ctx)
 }
 

@@ -146,7 +146,7 @@ def _many_sets(share):
 @pytest.mark.parametrize("share", [False, True])
 def test_repeated_search_that_finds_no_room(gpu, oracle_factory, share):
     """A prepared batch whose lists are full and whose second set of tables, for the search of every plan, finds no
-    room: an error, and with room again the same batch can be searched."""
+    room: an error that leaves the caller's arrays alone, and with room again the same batch can be searched."""
     profile, opts, sets = _many_sets(share)
     orc = oracle_factory(profile, opts)
     want = [orc.search(f)[0] for f in sets[:8]]
@@ -157,11 +157,15 @@ def test_repeated_search_that_finds_no_room(gpu, oracle_factory, share):
         gpu.cm_search_batch(ctx, sets[:600], opts)   # (loads the kernels)
         packed = gpu.PackedScenarios(sets)
         batch, _ = packed.prepare(ctx, opts)
+        for array in (packed.best, packed.per_policy):
+            C.memset(array, 0xa5, C.sizeof(array))
         with _Hog(0):
             for _ in range(2):
                 with pytest.raises(gpu.ChameleonError) as e:
                     packed.search_prepared(ctx, batch)
                 assert e.value.status == gpu.CM_ENOMEM
+        for array in (packed.best, packed.per_policy):
+            assert bytes(array) == b"\xa5" * C.sizeof(array)
         packed.search_prepared(ctx, batch)
         assert gpu.cm_last_stats(ctx)["repeated"] == 1
         for plan, w in zip(gpu.plans_from_array(packed.best), want):
