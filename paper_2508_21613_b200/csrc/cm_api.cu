@@ -1470,6 +1470,32 @@ size_t last_bytes(const Batch &bt) {
     return (size_t)bt.B * (bt.parted ? 1 : 4) * sizeof(cm_plan) + tail;
 }
 
+// Work beside the context's stream, on pol_stream: forked from `st` and joined back into it, on the way out of
+// a call that fails as well, so that nothing still runs there when the next call uses the same buffers and events.
+struct Beside {
+    cm_ctx *ctx;
+    cudaStream_t st;
+    bool forked = false, recorded = false;
+    cudaError_t fork() {
+        cudaError_t e = cudaEventRecord(ctx->pol_fork, st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0);
+        forked = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t record() {   // the last of it is enqueued
+        recorded = true;
+        return cudaEventRecord(ctx->pol_join, ctx->pol_stream);
+    }
+    cudaError_t join() {
+        cudaError_t e = cudaSuccess;
+        if (forked && !recorded) e = record();
+        if (forked && e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->pol_join, 0);
+        forked = false;
+        return e;
+    }
+    ~Beside() { join(); }
+};
+
 // Enqueue the launch sequence of a search on `st`: clear, the two one-plan policies, search
 // pass, split reduction, tie-break pass, finalize, plans back to the host.  phase_events: record
 // the events between the phases (not while the sequence is being captured into a graph).
@@ -1491,11 +1517,9 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     const bool policies = (bt.policy_mask & ((1u << CM_REROUTE) | (1u << CM_REDUNDANT))) != 0;
     const bool beside = policies && (bt.policy_mask & (1u << CM_DYNPAR)) && ctx->pol_stream;
     bt.parted = beside && !bt.direct;
+    Beside side{ctx, st};
     if (policies) {
-        if (beside) {
-            CM_CUDA(ctx, cudaEventRecord(ctx->pol_fork, st));
-            CM_CUDA(ctx, cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0));
-        }
+        if (beside) CM_CUDA(ctx, side.fork());
         CM_CUDA(ctx, launch_policies(tb, bd, ctx->hp.n_dp, beside ? ctx->pol_stream : st));
         if (bt.parted) {   // their plans go home while the search runs
             CM_CUDA(ctx, launch_finalize(tb, bd, kFinalFixed, ctx->pol_stream));
@@ -1503,7 +1527,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
                                          cudaMemcpyDeviceToHost, ctx->pol_stream));
             ++launches;
         }
-        if (beside) CM_CUDA(ctx, cudaEventRecord(ctx->pol_join, ctx->pol_stream));
+        if (beside) CM_CUDA(ctx, side.record());
         ++launches;
     }
     if (bt.policy_mask & (1u << CM_DYNPAR)) {
@@ -1529,7 +1553,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
         }
         if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[5], st));
     }
-    if (beside) CM_CUDA(ctx, cudaStreamWaitEvent(st, ctx->pol_join, 0));
+    CM_CUDA(ctx, side.join());
     CM_CUDA(ctx, launch_finalize(tb, bd, bt.parted ? kFinalDyn : kFinalAll, st));
     ++launches;
     if (phase_events) CM_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
@@ -2211,20 +2235,15 @@ cm_status cm_select(cm_ctx *ctx, cm_space *const *spaces, int32_t n_spaces, cm_p
     const bool beside = n_dyn && n_dyn < n_spaces && ctx->pol_stream;
     const uint64_t h_enqueue = now_ns();
     CM_CUDA(ctx, cudaEventRecord(ctx->ev[0], st));
-    if (beside) {
-        CM_CUDA(ctx, cudaEventRecord(ctx->pol_fork, st));
-        CM_CUDA(ctx, cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0));
-    }
+    Beside side{ctx, st};
+    if (beside) CM_CUDA(ctx, side.fork());
     cm_status s = CM_OK;
     for (int i = 0; i < n_spaces && n_dyn == 1 && s == CM_OK; ++i)   // first what takes longest
         if (spaces[i]->policy == CM_DYNPAR) s = enqueue_search(ctx, *spaces[i]->own, st, true, &launches, &cost_launches);
     for (int i = 0; i < n_spaces && s == CM_OK; ++i)
         if (spaces[i]->policy != CM_DYNPAR) s = enqueue_search(ctx, *spaces[i]->own, beside ? ctx->pol_stream : st, false, &launches, &cost_launches);
-    if (beside) {   // joined even after a failure, so that no side stream runs ahead unobserved
-        const cudaError_t e1 = cudaEventRecord(ctx->pol_join, ctx->pol_stream), e2 = cudaStreamWaitEvent(st, ctx->pol_join, 0);
-        if (s == CM_OK) { CM_CUDA(ctx, e1); CM_CUDA(ctx, e2); }
-    }
     if (s != CM_OK) return s;
+    CM_CUDA(ctx, side.join());
     CM_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
     const uint64_t h_wait = now_ns();
     CM_CUDA(ctx, cudaStreamSynchronize(st));
@@ -2393,20 +2412,15 @@ cm_status cm_search_objective(cm_ctx *ctx, const uint32_t *failed_ids, const int
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[2], st));
     // (a matching is a chain in one warp, a plan's rounds are chains in eight: neither fills the GPU, neither needs the other)
     const bool beside = q.sync_rounds && ctx->pol_stream;
-    if (beside) {
-        CM_CUDA(ctx, cudaEventRecord(ctx->pol_fork, st));
-        CM_CUDA(ctx, cudaStreamWaitEvent(ctx->pol_stream, ctx->pol_fork, 0));
-    }
+    Beside side{ctx, st};
+    if (beside) CM_CUDA(ctx, side.fork());
     CM_CUDA(ctx, launch_plan_matching(tb, bd, od, st));
     ++obj_launches;
     if (q.sync_rounds) {
         CM_CUDA(ctx, launch_plan_rounds(tb, bd, od, beside ? ctx->pol_stream : st));
         ++obj_launches;
     }
-    if (beside) {
-        CM_CUDA(ctx, cudaEventRecord(ctx->pol_join, ctx->pol_stream));
-        CM_CUDA(ctx, cudaStreamWaitEvent(st, ctx->pol_join, 0));
-    }
+    CM_CUDA(ctx, side.join());
     CM_CUDA(ctx, cudaEventRecord(ctx->ev_obj[3], st));
     CM_CUDA(ctx, launch_objective(tb, bd, od, st));
     ++obj_launches;
