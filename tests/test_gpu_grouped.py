@@ -93,3 +93,39 @@ def test_plans_of_a_batch_come_in_two_parts(gpu, mode):
         assert any(feasible) and not all(feasible)
     finally:
         gpu.cm_destroy(ctx)
+
+
+def _pairs(n, dp_hi, lo, hi, G):
+    """(stages, micro-batches) that occur among the strategies of n survivors: a group of the work layout each."""
+    def parts(n, dp, least):
+        if dp == 1:
+            return [(n,)] if least <= n <= hi else []
+        return [(s, *rest) for s in range(least, hi + 1) for rest in parts(n - s, dp - 1, s)]
+    found = set()
+    for t in (t for dp in range(1, dp_hi + 1) for t in parts(n, dp, lo)):
+        m = [G * s // n for s in t]
+        found |= {(s, b + k) for s, b in zip(t, m) for k in ((0, 1) if sum(m) < G else (0,))}
+    return found
+
+
+@pytest.mark.parametrize("failures,many", [(2, False), (12, True)])
+def test_layouts_of_few_and_of_many_groups(gpu, oracle_factory, failures, many):
+    """A block finds its group of segments by a thread per group, or by halving where there are more groups."""
+    profile = _job(40, 20, 48, per_node=4)
+    opts = W.SearchOptions(1, 2, 14, 26, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15)
+    sets = [list(range(0, 3 * k, 3)) for k in range(1, failures + 1)]
+    groups = sum(len(_pairs(40 - k, 2, 14, 26, 96)) for k in range(1, failures + 1))
+    assert (groups > 128) == many
+    orc = oracle_factory(profile, opts)
+    wants = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets * 60, opts)[0])
+        st = gpu.cm_last_stats(ctx)
+        assert 0 < st["plans_run"] < st["plans_simulated"]
+        for b, plan in enumerate(best):
+            want = wants[b % failures]
+            assert plan.key() == want.key() and plan.cost == want.cost, (sets[b % failures], plan, want)
+    finally:
+        gpu.cm_destroy(ctx)
