@@ -112,6 +112,10 @@ __global__ void __launch_bounds__(kTieThreads) cm_tiebreak_kernel(Tables tb, Bat
 // one: three to a warp wait for the one that needs most attempts (1024 sets of the 256-device job 240 us, 160 above).
 // ----------------------------------------------------------------------------------
 constexpr int kTieWarps = 2, kTieMost = 8;
+// Pipelines from which they share: below, the GPU has room for a warp each, and eight in sequence are the longer chain.
+// Batches of the 32-device job, shared and a warp each: 60 sets (300 pipelines) 41 and 18 us, 400 sets 43 and 20, 700 sets 45
+// and 33, 1200 sets (6000) 49 and 47, 2500 sets 57 and 90; of the 8-device job, 700 sets (4900) 27 and 23, 1200 sets 29 and 31.
+constexpr uint64_t kTieBatchMin = 148 * 44;
 constexpr uint32_t kTieTiles = 64;   // of kTile candidates
 
 template <typename T>
@@ -312,8 +316,8 @@ cudaError_t launch_tiebreak(const Tables &t, const BatchDev &b, uint64_t stages,
     // that its bound leaves nearly always is it.  1024 sets of the 256-device job: 133 us with a warp, 172 us with
     // two, where a plan-per-lane kernel per depth took 1300 us in all.
     const bool wide = nx <= 148 * 2;
-    // Several pipelines to a warp where they have few tiles each (a long walk would hold up the others).
-    if (!wide && t.sched != CM_SCHED_GPIPE && b.max_tiles_per_seg <= kTieTiles && !(stages >> kRegStagesMax)) {
+    // Several pipelines to a warp where there are many, of few tiles each (a long walk would hold up the others).
+    if (nx >= kTieBatchMin && t.sched != CM_SCHED_GPIPE && b.max_tiles_per_seg <= kTieTiles && !(stages >> kRegStagesMax)) {
         const unsigned ctas = (unsigned)((nx + kTieMost * kTieWarps - 1) / (kTieMost * kTieWarps));
         return native_i64(b) ? launch_next(cm_tie_batch_kernel<long long>, ctas, kTieWarps * 32, 0, st, t, b, (uint32_t)nx)
                              : launch_next(cm_tie_batch_kernel<double>, ctas, kTieWarps * 32, 0, st, t, b, (uint32_t)nx);

@@ -54,6 +54,27 @@ def test_batches_of_pipelines_that_share_warps(gpu, oracle_factory, name, mode, 
         gpu.cm_destroy(ctx)
 
 
+@pytest.mark.parametrize("mode,native", [(0, False), (1, False), (1, True)])
+@pytest.mark.parametrize("n", [3255, 3256, 5000])
+def test_tie_break_on_either_side_of_sharing_a_warp(gpu, oracle_factory, n, mode, native):
+    """Two shallow pipelines a set: a warp each up to 6511 of them, eight to a warp from 6512 on."""
+    profile = _job(36, 16, 24)
+    opts = W.SearchOptions(2, 2, 13, 16, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 14, mode)
+    sets = [[3], [0, 17], [5, 6, 16], [2, 9, 18, 30]]
+    orc = oracle_factory(profile, opts)
+    wants = [orc.search_policy(f, W.POLICY_DYNPAR) for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_set_int64_arithmetic(ctx, native)
+        _, pol, _ = gpu.cm_search_batch(ctx, [sets[b % 4] for b in range(n)], opts, per_policy=True)
+        for b, plan in enumerate(gpu.plans_from_array(pol)[W.POLICY_DYNPAR::3]):
+            want = wants[b % 4]
+            assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (sets[b % 4], plan, want)
+    finally:
+        gpu.cm_destroy(ctx)
+
+
 @pytest.mark.parametrize("per_node", [3, 8])
 def test_bounds_where_links_inside_nodes_are_the_dearer(gpu, oracle_factory, per_node):
     profile = _job(36, 16, 24, per_node=per_node, intra=15, inter=200)
