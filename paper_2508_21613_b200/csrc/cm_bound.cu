@@ -54,6 +54,13 @@ __device__ __forceinline__ unsigned long long least_bound(const float4 *comp, co
     return ((unsigned long long)__float_as_uint(least) << 32) | (uint32_t)at;
 }
 
+// Segments up to which, where one of them crosses more dear boundaries than are kept in a list, the lanes keep a composition
+// each and go through the segments, with a reduction per segment: a lane per segment leaves most lanes idle there and goes
+// through 32 compositions in a long chain (one failure of the 64-device job, a device per node and up to 47 dear
+// boundaries: 198 us a call with a lane per segment, 161 up to 8 segments, 149 up to 32).  A short chain takes the same either
+// way (256-device job, 4 dear boundaries: 139 and 139, 12 sets of it 268 with a lane per segment, 275 up to 32).
+constexpr int kFewSegs = 32;
+
 template <typename T, bool UNI_X>
 __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, BatchDev bd, BoundDev bo) {
     __shared__ SProf<T> sp;
@@ -61,10 +68,13 @@ __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, Batc
     __shared__ float4 comp[kBoundThreads];
     __shared__ SegLite segs[kBoundSegs];
     __shared__ unsigned long long word[kBoundThreads / 32][kBoundSegs];
+    __shared__ SegHot few[kFewSegs];
+    __shared__ bool long_chain;   // a segment crosses more dear boundaries than a list holds (looked at where it matters)
     extern __shared__ __align__(16) unsigned char terms[];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     find_bucket(bo, blockIdx.x, &bks);
     stage_profile(sp, tb);
+    if (tid == 0) long_chain = false;
     __syncthreads();
     const BBucket &bk = bks;
     const BoundJob job = bound_job(bk, blockIdx.x);
@@ -77,6 +87,7 @@ __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, Batc
         if ((int)tid >= n_seg) return;
         const BoundSeg g = bound_segment(bd, bk, base + tid);
         segs[tid] = seg_lite(g.tier, g.row, g.n_sync, sp.bw_sync);
+        if (n_seg <= kFewSegs && __popcll(dear_bits(g.tier, dear, S)) > kDearMax) long_chain = true;   // (nothing else is written)
         if (job.tile == 0) bo.rec[bk.seg_first + base + tid] = seg_record(g);
     };
     LaneBound v;
@@ -107,7 +118,17 @@ __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, Batc
             take_segments(base, n_seg);
             __syncthreads();
         }
-        for (int g = warp / parts * 32; g < n_seg; g += 128 / parts) {
+        const bool comp_lanes = n_seg <= kFewSegs && long_chain;   // uniform
+        if (comp_lanes) {
+            if ((int)tid < n_seg) few[tid] = seg_hot<UNI_X>(segs[tid], S, dear, delta, gpipe);
+            __syncthreads();
+            for (int s = 0; s < n_seg && (int)warp < parts; ++s) {
+                const uint32_t value = __float_as_uint(bound_value_of<UNI_X>(v, terms + tid * kTermSize<UNI_X>, few[s], delta));
+                const uint32_t least = __reduce_min_sync(0xffffffffu, value), who = __ballot_sync(0xffffffffu, value == least);
+                if (lane == 0) word[warp][s] = ((unsigned long long)least << 32) | (32 * warp + __ffs((int)who) - 1);
+            }
+        }
+        for (int g = warp / parts * 32; g < n_seg && !comp_lanes; g += 128 / parts) {
             const SegHot h = seg_hot<UNI_X>(segs[min(g + (int)lane, n_seg - 1)], S, dear, delta, gpipe);
             unsigned long long key;
 #define CM_NF(N) case N: key = least_bound<UNI_X, N>(comp, terms, h, delta, c0, c1); break;

@@ -315,6 +315,13 @@ __device__ __forceinline__ float bound_value(float v_best, float v_u0, float v_g
     }
     return fmaxf(__fmaf_rd(v_g, h.coef, __fadd_rd(__fadd_rd(v_u0, extra), best)), 0.0f);
 }
+// The same for a composition per lane and one segment for all of them.
+template <bool UNI_X>
+__device__ __forceinline__ float bound_value_of(const LaneBound &v, const unsigned char *term_col, const SegHot &h, float delta) {
+    return h.n <= 2 ? bound_value<UNI_X, 2>(v.best, v.u0, v.g, term_col, h, delta)
+         : h.n <= kDearMax ? bound_value<UNI_X, kDearMax>(v.best, v.u0, v.g, term_col, h, delta)
+                           : bound_value<UNI_X, -1>(v.best, v.u0, v.g, term_col, h, delta);
+}
 // slack: 1 where the synchronisation quotient floors
 __device__ __forceinline__ float bound_of(float value, float slack) {
     return fmaxf(__fmul_rd(__fsub_rd(value, slack), kFloatSlack), 0.0f);

@@ -172,11 +172,7 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
         for (int s = s0; s < n_act && s < s0 + kRefineSegs; ++s) {
             bool take = false;
             if (v.ok) {
-                const SegHot &h = sm.hot[s];
-                const float value = h.n <= 2 ? bound_value<UNI_X, 2>(v.best, v.u0, v.g, term_col, h, delta)
-                                  : h.n <= kDearMax ? bound_value<UNI_X, kDearMax>(v.best, v.u0, v.g, term_col, h, delta)
-                                                    : bound_value<UNI_X, -1>(v.best, v.u0, v.g, term_col, h, delta);
-                const float lb = bound_of(value, slack);
+                const float lb = bound_of(bound_value_of<UNI_X>(v, term_col, sm.hot[s], delta), slack);
                 take = lb <= sm.open[s].lim && lb > sm.open[s].ev;
             }
             const uint32_t who = __ballot_sync(0xffffffffu, take);

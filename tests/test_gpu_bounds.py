@@ -388,3 +388,34 @@ def test_bounds_of_pipelines_over_many_nodes(gpu, oracle_factory, per_node, mode
             assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (sets[b % 3], plan, want)
     finally:
         gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode,native", [(0, False), (1, False), (1, True)])
+@pytest.mark.parametrize("per_node,layered", [(1, False), (1, True), (8, False), (8, True)])
+def test_bounds_of_few_segments(gpu, oracle_factory, per_node, layered, mode, native):
+    """Four to 33 segments to a block, over two or three dear boundaries and over sixteen and more: up to 32 segments
+    over more than six boundaries the lanes take a composition each, else a segment each.  Groups of one, 22 and thousands of
+    compositions."""
+    rng = np.random.default_rng(83)
+    L = 45
+    fwd = rng.uniform(2.5e6, 3.5e6, L).round()
+    p2p = 8_000_000 if not layered else rng.integers(4_000_000, 12_000_000, L)
+    profile = W.make_profile_ns(L, 2, 20, 96, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, p2p,
+                                [round(i * L / 20) for i in range(21)], 80_000_000_000, per_node, 300, 20)
+    opts = W.SearchOptions(2, 2, 17, 22, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 16000, mode)
+    sets = [[3], [20]]
+    orc = oracle_factory(profile, opts)
+    wants = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        gpu.cm_set_int64_arithmetic(ctx, native)
+        for n in (4, 7, 8, 9, 32, 33):
+            best = gpu.plans_from_array(gpu.cm_search_batch(ctx, [sets[b % 2] for b in range(n)], opts)[0])
+            st = gpu.cm_last_stats(ctx)
+            assert 0 < st["plans_run"] < st["plans_simulated"]
+            for b, plan in enumerate(best):
+                want = wants[b % 2]
+                assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (n, sets[b % 2], plan, want)
+    finally:
+        gpu.cm_destroy(ctx)
