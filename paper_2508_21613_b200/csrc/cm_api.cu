@@ -1496,6 +1496,11 @@ struct Beside {
     ~Beside() { join(); }
 };
 
+// Scenarios from which plans go home in two parts: a launch, a copy and an event more for the host, which cost more than they
+// save below (32-device job, whole and in parts: 8 sets 183 and 191 us, 120 sets 219 either way, 250 sets 248 and 243, 2500
+// sets 661 and 567; 256-device job 8 sets 255 and 258, 120 sets 351 and 354, 250 sets 497 and 490).
+constexpr int kPartedMin = 192;
+
 // Enqueue the launch sequence of a search on `st`: clear, the two one-plan policies, search
 // pass, split reduction, tie-break pass, finalize, plans back to the host.  phase_events: record
 // the events between the phases (not while the sequence is being captured into a graph).
@@ -1516,7 +1521,7 @@ cm_status enqueue_search(cm_ctx *ctx, Batch &bt, cudaStream_t st, bool phase_eve
     }
     const bool policies = (bt.policy_mask & ((1u << CM_REROUTE) | (1u << CM_REDUNDANT))) != 0;
     const bool beside = policies && (bt.policy_mask & (1u << CM_DYNPAR)) && ctx->pol_stream;
-    bt.parted = beside && !bt.direct;
+    bt.parted = beside && !bt.direct && bt.B >= kPartedMin;
     Beside side{ctx, st};
     if (policies) {
         if (beside) CM_CUDA(ctx, side.fork());

@@ -95,12 +95,13 @@ def test_bounds_where_links_inside_nodes_are_the_dearer(gpu, oracle_factory, per
 
 
 @pytest.mark.parametrize("mode", [0, 1])
-def test_plans_of_a_batch_come_in_two_parts(gpu, mode):
-    """Sets that every policy survives, that rerouting does not (a stage lost in every pipeline), and that nothing
+@pytest.mark.parametrize("n", [54, 191, 192, 401])
+def test_plans_of_a_batch_come_in_two_parts(gpu, n, mode):
+    """From 192 on.  Sets that every policy survives, that rerouting does not (a stage lost in every pipeline), and that nothing
     does (no strategy for the survivors): the same plans as one failure at a time, with and without those per policy."""
     profile = _job(12, 4, 8, per_node=4)
     opts = W.SearchOptions(2, 2, 3, 4, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15, mode)
-    sets = [[1], [1, 5], [0, 4], [0, 4, 1], [], [7]] * 9
+    sets = ([[1], [1, 5], [0, 4], [0, 4, 1], [], [7]] * 67)[:n]
     ctx = gpu.cm_create(0)
     try:
         gpu.cm_load_profile(ctx, profile)
