@@ -369,7 +369,9 @@ cudaError_t launch_gather(const Tables &t, const BatchDev &b, const BoundDev &bo
 // ----------------------------------------------------------------------------------
 // The recurrence on the listed plans.  Pipelines of at most 16 stages: a thread per plan, state in
 // registers; deeper ones in lock step, 2(S+m) slots (a thread would need ~100 us for its chain of 2 S m cells): a
-// warp per plan where the warps are enough for the list, three plans per warp (two beyond 40 stages) where not.
+// warp per plan up to two and a half plans for each of its 2960 warps, three plans per warp (two beyond 40 stages) beyond:
+// few groups of three leave most warps idle (passes of the 256-device job, a plan and three per warp: 140 sets, 3058 plans, 204
+// and 244 us, 260 sets, 5625 plans, 286 and 310, 350 sets, 7509 plans, 348 and 349, 1000 sets, 21375 plans, 792 and 759).
 // ----------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t list_length(const BoundDev &bo, int list) {
     const uint32_t n = bo.count[list] + 1u, room = bo.list_first[list + 1] - bo.list_first[list];
@@ -427,7 +429,7 @@ __global__ void __launch_bounds__(kChunk, 5) cm_list_deep_kernel(Tables tb, Batc
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t n_warps = gridDim.x * (kChunk / 32), first = blockIdx.x * (kChunk / 32) + warp;
     unsigned long long work = 0;
-    if (n <= n_warps || sp.sched == CM_SCHED_GPIPE) {
+    if (2ull * n <= 5ull * n_warps || sp.sched == CM_SCHED_GPIPE) {
         for (uint32_t i = first; i < n; i += n_warps) {
             const uint4 e = entries[i];
             const SegView g = seg_view(bd, e.x, e.y);

@@ -27,16 +27,18 @@ def _job(L, pp, micro, seed=5, per_node=8, intra=300, inter=20):
                              80_000_000_000, per_node, intra, inter)
 
 
-# depths on either side of 16 and 40 stages, where the pipelines that share a warp go from eight to three to two;
-# odd and even ones side by side; fewer micro-batches than stages as well
-DEPTHS = {"15-18": (36, 16, 24, (2, 2, 15, 18)), "39-42": (84, 41, 48, (2, 2, 39, 42)), "few-micro-batches": (40, 18, 12, (2, 2, 16, 20))}
+# depths on either side of 16 and 40 stages, where the pipelines that share a warp go from eight to three to two; odd and
+# even ones side by side; fewer micro-batches than stages as well.  The last number: plans listed at least, in two lists; they
+# begin to share warps beyond 7400 to a list
+DEPTHS = {"15-16": (36, 16, 24, (2, 2, 15, 16), 0), "17-22": (44, 20, 48, (2, 2, 17, 22), 14801), "39-42": (84, 41, 48, (2, 2, 39, 42), 14801),
+          "few-micro-batches": (40, 18, 12, (2, 2, 16, 20), 14801)}
 
 
 @pytest.mark.parametrize("mode,native", [(0, False), (1, False), (1, True)])
 @pytest.mark.parametrize("name", sorted(DEPTHS))
 def test_batches_of_pipelines_that_share_warps(gpu, oracle_factory, name, mode, native):
-    """800 failure sets: more listed plans than warps, and more pipelines to complete."""
-    L, pp, micro, window = DEPTHS[name]
+    """5000 failure sets: more listed plans than warps, and more pipelines to complete."""
+    L, pp, micro, window, listed = DEPTHS[name]
     profile = _job(L, pp, micro)
     opts = W.SearchOptions(*window, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 4000, mode)
     sets = [[3], [0, pp + 1], [5, 6, pp]]
@@ -46,7 +48,10 @@ def test_batches_of_pipelines_that_share_warps(gpu, oracle_factory, name, mode, 
     try:
         gpu.cm_load_profile(ctx, profile)
         gpu.cm_set_int64_arithmetic(ctx, native)
-        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, [sets[b % 3] for b in range(800)], opts)[0])
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, [sets[b % 3] for b in range(5000)], opts)[0])
+        st = gpu.cm_last_stats(ctx)
+        if listed:
+            assert listed <= st["plans_run"] < st["plans_simulated"]
         for b, plan in enumerate(best):
             want = wants[b % 3]
             assert plan.key() == want.key() and plan.cost == want.cost and plan.cost_ns == want.cost_ns, (sets[b % 3], plan, want)
