@@ -176,3 +176,98 @@ def test_repeated_search_that_finds_no_room(gpu, oracle_factory, share):
         gpu.cm_batch_free(batch)
     finally:
         gpu.cm_destroy(ctx)
+
+
+def _one_heavy_layer():
+    """One layer takes nearly all of the time: a pipeline's is its micro-batches times that layer's, so that all
+    strategies whose deepest pipeline is equally deep come out alike."""
+    L, n_dp, n_pp = 14, 9, 7
+    fwd = np.full(L, 1e3)
+    fwd[5] = 5e7
+    return W.make_profile_ns(L, n_dp, n_pp, 61, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 0,
+                             [round(i * L / n_pp) for i in range(n_pp + 1)], 80_000_000_000, 4, 300, 20)
+
+
+def _many_strategies():
+    L, n_dp, n_pp = 32, 5, 8
+    fwd = np.random.default_rng(11).uniform(2.5e6, 3.5e6, L).round()
+    return W.make_profile_ns(L, n_dp, n_pp, 16, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 8_000_000,
+                             [4 * i for i in range(9)], 80_000_000_000, 8, 300, 20)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_more_strategies_within_reach_than_a_list_holds(gpu, oracle_factory, mode):
+    """A scenario's strategies within reach are kept in a list of 14: here 15 and more have the same step time."""
+    profile = _one_heavy_layer()
+    opts = W.SearchOptions(10, 10, 2, 7, W.LAYERS_FULL, W.BATCH_REMAINDER, 1 << 14, mode)   # 61 survivors: 23 strategies
+    sets = [[3, 4], [0, 17]]
+    orc = oracle_factory(profile, opts)
+    obj = W.ObjectiveOptions(topk=16)
+    for f in sets:
+        short = orc.search_objective(f, obj)[1].shortlist
+        assert len({p.strategy for p in short}) > 14 and len({(p.cost, p.cost_ns) for p in short}) == 1
+    want = [orc.search(f)[0] for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        best = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets * 600, opts)[0])
+        st = gpu.cm_last_stats(ctx)
+        assert 0 < st["plans_run"] < st["plans_simulated"]
+        for b, plan in enumerate(best):
+            _same(plan, want[b % 2])
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("topk", [1, 9])
+def test_more_strategies_than_are_kept(gpu, oracle_factory, topk):
+    """Step times from bounds of up to 2048 strategies are kept from the first look to the second."""
+    profile = _many_strategies()
+    opts = W.SearchOptions(4, 7, 2, 24, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 300)
+    sets = [[3], [0, 17]]
+    orc = oracle_factory(profile, opts)
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        if topk == 1:
+            got = gpu.plans_from_array(gpu.cm_search_batch(ctx, sets * 300, opts)[0])
+            want = [orc.search(f)[0] for f in sets]
+        else:
+            obj = W.ObjectiveOptions(topk=topk)
+            got = gpu.plans_from_array(gpu.cm_search_objective(ctx, sets * 300, opts, obj, shortlist=True)[2])
+            want = [p for f in sets for p in orc.search_objective(f, obj)[1].shortlist]
+            assert len(want) == 2 * topk
+        st = gpu.cm_last_stats(ctx)
+        assert 0 < st["plans_run"] < st["plans_simulated"] and st["strategies"] > 2 * 2048   # (of two survivor counts)
+        for b, plan in enumerate(got):
+            _same(plan, want[b % len(want)])
+    finally:
+        gpu.cm_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("deep", [False, True])
+def test_shortlists_over_slow_links(gpu, oracle_factory, deep, mode):
+    """Results that come out later than their bounds: the strategies within reach of the bounds then hold too few step
+    times for the shortlist, and all of them are looked at again."""
+    profile, opts = _slow_links(deep, 8_000_000 if deep else 16_777_216, 3)
+    opts = opts.with_cost_mode(mode)
+    sets = [[3], [0, 9]]
+    orc = oracle_factory(profile, opts)
+    obj = W.ObjectiveOptions(topk=16)
+    want = [orc.search_objective(f, obj) for f in sets]
+    ctx = gpu.cm_create(0)
+    try:
+        gpu.cm_load_profile(ctx, profile)
+        best, _, short, moved, _ = gpu.cm_search_objective(ctx, sets * (10 if deep else 60), opts, obj, shortlist=True)
+        st = gpu.cm_last_stats(ctx)
+        assert 0 < st["plans_run"] < st["plans_simulated"]
+        best, short = gpu.plans_from_array(best), gpu.plans_from_array(short)
+        for b, plan in enumerate(best):
+            _same(plan, want[b % 2][0])
+            got = [short[16 * b + r] for r in range(16) if moved[b, r] >= 0]
+            assert len(got) == len(want[b % 2][1].shortlist)
+            for p, w in zip(got, want[b % 2][1].shortlist):
+                _same(p, w)
+    finally:
+        gpu.cm_destroy(ctx)

@@ -19,11 +19,12 @@ def gpu():
     return binding
 
 
-def _job(L, pp, micro, seed=5, per_node=8, intra=300, inter=20):
+def _job(L, pp, micro, seed=5, per_node=8, intra=300, inter=20, layered=False):
     rng = np.random.default_rng(seed)
     fwd = rng.uniform(2.5e6, 3.5e6, L).round()
+    p2p = rng.integers(4_000_000, 12_000_000, L) if layered else 8_000_000
     cuts = [round(i * L / pp) for i in range(pp + 1)]
-    return W.make_profile_ns(L, 2, pp, micro, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, 8_000_000, cuts,
+    return W.make_profile_ns(L, 2, pp, micro, fwd, 2.0 * fwd, 1_000_000, 50_000_000, 300_000_000, p2p, cuts,
                              80_000_000_000, per_node, intra, inter)
 
 
@@ -80,9 +81,10 @@ def test_tie_break_on_either_side_of_sharing_a_warp(gpu, oracle_factory, n, mode
         gpu.cm_destroy(ctx)
 
 
+@pytest.mark.parametrize("layered", [False, True])
 @pytest.mark.parametrize("per_node", [3, 8])
-def test_bounds_where_links_inside_nodes_are_the_dearer(gpu, oracle_factory, per_node):
-    profile = _job(36, 16, 24, per_node=per_node, intra=15, inter=200)
+def test_bounds_where_links_inside_nodes_are_the_dearer(gpu, oracle_factory, per_node, layered):
+    profile = _job(36, 16, 24, per_node=per_node, intra=15, inter=200, layered=layered)
     opts = W.SearchOptions(2, 2, 13, 18, W.LAYERS_REMAINDER, W.BATCH_REMAINDER, 1 << 15)
     sets = [[3], [0, 17]]
     orc = oracle_factory(profile, opts)
