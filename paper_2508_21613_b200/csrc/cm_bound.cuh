@@ -42,7 +42,8 @@ namespace cm {
 constexpr double kBoundSlack = 1.0 - 1.0 / (1ull << 36);
 
 // A list of the bounded search pass was full: the host repeats the search without bounds, and what is left of
-// this one need not run.
+// this one need not run.  Threads of a CTA may each look only in kernels beside which none runs that lists plans (all but
+// cm_refine_kernel, whose CTAs list them themselves, and cm_gather_kernel): there all of them see the same.
 __device__ __forceinline__ bool lists_full(const BatchDev &bd) { return *(volatile unsigned long long *)(bd.counters + 4) == 0ull; }
 
 // Layer cuts of a plan in a shared-memory column, one byte per stage, a plan per thread:

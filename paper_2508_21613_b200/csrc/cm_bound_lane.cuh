@@ -1,5 +1,5 @@
-// What the kernels of the bounded search pass (cm_bound.cu, cm_refine.cu) share: a layer composition's
-// terms in a lane's registers, the segments of a CTA, the bound of (composition, segment) in floats.
+// What the kernels of the bounded search pass (cm_bound.cu, cm_refine.cu) share: a layer composition's terms, a column
+// of shared memory that its thread sets up, the segments of a CTA, the bound of (composition, segment) in floats.
 #pragma once
 
 #include "cm_bound.cuh"
@@ -7,8 +7,8 @@
 
 namespace cm {
 
-// Bounds of whole buckets are floats rounded down: the per-plan inner loop costs one addition and one
-// maximum per stage at full rate (in double arithmetic an addition and a compare-and-select take six
+// Bounds of whole buckets are floats rounded down: the per-plan inner loop costs one look-up, one addition and one
+// maximum per dear boundary at full rate (in double arithmetic an addition and a compare-and-select take six
 // issue slots).
 constexpr float kFloatSlack = 1.0f - 1.0f / (1 << 22);
 constexpr float kTieWindow = 1.0f / (1 << 18);     // bounds this close to the least one of a segment are compared bit for bit

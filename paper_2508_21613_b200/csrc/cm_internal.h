@@ -241,9 +241,10 @@ struct BoundDev {
     int uniform_x;
 };
 constexpr int kCounters = 8;   // work counters of a search (BatchDev::counters)
-// Recurrence cells of a search (a shallow one counting a quarter) from which bounds pay for their extra
-// launches: 33 sets of the 32-device job with the full objective (just below) 506 us directly, 745 by bounds;
-// one failure of the 256-device job (4e8) 380 us directly, 259 by bounds when they came, 155 now.
+// Recurrence cells of a search (a shallow one counting a quarter) from which it goes by bounds, which take some eight more
+// launches.  The line is from when a bound cost a term per stage, and lies on the safe side now: directly and by bounds, 4
+// sets of the 32-device job take 148 and 161 us, 8 sets 179 and 175, 32 sets (the last below it) 300 and 204; one set of the
+// 64-device job 143 and 156, two 302 and 165; one of the 256-device job (4e8 cells) 433 and 178.
 constexpr uint64_t kBoundMinCells = 200000000ull;
 constexpr uint64_t kTileMinMax = 1ull << 24;     // entries of BoundDev::tile_min, at most (64 MB)
 constexpr uint32_t kBoundListMin = 65536;        // plans a list has room for, at least (if there are as many)

@@ -679,8 +679,8 @@ __device__ __forceinline__ bool warp_plan_cost(const SProf<T> &sp, const Tables 
 
 // Costs of several plans at a time, each on `width` >= (S + 3) / 4 lanes with four stages per lane: half the
 // instructions per plan of warp_plan_cost where there are more plans than warps.  1F1B.  Arguments are those of
-// the lane's plan: `mine`, whether it has one, `gl`, the lane's number within it, `cuts`, kMaxS + 8
-// bytes of its own.  The cost is returned in the plan's first lane; false: no plan, or infeasible.
+// the lane's plan: `mine`, whether it has one, `gl`, the lane's number within it, `cuts`, S + 1
+// bytes of its own (untouched where `mine` is false).  The cost is returned in the plan's first lane; false: no plan, or infeasible.
 template <typename T>
 __device__ __forceinline__ bool group_plan_cost(const SProf<T> &sp, const Tables &tb, int layer_mode, const SegView &g, const Cand &cand, bool mine,
                                                 int gl, int width, uint8_t *cuts, T &cost) {

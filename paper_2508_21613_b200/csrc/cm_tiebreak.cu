@@ -121,11 +121,11 @@ constexpr uint32_t kTieTiles = 64;   // of kTile candidates
 template <typename T>
 __global__ void __launch_bounds__(kTieWarps * 32) cm_tie_batch_kernel(Tables tb, BatchDev bd, uint32_t n_items) {
     __shared__ SProf<T> sp;
-    __shared__ uint8_t cuts_s[kTieWarps][kTieMost][kRegStagesMax + 8];   // (per pipeline)
+    __shared__ uint8_t cuts_s[kTieWarps][kTieMost][kRegStagesMax + 8];   // (per pipeline; none is deeper: launch_tiebreak)
     __shared__ uint8_t cut_col[kTieWarps][kRegStagesMax * 32];
     stage_profile(sp, tb);
     after_previous();
-    if (lists_full(bd)) return;   // uniform
+    if (lists_full(bd)) return;   // uniform: no kernel that may run beside this one writes the flag
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int width = 32 / kTieMost;
