@@ -60,6 +60,15 @@ __device__ __forceinline__ unsigned long long least_bound(const float4 *comp, co
 // boundaries: 198 us a call with a lane per segment, 161 up to 8 segments, 149 up to 32).  A short chain takes the same either
 // way (256-device job, 4 dear boundaries: 139 and 139, 12 sets of it 268 with a lane per segment, 275 up to 32).
 constexpr int kFewSegs = 32;
+template <bool UNI_X>   // (out of line: the kernel's other path is the one that most calls take)
+__device__ __noinline__ void least_of_lanes(const LaneBound &v, const unsigned char *term_col, const SegHot *segs, int n_seg, float delta, unsigned long long *word) {
+    const uint32_t lane = threadIdx.x & 31;
+    for (int s = 0; s < n_seg; ++s) {
+        const uint32_t value = __float_as_uint(bound_value_of<UNI_X>(v, term_col, segs[s], delta));
+        const uint32_t least = __reduce_min_sync(0xffffffffu, value), who = __ballot_sync(0xffffffffu, value == least);
+        if (lane == 0) word[s] = ((unsigned long long)least << 32) | (threadIdx.x + __ffs((int)who) - 1);
+    }
+}
 
 template <typename T, bool UNI_X>
 __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, BatchDev bd, BoundDev bo) {
@@ -122,11 +131,7 @@ __global__ void __launch_bounds__(kBoundThreads) cm_bound_kernel(Tables tb, Batc
         if (comp_lanes) {
             if ((int)tid < n_seg) few[tid] = seg_hot<UNI_X>(segs[tid], S, dear, delta, gpipe);
             __syncthreads();
-            for (int s = 0; s < n_seg && (int)warp < parts; ++s) {
-                const uint32_t value = __float_as_uint(bound_value_of<UNI_X>(v, terms + tid * kTermSize<UNI_X>, few[s], delta));
-                const uint32_t least = __reduce_min_sync(0xffffffffu, value), who = __ballot_sync(0xffffffffu, value == least);
-                if (lane == 0) word[warp][s] = ((unsigned long long)least << 32) | (32 * warp + __ffs((int)who) - 1);
-            }
+            if ((int)warp < parts) least_of_lanes<UNI_X>(v, terms + tid * kTermSize<UNI_X>, few, n_seg, delta, word[warp]);
         }
         for (int g = warp / parts * 32; g < n_seg && !comp_lanes; g += 128 / parts) {
             const SegHot h = seg_hot<UNI_X>(segs[min(g + (int)lane, n_seg - 1)], S, dear, delta, gpipe);

@@ -60,6 +60,7 @@ struct RefineSmem {
     RefineSeg open[kBoundSegs];
     unsigned long long word[kBoundSegs];   // phase 1: least walk cost
     int n_queue;
+    bool full;                             // the lists, when the segments were looked at
     uint16_t queue[kRefineSegs * kBoundThreads];   // plans to walk: segment << 7 | thread whose composition it is
 };
 
@@ -129,12 +130,11 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
     const uint32_t per_cta = bo.parts * (kBoundSegs / size), cta = item / per_cta, part = item - cta * per_cta;
     find_bucket(bo, cta, &bks);
     if (ahead) stage_profile(sp, tb);
-    else after_previous();
-    if (tid == 0) n_open = phase == 2 && lists_full(bd) ? -1 : 0;
+    if (tid == 0) n_open = 0;
     __syncthreads();
-    if (n_open < 0) return;   // uniform (it only grows from 0)
     const BBucket &bk = bks;
     const RefineJob job = refine_job(bk, cta, part, size);
+    if (!ahead) after_previous();
     const int S = bk.S, W = bk.width, dear = dear_tier(tb);
     unsigned char *term_col = dyn + tid * kTermSize<UNI_X>;
     uint8_t *cuts = dyn + bo.dyn_cuts;
@@ -146,6 +146,7 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
         v = lane_of<T, UNI_X, true>(sp, tb, bd, bk, any, cand, dear, term_col, cuts + tid);
         after_previous();
     }
+    const bool full = tid == 0 && phase == 2 && lists_full(bd);   // (on its way with the segments)
     SegRec g;
     RefineSeg rs;
     if (thread_open<T>(bd, bo, bk, job, phase, g, rs)) {
@@ -154,9 +155,10 @@ __device__ __forceinline__ void refine_part(const Tables &tb, const BatchDev &bd
         sm.open[at] = rs;
         sm.word[at] = ~0ull;
     }
+    if (tid == 0) sm.full = full;
     __syncthreads();
     const int n_act = n_open;
-    if (n_act == 0) return;   // uniform
+    if (n_act == 0 || sm.full) return;   // uniform
     if (!ahead) {
         stage_profile(sp, tb);
         __syncthreads();
