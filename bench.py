@@ -53,8 +53,8 @@ KERNEL_PROFILES = {
 }
 # Large batches decide most plans by a lower bound (cm_bound_kernel) and run the recurrence on the few it
 # leaves: there the unit of work is one plan bounded, with I_plan thread-instructions.
-BOUND_PROFILE = {"i_plan": 87.0, "issue_active": 0.540, "dram_bytes_per_plan": 1044736 / 7.289e6,
-                 "profile": "profiles/cm_bound_kernel_256dev-64.md"}
+BOUND_PROFILE = {"i_plan": 43.1, "issue_active": 0.66, "dram_bytes_per_plan": 2773504 / 73.34e6,
+                 "profile": "profiles/cm_bound_kernel_256dev-1024.md"}
 KERNEL_NAMES = {"regs": "cm_cost_regs_kernel", "regs_pair": "cm_cost_regs_pair_kernel", "wide": "cm_cost_wide_kernel",
                 "pair": "cm_cost_pair_kernel"}
 FP64_INSTR_PER_CELL = 3.0          # 2 DADD + 1 DSETP; an FP64 warp instruction occupies its pipe for 2 cycles
